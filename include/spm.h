@@ -331,10 +331,10 @@ spm_status spm_scene_phase_ms(spm_scene *scene, float *vertex_ms, float *cull_ms
  *   from geometry alone (every generator's visible tiles, no shadow cone) on
  *   the scene's own side stream, concurrently with the vertex phase; the
  *   pixel pass then applies costs and cones.
- * hidden_chunk: first chunk of lb-ordered candidates whose tiles are tested
- *   for being hidden (32..256; later chunks double).
- * tile: pixel tile side, 16 or 32 (default 16 when a pixel spans 8 world
- *   units or more, else 32): each tile is one CTA of the pixel pass.
+ * hidden_chunk: 32..256, checked and reported; the pixel pass takes its
+ *   candidates one by one in order of their lower bounds, so it has no effect.
+ * tile: side of the tiles that carry the candidate lists, 16 or 32 pixels
+ *   (default 16 when a pixel spans 8 world units or more, else 32).
  * maps: 1 = the flood keeps each point generator's angular depth map and the
  *   pixel pass decides most pixels' visibility from it (exact bounds; only
  *   the undecided pixels take the exact polygon test), 0 = every pixel takes
@@ -366,10 +366,9 @@ spm_status spm_scene_get_tuning(const spm_scene *scene, spm_tuning *out);
 spm_status spm_scene_set_tuning(spm_scene *scene, const spm_tuning *tuning);
 
 /* Autotuner: times spm_compute on this scene (device events on `stream`,
- * warm-up then the median of 3 runs) for every flood_mode x hidden_chunk x
- * tile x maps combination in {1, 2, 3} x {32, 256} x {16, 32} x {0, 1} (maps
- * only with a flood), keeps the fastest and
- * writes it to *chosen (may be NULL). Synchronous. Allocates the scene's
+ * warm-up then the median of 3 runs) for every flood_mode x tile x maps
+ * combination in {1, 2, 3} x {16, 32} x {0, 1} (maps only with a flood), keeps
+ * the fastest and writes it to *chosen (may be NULL). Synchronous. Allocates the scene's
  * output staging planes on first use; call it at set-up, not inside a
  * captured stream. */
 spm_status spm_scene_autotune(spm_scene *scene, void *stream, spm_tuning *chosen);

@@ -260,11 +260,15 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
     ds.Wx = hs.Wx; ds.Wy = hs.Wy; ds.Nx = hs.Nx; ds.Ny = hs.Ny; ds.S = hs.S;
     ds.hx = (float)hs.Wx / (float)hs.Nx;
     ds.hy = (float)hs.Wy / (float)hs.Ny;
+    ds.inv_S = 1.0f / (float)hs.S;
+    ds.pitch_x = hs.S * hs.Wx / hs.Nx;
+    ds.pitch_y = hs.S * hs.Wy / hs.Ny;
     ds.n_poly = (int32_t)hs.poly_off.size() - 1;
     ds.n_gen = hs.n_gen; ds.n_src = hs.n_src; ds.n_vert = hs.n_vert;
     ds.n_seg = (int32_t)hs.segs.size() / 4;
     ds.bin_x0 = hs.bin_x0; ds.bin_y0 = hs.bin_y0; ds.bin_size = hs.bin_size;
     ds.bin_nx = hs.bin_nx; ds.bin_ny = hs.bin_ny;
+    ds.bin_inv = 1.0f / (float)hs.bin_size;
     if (hs.n_gen > (1 << 20)) {
         delete s;
         return set_err(nullptr, SPM_ERR_CAPACITY, "more than 2^20 generators");
@@ -339,6 +343,8 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
     ds.gen_costf = dalloc<float>(s, hs.n_gen);
     ds.gen_cost = dalloc<double>(s, hs.n_gen);
     ds.gen_par = dalloc<int32_t>(s, hs.n_gen);
+    ds.gen_rec = dalloc<float4>(s, hs.n_gen);
+    ds.gen_cull = dalloc<int4>(s, hs.n_gen);
     ds.gen_cone = dalloc<int4>(s, hs.n_gen);
     ds.gen_ctype = dalloc<int32_t>(s, hs.n_gen);
     ds.dirty = dalloc<uint32_t>(s, (hs.n_gen + 31) / 32);
@@ -918,8 +924,12 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         return (double)descs[k].n_gen / std::sqrt((double)std::max(1, descs[k].tiles_x * descs[k].tiles_y));
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return tile_cost(a) > tile_cost(c); });
-    for (int k = 0; k < n; ++k)
-        tile_off[k + 1] = tile_off[k] + descs[order[k]].tiles_x * descs[order[k]].tiles_y;
+    std::vector<int32_t> blk_off(n + 1, 0);
+    for (int k = 0; k < n; ++k) {
+        const spm::DevScene &d = descs[order[k]];
+        tile_off[k + 1] = tile_off[k] + d.tiles_x * d.tiles_y;
+        blk_off[k + 1] = blk_off[k] + d.tiles_x * d.tiles_y * (d.tile == spm::kTile ? 4 : 1);
+    }
     bool ok = true;
     spm::BatchDev &bd = b->dev;
     bd.n = n;
@@ -936,7 +946,8 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     b->src_tiles = src_tile_off[n];
     bd.order = bupload(b, order, ok);
     bd.tile_off = bupload(b, tile_off, ok);
-    bd.total_tiles = tile_off[n];
+    bd.blk_off = bupload(b, blk_off, ok);
+    bd.total_blocks = blk_off[n];
     bd.tile_counter = balloc<int32_t>(b, 1);
     bd.dist = bupload(b, dv, ok);
     bd.parent = bupload(b, pv, ok);
@@ -1254,7 +1265,7 @@ spm_status spm_scene_autotune(spm_scene *s, void *stream, spm_tuning *chosen) {
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess)
         return set_err(s, SPM_ERR_CUDA, "event creation failed");
-    const int modes[3] = {1, 2, 3}, chunks[2] = {32, 256}, tiles[2] = {spm::kTileSmall, spm::kTile};
+    const int modes[3] = {1, 2, 3}, tiles[2] = {spm::kTileSmall, spm::kTile};
     float best = 3.4e38f;
     spm_tuning pick{};
     pick.flood_mode = s->ds.flood_mode;
@@ -1267,35 +1278,30 @@ spm_status spm_scene_autotune(spm_scene *s, void *stream, spm_tuning *chosen) {
     for (int mi = 0; mi < 3; ++mi) {
         if (modes[mi] != 2 && !s->ds.use_flood) continue;
         if (ui == 1 && (modes[mi] == 2 || !s->ds.gen_maps)) continue;  // maps need a flood
-        for (int ci = 0; ci < 2; ++ci) {
-            s->ds.flood_mode = modes[mi];
-            s->ds.hidden_chunk = chunks[ci];
-            s->ds.use_maps = ui;
-            set_tile(s->ds, tiles[ti]);
-            float t[3];
-            st = spm_compute(s, stream, s->stage_dist, s->stage_par);  // warm-up
-            for (int k = 0; k < 3 && st == SPM_OK; ++k) {
-                cudaEventRecord(a, cs);
-                st = spm_compute(s, stream, s->stage_dist, s->stage_par);
-                cudaEventRecord(b, cs);
-                cudaEventSynchronize(b);
-                cudaEventElapsedTime(&t[k], a, b);
-            }
-            if (st != SPM_OK) break;
-            std::sort(t, t + 3);
-            if (t[1] < best) {
-                best = t[1];
-                pick.flood_mode = modes[mi];
-                pick.hidden_chunk = chunks[ci];
-                pick.tile = tiles[ti];
-                pick.maps = ui;
-            }
+        s->ds.flood_mode = modes[mi];
+        s->ds.use_maps = ui;
+        set_tile(s->ds, tiles[ti]);
+        float t[3];
+        st = spm_compute(s, stream, s->stage_dist, s->stage_par);  // warm-up
+        for (int k = 0; k < 3 && st == SPM_OK; ++k) {
+            cudaEventRecord(a, cs);
+            st = spm_compute(s, stream, s->stage_dist, s->stage_par);
+            cudaEventRecord(b, cs);
+            cudaEventSynchronize(b);
+            cudaEventElapsedTime(&t[k], a, b);
+        }
+        if (st != SPM_OK) break;
+        std::sort(t, t + 3);
+        if (t[1] < best) {
+            best = t[1];
+            pick.flood_mode = modes[mi];
+            pick.tile = tiles[ti];
+            pick.maps = ui;
         }
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     s->ds.flood_mode = pick.flood_mode;
-    s->ds.hidden_chunk = pick.hidden_chunk;
     s->ds.use_maps = pick.maps;
     set_tile(s->ds, pick.tile);
     if (chosen) *chosen = pick;

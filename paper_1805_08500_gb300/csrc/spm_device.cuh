@@ -60,37 +60,31 @@ __device__ __forceinline__ bool poly_blocks(const int2 *V, int m, int px, int py
     return pos && neg;
 }
 
-__device__ __forceinline__ unsigned edge_mask(const int2 *V, int m, int qx, int qy) {
-    unsigned mq = 0;
-    for (int i = 0; i < m; ++i) {
-        int2 a = V[i], b = V[i + 1 == m ? 0 : i + 1];
-        if (orient32(a.x, a.y, b.x, b.y, qx, qy) > 0) mq |= 1u << i;
-    }
-    return mq;
-}
-
-// Same test with q = perpendicular foot of p on segment source A->B (Sec. 4),
-// f = A + (num/den)(B - A), 0 < num < den. oA[i], oB[i] = orient(e_i, A / B).
-// orient(e_i, f) has the sign of (den - num) * oA[i] + num * oB[i] (int64).
-// The line p->f is parallel to perp(B - A) = (nx, ny).
-__device__ __forceinline__ bool poly_blocks_foot(const int2 *V, int m, const int *oA,
-                                                 const int *oB, int px, int py, long long num,
-                                                 long long den, int nx, int ny) {
-    unsigned mp = 0, mf = 0;
-    for (int i = 0; i < m; ++i) {
-        int2 a = V[i], b = V[i + 1 == m ? 0 : i + 1];
-        if (orient32(a.x, a.y, b.x, b.y, px, py) > 0) mp |= 1u << i;
-        long long of = (den - num) * (long long)oA[i] + num * (long long)oB[i];
-        if (of > 0) mf |= 1u << i;
-    }
-    if ((mp | mf) != ((1u << m) - 1u)) return false;
+// Same test with q = perpendicular foot of p on segment source A->B = seg
+// (Sec. 4), f = A + (num/den)(B - A), 0 < num < den: orient(e_i, f) has the
+// sign of (den - num) * orient(e_i, A) + num * orient(e_i, B) (int64). The
+// line p->f is parallel to perp(B - A).
+__device__ __forceinline__ bool foot_meets_poly(const int2 *V, int m, int4 seg, int px, int py, long long num,
+                                                long long den) {
+    const int nx = -(seg.w - seg.y), ny = seg.z - seg.x;
     bool pos = false, neg = false;
     for (int i = 0; i < m; ++i) {
-        int s = nx * (V[i].y - py) - ny * (V[i].x - px);
+        const int2 a = V[i];
+        const int s = nx * (a.y - py) - ny * (a.x - px);
         pos |= s > 0;
         neg |= s < 0;
     }
-    return pos && neg;
+    if (!(pos && neg)) return false;
+    int2 a = V[m - 1];
+    for (int i = 0; i < m; ++i) {
+        const int2 b = V[i];
+        if (orient32(a.x, a.y, b.x, b.y, px, py) <= 0 &&
+            (den - num) * (long long)orient32(a.x, a.y, b.x, b.y, seg.x, seg.y) +
+                    num * (long long)orient32(a.x, a.y, b.x, b.y, seg.z, seg.w) <= 0)
+            return false;
+        a = b;
+    }
+    return true;
 }
 
 // Cone membership of direction w for a vertex generator: wedge cones are the
@@ -193,46 +187,82 @@ __device__ __forceinline__ bool walk_bins(const DevScene &ds, float px, float py
     return false;
 }
 
-// Does the (float, lattice units) segment p->q come within r of box [x0,x1]x[y0,y1]?
-// Slab test on the box grown by r + 1: conservative (the 1e-4 slack on the
-// segment parameter is far above the error of the fast divisions).
-__device__ __forceinline__ bool seg_near_box(float px, float py, float qx, float qy, float r, int4 box) {
-    const float m = r + 1.0f;
-    float lo = 0.f, hi = 1.f;
-    float d[2] = {qx - px, qy - py}, p[2] = {px, py};
-    float bl[2] = {(float)box.x - m, (float)box.y - m}, bh[2] = {(float)box.z + m, (float)box.w + m};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        if (fabsf(d[k]) < 1e-6f) {
-            if (p[k] < bl[k] || p[k] > bh[k]) return false;
-        } else {
-            const float id = __fdividef(1.0f, d[k]);
-            float t0 = (bl[k] - p[k]) * id, t1 = (bh[k] - p[k]) * id;
-            lo = fmaxf(lo, fminf(t0, t1));
-            hi = fminf(hi, fmaxf(t0, t1));
-        }
+// Does the open segment p->q meet the open interior of convex polygon V[0..m)?
+// The predicate of poly_blocks, the side test first: most polygons near a
+// segment lie on one side of its line.
+__device__ __forceinline__ bool segment_meets_poly(const int2 *V, int m, int px, int py, int qx, int qy) {
+    const int dx = qx - px, dy = qy - py;
+    bool pos = false, neg = false;
+#pragma unroll 4
+    for (int i = 0; i < m; ++i) {
+        const int2 a = __ldg(V + i);
+        const int s = dx * (a.y - py) - dy * (a.x - px);
+        pos |= s > 0;
+        neg |= s < 0;
     }
-    return lo <= hi + 1e-4f;
+    if (!(pos && neg)) return false;
+    bool apart = false;  // an edge has both ends on its closed outer side
+    int2 a = __ldg(V + m - 1);
+#pragma unroll 4
+    for (int i = 0; i < m; ++i) {
+        const int2 b = __ldg(V + i);
+        apart |= orient32(a.x, a.y, b.x, b.y, px, py) <= 0 && orient32(a.x, a.y, b.x, b.y, qx, qy) <= 0;
+        a = b;
+    }
+    return !apart;
 }
 
 // Exact visibility between lattice point p and generator target q (a point),
-// one thread: walks the bins along the segment and tests every polygon there.
-__device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int py, int qx, int qy) {
+// one thread: walks the bins the segment crosses, cell to cell, and tests
+// every polygon there. Only the first share `part` of the segment from p is
+// walked: 1, or less when no obstacle is met beyond it (a polygon that blocks
+// the segment then meets that part, and is listed in one of its bins). The
+// float steps are off by far less than the unit the polygons' boxes are grown
+// by when they are binned. (A walk by columns with both their row ranges,
+// grown by a margin, took four divisions a column and visited about 1.6 x
+// the bins.)
+__device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int py, int qx, int qy, float part = 1.f) {
     if (px == qx && py == qy) return true;
-    int4 sb = make_int4(min(px, qx), min(py, qy), max(px, qx), max(py, qy));
-    bool blocked = walk_bins(ds, (float)px, (float)py, (float)qx, (float)qy, 0.f, [&](int bin) {
+    const float dx = (float)(qx - px), dy = (float)(qy - py);
+    const float u = (float)(px - ds.bin_x0) * ds.bin_inv, v = (float)(py - ds.bin_y0) * ds.bin_inv;
+    const float du = dx * part * ds.bin_inv, dv = dy * part * ds.bin_inv;
+    auto cell = [](float w, int n) { return min(max((int)floorf(w), 0), n - 1); };
+    int cx = cell(u, ds.bin_nx), cy = cell(v, ds.bin_ny);
+    const int ex = cell(u + du, ds.bin_nx), ey = cell(v + dv, ds.bin_ny);
+    const int sx = ex >= cx ? 1 : -1, sy = ey >= cy ? 1 : -1;
+    // segment parameter of the next crossing of a column / row border
+    const float ix = __fdividef(1.f, fabsf(du)), iy = __fdividef(1.f, fabsf(dv));
+    float nx = (float)(sx > 0 ? cx + 1 : cx), ny = (float)(sy > 0 ? cy + 1 : cy);
+    float tx = ex == cx ? INFINITY : fabsf(nx - u) * ix, ty = ey == cy ? INFINITY : fabsf(ny - v) * iy;
+    const int bx0 = min(px, qx), bx1 = max(px, qx), by0 = min(py, qy), by1 = max(py, qy);
+    for (int left = abs(ex - cx) + abs(ey - cy);; --left) {
         SPM_CNT(24, 1);  // a bin walked
-        for (int it = ds.bin_start[bin]; it < ds.bin_start[bin + 1]; ++it) {
-            const BinRec rec = ds.bin_recs[it];
-            const int4 bx = rec.box;
-            if (bx.z < sb.x || bx.x > sb.z || bx.w < sb.y || bx.y > sb.w) continue;
+        const int bin = cy * ds.bin_nx + cx, end = __ldg(ds.bin_start + bin + 1);
+        for (int it = __ldg(ds.bin_start + bin); it < end; ++it) {
+            const int4 *rp = reinterpret_cast<const int4 *>(ds.bin_recs + it);
+            const int4 bx = __ldg(rp);
+            if (bx.z < bx0 || bx.x > bx1 || bx.w < by0 || bx.y > by1) continue;
+            // the segment's line against the box, with half a unit of slack
+            // (the float roundings are below 2^-8 of a unit)
+            const float hx = 0.5f * (float)(bx.z - bx.x), hy = 0.5f * (float)(bx.w - bx.y);
+            const float mx = 0.5f * (float)(bx.x + bx.z) - (float)px, my = 0.5f * (float)(bx.y + bx.w) - (float)py;
+            const float reach = fabsf(dx) * (hy + 0.5f) + fabsf(dy) * (hx + 0.5f);
+            if (fabsf(dx * my - dy * mx) > reach) continue;
+            const int4 rec = __ldg(rp + 1);
             SPM_CNT(25, 1);  // a polygon tested
-            const int2 *V = ds.poly_v + rec.voff;
-            if (poly_blocks(V, rec.m, px, py, qx, qy, edge_mask(V, rec.m, qx, qy))) return true;
+            if (segment_meets_poly(ds.poly_v + rec.y, rec.z, px, py, qx, qy)) return false;
         }
-        return false;
-    });
-    return !blocked;
+        if (left <= 0) return true;
+        if (tx < ty) {
+            cx += sx;
+            nx += (float)sx;
+            tx = cx == ex ? INFINITY : fabsf(nx - u) * ix;
+        } else {
+            cy += sy;
+            ny += (float)sy;
+            ty = cy == ey ? INFINITY : fabsf(ny - v) * iy;
+        }
+    }
 }
 
 // Exact visibility between lattice point p and its perpendicular foot on
@@ -249,7 +279,6 @@ __device__ __forceinline__ bool visible_foot(const DevScene &ds, int s, int px, 
     float fx = (float)(L.x + t * ux), fy = (float)(L.y + t * uy);
     int4 sb = make_int4((int)floorf(fminf((float)px, fx)) - 1, (int)floorf(fminf((float)py, fy)) - 1,
                         (int)ceilf(fmaxf((float)px, fx)) + 1, (int)ceilf(fmaxf((float)py, fy)) + 1);
-    const int nx = -uy, ny = ux;
     const float wx0 = from_foot ? fx : (float)px, wy0 = from_foot ? fy : (float)py;
     const float wx1 = from_foot ? (float)px : fx, wy1 = from_foot ? (float)py : fy;
     bool blocked = walk_bins(ds, wx0, wy0, wx1, wy1, 0.f, [&](int bin) {
@@ -257,15 +286,7 @@ __device__ __forceinline__ bool visible_foot(const DevScene &ds, int s, int px, 
             const BinRec rec = ds.bin_recs[it];
             const int4 bx = rec.box;
             if (bx.z < sb.x || bx.x > sb.z || bx.w < sb.y || bx.y > sb.w) continue;
-            const int m = rec.m;
-            const int2 *V = ds.poly_v + rec.voff;
-            int oA[kMaxPolyVerts], oB[kMaxPolyVerts];
-            for (int i = 0; i < m; ++i) {
-                int2 a = V[i], bb = V[i + 1 == m ? 0 : i + 1];
-                oA[i] = orient32(a.x, a.y, bb.x, bb.y, L.x, L.y);
-                oB[i] = orient32(a.x, a.y, bb.x, bb.y, L.z, L.w);
-            }
-            if (poly_blocks_foot(V, m, oA, oB, px, py, num, den, nx, ny)) return true;
+            if (foot_meets_poly(ds.poly_v + rec.voff, rec.m, L, px, py, num, den)) return true;
         }
         return false;
     });
@@ -338,97 +359,5 @@ static __device__ unsigned long long g_time[8];
 #define SPM_LAP(i) ((void)0)
 #define SPM_TFLUSH() ((void)0)
 #endif
-
-// True when one polygon hides every point of the box from the point
-// generator at lattice point g. The set of points whose open segment to g
-// meets a convex polygon's interior is convex, so it suffices that the four
-// corners of the pixel-centre box are hidden by the same polygon. Walks the
-// bins of the thick segment (tile centre -> g, radius r) from the tile side
-// and stops at the first such polygon.
-__device__ __forceinline__ bool box_hidden(const DevScene &ds, int2 g, int4 box, float cx, float cy, float r,
-                                           float max_len = 3.4e38f) {
-    // walk toward g, optionally only the first max_len units (any subset of
-    // polygons keeps the test exact)
-    float tx = (float)g.x, ty = (float)g.y;
-    const float dx = tx - cx, dy = ty - cy, len = sqrtf(dx * dx + dy * dy);
-    if (len > max_len) {
-        tx = cx + dx * (max_len / len);
-        ty = cy + dy * (max_len / len);
-    }
-    return walk_bins(ds, cx, cy, tx, ty, r, [&](int bin) {
-        for (int it = ds.bin_start[bin]; it < ds.bin_start[bin + 1]; ++it) {
-            const BinRec rec = ds.bin_recs[it];
-            if (!seg_near_box(cx, cy, tx, ty, r, rec.box)) continue;
-            const int m = rec.m;
-            const int2 *V = ds.poly_v + rec.voff;
-            const unsigned mg = edge_mask(V, m, g.x, g.y);
-            if (poly_blocks(V, m, box.x, box.y, g.x, g.y, mg) && poly_blocks(V, m, box.z, box.y, g.x, g.y, mg) &&
-                poly_blocks(V, m, box.x, box.w, g.x, g.y, mg) && poly_blocks(V, m, box.z, box.w, g.x, g.y, mg))
-                return true;
-        }
-        return false;
-    });
-}
-
-// Warp-cooperative form of box_hidden (every lane must call it with the same
-// arguments): the thick segment from the box centre to g is cut into strips
-// one bin wide along its major axis; lane l takes strips l, l + 32, ...
-// (nearest the box first) and the warp stops at the first round in which
-// some lane found a polygon hiding all four corners.
-__device__ __forceinline__ bool box_hidden_warp(const DevScene &ds, int2 g, int4 box, float cx, float cy,
-                                                float r) {
-    const int lane = threadIdx.x & 31;
-    const float tx = (float)g.x, ty = (float)g.y;
-    const float bs = (float)ds.bin_size, m = r + 1.0f;
-    const bool xmaj = fabsf(tx - cx) >= fabsf(ty - cy);
-    // major axis: u (bins along it), minor: w
-    const float pu = xmaj ? cx : cy, pw = xmaj ? cy : cx, qu = xmaj ? tx : ty, qw = xmaj ? ty : tx;
-    const float ou = xmaj ? (float)ds.bin_x0 : (float)ds.bin_y0, ow = xmaj ? (float)ds.bin_y0 : (float)ds.bin_x0;
-    const int nu = xmaj ? ds.bin_nx : ds.bin_ny, nw = xmaj ? ds.bin_ny : ds.bin_nx;
-    auto bin_of = [&](float v, float o, int n) {
-        int b = (int)floorf((v - o) / bs);
-        return b < 0 ? 0 : (b >= n ? n - 1 : b);
-    };
-    const int u0 = bin_of(fminf(pu, qu) - m, ou, nu), u1 = bin_of(fmaxf(pu, qu) + m, ou, nu);
-    const int ustep = qu >= pu ? 1 : -1, us = ustep > 0 ? u0 : u1;
-    const int nstrips = u1 - u0 + 1;
-    const float du = qu - pu, dw = qw - pw;
-    for (int base = 0; base < nstrips; base += 32) {
-        bool found = false;
-        const int sidx = base + lane;
-        if (sidx < nstrips) {
-            const int u = us + ustep * sidx;
-            float wlo, whi;
-            if (fabsf(du) < 0.5f) {
-                wlo = fminf(pw, qw);
-                whi = fmaxf(pw, qw);
-            } else {
-                const float a = ou + u * bs - m, b = ou + (u + 1) * bs + m;
-                const float t0 = (a - pu) / du, t1 = (b - pu) / du;
-                float tl = fmaxf(0.f, fminf(t0, t1)), th = fminf(1.f, fmaxf(t0, t1));
-                if (tl > th) { tl = 0.f; th = 1.f; }
-                const float wa = pw + tl * dw, wb = pw + th * dw;
-                wlo = fminf(wa, wb);
-                whi = fmaxf(wa, wb);
-            }
-            const int w0 = bin_of(wlo - m, ow, nw), w1 = bin_of(whi + m, ow, nw);
-            for (int w = w0; w <= w1 && !found; ++w) {
-                const int bin = xmaj ? w * ds.bin_nx + u : u * ds.bin_nx + w;
-                for (int it = ds.bin_start[bin]; it < ds.bin_start[bin + 1] && !found; ++it) {
-                    const BinRec rec = ds.bin_recs[it];
-                    if (!seg_near_box(cx, cy, tx, ty, r, rec.box)) continue;
-                    const int2 *V = ds.poly_v + rec.voff;
-                    const unsigned mg = edge_mask(V, rec.m, g.x, g.y);
-                    found = poly_blocks(V, rec.m, box.x, box.y, g.x, g.y, mg) &&
-                            poly_blocks(V, rec.m, box.z, box.y, g.x, g.y, mg) &&
-                            poly_blocks(V, rec.m, box.x, box.w, g.x, g.y, mg) &&
-                            poly_blocks(V, rec.m, box.z, box.w, g.x, g.y, mg);
-                }
-            }
-        }
-        if (__any_sync(0xffffffffu, found)) return true;
-    }
-    return false;
-}
 
 }  // namespace spm

@@ -14,12 +14,9 @@ namespace spm {
 
 constexpr int kMaxPolyVerts = 16;    // convex polygon vertex limit
 constexpr int kAngBins = 2048;       // pseudo-angle bins of a generator's depth map
-constexpr int kTile = 32;            // largest pixel tile side (one CTA per tile)
+constexpr int kTile = 32;            // largest pixel tile side (tiles carry the candidate lists)
 constexpr int kTileSmall = 16;       // small tile side, for coarse grids
-constexpr int kPixelThreads = 256;   // 32x32 tiles: 4 pixels per thread; 16x16: 1
-constexpr int kCandCap = 1024;       // candidate generators per batch (smem)
-constexpr int kBlockCap = 96;        // blocker polygons per chunk (smem)
-constexpr int kDedupBits = 8192;     // polygon-id dedup bitmap (smem)
+constexpr int kPixelThreads = 256;   // CTA of the free-space mask
 constexpr int kMaxRounds = 1 << 20;  // hard cap on vertex-fixpoint rounds
 constexpr int kSeqMaxGen = 1 << 16;  // generators the sequential (paper-schedule) kernel takes
 constexpr int kLocBins = 256;        // pseudo-angle bins of an obstacle vertex's local depth map
@@ -80,12 +77,15 @@ struct __align__(16) BinRec {
 struct DevScene {
     int32_t Wx, Wy, Nx, Ny, S;
     float hx, hy;                      // pixel size in world units
+    int32_t pitch_x, pitch_y;          // pixel size in lattice units
+    float inv_S;                       // 1 / S
     int32_t n_poly, n_gen, n_src, n_vert, n_seg;
     // polygons
     const int32_t *poly_off;
     const int2 *poly_v;
     const int4 *poly_box;
     int32_t bin_x0, bin_y0, bin_size, bin_nx, bin_ny;
+    float bin_inv;                     // 1 / bin_size
     const int32_t *bin_start, *bin_items;
     const BinRec *bin_recs;            // parallel to bin_items
     const uint32_t *free_bits;         // free-space mask of pixel centres, free_words words per grid row
@@ -155,6 +155,13 @@ struct DevScene {
     float *gen_costf;                  // n_gen (inf when unreached)
     double *gen_cost;                  // n_gen
     int32_t *gen_par;                  // n_gen
+    // the pixel pass's view of a generator, one 16-byte load: world x, y, FP32
+    // cost, and kind | cone type << 3 (as bits)
+    float4 *gen_rec;
+    // and what it culls by, one 16-byte load: lattice position, the cone's two
+    // directions (zero: no cone) as 16-bit pairs, and the FP32 cost (+inf when
+    // it can win nowhere, -1 for a segment interior)
+    int4 *gen_cull;
     int4 *gen_cone;                    // c1.x c1.y c2.x c2.y (lattice directions)
     int32_t *gen_ctype;                // ConeType
     uint32_t *status;                  // latched status bits
@@ -207,7 +214,8 @@ struct BatchDev {
     // pixel pass: scenes in processing order (costliest tiles first)
     const int32_t *order;              // n scene indices
     const int32_t *tile_off;           // n + 1 prefix of tiles in that order
-    int32_t total_tiles;
+    const int32_t *blk_off;            // n + 1 prefix of 16 x 16 pixel blocks in that order
+    int32_t total_blocks;
     int32_t *tile_counter;             // persistent-kernel work counter
     float *const *dist;                // n output planes (device pointers)
     int32_t *const *parent;

@@ -3,32 +3,27 @@
 // arxiv 1805.08500 Sec. 3.1, Procedure 3 ("Cone"): a pixel that sees generator
 // g takes cost(g) + |p - g| when that is smaller than what it holds; Sec. 4:
 // a segment interior reaches p through its perpendicular foot. Instead of one
-// full-screen pass per generator, one CTA owns a 32 x 32 (or 16 x 16) pixel
-// tile and gathers only the generators that can win somewhere in it:
+// full-screen pass per generator, one warp owns a block of 16 x 16 pixels and
+// gathers only the generators that can win somewhere in it:
 //   * free space: the pixels inside obstacles come from the scene's
 //     free-space mask (built once, one bit per pixel);
-//   * candidates: the tile's list from the flood, or every generator;
-//   * cull: finite cost, shadow cone (or perpendicular strip) meets the tile,
-//     lower bound lb = cost + dist(g, tile) below the tile's current worst;
-//   * order: candidates sorted by lb; the CTA stops once every pixel's best is
-//     <= lb (no later candidate can win);
-//   * hidden tiles: in lb order, in chunks of 32, 64, 128, then 256
-//     candidates (the early exit usually comes within the first chunk), each
-//     thread walks
-//     the polygon bins from the tile toward one candidate and drops it when a
-//     single polygon hides all four corners of the tile (the region a convex
-//     polygon hides from a point is convex, so the whole tile is hidden);
-//   * depth maps (when the flood kept them): a pixel nearer than the lower
-//     bound of its bin sees the candidate, one beyond the full-blocking upper
-//     bound does not; only the pixels in between take the exact test below;
-//   * visibility: for each candidate still useful to some pixel, the CTA
-//     builds the list of polygons whose interior meets the hull of (tile, g)
-//     (exact separating-axis filter), then every pixel runs the exact integer
+//   * candidates: the list of the block's tile from the flood, or every
+//     generator;
+//   * cull: finite cost, shadow cone (or perpendicular strip) meets the block,
+//     lower bound lb = cost + dist(g, block) below the block's current worst;
+//   * order: candidates in order of lb; the warp stops once every pixel's best
+//     is <= lb (no later candidate can win);
+//   * depth maps (when the flood kept them): the bins the block spans may show
+//     that it sees the candidate as a whole or not at all; otherwise a pixel
+//     nearer than the lower bound of its bin sees it, one beyond the
+//     full-blocking upper bound does not, and only the pixels in between take
+//     the exact test below;
+//   * visibility: the warp lists the polygons whose interior may meet the hull
+//     of (block, g), and every undecided pixel runs the exact integer
 //     separating-axis test against that list (none when the list is empty);
-//   * argmin: a per-pixel u64 key (FP32 distance bits << 32 | generator id),
-//     so "smaller distance, then smaller id" is one unsigned compare;
-//   * output: each thread owns 4 consecutive pixels of a row and writes them
-//     with one 16-byte store per plane (dist, parent).
+//   * argmin: smaller distance, then smaller id;
+//   * output: each lane writes four consecutive pixels of a row with one
+//     16-byte store per plane (dist, parent).
 #include <cuda_runtime.h>
 
 #include "spm_device.cuh"
@@ -37,698 +32,643 @@
 namespace spm {
 namespace {
 
-constexpr int NT = kPixelThreads;
-#ifndef SPM_PIX16_MINB
-#define SPM_PIX16_MINB 4  // resident CTAs per SM the 16 x 16 kernel is compiled for
-#endif
-#ifndef SPM_PIX32_MINB
-#define SPM_PIX32_MINB 4  // the same for the 32 x 32 kernel
-#endif
-#ifndef SPM_PIXB_MINB
-#define SPM_PIXB_MINB 3   // the same for the batched kernel (both tile sizes inlined)
-#endif
-constexpr unsigned long long kUnset = 0x7F800000FFFFFFFFull;  // (+inf, id max)
+constexpr int NT = kPixelThreads;  // threads of the free-space mask's CTAs
 
-// Work counters of an instrumentation build (-DSPM_COUNT); compiled out otherwise.
-
-
-// Convex hull (counter-clockwise, no repeated or collinear vertices) of the
-// tile's pixel-centre box and the lattice point t, by Andrew's monotone chain
-// over the 5 points. The box may be degenerate (a one-pixel row or column),
-// so the hull may be a segment (2 vertices) or a point (1).
-struct Hull {
-    int2 v[5];
-    int n;
-};
-
-__device__ __forceinline__ Hull hull_box_point(int4 box, int tx, int ty) {
-    int2 p[5] = {make_int2(box.x, box.y), make_int2(box.z, box.y), make_int2(box.z, box.w), make_int2(box.x, box.w),
-                 make_int2(tx, ty)};
+// Lower bound of the distance from segment source s's interior to any pixel of
+// the box (lattice box, world fbox), or -1 when no pixel's perpendicular foot
+// lies strictly inside the segment.
+__device__ __forceinline__ float segment_lower_bound(const DevScene &ds, int s, int4 box, float4 fbox) {
+    const int4 L = ds.seg_lat[s];
+    const long long ux = L.z - L.x, uy = L.w - L.y, den = ux * ux + uy * uy;
+    bool all_lo = true, all_hi = true;
+    const int cx[4] = {box.x, box.z, box.x, box.z}, cy[4] = {box.y, box.y, box.w, box.w};
 #pragma unroll
-    for (int i = 1; i < 5; ++i)  // sort by (x, y)
-#pragma unroll
-        for (int j = i; j > 0; --j)
-            if (p[j].x < p[j - 1].x || (p[j].x == p[j - 1].x && p[j].y < p[j - 1].y)) {
-                const int2 t = p[j];
-                p[j] = p[j - 1];
-                p[j - 1] = t;
-            }
-    int2 st[10];
-    int k = 0;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {  // lower chain
-        while (k >= 2 && orient32(st[k - 2].x, st[k - 2].y, st[k - 1].x, st[k - 1].y, p[i].x, p[i].y) <= 0) --k;
-        st[k++] = p[i];
+    for (int k = 0; k < 4; ++k) {
+        const long long num = (cx[k] - L.x) * ux + (cy[k] - L.y) * uy;
+        all_lo &= num <= 0;
+        all_hi &= num >= den;
     }
-    const int lower = k + 1;
+    if (all_lo || all_hi) return -1.f;
+    const float4 F = ds.seg_pos[s];
+    const float fx = F.z - F.x, fy = F.w - F.y, il = rsqrtf(fx * fx + fy * fy);
+    const float qx[4] = {fbox.x, fbox.z, fbox.x, fbox.z}, qy[4] = {fbox.y, fbox.y, fbox.w, fbox.w};
+    float mn = INFINITY;
+    bool pos = false, neg = false;
 #pragma unroll
-    for (int i = 3; i >= 0; --i) {  // upper chain
-        while (k >= lower && orient32(st[k - 2].x, st[k - 2].y, st[k - 1].x, st[k - 1].y, p[i].x, p[i].y) <= 0) --k;
-        st[k++] = p[i];
+    for (int k = 0; k < 4; ++k) {
+        const float sd = (fx * (qy[k] - F.y) - fy * (qx[k] - F.x)) * il;
+        pos |= sd > 0.f;
+        neg |= sd < 0.f;
+        mn = fminf(mn, fabsf(sd));
     }
-    Hull h;
-    h.n = k > 1 ? k - 1 : 1;  // the last point repeats the first
-    if (h.n == 2 && st[0].x == st[1].x && st[0].y == st[1].y) h.n = 1;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) h.v[i] = st[i < h.n ? i : 0];
-    return h;
+    return (pos && neg) ? 0.f : mn * 0.999999f;
 }
 
-// Per-candidate generator data staged in shared memory for the first
-// kStage candidates of a sorted batch: one parallel load replaces a dependent
-// global load per candidate in the lb-ordered loop.
-constexpr int kStage = 64;
-struct CandRec {
-    int4 cone;
-    int2 lat;
-    float2 pos;
-    float cf;
-    int kind, ctype, map_ok;
+// ---------------------------------------------------------------------------
+// One warp, one block of 16 x 16 pixels (eight pixels a lane), no barrier.
+// ---------------------------------------------------------------------------
+constexpr int kBlk = 16;         // block side in pixels
+#ifndef SPM_BLK_WARPS
+#define SPM_BLK_WARPS 4
+#endif
+constexpr int kBlkWarps = SPM_BLK_WARPS;  // warps (blocks) per CTA
+constexpr int kWarpCand = 96;    // candidates a warp holds before it works them off
+constexpr int kWarpPoly = 64;    // blocker polygons a warp lists at a time
+constexpr int kBlocked = 1 << 15; // an undecided pixel found blocked
+
+// A candidate's flags, above its generator id (below 2^20).
+constexpr int kCandId = (1 << 20) - 1;
+constexpr int kCandInCone = 1 << 20;  // the whole block lies in the shadow cone (or there is none)
+constexpr int kCandMap = 1 << 21;     // its depth map is complete
+
+// The pixels' state lives in shared memory (a lane's eight pixels at
+// k * 32 + lane), not in registers: the loops over them stay rolled, nothing
+// spills around the exact tests, and more warps are resident.
+struct WarpSmem {
+    float bd[256];               // best distance so far (-inf: not a free pixel of the grid)
+    int bi[256];                 // and its generator
+    float lb[kWarpCand];         // candidates: least cost + distance over the block
+    int cand[kWarpCand];         // generator id and flags
+    int3 poly[kWarpPoly];        // blocker polygons: id, first vertex, vertices
+    unsigned short item[256];    // undecided pixels, lane * 8 + k, and kBlocked
 };
 
-struct PixSmem {
-    CandRec rec[kStage];
-    int cand_id[kCandCap];
-    float cand_lb[kCandCap];
-    unsigned dedup[kDedupBits / 32];
-    int2 blk_v[kBlockCap][kMaxPolyVerts];
-    int blk_oA[kBlockCap][kMaxPolyVerts];
-    int blk_oB[kBlockCap][kMaxPolyVerts];
-    unsigned blk_mask[kBlockCap];
-    int blk_m[kBlockCap];
-    unsigned char hidden[kCandCap];
-    int n_cand, n_block, overflow;
-    float tile_ub;
-    Hull hull;  // of the tile box and the current point target
+// One warp's block of pixels. A lane holds four consecutive pixels (k & 3) of
+// rows lane / 4 and lane / 4 + 8 (k >> 2).
+struct Block {
+    int4 box;    // lattice box of its pixel centres
+    int i0, j0;  // its first pixel
+    int i, j;    // the lane's first pixel
+    float worst; // largest best distance of the lane's pixels
+    bool lists;  // the candidates come from flooded lists
 };
 
-// Does the interior of convex polygon V meet the closed convex hull H?
-// Separating-axis test over the edges of both (an edge separates when the
-// other body lies on its closed outer side).
-__device__ bool poly_meets_hull(const int2 *V, int m, const Hull &H) {
-    for (int i = 0; i < m; ++i) {  // polygon edges (outward side is orient < 0)
-        const int2 a = V[i], b = V[i + 1 == m ? 0 : i + 1];
-        bool all_out = true;
-        for (int k = 0; k < H.n && all_out; ++k) all_out = orient32(a.x, a.y, b.x, b.y, H.v[k].x, H.v[k].y) <= 0;
-        if (all_out) return false;
+__device__ __forceinline__ float point_dist(float cf, float dx, float dy) { return cf + sqrtf(dx * dx + dy * dy); }
+__device__ __forceinline__ float pixel_x(const DevScene &ds, int i) { return ((float)i + 0.5f) * ds.hx; }
+__device__ __forceinline__ float pixel_y(const DevScene &ds, int j) { return ((float)j + 0.5f) * ds.hy; }
+
+// Generator g as a candidate of the block: its lower bound and flags; false
+// when it cannot win anywhere in the block. Most entries of a list go by their
+// cost or cone, one 16-byte load.
+__device__ __forceinline__ bool block_candidate(const DevScene &ds, int g, const Block &b, float ub, bool maps,
+                                                float &lb, int &cand) {
+    const int4 q = __ldg(ds.gen_cull + g);
+    const float cost = __int_as_float(q.w);
+    const int4 box = b.box;
+    cand = g;
+    if (cost < 0.f) {  // a segment interior
+        const float4 fbox = make_float4(pixel_x(ds, b.i0), pixel_y(ds, b.j0), pixel_x(ds, min(b.i0 + kBlk, ds.Nx) - 1),
+                                        pixel_y(ds, min(b.j0 + kBlk, ds.Ny) - 1));
+        lb = segment_lower_bound(ds, ds.gen_aux[g], box, fbox);
+        return lb >= 0.f && lb <= ub;
     }
-    for (int j = 0; j < H.n; ++j) {  // hull edges
-        const int2 a = H.v[j], b = H.v[j + 1 == H.n ? 0 : j + 1];
-        if (a.x == b.x && a.y == b.y) continue;  // a one-point hull has no edge
-        bool all_out = true;
-        for (int i = 0; i < m && all_out; ++i) all_out = orient32(a.x, a.y, b.x, b.y, V[i].x, V[i].y) <= 0;
-        if (all_out) return false;
-    }
+    const int2 l = make_int2((short)q.x, q.x >> 16);
+    const int x0 = box.x - l.x, x1 = box.z - l.x, y0 = box.y - l.y, y1 = box.w - l.y;
+    const float dx = (float)max(max(x0, -x1), 0), dy = (float)max(max(y0, -y1), 0);
+    // a source lies within a lattice unit of its lattice point, a vertex on it
+    const float d = sqrtf(dx * dx + dy * dy) - (g < ds.n_src ? 1.f : 0.f);
+    lb = (cost + fmaxf(d, 0.f) * ds.inv_S) * 0.999999f;
+    // cross(c1, w) and cross(w, c2) are linear in w: their extremes over the
+    // box lie at the corners their signs choose (no cone: all zero)
+    const int kx = (short)q.y, ky = q.y >> 16, kz = (short)q.z, kw = q.z >> 16;
+    const int hi1 = kx * (kx > 0 ? y1 : y0) - ky * (ky > 0 ? x0 : x1);
+    const int hi2 = kw * (kw > 0 ? x1 : x0) - kz * (kz > 0 ? y0 : y1);
+    if (!(lb <= ub) || !(cost < INFINITY) || (hi1 | hi2) < 0) return false;
+    const int lo1 = kx * (kx > 0 ? y0 : y1) - ky * (ky > 0 ? x1 : x0);
+    const int lo2 = kw * (kw > 0 ? x0 : x1) - kz * (kz > 0 ? y1 : y0);
+    // a ray's two directions are the same: the box would lie on its line
+    if ((lo1 | lo2) >= 0 && (q.y != q.z || q.y == 0)) cand |= kCandInCone;
+    if (maps && ds.gen_map_ok[g]) cand |= kCandMap;
     return true;
 }
 
-__device__ __forceinline__ float key_dist(unsigned long long k) { return __uint_as_float((unsigned)(k >> 32)); }
-
-// Lower bound of cost(g) + distance from g to any pixel of the tile, or -1 if
-// g cannot be valid anywhere in the tile.
-__device__ float tile_lower_bound(const DevScene &ds, int g, int4 box, float4 fbox) {
-    // every field is loaded up front (independent loads, in flight together)
-    const float cf = __ldg(ds.gen_costf + g);
-    const int kind = __ldg(ds.gen_kind + g);
-    const int ctype = __ldg(ds.gen_ctype + g);
-    const int4 cone = __ldg(ds.gen_cone + g);
-    const int2 gv = __ldg(ds.gen_lat + g);
-    const float2 gpos = __ldg(ds.gen_pos + g);
-    if (!(cf < INFINITY)) return -1.f;
-    if (kind == kSegI) {
-        const int s = ds.gen_aux[g];
-        const int4 L = ds.seg_lat[s];
-        const long long ux = L.z - L.x, uy = L.w - L.y, den = ux * ux + uy * uy;
-        bool all_lo = true, all_hi = true;
-        const int cx[4] = {box.x, box.z, box.x, box.z}, cy[4] = {box.y, box.y, box.w, box.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            long long num = (cx[k] - L.x) * ux + (cy[k] - L.y) * uy;
-            all_lo &= num <= 0;
-            all_hi &= num >= den;
-        }
-        if (all_lo || all_hi) return -1.f;
-        const float4 F = ds.seg_pos[s];
-        const float fx = F.z - F.x, fy = F.w - F.y, il = rsqrtf(fx * fx + fy * fy);
-        const float qx[4] = {fbox.x, fbox.z, fbox.x, fbox.z}, qy[4] = {fbox.y, fbox.y, fbox.w, fbox.w};
-        float mn = INFINITY;
-        bool pos = false, neg = false;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            float sd = (fx * (qy[k] - F.y) - fy * (qx[k] - F.x)) * il;
-            pos |= sd > 0.f;
-            neg |= sd < 0.f;
-            mn = fminf(mn, fabsf(sd));
-        }
-        return (pos && neg) ? 0.f : mn * 0.999999f;
+// What the depth map says about the whole block: 0 every pixel sees the
+// generator, 1 none does, 2 neither is shown. The block's box spans less than
+// half a turn seen from a point outside it, so its corners bound its angles.
+__device__ __forceinline__ int block_class(const float2 *map, int2 gl, const int4 box) {
+    const int lane = threadIdx.x & 31;
+    if (gl.x >= box.x - 1 && gl.x <= box.z + 1 && gl.y >= box.y - 1 && gl.y <= box.w + 1) return 2;
+    const float x0 = (float)(box.x - gl.x), x1 = (float)(box.z - gl.x), y0 = (float)(box.y - gl.y),
+                y1 = (float)(box.w - gl.y);
+    const float a = pang(lane & 1 ? x1 : x0, lane & 2 ? y1 : y0);
+    const float a0 = __shfl_sync(0xffffffffu, a, 0);
+    float d = a - a0;
+    if (d > 2.f) d -= 4.f;
+    if (d < -2.f) d += 4.f;
+    const float d1 = __shfl_xor_sync(0xffffffffu, d, 1);
+    float lo = fminf(d, d1), hi = fmaxf(d, d1);
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 2));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 2));
+    const int k0 = (int)floorf((a0 + lo - kAngEps) / kAngW), k1 = (int)floorf((a0 + hi + kAngEps) / kAngW);
+    if (k1 - k0 >= 256) return 2;  // a generator next to the block: pixel by pixel
+    float up = 0.f, low = INFINITY;
+    for (int k = k0 + lane; k <= k1; k += 32) {
+        const float2 b = __ldg(map + ((k + kAngBins) & (kAngBins - 1)));
+        up = fmaxf(up, b.x);
+        low = fminf(low, b.y);
     }
-    if (kind == kVert) {
-        const int ct = ctype;
-        if (ct == kConeEmpty) return -1.f;
-        const int4 c = cone;
-        const int2 v = gv;
-        const int cx[4] = {box.x, box.z, box.x, box.z}, cy[4] = {box.y, box.y, box.w, box.w};
-        bool out1 = true, out2 = true;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int wx = cx[k] - v.x, wy = cy[k] - v.y;
-            out1 &= cross32(c.x, c.y, wx, wy) < 0;
-            out2 &= cross32(wx, wy, c.z, c.w) < 0;
-        }
-        if (out1 || out2) return -1.f;
-    }
-    const float2 p = gpos;
-    const float dx = fmaxf(fmaxf(fbox.x - p.x, p.x - fbox.z), 0.f);
-    const float dy = fmaxf(fmaxf(fbox.y - p.y, p.y - fbox.w), 0.f);
-    return (cf + sqrtf(dx * dx + dy * dy)) * 0.999999f;
+    // non-negative floats order as their bits
+    const float l = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(low)));
+    const float u = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(up)));
+    const float fx = fmaxf(fabsf(x0), fabsf(x1)), fy = fmaxf(fabsf(y0), fabsf(y1));
+    if (fmaf(fx, fx, fy * fy) * (1.f + 1e-5f) < l) return 0;
+    const float nx = fmaxf(fmaxf(x0, -x1), 0.f), ny = fmaxf(fmaxf(y0, -y1), 0.f);
+    if (fmaf(nx, nx, ny * ny) * (1.f - 1e-5f) >= u) return 1;
+    return 2;
 }
 
-// Bitonic sort of (lb, id) pairs, n padded to a power of two with +inf
-// (lists of more than 32; shorter ones take sort_small_warp).
-__device__ void sort_candidates(PixSmem &sm, int n) {
-    int P = 1;
-    while (P < n) P <<= 1;
-    for (int i = n + threadIdx.x; i < P; i += NT) {
-        sm.cand_lb[i] = INFINITY;
-        sm.cand_id[i] = 0x7fffffff;
+// Depth-map bins a pixel at offset (rx, ry) != 0 may lie in.
+__device__ __forceinline__ int2 pixel_bins(float rx, float ry) {
+    const float a = pang(rx, ry);
+    return make_int2(((int)floorf((a - kAngEps) / kAngW) + kAngBins) & (kAngBins - 1),
+                     (int)floorf((a + kAngEps) / kAngW) & (kAngBins - 1));
+}
+
+// The undecided pixels of a candidate (bit k of und: the lane's pixel k)
+// tested exactly; returns the lane's visible ones. gl: a point generator's
+// lattice position; seg_id: a segment interior's source, else -1. clear (with
+// a depth map): no obstacle is met nearer than that to the generator on any of
+// their segments.
+// The polygons that may block one of them are those whose boxes meet the thick
+// segment from the block's centre to the generator (or to the centre's foot on
+// the segment source: the other pixels' segments are its translates) and, for
+// a point, that no edge of theirs separates from the hull of the block's box
+// and the generator. They are listed kWarpPoly at a time, and each list is
+// tested against the undecided pixels, packed a lane each. Without flooded
+// lists a polygon that hides all four corners of the block's box hides the
+// block (the region a convex polygon hides is convex).
+// Every step is one load deep for the whole warp: a lane takes a bin of the
+// segment, then the bins' records are dealt to the lanes evenly, then a lane
+// takes a listed polygon. (Lanes walking bins of their own, record by record
+// and vertex by vertex, waited on some 80 loads in a row: 57k cycles a list on
+// the 2048^2 maze.)
+__device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem &ws, const Block &b, int2 gl, int seg_id,
+                                                   float clear, unsigned und) {
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) SPM_CNT(5, 1);
+    SPM_CNT(7, __popc(und));
+    // the undecided pixels, packed
+    const int mine = __popc(und);
+    int at = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += y;
     }
-    __syncthreads();
-    for (int k = 2; k <= P; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < P; i += NT) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const bool up = (i & k) == 0;
-                    const float a = sm.cand_lb[i], b = sm.cand_lb[ixj];
-                    const int ia = sm.cand_id[i], ib = sm.cand_id[ixj];
-                    const bool gt = (a > b) || (a == b && ia > ib);
-                    if (gt == up) {
-                        sm.cand_lb[i] = b; sm.cand_lb[ixj] = a;
-                        sm.cand_id[i] = ib; sm.cand_id[ixj] = ia;
-                    }
+    const int n_item = __shfl_sync(0xffffffffu, at, 31);
+    at -= mine;
+    __syncwarp();
+    {
+        int p = at;
+        for (unsigned m = und; m; m &= m - 1) ws.item[p++] = (unsigned short)(lane * 8 + __ffs(m) - 1);
+    }
+    const int4 box = b.box;
+    const float cx = 0.5f * ((float)box.x + (float)box.z), cy = 0.5f * ((float)box.y + (float)box.w);
+    float dx = (float)gl.x - cx, dy = (float)gl.y - cy;
+    if (seg_id >= 0) {
+        const int4 seg = ds.seg_lat[seg_id];
+        const float fux = (float)(seg.z - seg.x), fuy = (float)(seg.w - seg.y);
+        const float t = ((cx - seg.x) * fux + (cy - seg.y) * fuy) / (fux * fux + fuy * fuy);
+        dx = seg.x + t * fux - cx;
+        dy = seg.y + t * fuy - cy;
+    } else {
+        // the block's segments shrink toward the generator alike: what lies
+        // nearer than `clear` to it is the same last share of each
+        const float fx = fmaxf(fabsf((float)(box.x - gl.x)), fabsf((float)(box.z - gl.x)));
+        const float fy = fmaxf(fabsf((float)(box.y - gl.y)), fabsf((float)(box.w - gl.y)));
+        const float part = fmaxf(1.f - fmaxf(clear - 2.f, 0.f) * rsqrtf(fmaf(fx, fx, fy * fy)), 0.f);
+        dx *= part;
+        dy *= part;
+    }
+    const float ex = (float)(box.z - box.x), ey = (float)(box.w - box.y);
+    const float m = 0.5f * sqrtf(ex * ex + ey * ey) + 2.0f;  // half the segment's thickness
+    const float bs = (float)ds.bin_size, ibs = ds.bin_inv;
+    auto col_of = [&](float v) { return min(max((int)floorf((v - (float)ds.bin_x0) * ibs), 0), ds.bin_nx - 1); };
+    auto row_of = [&](float v) { return min(max((int)floorf((v - (float)ds.bin_y0) * ibs), 0), ds.bin_ny - 1); };
+    const int c0 = col_of(fminf(cx, cx + dx) - m), c1 = col_of(fmaxf(cx, cx + dx) + m);
+    const bool steep = fabsf(dx) < 0.5f;
+    const float idx = steep ? 0.f : __fdividef(1.0f, dx);
+    // rows a column's share of the segment may span: an upper bound, so that
+    // every (column, row) of it is an item of its own
+    const float span = (steep ? fabsf(dy) : fminf(fabsf(dy * idx) * (bs + 2.f * m), fabsf(dy))) + 2.f * m;
+    const int K = min((int)(span * ibs) + 3, ds.bin_ny), items = (c1 - c0 + 1) * K;
+    int n = 0, first = 0, cnt = 0, incl = 0, recs = 0, r0 = 0;
+    for (int j0 = 0;;) {
+        while (r0 >= recs && j0 < items) {  // the next 32 bins
+            cnt = 0;
+            if (j0 + lane < items) {
+                const int c = (j0 + lane) / K, kr = j0 + lane - c * K;
+                float ylo = fminf(0.f, dy), yhi = fmaxf(0.f, dy);
+                if (!steep) {
+                    const float xa = (float)(ds.bin_x0 + (c0 + c) * ds.bin_size) - cx;
+                    const float ta = (xa - m) * idx, tb = (xa + bs + m) * idx;
+                    const float ya = __saturatef(fminf(ta, tb)) * dy, yb = __saturatef(fmaxf(ta, tb)) * dy;
+                    ylo = fminf(ya, yb);
+                    yhi = fmaxf(ya, yb);
+                }
+                const int row = row_of(cy + ylo - m) + kr;
+                if (row <= row_of(cy + yhi + m)) {
+                    const int bin = row * ds.bin_nx + c0 + c;
+                    first = __ldg(ds.bin_start + bin);
+                    cnt = __ldg(ds.bin_start + bin + 1) - first;
                 }
             }
-            __syncthreads();
-        }
-}
-
-// The generator data the candidate loop reads, staged in shared memory.
-template <bool MAPS>
-__device__ __forceinline__ CandRec stage_candidate(const DevScene &ds, int g) {
-    CandRec r;
-    r.kind = ds.gen_kind[g];
-    r.cf = ds.gen_costf[g];
-    r.lat = ds.gen_lat[g];
-    r.pos = ds.gen_pos[g];
-    r.ctype = r.kind == kVert ? ds.gen_ctype[g] : kConeNone;
-    r.cone = r.kind == kVert ? ds.gen_cone[g] : make_int4(0, 0, 0, 0);
-    r.map_ok = MAPS && ds.gen_map_ok ? ds.gen_map_ok[g] : 0;
-    return r;
-}
-
-// Up to 32 (lb, id) pairs, nearly every tile's list, sorted by the first warp
-// in registers with shuffles (a bitonic network of the next power of two
-// above n), each lane then staging its candidate's generator data; the CTA
-// waits once.
-template <bool MAPS>
-__device__ void sort_small_warp(const DevScene &ds, PixSmem &sm, int n) {
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        float lb = lane < n ? sm.cand_lb[lane] : INFINITY;
-        int id = lane < n ? sm.cand_id[lane] : 0x7fffffff;
-        int P = 1;
-        while (P < n) P <<= 1;
-        for (int k = 2; k <= P; k <<= 1)
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                const float olb = __shfl_xor_sync(0xffffffffu, lb, j);
-                const int oid = __shfl_xor_sync(0xffffffffu, id, j);
-                // the lower lane of a pair keeps the smaller key in an
-                // ascending run ((lane & k) == 0), the larger otherwise
-                const bool lower = (lane & j) == 0, up = (lane & k) == 0;
-                const bool o_less = olb < lb || (olb == lb && oid < id);
-                if (o_less == (lower == up)) {
-                    lb = olb;
-                    id = oid;
-                }
+            incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
             }
-        if (lane < n) {
-            sm.cand_lb[lane] = lb;
-            sm.cand_id[lane] = id;
-            sm.rec[lane] = stage_candidate<MAPS>(ds, id);  // kStage >= 32
+            recs = __shfl_sync(0xffffffffu, incl, 31);
+            r0 = 0;
+            j0 += 32;
         }
-    }
-    __syncthreads();
-}
-
-// Conservative bin enumeration for the thick segment c->t (lattice units,
-// radius r): column-wise, one (column, bin) item per thread, so that every
-// thread scans one bin's records. Each polygon found is filtered against the
-// thick segment and appended (deduplicated) to smem.
-__device__ void build_blockers(const DevScene &ds, PixSmem &sm, float cx, float cy, float tx, float ty,
-                               float r, int kind, int2 tl, int4 seg, int4 box) {
-    // Float steps here only choose bins; their errors (~1e-3 lattice units)
-    // stay far inside the margin m, so fast reciprocals are safe.
-    const float bs = (float)ds.bin_size, ibs = 1.0f / bs, x0 = (float)ds.bin_x0, y0 = (float)ds.bin_y0;
-    const float m = r + 1.0f;
-    auto bin_of = [&](float v, float o, int n) {
-        int b = (int)floorf((v - o) * ibs);
-        return b < 0 ? 0 : (b >= n ? n - 1 : b);
-    };
-    const int c0 = bin_of(fminf(cx, tx) - m, x0, ds.bin_nx), c1 = bin_of(fmaxf(cx, tx) + m, x0, ds.bin_nx);
-    const float dx = tx - cx, dy = ty - cy;
-    const bool dedup = ds.n_poly <= kDedupBits;
-    // items per column: about the rows one column spans (its x extent is
-    // bs + 2m, the segment rises |dy/dx| per unit along it, plus m on both
-    // sides); each item strides by K, so any K covers every row
-    const float idx = fabsf(dx) < 0.5f ? 0.f : __fdividef(1.0f, dx);
-    const float span = fabsf(dx) < 0.5f ? fabsf(dy) + 2.f * m : fabsf(dy * idx) * (bs + 2.f * m) + 2.f * m;
-    const int K = min((int)(span * ibs) + 2, ds.bin_ny);
-    const int items = (c1 - c0 + 1) * K;
-    for (int j = threadIdx.x; j < items; j += NT) {
-        const int col = c0 + j / K, kr = j - (j / K) * K;
-        float ylo, yhi;
-        if (fabsf(dx) < 0.5f) {
-            ylo = fminf(cy, ty);
-            yhi = fmaxf(cy, ty);
-        } else {
-            float a = x0 + col * bs - m, b = x0 + (col + 1) * bs + m;
-            float t0 = (a - cx) * idx, t1 = (b - cx) * idx;
-            float tlo = fmaxf(0.f, fminf(t0, t1)), thi = fminf(1.f, fmaxf(t0, t1));
-            if (tlo > thi) { tlo = 0.f; thi = 1.f; }
-            float ya = cy + tlo * dy, yb = cy + thi * dy;
-            ylo = fminf(ya, yb);
-            yhi = fmaxf(ya, yb);
-        }
-        const int r0 = bin_of(ylo - m, y0, ds.bin_ny), r1 = bin_of(yhi + m, y0, ds.bin_ny);
-        for (int row = r0 + kr; row <= r1; row += K) {  // rows kr, kr + K, ...: every row once
-            const int bin = row * ds.bin_nx + col;
-            const int e = __ldg(ds.bin_start + bin + 1);
-            for (int it = __ldg(ds.bin_start + bin); it < e; ++it) {
+        if (r0 < recs) {  // 32 of their records
+            const int r = r0 + lane;
+            int own = 0;  // the first lane whose records end beyond r
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, incl, (own + o - 1) & 31) <= r) own += o;
+            own &= 31;
+            const int it = __shfl_sync(0xffffffffu, first, own) + r -
+                           (__shfl_sync(0xffffffffu, incl, own) - __shfl_sync(0xffffffffu, cnt, own));
+            int4 rec = make_int4(-1 - lane, 0, 0, 0);
+            bool hit = false;
+            if (r < recs) {
                 const int4 *rp = reinterpret_cast<const int4 *>(ds.bin_recs + it);
-                const BinRec rec = {__ldg(rp), __ldg(rp + 1).x, __ldg(rp + 1).y, __ldg(rp + 1).z, 0};
-                const int k = rec.poly;
-                if (dedup) {
-                    const unsigned bit = 1u << (k & 31);
-                    if (atomicOr(&sm.dedup[k >> 5], bit) & bit) continue;
-                }
-                if (!seg_near_box(cx, cy, tx, ty, r, rec.box)) continue;
-                if (kind != kSegI && !poly_meets_hull(ds.poly_v + rec.voff, rec.m, sm.hull)) continue;
-                const int slot = atomicAdd(&sm.n_block, 1);
-                if (slot >= kBlockCap) {
-                    sm.overflow = 1;
-                    continue;
-                }
-                const int b = rec.voff, nv = rec.m;
-                sm.blk_m[slot] = nv;
-                for (int i = 0; i < nv; ++i) sm.blk_v[slot][i] = ds.poly_v[b + i];
-                if (kind == kSegI) {
-                    for (int i = 0; i < nv; ++i) {
-                        const int2 a = sm.blk_v[slot][i], bb = sm.blk_v[slot][i + 1 == nv ? 0 : i + 1];
-                        sm.blk_oA[slot][i] = orient32(a.x, a.y, bb.x, bb.y, seg.x, seg.y);
-                        sm.blk_oB[slot][i] = orient32(a.x, a.y, bb.x, bb.y, seg.z, seg.w);
+                const int4 bx = __ldg(rp);
+                rec = __ldg(rp + 1);
+                // its box against the thick segment: the line, then the extent
+                const float hx = 0.5f * (float)(bx.z - bx.x) + m, hy = 0.5f * (float)(bx.w - bx.y) + m;
+                const float qx = 0.5f * (float)(bx.x + bx.z) - cx, qy = 0.5f * (float)(bx.y + bx.w) - cy;
+                hit = fabsf(dx * qy - dy * qx) <= fabsf(dx) * hy + fabsf(dy) * hx &&
+                      fabsf(qx - 0.5f * dx) <= 0.5f * fabsf(dx) + hx && fabsf(qy - 0.5f * dy) <= 0.5f * fabsf(dy) + hy;
+            }
+            // a polygon lies in several bins: its first record here counts
+            const unsigned same = __match_any_sync(0xffffffffu, rec.x);
+            hit = hit && (same & ((1u << lane) - 1u)) == 0;
+            for (int q = 0; q < n; ++q) hit = hit && ws.poly[q].x != rec.x;
+            const unsigned bal = __ballot_sync(0xffffffffu, hit);
+            if (hit) ws.poly[n + __popc(bal & ((1u << lane) - 1u))] = make_int3(rec.x, rec.y, rec.z);
+            n += __popc(bal);
+            r0 += 32;
+            __syncwarp();
+        }
+        const bool done = r0 >= recs && j0 >= items;
+        if (!done && n <= kWarpPoly - 32) continue;
+        if (lane == 0) SPM_CNT(6, n);
+        // the listed polygons against the undecided pixels
+        if (seg_id < 0) {
+            bool hides = false;
+            int kept = 0;
+            for (int q0 = 0; q0 < n; q0 += 32) {
+                bool keep = false;
+                int3 pl = make_int3(0, 0, 0);
+                if (q0 + lane < n) {
+                    pl = ws.poly[q0 + lane];
+                    const int2 *V = ds.poly_v + pl.y;
+                    bool apart = false;
+                    unsigned mask = 0;
+                    int2 a = __ldg(V + pl.z - 1);
+#pragma unroll 4
+                    for (int i = 0; i < pl.z; ++i) {
+                        const int2 e = __ldg(V + i);
+                        const int nx = -(e.y - a.y), ny = e.x - a.x;  // orient(a, e, p) = n . (p - a)
+                        const int far = nx * ((nx > 0 ? box.z : box.x) - a.x) + ny * ((ny > 0 ? box.w : box.y) - a.y);
+                        const bool in = nx * (gl.x - a.x) + ny * (gl.y - a.y) > 0;
+                        if (in) mask |= 1u << (i == 0 ? pl.z - 1 : i - 1);
+                        apart |= !in && far <= 0;
+                        a = e;
                     }
-                } else {
-                    sm.blk_mask[slot] = edge_mask(sm.blk_v[slot], nv, tl.x, tl.y);
+                    keep = !apart;
+                    if (keep && !b.lists)
+                        hides |= poly_blocks(V, pl.z, box.x, box.y, gl.x, gl.y, mask) &&
+                                 poly_blocks(V, pl.z, box.z, box.y, gl.x, gl.y, mask) &&
+                                 poly_blocks(V, pl.z, box.x, box.w, gl.x, gl.y, mask) &&
+                                 poly_blocks(V, pl.z, box.z, box.w, gl.x, gl.y, mask);
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                __syncwarp();
+                if (keep) ws.poly[kept + __popc(bal & ((1u << lane) - 1u))] = pl;
+                kept += __popc(bal);
+                __syncwarp();
+            }
+            n = kept;
+            if (__any_sync(0xffffffffu, hides)) return 0u;
+        }
+        for (int e = lane; e < n_item && n > 0; e += 32) {
+            const int it = ws.item[e], l = it >> 3, k = it & 7;
+            if (it & kBlocked) continue;
+            const int px = ds.pitch_x * (b.i0 + (l & 3) * 4 + (k & 3)) + ds.pitch_x / 2;
+            const int py = ds.pitch_y * (b.j0 + (l >> 2) + (k >> 2) * 8) + ds.pitch_y / 2;
+            bool v = true;
+            if (seg_id < 0) {
+                if (px != gl.x || py != gl.y)
+                    for (int q = 0; q < n && v; ++q) {
+                        SPM_CNT(10, 1);
+                        v = !segment_meets_poly(ds.poly_v + ws.poly[q].y, ws.poly[q].z, px, py, gl.x, gl.y);
+                    }
+            } else {
+                const int4 seg = ds.seg_lat[seg_id];
+                const long long ux = seg.z - seg.x, uy = seg.w - seg.y, den = ux * ux + uy * uy;
+                const long long num = (px - seg.x) * ux + (py - seg.y) * uy;
+                if (cross32((int)ux, (int)uy, px - seg.x, py - seg.y) != 0)
+                    for (int q = 0; q < n && v; ++q)
+                        v = !foot_meets_poly(ds.poly_v + ws.poly[q].y, ws.poly[q].z, seg, px, py, num, den);
+            }
+            if (!v) ws.item[e] = (unsigned short)(it | kBlocked);
+        }
+        __syncwarp();
+        n = 0;
+        if (done) break;
+    }
+    unsigned vis = 0;
+    for (unsigned w = und; w; w &= w - 1)
+        if (!(ws.item[at++] & kBlocked)) vis |= w & -w;
+    return vis;
+}
+
+// Candidate c against the block's pixels.
+__device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem &ws, Block &b, int c) {
+    const int lane = threadIdx.x & 31, g = c & kCandId;
+    const float4 rec = __ldg(ds.gen_rec + g);
+    const int4 q = __ldg(ds.gen_cull + g);
+    const int2 gl = make_int2((short)q.x, q.x >> 16);
+    const bool seg = (__float_as_int(rec.w) & 7) == kSegI;
+    const int seg_id = seg ? ds.gen_aux[g] : -1;
+    const float2 *map = c & kCandMap ? ds.gen_maps + (size_t)g * kAngBins : nullptr;
+    const int cls = map ? block_class(map, gl, b.box) : 2;
+    if (lane == 0) SPM_CNT(cls == 0 ? 2 : cls == 1 ? 3 : 8, 1);
+    if (cls == 1) return;
+    float4 sf = make_float4(0.f, 0.f, 0.f, 0.f);
+    float il = 0.f;
+    if (seg) {
+        sf = ds.seg_pos[seg_id];
+        const float fux = sf.z - sf.x, fuy = sf.w - sf.y;
+        il = 1.0f / sqrtf(fux * fux + fuy * fuy);
+    }
+    auto dist_at = [&](int k) {
+        const float fx = pixel_x(ds, b.i + (k & 3)), fy = pixel_y(ds, b.j + (k >> 2) * 8);
+        return seg ? fabsf((sf.z - sf.x) * (fy - sf.y) - (sf.w - sf.y) * (fx - sf.x)) * il
+                   : point_dist(rec.z, fx - rec.x, fy - rec.y);
+    };
+    const bool take_all = cls == 0 && (c & kCandInCone);
+    unsigned want = 0;
+    float worst = -INFINITY;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int k4 = 0; k4 < 4; ++k4) {
+            const int k = 4 * h + k4, at = k * 32 + lane;
+            const float d = dist_at(k);
+            float old = ws.bd[at];
+            bool better = d < old;
+            if (d == old) better = g < ws.bi[at];
+            if (better) want |= 1u << k;
+            if (take_all && better) {
+                ws.bd[at] = d;
+                ws.bi[at] = g;
+                old = d;
+            }
+            worst = fmaxf(worst, old);
+        }
+    }
+    SPM_CNT(14, __popc(want));
+    if (take_all) {
+        b.worst = worst;
+        return;
+    }
+    unsigned vis = 0, und = 0;
+    float clear = INFINITY;
+    const int rx0 = ds.pitch_x * b.i + ds.pitch_x / 2 - gl.x, ry0 = ds.pitch_y * b.j + ds.pitch_y / 2 - gl.y;
+    if (seg) {  // the perpendicular foot strictly inside the segment
+        const int4 L = ds.seg_lat[seg_id];
+        const long long ux = L.z - L.x, uy = L.w - L.y, den = ux * ux + uy * uy;
+#pragma unroll 1
+        for (unsigned m = want; m; m &= m - 1) {
+            const int k = __ffs(m) - 1;
+            const int px = ds.pitch_x * (b.i + (k & 3)) + ds.pitch_x / 2;
+            const int py = ds.pitch_y * (b.j + (k >> 2) * 8) + ds.pitch_y / 2;
+            const long long nm = (px - L.x) * ux + (py - L.y) * uy;
+            if (nm > 0 && nm < den) und |= m & -m;
+        }
+    } else {
+        const int4 cone = make_int4((short)q.y, q.y >> 16, (short)q.z, q.z >> 16);
+        const int ct = (__float_as_int(rec.w) >> 3) & 3;
+#pragma unroll 1
+        for (unsigned m = want; m; m &= m - 1) {
+            const int k = __ffs(m) - 1;
+            const int ix = rx0 + (k & 3) * ds.pitch_x, iy = ry0 + (k >> 2) * 8 * ds.pitch_y;
+            if (!(c & kCandInCone) && !in_cone(ct, cone, ix, iy)) continue;
+            if (cls == 0) {
+                vis |= m & -m;
+            } else if (!map) {
+                und |= m & -m;
+            } else {
+                const float rx = (float)ix, ry = (float)iy, r2 = fmaf(rx, rx, ry * ry);
+                const int2 bin = pixel_bins(rx, ry);
+                const float2 m0 = __ldg(map + bin.x), m1 = __ldg(map + bin.y);
+                const float low = fminf(m0.y, m1.y);
+                if (r2 == 0.f || r2 * (1.f + 1e-5f) < low) {  // visible (or the generator's own pixel)
+                    SPM_CNT(12, 1);
+                    vis |= m & -m;
+                } else if (r2 * (1.f - 1e-5f) < fmaxf(m0.x, m1.x)) {
+                    und |= m & -m;
+                    clear = fminf(clear, low);
+                } else {  // hidden
+                    SPM_CNT(13, 1);
                 }
             }
         }
     }
+    if (__any_sync(0xffffffffu, und)) {
+        // squared distances are non-negative: they order as their bits
+        const float near = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(clear)));
+        vis |= resolve_pixels(ds, ws, b, gl, seg_id, map ? sqrtf(near) : 0.f, und);
+    }
+    if (vis) {
+#pragma unroll 1
+        for (unsigned m = vis; m; m &= m - 1) {
+            const int k = __ffs(m) - 1;
+            ws.bd[k * 32 + lane] = dist_at(k);
+            ws.bi[k * 32 + lane] = g;
+        }
+        worst = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) worst = fmaxf(worst, ws.bd[k * 32 + lane]);
+        b.worst = worst;
+    }
 }
 
-// One tile of one scene, by one CTA: 32 x 32 pixels with PX = 4 pixels per
-// thread (consecutive in a row), or 16 x 16 with PX = 1. allow_lists = false
-// ignores flooded candidate lists (the batched form scans every generator).
-template <int PX, bool MAPS>
-__device__ __forceinline__ void pixel_tile(const DevScene &ds, const int tile, float *__restrict__ dist,
-                                           int32_t *__restrict__ parent, PixSmem &sm, const bool allow_lists) {
-    constexpr int T = PX == 4 ? 32 : 16;
-    constexpr int TPR = T / PX;  // threads per tile row
-    SPM_T0();
-    const int i0 = (tile % ds.tiles_x) * T, j0 = (tile / ds.tiles_x) * T;
-    const int row = threadIdx.x / TPR, c4 = (threadIdx.x % TPR) * PX;
-    const int j = j0 + row;
-    const int pitch_x = ds.S * ds.Wx / ds.Nx, pitch_y = ds.S * ds.Wy / ds.Ny;
-    const int py = pitch_y * j + pitch_y / 2;
-    const float fy = ((float)j + 0.5f) * ds.hy;
-    int px[PX];
-    float fx[PX];
-    unsigned long long key[PX];
+// The n candidates the warp holds, in order of their lower bounds, until none
+// can improve a pixel.
+__device__ __forceinline__ void apply_candidates(const DevScene &ds, WarpSmem &ws, int n, Block &b) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    unsigned l[kWarpCand / 32];
+#pragma unroll
+    for (int k = 0; k < kWarpCand / 32; ++k)
+        l[k] = lane + 32 * k < n ? __float_as_uint(ws.lb[lane + 32 * k]) : 0xffffffffu;
+    for (;;) {
+        unsigned mine = l[0];
+#pragma unroll
+        for (int k = 1; k < kWarpCand / 32; ++k) mine = min(mine, l[k]);
+        const unsigned least = __reduce_min_sync(0xffffffffu, mine);
+        if (least == 0xffffffffu) break;
+        if (!__any_sync(0xffffffffu, b.worst > __uint_as_float(least))) break;
+        const int from = __ffs(__ballot_sync(0xffffffffu, mine == least)) - 1;
+        int c = 0;
+        if (lane == from) {
+#pragma unroll
+            for (int k = kWarpCand / 32 - 1; k >= 0; --k)
+                if (l[k] == least) c = k;
+#pragma unroll
+            for (int k = 0; k < kWarpCand / 32; ++k)
+                if (k == c) l[k] = 0xffffffffu;
+        }
+        c = __shfl_sync(0xffffffffu, c, from);
+        if (lane == 0) SPM_CNT(4, 1);
+        apply_candidate(ds, ws, b, ws.cand[32 * c + from]);
+    }
+    __syncwarp();
+}
+
+__device__ __forceinline__ void pixel_block(const DevScene &ds, const int tile, const int sub, float *__restrict__ dist,
+                                            int32_t *__restrict__ parent, WarpSmem &ws) {
+    const int lane = threadIdx.x & 31;
+    Block b;
+    b.i0 = (tile % ds.tiles_x) * ds.tile + (sub & 1) * kBlk;
+    b.j0 = (tile / ds.tiles_x) * ds.tile + (sub >> 1) * kBlk;
+    if (b.i0 >= ds.Nx || b.j0 >= ds.Ny) return;
+    b.i = b.i0 + (lane & 3) * 4;
+    b.j = b.j0 + (lane >> 2);
     unsigned live = 0;
 #pragma unroll
-    for (int k = 0; k < PX; ++k) {
-        const int i = i0 + c4 + k;
-        px[k] = pitch_x * i + pitch_x / 2;
-        fx[k] = ((float)i + 0.5f) * ds.hx;
-        key[k] = kUnset;
-        if (i < ds.Nx && j < ds.Ny) live |= 1u << k;
-    }
-    // free space: not in the open interior of any polygon (the scene's
-    // free-space mask; the PX pixels of a thread share one word)
-    if (j < ds.Ny) {
-        const uint32_t fw = __ldg(ds.free_bits + (size_t)j * ds.free_words + ((i0 + c4) >> 5));
+    for (int h = 0; h < 2; ++h)
+        if (b.j + 8 * h < ds.Ny)  // the scene's free-space mask: outside every obstacle's open interior, inside the grid
+            live |= ((__ldg(ds.free_bits + (size_t)(b.j + 8 * h) * ds.free_words + (b.i >> 5)) >> (b.i & 31)) & 15u) << (4 * h);
 #pragma unroll
-        for (int k = 0; k < PX; ++k)
-            if (!((fw >> ((i0 + c4 + k) & 31)) & 1u)) live &= ~(1u << k);
+    for (int k = 0; k < 8; ++k) {
+        ws.bd[k * 32 + lane] = (live >> k) & 1u ? INFINITY : -INFINITY;
+        ws.bi[k * 32 + lane] = -1;
     }
-    const int ni = min(T, ds.Nx - i0), nj = min(T, ds.Ny - j0);
-    const int4 box = make_int4(pitch_x * i0 + pitch_x / 2, pitch_y * j0 + pitch_y / 2,
-                               pitch_x * (i0 + ni - 1) + pitch_x / 2, pitch_y * (j0 + nj - 1) + pitch_y / 2);
-    const float4 fbox = make_float4(((float)i0 + 0.5f) * ds.hx, ((float)j0 + 0.5f) * ds.hy,
-                                    ((float)(i0 + ni - 1) + 0.5f) * ds.hx, ((float)(j0 + nj - 1) + 0.5f) * ds.hy);
-    const float bcx = 0.5f * ((float)box.x + (float)box.z), bcy = 0.5f * ((float)box.y + (float)box.w);
-    const float brad = 0.5f * sqrtf((float)(box.z - box.x) * (float)(box.z - box.x) +
-                                    (float)(box.w - box.y) * (float)(box.w - box.y)) + 1.0f;
-    const bool any_live = __syncthreads_or(live != 0);
-    if (threadIdx.x == 0) SPM_CNT(0, 1);
-    if (threadIdx.x == 0) {
-        sm.n_cand = 0;
-        sm.tile_ub = INFINITY;
-    }
-    __syncthreads();
-    SPM_LAP(0);
-    // candidate source: the tile's flooded lists (the obstacle vertices' kept
-    // list, when this compute reuses it, then this flood's list) plus the
-    // global list, or every generator when the lists are unavailable
-    const bool lists = allow_lists && ds.use_flood && ds.flood_counts[2] == 0;
-    const bool stat = lists && ds.static_lists;
-    const int tix = tile;
-    const int s0 = stat ? ds.static_tile_start[tix] : 0;
-    const int ns = stat ? ds.static_tile_start[tix + 1] - s0 : 0;
-    const int l0 = lists ? ds.tile_start[tix] : 0;
-    const int nl = ns + (lists ? ds.tile_start[tix + 1] - l0 : 0);
-    const int ntotal = lists ? nl + ds.flood_counts[1] : ds.n_gen;
-    for (int g0 = 0; any_live && g0 < ntotal; g0 += NT) {
-        const int i = g0 + threadIdx.x;
-        int g = i;
-        if (lists && i < ntotal)
-            g = i < ns ? ds.static_tile_items[s0 + i] : i < nl ? ds.tile_items[l0 + i - ns] : ds.glob_list[i - nl];
-        float lb = -1.f;
-        if (i < ntotal) lb = tile_lower_bound(ds, g, box, fbox);
-        const bool keep = lb >= 0.f && lb <= sm.tile_ub;
-        const unsigned bal = __ballot_sync(0xffffffffu, keep);
-        int base = 0;
-        if ((threadIdx.x & 31) == 0 && bal) base = atomicAdd(&sm.n_cand, __popc(bal));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (keep) {
-            const int slot = base + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
-            sm.cand_id[slot] = g;
-            sm.cand_lb[slot] = lb;
-        }
-        __syncthreads();
-        SPM_LAP(1);
-        const int nc = sm.n_cand;
-        const bool last = g0 + NT >= ntotal;
-        if (nc > kCandCap - NT || (last && nc > 0)) {
-            static_assert(kStage >= 32, "a warp-sorted list is staged whole");
-            if (nc <= 32) {
-                sort_small_warp<MAPS>(ds, sm, nc);
-            } else {
-                sort_candidates(sm, nc);
-                for (int t = threadIdx.x; t < min(nc, kStage); t += NT) sm.rec[t] = stage_candidate<MAPS>(ds, sm.cand_id[t]);
-                __syncthreads();
+    b.worst = live ? INFINITY : -INFINITY;
+    if (lane == 0) SPM_CNT(0, 1);
+    if (__any_sync(0xffffffffu, live)) {
+        const int ni = min(kBlk, ds.Nx - b.i0), nj = min(kBlk, ds.Ny - b.j0);
+        b.box = make_int4(ds.pitch_x * b.i0 + ds.pitch_x / 2, ds.pitch_y * b.j0 + ds.pitch_y / 2,
+                          ds.pitch_x * (b.i0 + ni - 1) + ds.pitch_x / 2, ds.pitch_y * (b.j0 + nj - 1) + ds.pitch_y / 2);
+        b.lists = ds.use_flood && ds.flood_counts[2] == 0;
+        const bool stat = b.lists && ds.static_lists, maps = b.lists && ds.use_maps && ds.gen_maps;
+        const int s0 = stat ? ds.static_tile_start[tile] : 0, ns = stat ? ds.static_tile_start[tile + 1] - s0 : 0;
+        const int l0 = b.lists ? ds.tile_start[tile] : 0, nl = ns + (b.lists ? ds.tile_start[tile + 1] - l0 : 0);
+        const int total = b.lists ? nl + ds.flood_counts[1] : ds.n_gen;
+        float ub = INFINITY;  // no pixel of the block can take more
+        int n = 0;
+        for (int e0 = 0; e0 < total; e0 += 32) {
+            const int e = e0 + lane;
+            bool keep = false;
+            float lb = 0.f;
+            int c = 0;
+            if (e < total) {
+                const int32_t *at = e < ns ? ds.static_tile_items + s0 + e
+                                           : e < nl ? ds.tile_items + l0 + e - ns : ds.glob_list + e - nl;
+                keep = block_candidate(ds, b.lists ? __ldg(at) : e, b, ub, maps, lb, c);
             }
-            SPM_LAP(2);
-            if (threadIdx.x == 0) SPM_CNT(1, nc);
-            bool done = false;
-            int tested = 0, chunk = ds.hidden_chunk;
-            for (int c = 0; c < nc && !done; ++c) {
-                const float lb_c = sm.cand_lb[c];
-                bool act = false;
-#pragma unroll
-                for (int k = 0; k < PX; ++k) act |= (live >> k & 1u) && key_dist(key[k]) > lb_c;
-                if (!__syncthreads_or(act)) {
-                    done = true;
-                    SPM_LAP(3);
-                    break;
-                }
-                SPM_LAP(3);
-                // flooded lists were already tested on the whole tile area:
-                // no hidden-tile tests (nor their barriers) with lists
-                if (!lists && c == tested) {  // hidden-tile test for the next chunk, in parallel
-                    const int cc = c + threadIdx.x;
-                    if (threadIdx.x < chunk && cc < nc) {
-                        SPM_CNT(2, 1);
-                        const int g2 = sm.cand_id[cc];
-                        sm.hidden[cc] = ds.gen_kind[g2] != kSegI && box_hidden(ds, ds.gen_lat[g2], box, bcx, bcy, brad);
-                    }
-                    tested += chunk;
-                    chunk = min(2 * chunk, NT);  // most tiles exit within the first chunk
-                    __syncthreads();
-                }
-                if (!lists && sm.hidden[c]) {
-                    if (threadIdx.x == 0) SPM_CNT(3, 1);
-                    continue;
-                }
-                if (threadIdx.x == 0) SPM_CNT(4, 1);
-                const int gc = sm.cand_id[c];
-                const bool staged = c < kStage;
-                const int kind = staged ? sm.rec[c].kind : ds.gen_kind[gc];
-                const float cf = staged ? sm.rec[c].cf : ds.gen_costf[gc];
-                const int2 gl = staged ? sm.rec[c].lat : ds.gen_lat[gc];
-                const float2 gp = staged ? sm.rec[c].pos : ds.gen_pos[gc];
-                int ct = kConeNone;
-                int4 cone = make_int4(0, 0, 0, 0);
-                int4 seg = make_int4(0, 0, 0, 0);
-                float4 segf = make_float4(0.f, 0.f, 0.f, 0.f);
-                long long den = 0;
-                float seg_il = 0.f;
-                if (kind == kVert) {
-                    ct = staged ? sm.rec[c].ctype : ds.gen_ctype[gc];
-                    cone = staged ? sm.rec[c].cone : ds.gen_cone[gc];
-                } else if (kind == kSegI) {
-                    seg = ds.seg_lat[ds.gen_aux[gc]];
-                    segf = ds.seg_pos[ds.gen_aux[gc]];
-                    const long long ux = seg.z - seg.x, uy = seg.w - seg.y;
-                    den = ux * ux + uy * uy;
-                    const float fux = segf.z - segf.x, fuy = segf.w - segf.y;
-                    seg_il = 1.0f / sqrtf(fux * fux + fuy * fuy);
-                }
-                unsigned need = 0, want = 0;
-                unsigned long long nk[PX];
-                long long num[PX];
-                // the flood's depth map of a point generator decides most pixels:
-                // nearer than any obstacle on their ray -> visible; beyond a full
-                // blocking -> hidden; only the rest need the exact test below
-                const float2 *gmap = MAPS && lists && ds.use_maps && ds.gen_maps && kind != kSegI &&
-                                             (staged ? sm.rec[c].map_ok : ds.gen_map_ok[gc])
-                                         ? ds.gen_maps + (size_t)gc * kAngBins
-                                         : nullptr;
-                // first pass: each pixel's key and depth-map bins, without
-                // branches around the loads, so that all of the thread's map
-                // loads are in flight together
-                float r2[PX];
-                int bA[PX], bB[PX];
-#pragma unroll
-                for (int k = 0; k < PX; ++k) {
-                    bool ok = ((live >> k) & 1u) && key_dist(key[k]) > lb_c;
-                    float d;
-                    num[k] = 0;
-                    if (kind == kSegI) {
-                        const long long nm = (long long)(px[k] - seg.x) * (seg.z - seg.x) +
-                                             (long long)(py - seg.y) * (seg.w - seg.y);
-                        ok = ok && nm > 0 && nm < den;
-                        num[k] = nm;
-                        d = fabsf((segf.z - segf.x) * (fy - segf.y) - (segf.w - segf.y) * (fx[k] - segf.x)) * seg_il;
-                    } else {
-                        ok = ok && (kind != kVert || in_cone(ct, cone, px[k] - gl.x, py - gl.y));
-                        const float ddx = fx[k] - gp.x, ddy = fy - gp.y;
-                        d = cf + sqrtf(ddx * ddx + ddy * ddy);
-                    }
-                    nk[k] = ((unsigned long long)__float_as_uint(d) << 32) | (unsigned)gc;
-                    if (ok && nk[k] < key[k]) want |= 1u << k;
-                    const int rx = px[k] - gl.x, ry = py - gl.y;
-                    // float products (|rx|, |ry| < 2^15: relative error below 2^-22,
-                    // inside the 1e-5 margins of the map tests below)
-                    r2[k] = fmaf((float)rx, (float)rx, (float)ry * (float)ry);
-                    const float a = (rx | ry) ? pang((float)rx, (float)ry) : 0.f;
-                    bA[k] = ((int)floorf((a - kAngEps) / kAngW) + kAngBins) & (kAngBins - 1);
-                    bB[k] = (int)floorf((a + kAngEps) / kAngW) & (kAngBins - 1);
-                }
-                if (MAPS && gmap) {
-                    float2 m0[PX], m1[PX];
-#pragma unroll
-                    for (int k = 0; k < PX; ++k) {
-                        m0[k] = make_float2(0.f, 0.f);
-                        m1[k] = m0[k];
-                        if ((want >> k) & 1u) {
-                            m0[k] = __ldg(gmap + bA[k]);
-                            m1[k] = __ldg(gmap + bB[k]);
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < PX; ++k) {
-                        if (!((want >> k) & 1u)) continue;
-                        SPM_CNT(14, 1);  // a pixel-candidate pair that needs a visibility decision
-                        if (px[k] == gl.x && py == gl.y) {  // the generator's own pixel
-                            key[k] = nk[k];
-                            continue;
-                        }
-                        if (r2[k] * (1.f - 1e-5f) >= fmaxf(m0[k].x, m1[k].x)) {  // hidden
-                            SPM_CNT(13, 1);
-                            continue;
-                        }
-                        if (r2[k] * (1.f + 1e-5f) < fminf(m0[k].y, m1[k].y)) {  // visible
-                            SPM_CNT(12, 1);
-                            key[k] = nk[k];
-                            continue;
-                        }
-                        need |= 1u << k;
-                    }
-                } else {
-                    need = want;
-                    SPM_CNT(14, __popc(want));
-                }
-                if (!__syncthreads_or(need != 0)) {
-                    SPM_LAP(4);
-                    continue;
-                }
-                SPM_LAP(4);
-                if (threadIdx.x == 0) SPM_CNT(5, 1);
-                // blockers of the hull of (tile, target)
-                float tx, ty;
-                if (kind == kSegI) {
-                    const float ux = (float)(seg.z - seg.x), uy = (float)(seg.w - seg.y);
-                    const float t = ((bcx - seg.x) * ux + (bcy - seg.y) * uy) / (ux * ux + uy * uy);
-                    tx = seg.x + t * ux;
-                    ty = seg.y + t * uy;
-                } else {
-                    tx = (float)gl.x;
-                    ty = (float)gl.y;
-                }
-                for (int w = threadIdx.x; w < kDedupBits / 32; w += NT) sm.dedup[w] = 0u;
-                if (threadIdx.x == 0) {
-                    sm.n_block = 0;
-                    sm.overflow = 0;
-                    if (kind != kSegI) sm.hull = hull_box_point(box, gl.x, gl.y);
-                }
-                __syncthreads();
-                build_blockers(ds, sm, bcx, bcy, tx, ty, brad, kind, gl, seg, box);
-                __syncthreads();
-                SPM_LAP(5);
-                const int nb = min(sm.n_block, kBlockCap);
-                const bool ovf = sm.overflow != 0;
-                if (threadIdx.x == 0) {
-                    SPM_CNT(6, nb);
-                    SPM_CNT(8, ovf ? 1 : 0);
-                    if (nb == 0) SPM_CNT(9, 1);
-                }
-                SPM_CNT(7, __popc(need));
-                const int nx = -(seg.w - seg.y), ny = seg.z - seg.x;
-#pragma unroll
-                for (int k = 0; k < PX; ++k) {
-                    if (!((need >> k) & 1u)) continue;
-                    bool vis;
-                    if (ovf) {
-                        vis = kind == kSegI ? visible_foot(ds, ds.gen_aux[gc], px[k], py, num[k], den)
-                                            : visible_points(ds, px[k], py, gl.x, gl.y);
-                    } else if (kind == kSegI) {
-                        vis = true;
-                        if (cross32(seg.z - seg.x, seg.w - seg.y, px[k] - seg.x, py - seg.y) != 0)
-                            for (int b = 0; b < nb && vis; ++b)
-                                vis = !poly_blocks_foot(sm.blk_v[b], sm.blk_m[b], sm.blk_oA[b], sm.blk_oB[b],
-                                                        px[k], py, num[k], den, nx, ny);
-                    } else {
-                        vis = true;
-                        if (px[k] != gl.x || py != gl.y)
-                            for (int b = 0; b < nb && vis; ++b)
-                            {
-                                vis = !poly_blocks(sm.blk_v[b], sm.blk_m[b], px[k], py, gl.x, gl.y, sm.blk_mask[b]);
-                                SPM_CNT(10, 1);
-                                SPM_CNT(11, sm.blk_m[b]);  // orientations of the polygon's edge pass
-                            }
-                    }
-                    if (vis) key[k] = nk[k];
-                }
-                __syncthreads();
-                SPM_LAP(6);
+            const unsigned bal = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const int slot = n + __popc(bal & ((1u << lane) - 1u));
+                ws.lb[slot] = lb;
+                ws.cand[slot] = c;
             }
-            // tile upper bound for the next batch's candidate pruning (worst
-            // best over live pixels); after the last batch nothing reads it
-            if (!last) {
-                float worst = 0.f;
+            n += __popc(bal);
+            const bool last = e0 + 32 >= total;
+            if (n > kWarpCand - 32 || (last && n > 0)) {
+                if (lane == 0) SPM_CNT(1, n);
+                apply_candidates(ds, ws, n, b);
+                n = 0;
+                if (!last) {
+                    float w = b.worst;
 #pragma unroll
-                for (int k = 0; k < PX; ++k)
-                    if ((live >> k) & 1u) worst = fmaxf(worst, key_dist(key[k]));
-                for (int o = 16; o > 0; o >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, o));
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    sm.n_cand = 0;
-                    sm.tile_ub = 0.f;
+                    for (int o = 16; o > 0; o >>= 1) w = fmaxf(w, __shfl_xor_sync(0xffffffffu, w, o));
+                    ub = w;
                 }
-                __syncthreads();
-                if ((threadIdx.x & 31) == 0) atomicMax((int *)&sm.tile_ub, __float_as_int(worst));
-                __syncthreads();
             }
         }
     }
-
-    if (j < ds.Ny) {
-        float od[PX];
-        int op[PX];
+    // 16-byte stores where every row of both planes starts on such a boundary
+    const bool vec = (ds.Nx & 3) == 0 && ((reinterpret_cast<size_t>(dist) | reinterpret_cast<size_t>(parent)) & 15) == 0;
 #pragma unroll
-        for (int k = 0; k < PX; ++k) {
-            const bool ok = ((live >> k) & 1u) && key[k] != kUnset;
-            od[k] = ok ? key_dist(key[k]) : INFINITY;
-            op[k] = ok ? (int)(unsigned)(key[k] & 0xffffffffu) : -1;
+    for (int h = 0; h < 2; ++h) {
+        if (b.j + 8 * h >= ds.Ny) continue;
+        float od[4];
+        int op[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            op[k] = ws.bi[(4 * h + k) * 32 + lane];
+            od[k] = op[k] >= 0 ? ws.bd[(4 * h + k) * 32 + lane] : INFINITY;
         }
-        const size_t base = (size_t)j * ds.Nx + i0 + c4;
-        if (PX == 4 && (ds.Nx & 3) == 0 && i0 + c4 + 3 < ds.Nx) {
-            *reinterpret_cast<float4 *>(dist + base) = make_float4(od[0], od[PX > 1 ? 1 : 0], od[PX > 2 ? 2 : 0], od[PX > 3 ? 3 : 0]);
-            *reinterpret_cast<int4 *>(parent + base) = make_int4(op[0], op[PX > 1 ? 1 : 0], op[PX > 2 ? 2 : 0], op[PX > 3 ? 3 : 0]);
+        const size_t base = (size_t)(b.j + 8 * h) * ds.Nx + b.i;
+        if (vec) {
+            if (b.i < ds.Nx) {
+                *reinterpret_cast<float4 *>(dist + base) = make_float4(od[0], od[1], od[2], od[3]);
+                *reinterpret_cast<int4 *>(parent + base) = make_int4(op[0], op[1], op[2], op[3]);
+            }
         } else {
-            for (int k = 0; k < PX; ++k)
-                if (i0 + c4 + k < ds.Nx) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (b.i + k < ds.Nx) {
                     dist[base + k] = od[k];
                     parent[base + k] = op[k];
                 }
         }
     }
-    SPM_LAP(7);
-    SPM_TFLUSH();
 }
 
-// One CTA per tile; one kernel per tile size, so each gets its own register
-// allocation (32 x 32 tiles: 4 pixels a thread, 16 x 16: 1).
-template <int PX, bool MAPS>
-__global__ void __launch_bounds__(NT, PX == 4 ? SPM_PIX32_MINB : SPM_PIX16_MINB) k_pixels(const __grid_constant__ DevScene ds,
-                                                                         float *__restrict__ dist,
-                                                                         int32_t *__restrict__ parent, int tile0) {
-    __shared__ PixSmem sm;
-    pixel_tile<PX, MAPS>(ds, tile0 + blockIdx.x, dist, parent, sm, true);
+#ifndef SPM_BLK_MINB
+#define SPM_BLK_MINB (24 / SPM_BLK_WARPS)  // resident CTAs per SM the kernel is compiled for
+#endif
+__global__ void __launch_bounds__(32 * kBlkWarps, SPM_BLK_MINB) k_pixel_blocks(const __grid_constant__ DevScene ds,
+                                                                               float *__restrict__ dist,
+                                                                               int32_t *__restrict__ parent, int tile0,
+                                                                               int tile1) {
+    __shared__ WarpSmem sm[kBlkWarps];
+    const int warp = threadIdx.x >> 5;
+    // a warp a block: four blocks to a 32-pixel tile, one to a 16-pixel one
+    const int per = ds.tile == kTile ? 4 : 1, blk = blockIdx.x * kBlkWarps + warp, t = tile0 + blk / per;
+    if (t < tile1) pixel_block(ds, t, blk % per, dist, parent, sm[warp]);
 }
 
-// Persistent form over a batch of scenes: each CTA takes the next
-// (scene, tile) from a global counter (costliest tiles first), copies
-// that scene's descriptor into shared memory and runs the same tile code.
-template <bool ANY_MAPS>  // some scene of the batch uses depth maps
-__global__ void __launch_bounds__(NT, SPM_PIXB_MINB) k_pixels_batched(const __grid_constant__ BatchDev b) {
-    __shared__ PixSmem sm;
-    __shared__ DevScene sds;
-    __shared__ int cur, cur_scene;
+// Persistent form over a batch of scenes: each warp takes the next
+// (scene, block) from a global counter (costliest tiles first), copies that
+// scene's descriptor into shared memory and runs the same code.
+__global__ void __launch_bounds__(32 * kBlkWarps, SPM_BLK_MINB) k_pixel_blocks_b(const __grid_constant__ BatchDev b) {
+    __shared__ WarpSmem sm[kBlkWarps];
+    __shared__ DevScene sds[kBlkWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    DevScene &ds = sds[warp];
+    int held = -1;
     for (;;) {
-        if (threadIdx.x == 0) {
-            const int t = atomicAdd(b.tile_counter, 1);
-            cur = t;
-            if (t < b.total_tiles) {
-                int lo = 0, hi = b.n;  // last order index with tile_off <= t
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (b.tile_off[mid] <= t) lo = mid;
-                    else hi = mid;
-                }
-                cur_scene = lo;
-            }
+        int t = 0;
+        if (lane == 0) t = atomicAdd(b.tile_counter, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= b.total_blocks) break;
+        int lo = 0, hi = b.n;  // last order index with blk_off <= t
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (__ldg(b.blk_off + mid) <= t) lo = mid;
+            else hi = mid;
         }
-        __syncthreads();
-        const int t = cur;
-        if (t >= b.total_tiles) break;
-        const int oi = cur_scene, sc = b.order[oi];
-        for (int w = threadIdx.x; w < (int)(sizeof(DevScene) / 4); w += NT)
-            reinterpret_cast<int *>(&sds)[w] = reinterpret_cast<const int *>(&b.scenes[sc])[w];
-        __syncthreads();
-        if (sds.tile == kTile) pixel_tile<4, ANY_MAPS>(sds, t - b.tile_off[oi], b.dist[sc], b.parent[sc], sm, true);
-        else pixel_tile<1, ANY_MAPS>(sds, t - b.tile_off[oi], b.dist[sc], b.parent[sc], sm, true);
-        __syncthreads();
+        const int sc = __ldg(b.order + lo), blk = t - __ldg(b.blk_off + lo);
+        if (sc != held) {
+            __syncwarp();
+            for (int w = lane; w < (int)(sizeof(DevScene) / 4); w += 32)
+                reinterpret_cast<int *>(&ds)[w] = __ldg(reinterpret_cast<const int *>(&b.scenes[sc]) + w);
+            __syncwarp();
+            held = sc;
+        }
+        const int per = ds.tile == kTile ? 4 : 1;
+        pixel_block(ds, blk / per, blk % per, b.dist[sc], b.parent[sc], sm[warp]);
     }
 }
 
@@ -844,13 +784,8 @@ void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_
     const int tiles = ds.tiles_x * (tile_row1 - tile_row0);
     if (tiles <= 0) return;
     const int t0 = tile_row0 * ds.tiles_x;
-    if (ds.use_maps && ds.gen_maps) {
-        if (ds.tile == kTile) k_pixels<4, true><<<tiles, NT, 0, st>>>(ds, dist, parent, t0);
-        else k_pixels<1, true><<<tiles, NT, 0, st>>>(ds, dist, parent, t0);
-    } else {
-        if (ds.tile == kTile) k_pixels<4, false><<<tiles, NT, 0, st>>>(ds, dist, parent, t0);
-        else k_pixels<1, false><<<tiles, NT, 0, st>>>(ds, dist, parent, t0);
-    }
+    const int grid = (tiles * (ds.tile == kTile ? 4 : 1) + kBlkWarps - 1) / kBlkWarps;
+    k_pixel_blocks<<<grid, 32 * kBlkWarps, 0, st>>>(ds, dist, parent, t0, t0 + tiles);
 }
 
 void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st) {
@@ -858,11 +793,9 @@ void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st) {
     int per_sm = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b.any_maps ? k_pixels_batched<true> : k_pixels_batched<false>,
-                                                  NT, 0);
-    const int grid = max(1, min(b.total_tiles, sms * max(per_sm, 1)));
-    if (b.any_maps) k_pixels_batched<true><<<grid, NT, 0, st>>>(b);
-    else k_pixels_batched<false><<<grid, NT, 0, st>>>(b);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pixel_blocks_b, 32 * kBlkWarps, 0);
+    const int grid = max(1, min((b.total_blocks + kBlkWarps - 1) / kBlkWarps, sms * max(per_sm, 1)));
+    k_pixel_blocks_b<<<grid, 32 * kBlkWarps, 0, st>>>(b);
 }
 
 int count_kernel_launches_pixel() { return 1; }

@@ -282,7 +282,9 @@ spm_status prepare_scene(const spm_scene_desc &d, HostScene &hs, std::string &er
         hs.poly_box[4 * k] = (int32_t)x0; hs.poly_box[4 * k + 1] = (int32_t)y0;
         hs.poly_box[4 * k + 2] = (int32_t)x1; hs.poly_box[4 * k + 3] = (int32_t)y1;
     }
-    // bins: about four per polygon, square, covering world and polygons
+    // bins: about four per polygon, square, covering world and polygons. A
+    // polygon is listed in every bin its box grown by one unit overlaps, so
+    // that a walk along a segment may be off by that much
     {
         i64 bx0 = lo_x * S - 1, by0 = lo_y * S - 1, bx1 = hi_x * S + 1, by1 = hi_y * S + 1;
         double area = (double)(bx1 - bx0) * (double)(by1 - by0);
@@ -300,8 +302,9 @@ spm_status prepare_scene(const spm_scene_desc &d, HostScene &hs, std::string &er
                 hs.bin_items.assign(hs.bin_start[nb], 0);
             }
             for (int k = 0; k < P; ++k) {
-                int cx0 = (int)((hs.poly_box[4 * k] - bx0) / bs), cx1 = (int)((hs.poly_box[4 * k + 2] - bx0) / bs);
-                int cy0 = (int)((hs.poly_box[4 * k + 1] - by0) / bs), cy1 = (int)((hs.poly_box[4 * k + 3] - by0) / bs);
+                // (the bins' own box has that margin already)
+                int cx0 = (int)((hs.poly_box[4 * k] - 1 - bx0) / bs), cx1 = (int)((hs.poly_box[4 * k + 2] + 1 - bx0) / bs);
+                int cy0 = (int)((hs.poly_box[4 * k + 1] - 1 - by0) / bs), cy1 = (int)((hs.poly_box[4 * k + 3] + 1 - by0) / bs);
                 for (int cy = cy0; cy <= cy1; ++cy)
                     for (int cx = cx0; cx <= cx1; ++cx) {
                         int c = cy * hs.bin_nx + cx;

@@ -436,11 +436,20 @@ __global__ void k_static_lengths(const __grid_constant__ DevScene ds, double *le
             len[e] = edge_len(ds, ds.st_src[e], ds.n_src + vv);
 }
 
-// The finalised table entry of generator g (the pixel pass reads FP32 costs).
+// The finalised table entry of generator g, whose cone is set already
+// (the pixel pass reads FP32 costs, packed with what it culls by).
 __device__ __forceinline__ void finalize_gen(const DevScene &ds, int g, double c, int p) {
     ds.gen_cost[g] = c;
     ds.gen_par[g] = p;
     ds.gen_costf[g] = (float)c;
+    const int kind = ds.gen_kind[g], ct = ds.gen_ctype[g];
+    const float2 w = ds.gen_pos[g];
+    ds.gen_rec[g] = make_float4(w.x, w.y, (float)c, __int_as_float(kind | ct << 3));
+    const int2 l = ds.gen_lat[g];
+    const int4 k = ds.gen_cone[g];
+    auto pack = [](int x, int y) { return (x & 0xffff) | y << 16; };
+    const float cull = kind == kSegI ? -1.f : ct == kConeEmpty ? INFINITY : (float)c;
+    ds.gen_cull[g] = make_int4(pack(l.x, l.y), pack(k.x, k.y), pack(k.z, k.w), __float_as_int(cull));
 }
 
 // Jacobi rounds of the fixpoint on the whole GPU (cooperative launch, two

@@ -1032,3 +1032,40 @@ def test_source_snapping_effect_at_config_size(spm, oracle_mod):
     assert rel.max() <= 1e-4
     # where the label differs the distance is the same path length
     assert np.all(np.abs(gd[hard].astype(np.float64) - rd[hard]) <= 1e-3)
+
+
+@pytest.mark.parametrize("tile", [16, 32])
+@pytest.mark.parametrize("n", [1, 5, 16, 17, 33, 63])
+def test_pixel_blocks_at_their_edges(spm, oracle_mod, n, tile):
+    """The pixel pass's 16 x 16 blocks on grids that end inside, at and just
+    beyond a block, rows that are and are not a multiple of a 16-byte store,
+    output planes that start off a 16-byte boundary, with depth maps (block and
+    pixel decisions), without (every pixel tested exactly) and without lists;
+    a polygon cluster dense enough that a block lists many blockers."""
+    rng = np.random.default_rng(n)
+    W = 16 * n
+    polys = []
+    for _ in range(3 if n < 16 else 60):  # small, possibly overlapping triangles
+        x, y = rng.integers(2, W - 7, 2)
+        polys.append(np.array([(x, y), (x + int(rng.integers(3, 6)), y + 1), (x + 1, y + int(rng.integers(3, 6)))]))
+    keep = []
+    for p in polys:  # no shared points: triangles whose boxes stay apart
+        if all(p[:, 0].min() > q[:, 0].max() + 1 or p[:, 0].max() < q[:, 0].min() - 1 or
+               p[:, 1].min() > q[:, 1].max() + 1 or p[:, 1].max() < q[:, 1].min() - 1 for q in keep):
+            keep.append(p)
+    scene = sg.Scene((W, W), (n, n + 2 if n == 16 else n), keep, [(1.0, 1.0)], [(0.0, W - 1.0, W - 1.0, W - 1.0)])
+    if scene.grid[1] != n:
+        scene = sg.Scene((W, 16 * scene.grid[1]), scene.grid, keep, scene.points, scene.segs)
+    rd, rp, rd2, rp2 = oracle_mod.Oracle(scene).field()
+    s = spm.Scene(scene)
+    Nx, Ny = scene.grid
+    for mode, maps in ((3, 1), (1, 1), (3, 0), (0, 0), (2, 0)):
+        spm.spm_scene_set_tuning(s.handle, mode, 32, tile, maps)
+        flat_d = torch.full((Nx * Ny + 1,), -5.0, device="cuda")
+        flat_p = torch.full((Nx * Ny + 1,), -5, dtype=torch.int32, device="cuda")
+        for off in (0, 1):
+            d, p = flat_d[off:off + Nx * Ny], flat_p[off:off + Nx * Ny]
+            s.compute(d, p)
+            s.sync()
+            check_parity(scene, d.cpu().numpy().reshape(Ny, Nx), p.cpu().numpy().reshape(Ny, Nx), rd, rp, rd2,
+                         f"blocks n={n} tile={tile} mode={mode} maps={maps} off={off}", rp2)
