@@ -30,61 +30,27 @@ __device__ __forceinline__ int orient32(int ax, int ay, int bx, int by, int cx, 
 }
 __device__ __forceinline__ int cross32(int ax, int ay, int bx, int by) { return ax * by - ay * bx; }
 
-// Open segment p->q against the open interior of convex CCW polygon V[0..m).
-// Separating-axis test on the segment and the polygon (both convex): they are
-// disjoint in the interiors iff some outward edge normal of the polygon or the
-// normal of the segment weakly separates them, i.e. (a) both endpoints lie on
-// the closed outer side of one edge line, or (b) all polygon vertices lie on
-// one closed side of the line pq. maskQ carries bit i = [orient(e_i, q) > 0].
-__device__ __forceinline__ bool poly_blocks(const int2 *V, int m, int px, int py, int qx, int qy,
-                                            unsigned maskQ) {
-    unsigned mp = 0;
-    int2 a = V[m - 1];
-#pragma unroll 4
-    for (int i = 0; i < m; ++i) {
-        int2 b = V[i];
-        // edge (a -> b) is edge index m-1 for i == 0, else i-1
-        int e = (i == 0) ? m - 1 : i - 1;
-        if (orient32(a.x, a.y, b.x, b.y, px, py) > 0) mp |= 1u << e;
-        a = b;
-    }
-    if ((mp | maskQ) != ((1u << m) - 1u)) return false;
-    const int dx = qx - px, dy = qy - py;
-    bool pos = false, neg = false;
-#pragma unroll 4
-    for (int i = 0; i < m; ++i) {
-        int s = dx * (V[i].y - py) - dy * (V[i].x - px);
-        pos |= s > 0;
-        neg |= s < 0;
-    }
-    return pos && neg;
-}
-
-// Same test with q = perpendicular foot of p on segment source A->B = seg
+// The same test with q = perpendicular foot of p on segment source A->B = seg
 // (Sec. 4), f = A + (num/den)(B - A), 0 < num < den: orient(e_i, f) has the
 // sign of (den - num) * orient(e_i, A) + num * orient(e_i, B) (int64). The
 // line p->f is parallel to perp(B - A).
 __device__ __forceinline__ bool foot_meets_poly(const int2 *V, int m, int4 seg, int px, int py, long long num,
                                                 long long den) {
     const int nx = -(seg.w - seg.y), ny = seg.z - seg.x;
-    bool pos = false, neg = false;
+    bool pos = false, neg = false, apart = false;
+    int2 a = __ldg(V + m - 1);
+#pragma unroll 1
     for (int i = 0; i < m; ++i) {
-        const int2 a = V[i];
-        const int s = nx * (a.y - py) - ny * (a.x - px);
+        const int2 b = __ldg(V + i);
+        const int s = nx * (b.y - py) - ny * (b.x - px);
         pos |= s > 0;
         neg |= s < 0;
-    }
-    if (!(pos && neg)) return false;
-    int2 a = V[m - 1];
-    for (int i = 0; i < m; ++i) {
-        const int2 b = V[i];
-        if (orient32(a.x, a.y, b.x, b.y, px, py) <= 0 &&
-            (den - num) * (long long)orient32(a.x, a.y, b.x, b.y, seg.x, seg.y) +
-                    num * (long long)orient32(a.x, a.y, b.x, b.y, seg.z, seg.w) <= 0)
-            return false;
+        apart |= orient32(a.x, a.y, b.x, b.y, px, py) <= 0 &&
+                 (den - num) * (long long)orient32(a.x, a.y, b.x, b.y, seg.x, seg.y) +
+                         num * (long long)orient32(a.x, a.y, b.x, b.y, seg.z, seg.w) <= 0;
         a = b;
     }
-    return true;
+    return pos && neg && !apart;
 }
 
 // Cone membership of direction w for a vertex generator: wedge cones are the
@@ -187,42 +153,42 @@ __device__ __forceinline__ bool walk_bins(const DevScene &ds, float px, float py
     return false;
 }
 
-// Does the open segment p->q meet the open interior of convex polygon V[0..m)?
-// The predicate of poly_blocks, the side test first: most polygons near a
-// segment lie on one side of its line.
+// Does the open segment p->q meet the open interior of convex CCW polygon
+// V[0..m)? Separating-axis test on the segment and the polygon (both convex):
+// they are disjoint in the interiors iff some outward edge normal of the
+// polygon or the normal of the segment weakly separates them, i.e. (a) all
+// polygon vertices lie on one closed side of the line pq, or (b) both endpoints
+// lie on the closed outer side of one edge line. One short loop: the pixel
+// kernel's speed hangs on its code staying in the instruction caches.
 __device__ __forceinline__ bool segment_meets_poly(const int2 *V, int m, int px, int py, int qx, int qy) {
     const int dx = qx - px, dy = qy - py;
-    bool pos = false, neg = false;
-#pragma unroll 4
-    for (int i = 0; i < m; ++i) {
-        const int2 a = __ldg(V + i);
-        const int s = dx * (a.y - py) - dy * (a.x - px);
-        pos |= s > 0;
-        neg |= s < 0;
-    }
-    if (!(pos && neg)) return false;
-    bool apart = false;  // an edge has both ends on its closed outer side
+    bool pos = false, neg = false, apart = false;
     int2 a = __ldg(V + m - 1);
-#pragma unroll 4
+#pragma unroll 2
     for (int i = 0; i < m; ++i) {
         const int2 b = __ldg(V + i);
-        apart |= orient32(a.x, a.y, b.x, b.y, px, py) <= 0 && orient32(a.x, a.y, b.x, b.y, qx, qy) <= 0;
+        const int s = dx * (b.y - py) - dy * (b.x - px);
+        pos |= s > 0;
+        neg |= s < 0;
+        const int ex = b.x - a.x, ey = b.y - a.y;
+        apart |= ex * (py - a.y) - ey * (px - a.x) <= 0 && ex * (qy - a.y) - ey * (qx - a.x) <= 0;
         a = b;
     }
-    return !apart;
+    return pos && neg && !apart;
 }
 
-// Exact visibility between lattice point p and generator target q (a point),
-// one thread: walks the bins the segment crosses, cell to cell, and tests
-// every polygon there. Only the first share `part` of the segment from p is
-// walked: 1, or less when no obstacle is met beyond it (a polygon that blocks
-// the segment then meets that part, and is listed in one of its bins). The
-// float steps are off by far less than the unit the polygons' boxes are grown
-// by when they are binned. (A walk by columns with both their row ranges,
-// grown by a margin, took four divisions a column and visited about 1.6 x
-// the bins.)
-__device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int py, int qx, int qy, float part = 1.f) {
-    if (px == qx && py == qy) return true;
+// Calls f(V, m) for every polygon that blocks the open segment between lattice
+// points p and q (its open interior meets it) until f returns true; returns
+// whether one did. One thread: walks the bins the segment crosses, cell to
+// cell. Only the first share `part` of the segment from p is walked: 1, or
+// less when no obstacle is met beyond it (a polygon that blocks the segment
+// then meets that part, and is listed in one of its bins). The float steps are
+// off by far less than the unit the polygons' boxes are grown by when they are
+// binned. (A walk by columns with both their row ranges, grown by a margin,
+// took four divisions a column and visited more bins: vertex phase of the
+// 1024^2 polygons 0.106 -> 0.092 ms.)
+template <class F>
+__device__ __forceinline__ bool walk_blockers(const DevScene &ds, int px, int py, int qx, int qy, float part, F &&f) {
     const float dx = (float)(qx - px), dy = (float)(qy - py);
     const float u = (float)(px - ds.bin_x0) * ds.bin_inv, v = (float)(py - ds.bin_y0) * ds.bin_inv;
     const float du = dx * part * ds.bin_inv, dv = dy * part * ds.bin_inv;
@@ -250,9 +216,9 @@ __device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int p
             if (fabsf(dx * my - dy * mx) > reach) continue;
             const int4 rec = __ldg(rp + 1);
             SPM_CNT(25, 1);  // a polygon tested
-            if (segment_meets_poly(ds.poly_v + rec.y, rec.z, px, py, qx, qy)) return false;
+            if (segment_meets_poly(ds.poly_v + rec.y, rec.z, px, py, qx, qy) && f(ds.poly_v + rec.y, rec.z)) return true;
         }
-        if (left <= 0) return true;
+        if (left <= 0) return false;
         if (tx < ty) {
             cx += sx;
             nx += (float)sx;
@@ -263,6 +229,29 @@ __device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int p
             ty = cy == ey ? INFINITY : fabsf(ny - v) * iy;
         }
     }
+}
+
+// Exact visibility between lattice point p and generator target q (a point),
+// one thread.
+__device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int py, int qx, int qy) {
+    if (px == qx && py == qy) return true;
+    return !walk_blockers(ds, px, py, qx, qy, 1.f, [](const int2 *, int) { return true; });
+}
+
+// Does one polygon hide every point of the box from the point generator at
+// lattice point g? The set of points whose open segment to g meets a convex
+// polygon's interior is convex, so it suffices that it hides the four corners;
+// such a polygon also blocks any one point of the box, here one near its centre.
+__device__ __forceinline__ bool box_hidden(const DevScene &ds, int4 box, int2 g) {
+    const int cx = (box.x + box.z) >> 1, cy = (box.y + box.w) >> 1;
+    if (cx == g.x && cy == g.y) return false;
+    return walk_blockers(ds, cx, cy, g.x, g.y, 1.f, [&](const int2 *V, int m) {
+        bool all = true;
+#pragma unroll 1
+        for (int k = 0; k < 4 && all; ++k)
+            all = segment_meets_poly(V, m, k & 1 ? box.z : box.x, k & 2 ? box.w : box.y, g.x, g.y);
+        return all;
+    });
 }
 
 // Exact visibility between lattice point p and its perpendicular foot on

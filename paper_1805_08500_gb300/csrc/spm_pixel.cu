@@ -26,6 +26,8 @@
 //     16-byte store per plane (dist, parent).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "spm_device.cuh"
 #include "spm_internal.h"
 
@@ -40,38 +42,27 @@ constexpr int NT = kPixelThreads;  // threads of the free-space mask's CTAs
 __device__ __forceinline__ float segment_lower_bound(const DevScene &ds, int s, int4 box, float4 fbox) {
     const int4 L = ds.seg_lat[s];
     const long long ux = L.z - L.x, uy = L.w - L.y, den = ux * ux + uy * uy;
-    bool all_lo = true, all_hi = true;
-    const int cx[4] = {box.x, box.z, box.x, box.z}, cy[4] = {box.y, box.y, box.w, box.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const long long num = (cx[k] - L.x) * ux + (cy[k] - L.y) * uy;
-        all_lo &= num <= 0;
-        all_hi &= num >= den;
-    }
-    if (all_lo || all_hi) return -1.f;
+    bool all_lo = true, all_hi = true, pos = false, neg = false;
     const float4 F = ds.seg_pos[s];
     const float fx = F.z - F.x, fy = F.w - F.y, il = rsqrtf(fx * fx + fy * fy);
-    const float qx[4] = {fbox.x, fbox.z, fbox.x, fbox.z}, qy[4] = {fbox.y, fbox.y, fbox.w, fbox.w};
     float mn = INFINITY;
-    bool pos = false, neg = false;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float sd = (fx * (qy[k] - F.y) - fy * (qx[k] - F.x)) * il;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {  // the box's corners
+        const long long num = ((k & 1 ? box.z : box.x) - L.x) * ux + ((k & 2 ? box.w : box.y) - L.y) * uy;
+        all_lo &= num <= 0;
+        all_hi &= num >= den;
+        const float sd = (fx * ((k & 2 ? fbox.w : fbox.y) - F.y) - fy * ((k & 1 ? fbox.z : fbox.x) - F.x)) * il;
         pos |= sd > 0.f;
         neg |= sd < 0.f;
         mn = fminf(mn, fabsf(sd));
     }
+    if (all_lo || all_hi) return -1.f;
     return (pos && neg) ? 0.f : mn * 0.999999f;
 }
 
 // ---------------------------------------------------------------------------
-// One warp, one block of 16 x 16 pixels (eight pixels a lane), no barrier.
+// One warp, one block of pixels (16 x 16, smaller on small grids), no barrier.
 // ---------------------------------------------------------------------------
-constexpr int kBlk = 16;         // block side in pixels
-#ifndef SPM_BLK_WARPS
-#define SPM_BLK_WARPS 4
-#endif
-constexpr int kBlkWarps = SPM_BLK_WARPS;  // warps (blocks) per CTA
 constexpr int kWarpCand = 96;    // candidates a warp holds before it works them off
 constexpr int kWarpPoly = 64;    // blocker polygons a warp lists at a time
 constexpr int kBlocked = 1 << 15; // an undecided pixel found blocked
@@ -84,20 +75,30 @@ constexpr int kCandMap = 1 << 21;     // its depth map is complete
 // The pixels' state lives in shared memory (a lane's eight pixels at
 // k * 32 + lane), not in registers: the loops over them stay rolled, nothing
 // spills around the exact tests, and more warps are resident.
+template <int PX, int PY>
+struct Shape {                       // a lane's pixels: PX consecutive ones of PY rows
+    static constexpr int kPix = PX * PY;
+    static constexpr int kRow = PX == 1 ? 8 : 4;                  // lanes across the block
+    static constexpr int kW = PX * kRow, kH = PY * (32 / kRow);   // block size in pixels
+};
+
+template <int N>  // pixels a lane
 struct WarpSmem {
-    float bd[256];               // best distance so far (-inf: not a free pixel of the grid)
-    int bi[256];                 // and its generator
+    float bd[32 * N];            // best distance so far (-inf: not a free pixel of the grid)
+    int bi[32 * N];              // and its generator
+    float d[32 * N];             // the candidate's distances
     float lb[kWarpCand];         // candidates: least cost + distance over the block
     int cand[kWarpCand];         // generator id and flags
     int3 poly[kWarpPoly];        // blocker polygons: id, first vertex, vertices
-    unsigned short item[256];    // undecided pixels, lane * 8 + k, and kBlocked
+    unsigned short item[32 * N]; // undecided pixels, lane * N + k, and kBlocked
 };
 
-// One warp's block of pixels. A lane holds four consecutive pixels (k & 3) of
-// rows lane / 4 and lane / 4 + 8 (k >> 2).
+// One warp's block of pixels. A lane holds PX consecutive pixels (k % PX) of
+// PY rows, 32 / kRow apart (k / PX).
 struct Block {
     int4 box;    // lattice box of its pixel centres
     int i0, j0;  // its first pixel
+    int i1, j1;  // its last pixel within the grid
     int i, j;    // the lane's first pixel
     float worst; // largest best distance of the lane's pixels
     bool lists;  // the candidates come from flooded lists
@@ -117,8 +118,7 @@ __device__ __forceinline__ bool block_candidate(const DevScene &ds, int g, const
     const int4 box = b.box;
     cand = g;
     if (cost < 0.f) {  // a segment interior
-        const float4 fbox = make_float4(pixel_x(ds, b.i0), pixel_y(ds, b.j0), pixel_x(ds, min(b.i0 + kBlk, ds.Nx) - 1),
-                                        pixel_y(ds, min(b.j0 + kBlk, ds.Ny) - 1));
+        const float4 fbox = make_float4(pixel_x(ds, b.i0), pixel_y(ds, b.j0), pixel_x(ds, b.i1), pixel_y(ds, b.j1));
         lb = segment_lower_bound(ds, ds.gen_aux[g], box, fbox);
         return lb >= 0.f && lb <= ub;
     }
@@ -126,7 +126,8 @@ __device__ __forceinline__ bool block_candidate(const DevScene &ds, int g, const
     const int x0 = box.x - l.x, x1 = box.z - l.x, y0 = box.y - l.y, y1 = box.w - l.y;
     const float dx = (float)max(max(x0, -x1), 0), dy = (float)max(max(y0, -y1), 0);
     // a source lies within a lattice unit of its lattice point, a vertex on it
-    const float d = sqrtf(dx * dx + dy * dy) - (g < ds.n_src ? 1.f : 0.f);
+    const float d2 = fmaf(dx, dx, dy * dy);
+    const float d = d2 * rsqrtf(fmaxf(d2, 1e-20f)) - (g < ds.n_src ? 1.f : 0.f);
     lb = (cost + fmaxf(d, 0.f) * ds.inv_S) * 0.999999f;
     // cross(c1, w) and cross(w, c2) are linear in w: their extremes over the
     // box lie at the corners their signs choose (no cone: all zero)
@@ -194,16 +195,17 @@ __device__ __forceinline__ int2 pixel_bins(float rx, float ry) {
 // the segment source: the other pixels' segments are its translates) and, for
 // a point, that no edge of theirs separates from the hull of the block's box
 // and the generator. They are listed kWarpPoly at a time, and each list is
-// tested against the undecided pixels, packed a lane each. Without flooded
-// lists a polygon that hides all four corners of the block's box hides the
-// block (the region a convex polygon hides is convex).
+// tested against the undecided pixels, packed a lane each.
 // Every step is one load deep for the whole warp: a lane takes a bin of the
 // segment, then the bins' records are dealt to the lanes evenly, then a lane
 // takes a listed polygon. (Lanes walking bins of their own, record by record
 // and vertex by vertex, waited on some 80 loads in a row: 57k cycles a list on
 // the 2048^2 maze.)
-__device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem &ws, const Block &b, int2 gl, int seg_id,
+template <int PX, int PY>
+__device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem<PX * PY> &ws, const Block &b, int2 gl, int seg_id,
                                                    float clear, unsigned und) {
+    using S = Shape<PX, PY>;
+    constexpr int N = S::kPix;
     const int lane = threadIdx.x & 31;
     if (lane == 0) SPM_CNT(5, 1);
     SPM_CNT(7, __popc(und));
@@ -220,7 +222,7 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem 
     __syncwarp();
     {
         int p = at;
-        for (unsigned m = und; m; m &= m - 1) ws.item[p++] = (unsigned short)(lane * 8 + __ffs(m) - 1);
+        for (unsigned m = und; m; m &= m - 1) ws.item[p++] = (unsigned short)(lane * N + __ffs(m) - 1);
     }
     const int4 box = b.box;
     const float cx = 0.5f * ((float)box.x + (float)box.z), cy = 0.5f * ((float)box.y + (float)box.w);
@@ -228,7 +230,7 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem 
     if (seg_id >= 0) {
         const int4 seg = ds.seg_lat[seg_id];
         const float fux = (float)(seg.z - seg.x), fuy = (float)(seg.w - seg.y);
-        const float t = ((cx - seg.x) * fux + (cy - seg.y) * fuy) / (fux * fux + fuy * fuy);
+        const float t = __fdividef((cx - seg.x) * fux + (cy - seg.y) * fuy, fux * fux + fuy * fuy);
         dx = seg.x + t * fux - cx;
         dy = seg.y + t * fuy - cy;
     } else {
@@ -241,7 +243,7 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem 
         dy *= part;
     }
     const float ex = (float)(box.z - box.x), ey = (float)(box.w - box.y);
-    const float m = 0.5f * sqrtf(ex * ex + ey * ey) + 2.0f;  // half the segment's thickness
+    const float m = 0.5f * (ex * ex + ey * ey) * rsqrtf(fmaxf(ex * ex + ey * ey, 1.f)) + 2.0f;  // half the segment's thickness
     const float bs = (float)ds.bin_size, ibs = ds.bin_inv;
     auto col_of = [&](float v) { return min(max((int)floorf((v - (float)ds.bin_x0) * ibs), 0), ds.bin_nx - 1); };
     auto row_of = [&](float v) { return min(max((int)floorf((v - (float)ds.bin_y0) * ibs), 0), ds.bin_ny - 1); };
@@ -319,7 +321,6 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem 
         if (lane == 0) SPM_CNT(6, n);
         // the listed polygons against the undecided pixels
         if (seg_id < 0) {
-            bool hides = false;
             int kept = 0;
             for (int q0 = 0; q0 < n; q0 += 32) {
                 bool keep = false;
@@ -328,24 +329,16 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem 
                     pl = ws.poly[q0 + lane];
                     const int2 *V = ds.poly_v + pl.y;
                     bool apart = false;
-                    unsigned mask = 0;
                     int2 a = __ldg(V + pl.z - 1);
-#pragma unroll 4
+#pragma unroll 2
                     for (int i = 0; i < pl.z; ++i) {
                         const int2 e = __ldg(V + i);
                         const int nx = -(e.y - a.y), ny = e.x - a.x;  // orient(a, e, p) = n . (p - a)
                         const int far = nx * ((nx > 0 ? box.z : box.x) - a.x) + ny * ((ny > 0 ? box.w : box.y) - a.y);
-                        const bool in = nx * (gl.x - a.x) + ny * (gl.y - a.y) > 0;
-                        if (in) mask |= 1u << (i == 0 ? pl.z - 1 : i - 1);
-                        apart |= !in && far <= 0;
+                        apart |= far <= 0 && nx * (gl.x - a.x) + ny * (gl.y - a.y) <= 0;
                         a = e;
                     }
                     keep = !apart;
-                    if (keep && !b.lists)
-                        hides |= poly_blocks(V, pl.z, box.x, box.y, gl.x, gl.y, mask) &&
-                                 poly_blocks(V, pl.z, box.z, box.y, gl.x, gl.y, mask) &&
-                                 poly_blocks(V, pl.z, box.x, box.w, gl.x, gl.y, mask) &&
-                                 poly_blocks(V, pl.z, box.z, box.w, gl.x, gl.y, mask);
                 }
                 const unsigned bal = __ballot_sync(0xffffffffu, keep);
                 __syncwarp();
@@ -354,13 +347,12 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem 
                 __syncwarp();
             }
             n = kept;
-            if (__any_sync(0xffffffffu, hides)) return 0u;
         }
         for (int e = lane; e < n_item && n > 0; e += 32) {
-            const int it = ws.item[e], l = it >> 3, k = it & 7;
+            const int it = ws.item[e], l = it / N, k = it % N;
             if (it & kBlocked) continue;
-            const int px = ds.pitch_x * (b.i0 + (l & 3) * 4 + (k & 3)) + ds.pitch_x / 2;
-            const int py = ds.pitch_y * (b.j0 + (l >> 2) + (k >> 2) * 8) + ds.pitch_y / 2;
+            const int px = ds.pitch_x * (b.i0 + l % S::kRow * PX + k % PX) + ds.pitch_x / 2;
+            const int py = ds.pitch_y * (b.j0 + l / S::kRow + k / PX * (32 / S::kRow)) + ds.pitch_y / 2;
             bool v = true;
             if (seg_id < 0) {
                 if (px != gl.x || py != gl.y)
@@ -389,7 +381,9 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem 
 }
 
 // Candidate c against the block's pixels.
-__device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem &ws, Block &b, int c) {
+template <int PX, int PY>
+__device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX * PY> &ws, Block &b, int c) {
+    constexpr int kStep = 32 / Shape<PX, PY>::kRow;  // rows between a lane's pixels
     const int lane = threadIdx.x & 31, g = c & kCandId;
     const float4 rec = __ldg(ds.gen_rec + g);
     const int4 q = __ldg(ds.gen_cull + g);
@@ -408,7 +402,7 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem &ws
         il = 1.0f / sqrtf(fux * fux + fuy * fuy);
     }
     auto dist_at = [&](int k) {
-        const float fx = pixel_x(ds, b.i + (k & 3)), fy = pixel_y(ds, b.j + (k >> 2) * 8);
+        const float fx = pixel_x(ds, b.i + k % PX), fy = pixel_y(ds, b.j + k / PX * kStep);
         return seg ? fabsf((sf.z - sf.x) * (fy - sf.y) - (sf.w - sf.y) * (fx - sf.x)) * il
                    : point_dist(rec.z, fx - rec.x, fy - rec.y);
     };
@@ -416,16 +410,18 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem &ws
     unsigned want = 0;
     float worst = -INFINITY;
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < PY; ++h) {
 #pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4) {
-            const int k = 4 * h + k4, at = k * 32 + lane;
+        for (int k4 = 0; k4 < PX; ++k4) {
+            const int k = PX * h + k4, at = k * 32 + lane;
             const float d = dist_at(k);
             float old = ws.bd[at];
             bool better = d < old;
             if (d == old) better = g < ws.bi[at];
             if (better) want |= 1u << k;
-            if (take_all && better) {
+            if (!take_all) {
+                ws.d[at] = d;
+            } else if (better) {
                 ws.bd[at] = d;
                 ws.bi[at] = g;
                 old = d;
@@ -447,8 +443,8 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem &ws
 #pragma unroll 1
         for (unsigned m = want; m; m &= m - 1) {
             const int k = __ffs(m) - 1;
-            const int px = ds.pitch_x * (b.i + (k & 3)) + ds.pitch_x / 2;
-            const int py = ds.pitch_y * (b.j + (k >> 2) * 8) + ds.pitch_y / 2;
+            const int px = ds.pitch_x * (b.i + k % PX) + ds.pitch_x / 2;
+            const int py = ds.pitch_y * (b.j + k / PX * kStep) + ds.pitch_y / 2;
             const long long nm = (px - L.x) * ux + (py - L.y) * uy;
             if (nm > 0 && nm < den) und |= m & -m;
         }
@@ -456,27 +452,31 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem &ws
         const int4 cone = make_int4((short)q.y, q.y >> 16, (short)q.z, q.z >> 16);
         const int ct = (__float_as_int(rec.w) >> 3) & 3;
 #pragma unroll 1
-        for (unsigned m = want; m; m &= m - 1) {
-            const int k = __ffs(m) - 1;
-            const int ix = rx0 + (k & 3) * ds.pitch_x, iy = ry0 + (k >> 2) * 8 * ds.pitch_y;
-            if (!(c & kCandInCone) && !in_cone(ct, cone, ix, iy)) continue;
-            if (cls == 0) {
-                vis |= m & -m;
-            } else if (!map) {
-                und |= m & -m;
-            } else {
-                const float rx = (float)ix, ry = (float)iy, r2 = fmaf(rx, rx, ry * ry);
-                const int2 bin = pixel_bins(rx, ry);
-                const float2 m0 = __ldg(map + bin.x), m1 = __ldg(map + bin.y);
-                const float low = fminf(m0.y, m1.y);
-                if (r2 == 0.f || r2 * (1.f + 1e-5f) < low) {  // visible (or the generator's own pixel)
-                    SPM_CNT(12, 1);
-                    vis |= m & -m;
-                } else if (r2 * (1.f - 1e-5f) < fmaxf(m0.x, m1.x)) {
-                    und |= m & -m;
-                    clear = fminf(clear, low);
-                } else {  // hidden
-                    SPM_CNT(13, 1);
+        for (int h = 0; h < PY; ++h) {
+#pragma unroll
+            for (int k4 = 0; k4 < PX; ++k4) {
+                const unsigned bit = 1u << (PX * h + k4);
+                if (!(want & bit)) continue;
+                const int ix = rx0 + k4 * ds.pitch_x, iy = ry0 + h * kStep * ds.pitch_y;
+                if (!(c & kCandInCone) && !in_cone(ct, cone, ix, iy)) continue;
+                if (cls == 0) {
+                    vis |= bit;
+                } else if (!map) {
+                    und |= bit;
+                } else {
+                    const float rx = (float)ix, ry = (float)iy, r2 = fmaf(rx, rx, ry * ry);
+                    const int2 bin = pixel_bins(rx, ry);
+                    const float2 m0 = __ldg(map + bin.x), m1 = __ldg(map + bin.y);
+                    const float low = fminf(m0.y, m1.y);
+                    if (r2 == 0.f || r2 * (1.f + 1e-5f) < low) {  // visible (or the generator's own pixel)
+                        SPM_CNT(12, 1);
+                        vis |= bit;
+                    } else if (r2 * (1.f - 1e-5f) < fmaxf(m0.x, m1.x)) {
+                        und |= bit;
+                        clear = fminf(clear, low);
+                    } else {  // hidden
+                        SPM_CNT(13, 1);
+                    }
                 }
             }
         }
@@ -484,31 +484,33 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem &ws
     if (__any_sync(0xffffffffu, und)) {
         // squared distances are non-negative: they order as their bits
         const float near = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(clear)));
-        vis |= resolve_pixels(ds, ws, b, gl, seg_id, map ? sqrtf(near) : 0.f, und);
+        vis |= resolve_pixels<PX, PY>(ds, ws, b, gl, seg_id, map ? sqrtf(near) : 0.f, und);
     }
     if (vis) {
 #pragma unroll 1
         for (unsigned m = vis; m; m &= m - 1) {
             const int k = __ffs(m) - 1;
-            ws.bd[k * 32 + lane] = dist_at(k);
+            ws.bd[k * 32 + lane] = ws.d[k * 32 + lane];
             ws.bi[k * 32 + lane] = g;
         }
         worst = -INFINITY;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) worst = fmaxf(worst, ws.bd[k * 32 + lane]);
+        for (int k = 0; k < PX * PY; ++k) worst = fmaxf(worst, ws.bd[k * 32 + lane]);
         b.worst = worst;
     }
 }
 
 // The n candidates the warp holds, in order of their lower bounds, until none
 // can improve a pixel.
-__device__ __forceinline__ void apply_candidates(const DevScene &ds, WarpSmem &ws, int n, Block &b) {
+template <int PX, int PY, bool SCAN>
+__device__ __forceinline__ void apply_candidates(const DevScene &ds, WarpSmem<PX * PY> &ws, int n, Block &b) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
     unsigned l[kWarpCand / 32];
 #pragma unroll
     for (int k = 0; k < kWarpCand / 32; ++k)
         l[k] = lane + 32 * k < n ? __float_as_uint(ws.lb[lane + 32 * k]) : 0xffffffffu;
+    bool tested = false;
     for (;;) {
         unsigned mine = l[0];
 #pragma unroll
@@ -528,37 +530,63 @@ __device__ __forceinline__ void apply_candidates(const DevScene &ds, WarpSmem &w
         }
         c = __shfl_sync(0xffffffffu, c, from);
         if (lane == 0) SPM_CNT(4, 1);
-        apply_candidate(ds, ws, b, ws.cand[32 * c + from]);
+        apply_candidate<PX, PY>(ds, ws, b, ws.cand[32 * c + from]);
+        if (SCAN && !b.lists && !tested) {
+            // flooded lists were tested on the tile's area; a scan's candidates
+            // that one polygon hides from the block go here, a lane each,
+            // after the first has set a bound to what the rest are good for
+            tested = true;
+            const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(b.worst, 0.f))));
+#pragma unroll 1
+            for (int k = 0; k < kWarpCand / 32; ++k) {
+                unsigned lk = l[0];
+#pragma unroll
+                for (int q = 1; q < kWarpCand / 32; ++q) lk = q == k ? l[q] : lk;
+                if (lk == 0xffffffffu || !(__uint_as_float(lk) < most)) continue;
+                const int g = ws.cand[lane + 32 * k] & kCandId;
+                const int4 q4 = __ldg(ds.gen_cull + g);
+                const bool hidden = !(__int_as_float(q4.w) < 0.f) &&
+                                    box_hidden(ds, b.box, make_int2((short)q4.x, q4.x >> 16));
+#pragma unroll
+                for (int q = 0; q < kWarpCand / 32; ++q)
+                    if (q == k && hidden) l[q] = 0xffffffffu;
+            }
+        }
     }
     __syncwarp();
 }
 
-__device__ __forceinline__ void pixel_block(const DevScene &ds, const int tile, const int sub, float *__restrict__ dist,
-                                            int32_t *__restrict__ parent, WarpSmem &ws) {
+template <int PX, int PY, bool SCAN>
+__device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, const int j0, float *__restrict__ dist,
+                                            int32_t *__restrict__ parent, WarpSmem<PX * PY> &ws) {
+    using S = Shape<PX, PY>;
+    constexpr int kStep = 32 / S::kRow;
     const int lane = threadIdx.x & 31;
     Block b;
-    b.i0 = (tile % ds.tiles_x) * ds.tile + (sub & 1) * kBlk;
-    b.j0 = (tile / ds.tiles_x) * ds.tile + (sub >> 1) * kBlk;
-    if (b.i0 >= ds.Nx || b.j0 >= ds.Ny) return;
-    b.i = b.i0 + (lane & 3) * 4;
-    b.j = b.j0 + (lane >> 2);
+    b.i0 = i0;
+    b.j0 = j0;
+    b.i = b.i0 + lane % S::kRow * PX;
+    b.j = b.j0 + lane / S::kRow;
     unsigned live = 0;
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (b.j + 8 * h < ds.Ny)  // the scene's free-space mask: outside every obstacle's open interior, inside the grid
-            live |= ((__ldg(ds.free_bits + (size_t)(b.j + 8 * h) * ds.free_words + (b.i >> 5)) >> (b.i & 31)) & 15u) << (4 * h);
+    for (int h = 0; h < PY; ++h)
+        if (b.j + kStep * h < ds.Ny)  // the scene's free-space mask: outside every obstacle's open interior, inside the grid
+            live |= ((__ldg(ds.free_bits + (size_t)(b.j + kStep * h) * ds.free_words + (b.i >> 5)) >> (b.i & 31)) &
+                     ((1u << PX) - 1u)) << (PX * h);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < S::kPix; ++k) {
         ws.bd[k * 32 + lane] = (live >> k) & 1u ? INFINITY : -INFINITY;
         ws.bi[k * 32 + lane] = -1;
     }
     b.worst = live ? INFINITY : -INFINITY;
     if (lane == 0) SPM_CNT(0, 1);
     if (__any_sync(0xffffffffu, live)) {
-        const int ni = min(kBlk, ds.Nx - b.i0), nj = min(kBlk, ds.Ny - b.j0);
+        b.i1 = min(b.i0 + S::kW, ds.Nx) - 1;
+        b.j1 = min(b.j0 + S::kH, ds.Ny) - 1;
         b.box = make_int4(ds.pitch_x * b.i0 + ds.pitch_x / 2, ds.pitch_y * b.j0 + ds.pitch_y / 2,
-                          ds.pitch_x * (b.i0 + ni - 1) + ds.pitch_x / 2, ds.pitch_y * (b.j0 + nj - 1) + ds.pitch_y / 2);
+                          ds.pitch_x * b.i1 + ds.pitch_x / 2, ds.pitch_y * b.j1 + ds.pitch_y / 2);
         b.lists = ds.use_flood && ds.flood_counts[2] == 0;
+        const int sh = ds.tile == kTile ? 5 : 4, tile = (j0 >> sh) * ds.tiles_x + (i0 >> sh);  // tiles of 32 or 16 pixels
         const bool stat = b.lists && ds.static_lists, maps = b.lists && ds.use_maps && ds.gen_maps;
         const int s0 = stat ? ds.static_tile_start[tile] : 0, ns = stat ? ds.static_tile_start[tile + 1] - s0 : 0;
         const int l0 = b.lists ? ds.tile_start[tile] : 0, nl = ns + (b.lists ? ds.tile_start[tile + 1] - l0 : 0);
@@ -585,7 +613,7 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int tile, 
             const bool last = e0 + 32 >= total;
             if (n > kWarpCand - 32 || (last && n > 0)) {
                 if (lane == 0) SPM_CNT(1, n);
-                apply_candidates(ds, ws, n, b);
+                apply_candidates<PX, PY, SCAN>(ds, ws, n, b);
                 n = 0;
                 if (!last) {
                     float w = b.worst;
@@ -597,26 +625,27 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int tile, 
         }
     }
     // 16-byte stores where every row of both planes starts on such a boundary
-    const bool vec = (ds.Nx & 3) == 0 && ((reinterpret_cast<size_t>(dist) | reinterpret_cast<size_t>(parent)) & 15) == 0;
+    const bool vec = PX == 4 && (ds.Nx & 3) == 0 &&
+                     ((reinterpret_cast<size_t>(dist) | reinterpret_cast<size_t>(parent)) & 15) == 0;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (b.j + 8 * h >= ds.Ny) continue;
-        float od[4];
-        int op[4];
+    for (int h = 0; h < PY; ++h) {
+        if (b.j + kStep * h >= ds.Ny) continue;
+        float od[PX];
+        int op[PX];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            op[k] = ws.bi[(4 * h + k) * 32 + lane];
-            od[k] = op[k] >= 0 ? ws.bd[(4 * h + k) * 32 + lane] : INFINITY;
+        for (int k = 0; k < PX; ++k) {
+            op[k] = ws.bi[(PX * h + k) * 32 + lane];
+            od[k] = op[k] >= 0 ? ws.bd[(PX * h + k) * 32 + lane] : INFINITY;
         }
-        const size_t base = (size_t)(b.j + 8 * h) * ds.Nx + b.i;
+        const size_t base = (size_t)(b.j + kStep * h) * ds.Nx + b.i;
         if (vec) {
             if (b.i < ds.Nx) {
-                *reinterpret_cast<float4 *>(dist + base) = make_float4(od[0], od[1], od[2], od[3]);
-                *reinterpret_cast<int4 *>(parent + base) = make_int4(op[0], op[1], op[2], op[3]);
+                *reinterpret_cast<float4 *>(dist + base) = make_float4(od[0], od[1 % PX], od[2 % PX], od[3 % PX]);
+                *reinterpret_cast<int4 *>(parent + base) = make_int4(op[0], op[1 % PX], op[2 % PX], op[3 % PX]);
             }
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
+            for (int k = 0; k < PX; ++k)
                 if (b.i + k < ds.Nx) {
                     dist[base + k] = od[k];
                     parent[base + k] = op[k];
@@ -625,27 +654,31 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int tile, 
     }
 }
 
+constexpr long long kTwoWaves = 2 * 152 * 28;
 #ifndef SPM_BLK_MINB
-#define SPM_BLK_MINB (24 / SPM_BLK_WARPS)  // resident CTAs per SM the kernel is compiled for
+#define SPM_BLK_MINB 28  // warps per SM the kernels are compiled for
 #endif
-__global__ void __launch_bounds__(32 * kBlkWarps, SPM_BLK_MINB) k_pixel_blocks(const __grid_constant__ DevScene ds,
-                                                                               float *__restrict__ dist,
-                                                                               int32_t *__restrict__ parent, int tile0,
-                                                                               int tile1) {
-    __shared__ WarpSmem sm[kBlkWarps];
-    const int warp = threadIdx.x >> 5;
-    // a warp a block: four blocks to a 32-pixel tile, one to a 16-pixel one
-    const int per = ds.tile == kTile ? 4 : 1, blk = blockIdx.x * kBlkWarps + warp, t = tile0 + blk / per;
-    if (t < tile1) pixel_block(ds, t, blk % per, dist, parent, sm[warp]);
+// One warp a CTA, so that a finished block's place is taken at once: with four
+// warps a CTA (sharing nothing) the early ones waited for the slowest, 15 %
+// on the 4096^2 maze.
+template <int PX, int PY, bool SCAN>
+__global__ void __launch_bounds__(32, SPM_BLK_MINB) k_pixel_blocks(const __grid_constant__ DevScene ds,
+                                                                   float *__restrict__ dist,
+                                                                   int32_t *__restrict__ parent, int row0) {
+    __shared__ WarpSmem<PX * PY> sm;
+    using S = Shape<PX, PY>;
+    pixel_block<PX, PY, SCAN>(ds, blockIdx.x * S::kW, row0 + blockIdx.y * S::kH, dist, parent, sm);
 }
 
 // Persistent form over a batch of scenes: each warp takes the next
 // (scene, block) from a global counter (costliest tiles first), copies that
 // scene's descriptor into shared memory and runs the same code.
-__global__ void __launch_bounds__(32 * kBlkWarps, SPM_BLK_MINB) k_pixel_blocks_b(const __grid_constant__ BatchDev b) {
-    __shared__ WarpSmem sm[kBlkWarps];
-    __shared__ DevScene sds[kBlkWarps];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+constexpr int kBatchWarps = 4;  // per CTA: neighbouring blocks share their lists and maps in L1
+__global__ void __launch_bounds__(32 * kBatchWarps, SPM_BLK_MINB / kBatchWarps) k_pixel_blocks_b(const __grid_constant__ BatchDev b) {
+    __shared__ WarpSmem<8> sm[kBatchWarps];
+    __shared__ DevScene sds[kBatchWarps];
+    using S = Shape<4, 2>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     DevScene &ds = sds[warp];
     int held = -1;
     for (;;) {
@@ -667,8 +700,9 @@ __global__ void __launch_bounds__(32 * kBlkWarps, SPM_BLK_MINB) k_pixel_blocks_b
             __syncwarp();
             held = sc;
         }
-        const int per = ds.tile == kTile ? 4 : 1;
-        pixel_block(ds, blk / per, blk % per, b.dist[sc], b.parent[sc], sm[warp]);
+        const int across = (ds.Nx + S::kW - 1) / S::kW;
+        pixel_block<4, 2, false>(ds, blk % across * S::kW, blk / across * S::kH, b.dist[sc], b.parent[sc], sm[warp]);
+        __syncwarp();
     }
 }
 
@@ -781,11 +815,28 @@ void launch_free_mask(const DevScene &ds, cudaStream_t st, uint32_t *bits) {
 
 void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int tile_row0,
                         int tile_row1) {
-    const int tiles = ds.tiles_x * (tile_row1 - tile_row0);
-    if (tiles <= 0) return;
-    const int t0 = tile_row0 * ds.tiles_x;
-    const int grid = (tiles * (ds.tile == kTile ? 4 : 1) + kBlkWarps - 1) / kBlkWarps;
-    k_pixel_blocks<<<grid, 32 * kBlkWarps, 0, st>>>(ds, dist, parent, t0, t0 + tiles);
+    const int row0 = tile_row0 * ds.tile, rows = std::min(tile_row1 * ds.tile, ds.Ny) - row0;
+    if (rows <= 0) return;
+    auto run = [&](auto shape, auto kern) {
+        const dim3 grid((ds.Nx + shape.kW - 1) / shape.kW, (rows + shape.kH - 1) / shape.kH);
+        kern<<<grid, 32, 0, st>>>(ds, dist, parent, row0);
+    };
+    // The largest blocks that still give the GPU about two waves of warps
+    // (28 an SM): large blocks cull and order their candidates for more pixels
+    // at once, but a small grid of them waits for its slowest few. Pixel pass
+    // in us with 16 x 16 / 16 x 8 / 8 x 8 / 8 x 4 blocks: 256^2 rectangles 33 /
+    // 22 / 17 / 15, 512^2 polygons 73 / 47 / 34 / 41, 1024^2 polygons 92 / 81 /
+    // 90 / 118, 1501^2 156 / 161 / 210 / 421, maze 4096^2 264 / 334 / 447 / 860.
+    const bool scan = !ds.use_flood || ds.flood_mode == 2 || ds.flood_mode == 0;  // (or may, decided on the device)
+    auto pick = [&](auto shape, auto lists, auto scans) {
+        if (scan) run(shape, scans);
+        else run(shape, lists);
+    };
+    const long long blocks = (long long)((ds.Nx + 15) / 16) * ((rows + 15) / 16);
+    if (blocks * 8 <= kTwoWaves) pick(Shape<1, 1>(), k_pixel_blocks<1, 1, false>, k_pixel_blocks<1, 1, true>);
+    else if (blocks * 4 <= kTwoWaves) pick(Shape<2, 1>(), k_pixel_blocks<2, 1, false>, k_pixel_blocks<2, 1, true>);
+    else if (blocks * 2 <= kTwoWaves) pick(Shape<4, 1>(), k_pixel_blocks<4, 1, false>, k_pixel_blocks<4, 1, true>);
+    else pick(Shape<4, 2>(), k_pixel_blocks<4, 2, false>, k_pixel_blocks<4, 2, true>);
 }
 
 void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st) {
@@ -793,9 +844,9 @@ void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st) {
     int per_sm = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pixel_blocks_b, 32 * kBlkWarps, 0);
-    const int grid = max(1, min((b.total_blocks + kBlkWarps - 1) / kBlkWarps, sms * max(per_sm, 1)));
-    k_pixel_blocks_b<<<grid, 32 * kBlkWarps, 0, st>>>(b);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pixel_blocks_b, 32 * kBatchWarps, 0);
+    const int grid = max(1, min((b.total_blocks + kBatchWarps - 1) / kBatchWarps, sms * max(per_sm, 1)));
+    k_pixel_blocks_b<<<grid, 32 * kBatchWarps, 0, st>>>(b);
 }
 
 int count_kernel_launches_pixel() { return 1; }
