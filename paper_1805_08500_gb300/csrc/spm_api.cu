@@ -282,6 +282,14 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
         std::vector<int4> b(hs.poly_box.size() / 4);
         std::memcpy(b.data(), hs.poly_box.data(), sizeof(int32_t) * hs.poly_box.size());
         ds.poly_box = dupload(s, b, ok);
+        std::vector<int4> e(v.size());
+        for (int k = 0; k < ds.n_poly; ++k)
+            for (int i = hs.poly_off[k]; i < hs.poly_off[k + 1]; ++i) {
+                const int2 a = v[i], c = v[i + 1 == hs.poly_off[k + 1] ? hs.poly_off[k] : i + 1];
+                e[i] = make_int4(a.x, a.y, c.x, c.y);
+            }
+        ds.edges = dupload(s, e, ok);
+        ds.n_edge = (int32_t)e.size();
     }
     ds.bin_start = dupload(s, hs.bin_start, ok);
     ds.bin_items = dupload(s, hs.bin_items, ok);
@@ -383,6 +391,8 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
         ds.static_counts = ds.use_flood ? dalloc<int32_t>(s, 4) : nullptr;
         ds.static_lists = 0;
         ds.src_direct = 0;
+        ds.src_words = (hs.n_src + 31) / 32;
+        ds.src_mask = ds.use_flood ? dalloc<uint32_t>(s, (size_t)ntiles * ds.src_words) : nullptr;
     }
     ds.free_words = (hs.Nx + 31) / 32;
     uint32_t *free_bits = dalloc<uint32_t>(s, (size_t)hs.Ny * ds.free_words);
@@ -584,6 +594,7 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     const bool timed = cap == cudaStreamCaptureStatusNone;
     const bool side = s->ds.use_flood && s->ds.flood_mode == 3;  // geometric flood beside the vertex phase
     s->ds.static_lists = side && s->ds.static_tile_start ? 1 : 0;  // the pixel pass reads the kept lists too
+    s->ds.src_direct = s->ds.static_lists && spm::flood_sources_direct(s->ds) ? 1 : 0;
     NvtxRange range_all("spm_compute");
     if (timed) cudaEventRecord(s->ev[0], cs);
     // the geometric flood needs nothing from the vertex phase (costs and
@@ -905,8 +916,8 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         descs[k].src_direct = d.flood_reuse && spm::flood_sources_direct(d) ? 1 : 0;
         const long long direct = descs[k].src_direct, ntl = (long long)d.tiles_x * d.tiles_y;
         src_map_off[k + 1] = src_map_off[k] + direct * d.n_src * spm::kAngBins;
-        src_ins_off[k + 1] = src_ins_off[k] + direct * d.n_src * d.n_poly;
-        src_tile_off[k + 1] = src_tile_off[k] + direct * d.n_src * ntl;
+        src_ins_off[k + 1] = src_ins_off[k] + direct * d.n_src * spm::src_edge_warps(d.n_edge);
+        src_tile_off[k + 1] = src_tile_off[k] + direct * ntl;
         const bool floods = d.use_flood && d.flood_mode != 2;
         flood_off[k + 1] =
             flood_off[k] + (floods && !direct ? (d.flood_reuse ? d.n_src : d.n_gen) : 0);
@@ -972,6 +983,9 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     bd.sssp_blocks = spm::sssp_batched_grid_blocks();
     bd.flood_smem = 0;
     bd.any_maps = 0;
+    bd.any_lists = 0;
+    for (int k = 0; k < n; ++k)
+        bd.any_lists |= descs[k].use_flood && descs[k].flood_mode != 2 && !descs[k].src_direct;
     for (int k = 0; k < n; ++k) bd.any_maps |= descs[k].use_flood && descs[k].flood_mode != 2 && descs[k].use_maps;
     for (int k = 0; k < n; ++k)
         if (descs[k].use_flood && descs[k].flood_mode != 2)
@@ -1216,16 +1230,16 @@ spm_status spm_scene_info(spm_scene *s, int64_t *info) {
     info[9] = s->ds.flood_mode;
     const bool floods = s->ds.use_flood && s->ds.flood_mode != 2;
     // the geometric mode over kept obstacle-vertex lists: the sources' culling
-    // (list reset, then the walk, or maps from every polygon and the tile
-    // tests) and the list scan and fill
+    // (list reset, the walk and the list scan and fill, or maps from every
+    // polygon and the tile tests)
     const bool reuse = floods && s->ds.flood_mode == 3 && s->ds.static_tile_start;
-    const int src_cull = !spm::flood_sources_direct(s->ds) ? 2 : s->ds.n_poly > 0 ? 3 : 2;
+    const int src_cull = !spm::flood_sources_direct(s->ds) ? 4 : s->ds.n_poly > 0 ? 3 : 2;
     // vertex phase (prep, pairs, edges, the tree's kernels, fixpoint kernels,
     // and after the many-CTA one its finalisation); flood, list scan and
     // fill; pixels
     const int many_cta = s->ds.fix_launch & (spm::kFixSoloSure | spm::kFixClusterSure) ? 0 : 2;
     info[10] = 1 + (s->hs.n_vert > 0 ? 4 : 0) + (s->ds.warm && s->ds.vtab ? 4 : 0) + (s->ds.fix_launch & spm::kFixSolo ? 1 : 0) +
-               (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull + 2 : 3) : 0) + 1;
+               (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull : 3) : 0) + 1;
     return SPM_OK;
 }
 

@@ -15,6 +15,41 @@
 
 namespace spm {
 
+// Programmatic dependent launch along the chains of small kernels: a kernel
+// launched with programmatic stream serialization may be scheduled while its
+// predecessor in the stream still runs. Each chain kernel first lets its own
+// successor be scheduled (launch_dependents), then waits (griddepcontrol.wait)
+// until its predecessor has completed and that grid's memory is visible,
+// before it reads anything. Launched the ordinary way, both instructions do
+// nothing.
+__device__ __forceinline__ void chain_start() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launches a kernel of a chain with programmatic stream
+// serialization (it may be scheduled while its predecessor runs and waits
+// for it in chain_start); an ordinary launch if the attribute is refused.
+template <typename... KArgs, typename... Args>
+static void launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                           Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) {
+        cudaGetLastError();
+        kern<<<grid, block, smem, st>>>(args...);
+    }
+}
+
+
 // Work counters of an instrumentation build (-DSPM_COUNT); compiled out otherwise.
 #ifdef SPM_COUNT
 static __device__ unsigned long long g_count[32];  // one copy per translation unit

@@ -131,60 +131,83 @@ __device__ __forceinline__ bool box_hidden_ang_warp(const float *depth2, int2 g,
     return box_hidden_ang<32>(depth2, g, box, lane, 0xffffffffu, stride);
 }
 
+// A front-facing edge a -> c (g strictly on its outer side) as seen from g.
+// Its angle range goes counter-clockwise from c to a; n is its line's normal,
+// with n . (a - g) = N > 0 and n . u > 0 for every ray u that meets the edge.
+struct EdgeView {
+    int nx, ny, ex, ey;  // normal, direction a -> c
+    float N2, h2;        // N^2; the line's squared distance, rounded down
+    float lo, hi;        // pseudo-angles of c and a, hi unwrapped past lo
+    float c2, a2;        // their squared distances
+    float sc, sa;        // and their places along the line, 0 at the foot of g
+    int k0, k1;          // bins its closed angle range touches
+};
+__device__ __forceinline__ bool edge_view(int2 g, int4 e, EdgeView &v) {
+    const int ax = e.x - g.x, ay = e.y - g.y, cx = e.z - g.x, cy = e.w - g.y;
+    const int N = cross32(cx, cy, ax, ay);  // = -orient(a, c, g)
+    if (N <= 0) return false;
+    v.ex = e.z - e.x;
+    v.ey = e.w - e.y;
+    v.nx = -v.ey;
+    v.ny = v.ex;
+    v.N2 = (float)N * (float)N;
+    v.h2 = __fdividef(v.N2, (float)v.ex * (float)v.ex + (float)v.ey * (float)v.ey) * (1.f - 1e-5f);
+    v.lo = pang((float)cx, (float)cy);
+    float d = pang((float)ax, (float)ay) - v.lo;
+    if (d < 0.f) d += 4.f;
+    v.hi = v.lo + d;
+    v.c2 = (float)cx * (float)cx + (float)cy * (float)cy;
+    v.a2 = (float)ax * (float)ax + (float)ay * (float)ay;
+    v.sc = (float)v.ex * (float)cx + (float)v.ey * (float)cy;
+    v.sa = (float)v.ex * (float)ax + (float)v.ey * (float)ay;
+    v.k0 = (int)floorf((v.lo - kAngEps) / kAngW);
+    v.k1 = (int)floorf((v.hi + kAngEps) / kAngW);
+    return true;
+}
+
+// Edge v enters bin k. The crossing distance along the line is convex in the
+// ray's angle, so over the rays of the bin that meet the edge it is largest at
+// an end of their range, and smallest there too unless the foot of g lies
+// between. A bin wholly inside the edge's range takes the larger end as its
+// full-blocking bound; every bin the range touches takes the smallest distance
+// as a lower bound of where a ray can first meet an obstacle: a ray enters an
+// obstacle through a front-facing edge or a vertex of one. Boundary rays are
+// exact multiples of 1/kAngQ, so their products with n are exact in integers;
+// a 1e-5 margin covers the few float roundings.
+// check: read a bin first and leave it when the edge does not lower it (saves
+// the atomic, costs the load's latency).
+template <bool MAPS>
+__device__ __forceinline__ void edge_into_bin(const EdgeView &v, int k, float *up, float *low, int stride, bool check) {
+    auto at = [&](int mb, float &s) {  // squared crossing distance and place along the line at boundary mb
+        const int2 u = boundary_dir(mb);
+        const float D = (float)(v.nx * u.x + v.ny * u.y);  // |n| < 2^16, |u| <= kAngQ
+        s = (float)(v.ex * u.x + v.ey * u.y);
+        return __fdividef(v.N2 * (float)(u.x * u.x + u.y * u.y), D * D);
+    };
+    const float b0 = (float)k * kAngW, b1 = (float)(k + 1) * kAngW;
+    float s0 = v.sc, s1 = v.sa;
+    const float f0 = b0 <= v.lo ? v.c2 : at(k, s0), f1 = b1 >= v.hi ? v.a2 : at(k + 1, s1);
+    const int slot = stride * ((k + kAng) & (kAng - 1));
+    if (b0 >= v.lo + kAngEps && b1 <= v.hi - kAngEps) {
+        const float d = fmaxf(f0, f1) * (1.f + 1e-5f);
+        if (!check || up[slot] > d) atomicMin((int *)up + slot, __float_as_int(d));  // non-negative floats order as ints
+    }
+    if (MAPS) {
+        const float f = (s0 > 0.f) != (s1 > 0.f) ? v.h2 : fminf(f0, f1);
+        const float d = fmaxf(f * (1.f - 2e-5f) - 0.05f, 0.f);
+        if (!check || low[slot] > d) atomicMin((int *)low + slot, __float_as_int(d));
+    }
+}
+
 // One warp inserts polygon q's front-facing edges into the depth map, the
 // lanes spread over each edge's bins.
 template <bool MAPS>
-__device__ void insert_polygon_warp(const DevScene &ds, float *depth2, float *lo2, int2 g, int q, int lane,
-                                    float plen, int stride = 1) {
-    const int b = ds.poly_off[q], m = ds.poly_off[q + 1] - b;
-    const int2 mine = lane < m ? ds.poly_v[b + lane] : make_int2(0, 0);  // vertex `lane`, one load per lane
-    for (int i = 0; i < m; ++i) {
-        const int in = i + 1 == m ? 0 : i + 1;
-        const int2 a = make_int2(__shfl_sync(0xffffffffu, mine.x, i), __shfl_sync(0xffffffffu, mine.y, i));
-        const int2 c = make_int2(__shfl_sync(0xffffffffu, mine.x, in), __shfl_sync(0xffffffffu, mine.y, in));
-        if (orient32(a.x, a.y, c.x, c.y, g.x, g.y) >= 0) continue;  // not front-facing
-        // line normal n (left of a -> c); g is on its negative side, so
-        // n . (a - g) > 0 and n . u > 0 for every ray u that meets the edge
-        const int nx = -(c.y - a.y), ny = c.x - a.x;
-        const long long N = (long long)nx * (a.x - g.x) + (long long)ny * (a.y - g.y);
-        const float fN2 = (float)N * (float)N;
-        // no ray crosses the line closer than its distance from g
-        const float h2 = __fdividef(fN2, (float)nx * (float)nx + (float)ny * (float)ny) * (1.f - 1e-5f);
-        // the edge runs clockwise seen from g: its angle range goes
-        // counter-clockwise from c to a
-        const float lo = pang((float)(c.x - g.x), (float)(c.y - g.y));
-        const float hi = lo + fmodf(pang((float)(a.x - g.x), (float)(a.y - g.y)) - lo + 4.f, 4.f);
-        const int k0 = (int)ceilf((lo + kAngEps) / kAngW), k1 = (int)floorf((hi - kAngEps) / kAngW) - 1;
-        auto bdist2 = [&](int mb) {  // squared crossing distance along boundary ray mb, rounded up
-            const int2 u = boundary_dir(mb);
-            const float fD = (float)(nx * u.x + ny * u.y);  // exact: |n| < 2^16, |u| <= 512
-            return __fdividef(fN2 * (float)(u.x * u.x + u.y * u.y), fD * fD) * (1.f + 1e-5f);
-        };
-        for (int k = k0 + lane; k <= k1; k += 32) {
-            int *slot = (int *)&depth2[stride * (k & (kAng - 1))];
-            if (__int_as_float(*slot) <= h2) continue;  // this edge cannot lower the bin
-            atomicMin(slot, __float_as_int(fmaxf(bdist2(k), bdist2(k + 1))));  // non-negative floats order as ints
-        }
-        // Lower bound: a ray entering an obstacle crosses a front-facing edge
-        // (or passes a vertex of one) at a point of some piece of it, no
-        // nearer than that piece's distance from g. Pieces of at most plen
-        // lattice units; every bin touching a piece's closed angle range.
-        if (!MAPS) continue;
-        const float ax = (float)(a.x - g.x), ay = (float)(a.y - g.y), ex = (float)(c.x - a.x), ey = (float)(c.y - a.y);
-        const float el = sqrtf(ex * ex + ey * ey);
-        const int np = max(1, (int)ceilf(el / plen));
-        for (int j = lane; j < np; j += 32) {
-            const float t0 = (float)j / (float)np, t1 = j + 1 == np ? 1.f : (float)(j + 1) / (float)np;
-            const float px0 = ax + t0 * ex, py0 = ay + t0 * ey, px1 = ax + t1 * ex, py1 = ay + t1 * ey;
-            const float dx = px1 - px0, dy = py1 - py0, dd = dx * dx + dy * dy;
-            const float tt = dd > 0.f ? fminf(fmaxf(-(px0 * dx + py0 * dy) / dd, 0.f), 1.f) : 0.f;
-            const float cx = px0 + tt * dx, cy = py0 + tt * dy;
-            const float d2 = fmaxf((cx * cx + cy * cy) * (1.f - 2e-5f) - 0.05f, 0.f);
-            const float plo = pang(px1, py1), phi = plo + fmodf(pang(px0, py0) - plo + 4.f, 4.f);
-            const int b0 = (int)floorf((plo - kAngEps) / kAngW), b1 = (int)floorf((phi + kAngEps) / kAngW);
-            for (int k = b0; k <= b1; ++k)
-                atomicMin((int *)&lo2[stride * ((k + 2 * kAng) & (kAng - 1))], __float_as_int(d2));
-        }
+__device__ void insert_polygon_warp(const DevScene &ds, float *depth2, float *lo2, int2 g, int q, int lane) {
+    const int e0 = ds.poly_off[q], e1 = ds.poly_off[q + 1];
+    for (int e = e0; e < e1; ++e) {
+        EdgeView v;
+        if (!edge_view(g, __ldg(ds.edges + e), v)) continue;
+        for (int k = v.k0 + lane; k <= v.k1; k += 32) edge_into_bin<MAPS>(v, k, depth2, lo2, 1, true);
     }
 }
 
@@ -203,7 +226,6 @@ __device__ void flood_one(const DevScene &ds, FloodSmem &sm, unsigned *fdyn, int
     // mode 3 floods from geometry alone (every generator, no cone): it runs
     // before the vertex costs exist, and the pixel pass applies cost and cone
     const bool geometric = ds.flood_mode == 3;
-    const float plen = fmaxf(1.f, 0.125f * (float)min(tpx, tpy));  // lower-bound piece length
     constexpr bool maps = MAPS;
     if (ds.gen_map_ok && tid == 0) ds.gen_map_ok[g] = 0;  // set again when the map is complete
     SPM_T0();
@@ -291,7 +313,7 @@ __device__ void flood_one(const DevScene &ds, FloodSmem &sm, unsigned *fdyn, int
         SPM_LAP(1);
         const int ni = min(sm.n_ins, kInsCap);
         for (int q = tid >> 5; q < ni; q += kFloodThreads / 32)
-            insert_polygon_warp<MAPS>(ds, sm.depth2, lo2, gl, sm.ins[q], tid & 31, plen);
+            insert_polygon_warp<MAPS>(ds, sm.depth2, lo2, gl, sm.ins[q], tid & 31);
         __syncthreads();
         SPM_LAP(2);
 #ifdef SPM_TIME
@@ -376,91 +398,122 @@ __device__ void flood_one(const DevScene &ds, FloodSmem &sm, unsigned *fdyn, int
 // Direct culling of the sources (generators [0, n_src)) in the geometric
 // mode: few generators, each reaching much of the grid, which one CTA per
 // generator would walk a breadth-first level at a time. Instead every
-// polygon enters each source's depth map at once (a warp per (source,
-// polygon), atomics into the source's map in global memory), and then every
-// tile is tested against the complete map at once (a warp per (source,
-// tile)). A tile that the map does not hide gets the source in its list.
-// That is a superset of what the walk reaches -- the walk also stops at
-// tiles cut off by hidden ones -- and every tile where the source can win is
-// still in it: the map only hides points that lie beyond an obstacle
-// interior on their ray. With every polygon in it the map is complete, and
-// the pixel pass may use it.
+// polygon edge enters each source's depth map at once (a warp per source and
+// sixteen edges, atomics into the source's map in global memory), and then every tile
+// is tested against the complete maps at once (a warp a tile), which gives the
+// tile a bit per source. That is a superset of what the walk reaches -- the
+// walk also stops at tiles cut off by hidden ones -- and every tile where the
+// source can win is still in it: the map only hides points that lie beyond an
+// obstacle interior on their ray. With every polygon in it the map is
+// complete, and the pixel pass may use it.
 __device__ __forceinline__ bool src_on_grid(const DevScene &ds, int g) {
     const int2 gl = ds.gen_lat[g];
-    const int px = ds.S * ds.Wx / ds.Nx, py = ds.S * ds.Wy / ds.Ny;
-    return ds.gen_kind[g] != kSegI && gl.x >= 0 && gl.y >= 0 && gl.x <= ds.Nx * px && gl.y <= ds.Ny * py;
+    return ds.gen_kind[g] != kSegI && gl.x >= 0 && gl.y >= 0 && gl.x <= ds.Nx * ds.pitch_x && gl.y <= ds.Ny * ds.pitch_y;
 }
 
-// Before the sources' culling: empty maps and lists, the global list after
-// the obstacle vertices' entries, the overflow flag as their flood left it.
-__device__ __forceinline__ void src_prep(const DevScene &ds, int i0, int stride, bool counts) {
-    const int nmap = ds.n_src * kAng, ntiles = ds.tiles_x * ds.tiles_y;
-    for (int i = i0; i < max(nmap, ntiles); i += stride) {
-        if (i < nmap) ds.gen_maps[i] = make_float2(INFINITY, INFINITY);
-        if (i < ntiles) ds.tile_count[i] = 0;
-        if (i < ds.n_src) ds.gen_map_ok[i] = 0;
+// Before the sources' culling: empty maps, the global list and the overflow
+// flag as the obstacle vertices' flood left them.
+__device__ __forceinline__ void src_prep(const DevScene &ds, int i0, int stride) {
+    const bool maps = ds.use_maps && ds.gen_maps;
+    for (int i = i0; i < ds.n_src * kAng; i += stride) {
+        ds.gen_maps[i] = make_float2(INFINITY, INFINITY);
+        if (i < ds.n_src) ds.gen_map_ok[i] = maps && src_on_grid(ds, i);  // complete by the time the pixel pass reads it
     }
-    if (counts && i0 < 4) ds.flood_counts[i0] = i0 == 1 || i0 == 2 ? ds.static_counts[i0] : 0;
+    if (i0 < 4) ds.flood_counts[i0] = i0 == 1 || i0 == 2 ? ds.static_counts[i0] : 0;
 }
 
+// Edges e0 .. e0 + kSrcEdges - 1 into source g's map, one warp: a lane views
+// an edge, then the bins they span are dealt to the lanes evenly (a wall next
+// to the source spans hundreds, a far one two or three).
+constexpr int kSrcEdges = 16;
 template <bool MAPS>
-__device__ __forceinline__ void src_insert(const DevScene &ds, int g, int q, int lane) {
-    if (!src_on_grid(ds, g)) return;
-    const int tpx = ds.tile * (ds.S * ds.Wx / ds.Nx), tpy = ds.tile * (ds.S * ds.Wy / ds.Ny);
-    const float plen = fmaxf(1.f, 0.125f * (float)min(tpx, tpy));  // as in the flood
+__device__ __forceinline__ void src_insert(const DevScene &ds, int g, int e0) {
+    const int lane = threadIdx.x & 31;
+    if (!src_on_grid(ds, g)) return;  // the same for the whole warp
     float *mp = reinterpret_cast<float *>(ds.gen_maps + (size_t)g * kAng);
-    insert_polygon_warp<MAPS>(ds, mp, mp + 1, ds.gen_lat[g], q, lane, plen, 2);
+    EdgeView v = {};
+    int span = 0;
+    if (lane < kSrcEdges && e0 + lane < ds.n_edge && edge_view(ds.gen_lat[g], __ldg(ds.edges + e0 + lane), v))
+        span = v.k1 - v.k0 + 1;
+    int incl = span;
+#pragma unroll
+    for (int o = 1; o < kSrcEdges; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, kSrcEdges - 1);
+    for (int r0 = 0; r0 < total; r0 += 32) {
+        const int r = r0 + lane;
+        int own = 0;  // the first edge whose bins end beyond r
+#pragma unroll
+        for (int o = kSrcEdges / 2; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, incl, own + o - 1) <= r) own += o;
+        own = min(own, kSrcEdges - 1);
+        EdgeView o;
+        auto take = [&](float x) { return __shfl_sync(0xffffffffu, x, own); };
+        o.ex = __shfl_sync(0xffffffffu, v.ex, own);
+        o.ey = __shfl_sync(0xffffffffu, v.ey, own);
+        o.nx = -o.ey;
+        o.ny = o.ex;
+        o.N2 = take(v.N2);
+        o.h2 = take(v.h2);
+        o.lo = take(v.lo);
+        o.hi = take(v.hi);
+        o.c2 = take(v.c2);
+        o.a2 = take(v.a2);
+        o.sc = take(v.sc);
+        o.sa = take(v.sa);
+        const int k = r - __shfl_sync(0xffffffffu, incl - span - v.k0, own);
+        if (r < total) edge_into_bin<MAPS>(o, k, mp, mp + 1, 2, total <= 64);  // wide ones are near and lower most bins
+    }
 }
 
-constexpr int kSrcGrp = 8;  // lanes per (source, tile) test: most tiles span few bins
-template <bool MAPS>
-__device__ __forceinline__ void src_tile(const DevScene &ds, int g, int t, int lane, unsigned gmask) {
-    if (!src_on_grid(ds, g)) {  // segment interiors and sources off the grid: every tile scans them
-        if (t == 0 && lane == 0) push_global(ds, g);
-        return;
-    }
-    const int2 gl = ds.gen_lat[g];
+// Tile t's bits: a warp, its groups of kSrcGrp lanes a source each (most tiles
+// span few bins). Segment interiors and sources off the grid are candidates
+// of every tile.
+constexpr int kSrcGrp = 8;
+__device__ __forceinline__ void src_tile(const DevScene &ds, int t) {
+    const int lane = threadIdx.x & 31, gl8 = lane % kSrcGrp, grp = lane / kSrcGrp;
+    const unsigned gmask = ((1u << kSrcGrp) - 1u) << (grp * kSrcGrp);
     const int4 area = tile_area(ds, t % ds.tiles_x, t / ds.tiles_x);
-    const bool inside = gl.x >= area.x && gl.x <= area.z && gl.y >= area.y && gl.y <= area.w;
-    const float *mp = reinterpret_cast<const float *>(ds.gen_maps + (size_t)g * kAng);
-    if (MAPS && t == 0 && lane == 0) ds.gen_map_ok[g] = 1;  // complete: the pixel pass may read it
-    if (!inside && box_hidden_ang<kSrcGrp>(mp, gl, area, lane, gmask, 2)) return;
-    if (lane == 0) {
-        const int slot = atomicAdd(&ds.flood_counts[0], 1);
-        if (slot < ds.pair_cap) {
-            ds.pairs[slot] = make_int2(t, g);
-            atomicAdd(&ds.tile_count[t], 1);
-        } else {
-            atomicOr(&ds.flood_counts[2], 1);
+    for (int w = 0; w < ds.src_words; ++w) {
+        const int mine = 32 * w + lane;  // one load for the word's sources
+        const int2 lat = mine < ds.n_src ? ds.gen_lat[mine] : make_int2(0, 0);
+        const bool on = mine < ds.n_src && src_on_grid(ds, mine);
+        const bool inside = lat.x >= area.x && lat.x <= area.z && lat.y >= area.y && lat.y <= area.w;
+        const unsigned every = __ballot_sync(0xffffffffu, mine < ds.n_src && (inside || !on));
+        uint32_t bits = every;
+        const int n = min(32, ds.n_src - 32 * w);
+#pragma unroll 2
+        for (int j0 = 0; j0 < n; j0 += 32 / kSrcGrp) {
+            const int j = j0 + grp;
+            const int2 gl = make_int2(__shfl_sync(0xffffffffu, lat.x, j & 31), __shfl_sync(0xffffffffu, lat.y, j & 31));
+            bool seen = false;
+            if (j < n && !(every >> j & 1u))
+                seen = !box_hidden_ang<kSrcGrp>(reinterpret_cast<const float *>(ds.gen_maps + (size_t)(32 * w + j) * kAng),
+                                                gl, area, gl8, gmask, 2);
+            const unsigned bal = __ballot_sync(0xffffffffu, seen && gl8 == 0);
+#pragma unroll
+            for (int q = 0; q < 32 / kSrcGrp; ++q)
+                if (bal >> (q * kSrcGrp) & 1u) bits |= 1u << (j0 + q);
         }
+        if (lane == 0) ds.src_mask[(size_t)t * ds.src_words + w] = bits;
     }
 }
 
-__global__ void k_src_prep(DevScene ds) {
-    src_prep(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, true);
+__global__ void k_src_prep(const __grid_constant__ DevScene ds) {
+    src_prep(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 template <bool MAPS>
-__global__ void k_src_insert(DevScene ds) {
-    const long long n = (long long)ds.n_src * ds.n_poly;
-    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; w < n;
-         w += (gridDim.x * (long long)blockDim.x) >> 5)
-        src_insert<MAPS>(ds, (int)(w / ds.n_poly), (int)(w % ds.n_poly), threadIdx.x & 31);
+__global__ void k_src_insert(const __grid_constant__ DevScene ds) {  // grid: (edges, sources)
+    const int e0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kSrcEdges;
+    for (int g = blockIdx.y; g < ds.n_src; g += gridDim.y) src_insert<MAPS>(ds, g, e0);
 }
 
-// group of kSrcGrp lanes of the calling thread's warp
-__device__ __forceinline__ unsigned src_group_mask() {
-    return ((1u << kSrcGrp) - 1u) << ((threadIdx.x & 31) & ~(kSrcGrp - 1));
-}
-
-template <bool MAPS>
-__global__ void k_src_tiles(DevScene ds) {
-    const int ntiles = ds.tiles_x * ds.tiles_y;
-    const long long n = (long long)ds.n_src * ntiles;
-    const unsigned gmask = src_group_mask();
-    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / kSrcGrp; w < n;
-         w += (gridDim.x * (long long)blockDim.x) / kSrcGrp)
-        src_tile<MAPS>(ds, (int)(w / ntiles), (int)(w % ntiles), threadIdx.x % kSrcGrp, gmask);
+__global__ void k_src_tiles(const __grid_constant__ DevScene ds) {
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (t < ds.tiles_x * ds.tiles_y) src_tile(ds, t);  // whole warps
 }
 
 // Automatic mode: flood only sparse visibility graphs (mazes); a dense one
@@ -558,7 +611,7 @@ __global__ void k_flood_reset_b(const __grid_constant__ BatchDev b) {
             const DevScene &ds = b.scenes[sc];
             const long long e = m - b.src_map_off[sc];
             ds.gen_maps[e] = make_float2(INFINITY, INFINITY);
-            if (e % kAng == 0) ds.gen_map_ok[e / kAng] = 0;
+            if (e % kAng == 0) ds.gen_map_ok[e / kAng] = ds.use_maps && src_on_grid(ds, (int)(e / kAng));
         } else if (i < total) {
             const int oi = scene_of_b(b.tile_off, b.n, (int32_t)i), sc = b.order[oi];
             b.scenes[sc].tile_count[i - b.tile_off[oi]] = 0;
@@ -573,8 +626,8 @@ __global__ void k_flood_reset_b(const __grid_constant__ BatchDev b) {
     }
 }
 
-// Batched direct culling of sources: (scene, source, polygon) and then
-// (scene, source, tile) warp tasks over the scenes with src_direct.
+// Batched direct culling of sources: (scene, source, edges) and then
+// (scene, tile) warp tasks over the scenes with src_direct.
 template <bool ANY_MAPS>
 __global__ void k_src_insert_b(const __grid_constant__ BatchDev b) {
     const long long n = b.src_ins_off[b.n];
@@ -582,26 +635,18 @@ __global__ void k_src_insert_b(const __grid_constant__ BatchDev b) {
          w += (gridDim.x * (long long)blockDim.x) >> 5) {
         const int sc = scene_of_b(b.src_ins_off, b.n, w);
         const DevScene &ds = b.scenes[sc];
-        const long long e = w - b.src_ins_off[sc];
-        const int g = (int)(e / ds.n_poly), q = (int)(e % ds.n_poly);
-        if (ANY_MAPS && ds.use_maps) src_insert<true>(ds, g, q, threadIdx.x & 31);
-        else src_insert<false>(ds, g, q, threadIdx.x & 31);
+        const int i = (int)(w - b.src_ins_off[sc]), per = (ds.n_edge + kSrcEdges - 1) / kSrcEdges;
+        if (ANY_MAPS && ds.use_maps) src_insert<true>(ds, i / per, i % per * kSrcEdges);
+        else src_insert<false>(ds, i / per, i % per * kSrcEdges);
     }
 }
 
-template <bool ANY_MAPS>
 __global__ void k_src_tiles_b(const __grid_constant__ BatchDev b) {
     const long long n = b.src_tile_off[b.n];
-    const unsigned gmask = src_group_mask();
-    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / kSrcGrp; w < n;
-         w += (gridDim.x * (long long)blockDim.x) / kSrcGrp) {
+    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; w < n;
+         w += (gridDim.x * (long long)blockDim.x) >> 5) {
         const int sc = scene_of_b(b.src_tile_off, b.n, w);
-        const DevScene &ds = b.scenes[sc];
-        const int ntiles = ds.tiles_x * ds.tiles_y;
-        const long long e = w - b.src_tile_off[sc];
-        const int g = (int)(e / ntiles), t = (int)(e % ntiles);
-        if (ANY_MAPS && ds.use_maps) src_tile<true>(ds, g, t, threadIdx.x % kSrcGrp, gmask);
-        else src_tile<false>(ds, g, t, threadIdx.x % kSrcGrp, gmask);
+        src_tile(b.scenes[sc], (int)(w - b.src_tile_off[sc]));
     }
 }
 
@@ -677,12 +722,13 @@ __global__ void k_tiles_fill(DevScene ds, int to_static) {
 // batched: one CTA per scene for the scan, a row of CTAs per scene for the fill
 __global__ void __launch_bounds__(1024) k_tiles_scan_b(const __grid_constant__ BatchDev b) {
     const DevScene &ds = b.scenes[blockIdx.x];
-    if (ds.use_flood && ds.flood_mode != 2) tiles_scan_block(ds);
+    if (ds.use_flood && ds.flood_mode != 2 && !ds.src_direct) tiles_scan_block(ds);
 }
 
 __global__ void k_tiles_fill_b(const __grid_constant__ BatchDev b) {
     const DevScene &ds = b.scenes[blockIdx.y];
-    if (ds.use_flood && ds.flood_mode != 2) tiles_fill(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+    if (ds.use_flood && ds.flood_mode != 2 && !ds.src_direct)
+        tiles_fill(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 }  // namespace
@@ -730,21 +776,18 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
             k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 1);
             k_flood_static<<<sblocks, 256, 0, st>>>(ds, 1);
         }
-        if (flood_sources_direct(ds)) {  // the sources: the only lists a compute sorts
-            const int nmap = ds.n_src * kAng;
-            k_src_prep<<<max(1, min((max(nmap, ntiles) + 255) / 256, 152 * 4)), 256, 0, st>>>(ds);
-            auto wblocks = [](long long warps) { return (int)std::max(1LL, std::min((warps + 7) / 8, 152LL * 16)); };
-            if (ds.n_poly > 0) {
-                if (maps) k_src_insert<true><<<wblocks((long long)ds.n_src * ds.n_poly), 256, 0, st>>>(ds);
-                else k_src_insert<false><<<wblocks((long long)ds.n_src * ds.n_poly), 256, 0, st>>>(ds);
-            }
-            const long long tgroups = ((long long)ds.n_src * ntiles + 3) / 4;  // warps of four tests
-            if (maps) k_src_tiles<true><<<wblocks(tgroups), 256, 0, st>>>(ds);
-            else k_src_tiles<false><<<wblocks(tgroups), 256, 0, st>>>(ds);
-        } else {
-            k_flood_static<<<sblocks, 256, 0, st>>>(ds, 0);
-            flood(0, ds.n_src);
+        if (flood_sources_direct(ds)) {  // a bit per source and tile: nothing to sort
+            k_src_prep<<<std::min((ds.n_src * kAng + 255) / 256, 152 * 8), 256, 0, st>>>(ds);
+            // ordinary launches: a dependent one would hold SMs, waiting, that
+            // the vertex phase beside it needs
+            const dim3 grid((ds.n_edge + 4 * kSrcEdges - 1) / (4 * kSrcEdges), std::min(ds.n_src, 65535));
+            if (ds.n_edge > 0 && maps) k_src_insert<true><<<grid, 128, 0, st>>>(ds);
+            else if (ds.n_edge > 0) k_src_insert<false><<<grid, 128, 0, st>>>(ds);
+            k_src_tiles<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
+            return;
         }
+        k_flood_static<<<sblocks, 256, 0, st>>>(ds, 0);
+        flood(0, ds.n_src);
     }
     k_tiles_scan<<<1, 1024, 0, st>>>(ds, 0);
     k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 0);
@@ -754,6 +797,8 @@ bool flood_sources_direct(const DevScene &ds) {
     const long long ntiles = (long long)ds.tiles_x * ds.tiles_y;
     return ds.gen_maps && ds.n_src > 0 && (long long)ds.n_src * (ds.n_poly + ntiles) <= (1LL << 24);
 }
+
+int src_edge_warps(int n_edge) { return (n_edge + kSrcEdges - 1) / kSrcEdges; }
 
 int flood_smem_attr() {
     const int dyn = 200 * 1024 - (int)sizeof(FloodSmem);
@@ -775,10 +820,8 @@ void launch_flood_batched(const BatchDev &b, cudaStream_t st, long long src_ins,
         if (b.any_maps) k_src_insert_b<true><<<wblocks(src_ins), 256, 0, st>>>(b);
         else k_src_insert_b<false><<<wblocks(src_ins), 256, 0, st>>>(b);
     }
-    if (src_tiles > 0) {  // four tests per warp
-        if (b.any_maps) k_src_tiles_b<true><<<wblocks((src_tiles + 3) / 4), 256, 0, st>>>(b);
-        else k_src_tiles_b<false><<<wblocks((src_tiles + 3) / 4), 256, 0, st>>>(b);
-    }
+    if (src_tiles > 0) k_src_tiles_b<<<wblocks(src_tiles), 256, 0, st>>>(b);
+    if (!b.any_lists) return;  // no lists but the kept ones
     k_tiles_scan_b<<<b.n, 1024, 0, st>>>(b);
     k_tiles_fill_b<<<dim3(16, b.n), 256, 0, st>>>(b);
 }

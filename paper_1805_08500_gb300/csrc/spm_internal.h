@@ -84,6 +84,8 @@ struct DevScene {
     const int32_t *poly_off;
     const int2 *poly_v;
     const int4 *poly_box;
+    const int4 *edges;                 // every polygon edge a -> c, counter-clockwise: a.x a.y c.x c.y
+    int32_t n_edge;
     int32_t bin_x0, bin_y0, bin_size, bin_nx, bin_ny;
     float bin_inv;                     // 1 / bin_size
     const int32_t *bin_start, *bin_items;
@@ -199,7 +201,11 @@ struct DevScene {
     int32_t *static_counts;            // 4
     int32_t static_lists;              // the pixel pass reads the static lists as well (this compute)
     int32_t flood_reuse;               // in a batch's copy: flood the sources only, over the static part
-    int32_t src_direct;                // in a batch's copy: those sources culled directly (complete maps)
+    // this compute's sources are culled directly (complete maps): instead of
+    // pairs and lists, a bit per source, src_words words a tile
+    int32_t src_direct;
+    int32_t src_words;
+    uint32_t *src_mask;
 };
 
 // A batch of scenes computed together (device-side descriptor).
@@ -229,9 +235,10 @@ struct BatchDev {
     int32_t any_maps;                  // some scene keeps depth maps
     // direct culling of the sources of scenes with src_direct (n + 1 prefixes):
     const long long *src_map_off;      // map entries: n_src * kAngBins
-    const long long *src_ins_off;      // warp tasks of the map building: n_src * n_poly
-    const long long *src_tile_off;     // warp tasks of the tile tests: n_src * tiles
+    const long long *src_ins_off;      // warp tasks of the map building: n_src * src_edge_warps(n_edge)
+    const long long *src_tile_off;     // warp tasks of the tile tests: tiles
     int32_t walk_tasks;                // (scene, generator) walks of the batched flood
+    int32_t any_lists;                 // some scene sorts lists per compute (its sources are not culled directly)
     // vertex fixpoint on resident clusters, one scene at a time
     const int32_t *cl_order;           // n scene indices, most generators first
     int32_t *cl_done;                  // n flags: a cluster took the scene's fixpoint
@@ -284,6 +291,7 @@ int flood_smem_attr();
 // the geometric mode culls the sources directly (complete depth maps, every
 // tile tested at once) rather than by the per-generator walk
 bool flood_sources_direct(const DevScene &ds);
+int src_edge_warps(int n_edge);  // warps that put a scene's edges into one source's map
 int sssp_grid_blocks();  // co-resident CTAs for the cooperative fixpoint kernel
 int solo_smem_bytes();   // shared memory granted to the single-CTA fixpoint kernel (0 if refused)
 bool cluster_smem_ok();  // the cluster fixpoint can run (its shared memory was granted)

@@ -588,8 +588,12 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
         b.lists = ds.use_flood && ds.flood_counts[2] == 0;
         const int sh = ds.tile == kTile ? 5 : 4, tile = (j0 >> sh) * ds.tiles_x + (i0 >> sh);  // tiles of 32 or 16 pixels
         const bool stat = b.lists && ds.static_lists, maps = b.lists && ds.use_maps && ds.gen_maps;
+        // the kept list of obstacle vertices, this compute's entries (a bit per
+        // source, or a list), the global list; or every generator
+        const bool bits = stat && ds.src_direct;
         const int s0 = stat ? ds.static_tile_start[tile] : 0, ns = stat ? ds.static_tile_start[tile + 1] - s0 : 0;
-        const int l0 = b.lists ? ds.tile_start[tile] : 0, nl = ns + (b.lists ? ds.tile_start[tile + 1] - l0 : 0);
+        const int l0 = b.lists && !bits ? ds.tile_start[tile] : 0;
+        const int nl = ns + (bits ? ds.n_src : b.lists ? ds.tile_start[tile + 1] - l0 : 0);
         const int total = b.lists ? nl + ds.flood_counts[1] : ds.n_gen;
         float ub = INFINITY;  // no pixel of the block can take more
         int n = 0;
@@ -598,11 +602,18 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
             bool keep = false;
             float lb = 0.f;
             int c = 0;
-            if (e < total) {
-                const int32_t *at = e < ns ? ds.static_tile_items + s0 + e
-                                           : e < nl ? ds.tile_items + l0 + e - ns : ds.glob_list + e - nl;
-                keep = block_candidate(ds, b.lists ? __ldg(at) : e, b, ub, maps, lb, c);
+            int g = e;
+            bool in = e < total;
+            if (in && b.lists) {
+                const int r = e - ns;
+                if (r >= 0 && e < nl && bits) {
+                    g = r;
+                    in = __ldg(ds.src_mask + (size_t)tile * ds.src_words + (r >> 5)) >> (r & 31) & 1u;
+                } else {
+                    g = __ldg(r < 0 ? ds.static_tile_items + s0 + e : e < nl ? ds.tile_items + l0 + r : ds.glob_list + e - nl);
+                }
             }
+            if (in) keep = block_candidate(ds, g, b, ub, maps, lb, c);
             const unsigned bal = __ballot_sync(0xffffffffu, keep);
             if (keep) {
                 const int slot = n + __popc(bal & ((1u << lane) - 1u));

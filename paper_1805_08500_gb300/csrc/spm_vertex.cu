@@ -39,20 +39,6 @@
 #include "spm_device.cuh"
 #include "spm_internal.h"
 
-namespace spm {
-// Programmatic dependent launch along the vertex phase's chain of small
-// kernels: a kernel launched with programmatic stream serialization may be
-// scheduled while its predecessor in the stream still runs. Each chain
-// kernel first lets its own successor be scheduled (launch_dependents), then
-// waits (griddepcontrol.wait) until its predecessor has completed and that
-// grid's memory is visible, before it reads anything. Launched the ordinary
-// way, both instructions do nothing.
-__device__ __forceinline__ void chain_start() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-}  // namespace spm
-
 namespace cg = cooperative_groups;
 
 namespace spm {
@@ -1530,28 +1516,6 @@ __global__ void k_vertex_prep(const __grid_constant__ DevScene ds) {
             ds.counters[4] = 0;
             ds.counters[6] = 0;
         }
-    }
-}
-
-// Launches a kernel of the vertex phase's chain with programmatic stream
-// serialization (it may be scheduled while its predecessor runs and waits
-// for it in chain_start); an ordinary launch if the attribute is refused.
-template <typename... KArgs, typename... Args>
-static void launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                           Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, args...) != cudaSuccess) {
-        cudaGetLastError();
-        kern<<<grid, block, smem, st>>>(args...);
     }
 }
 
