@@ -324,13 +324,15 @@ spm_status spm_scene_phase_ms(spm_scene *scene, float *vertex_ms, float *cull_ms
                               float *pixel_ms);
 
 /* Tuning of the pixel pass's culling, per scene.
- * flood_mode: 0 = automatic (flood the per-tile candidate lists when the
- *   visibility graph among generators is sparse -- below 1% of all pairs,
- *   as in mazes -- otherwise let every tile scan every generator; decided on
- *   the device each compute), 1 = always flood, 2 = never flood, 3 = flood
- *   from geometry alone (every generator's visible tiles, no shadow cone) on
- *   the scene's own side stream, concurrently with the vertex phase; the
- *   pixel pass then applies costs and cones.
+ * flood_mode: 0 = automatic: mode 3 with depth maps (below) where the scene
+ *   has room for the maps; otherwise the per-tile candidate lists are flooded
+ *   when the visibility graph among generators is sparse (below 1% of all
+ *   pairs, as in mazes) and every tile scans every generator when it is not,
+ *   decided on the device each compute. 1 = always flood, 2 = never flood,
+ *   3 = flood from geometry alone (every generator's visible tiles, no shadow
+ *   cone) on the scene's own side stream, concurrently with the vertex phase;
+ *   the pixel pass then applies costs and cones. The obstacle vertices' part
+ *   is built by the scene's first such compute and kept.
  * hidden_chunk: 32..256, checked and reported; the pixel pass takes its
  *   candidates one by one in order of their lower bounds, so it has no effect.
  * tile: side of the tiles that carry the candidate lists, 16 or 32 pixels

@@ -176,6 +176,21 @@ void set_tile(spm::DevScene &ds, int tile) {
     ds.tiles_y = (ds.Ny + tile - 1) / tile;
 }
 
+// The descriptor a compute runs with. Automatic culling takes the geometric
+// flood with depth maps wherever the scene has room for them: the lists of the
+// obstacle vertices are kept, and a compute culls its sources beside the vertex
+// phase. (Scanning every generator, what it took on dense scenes before:
+// 512^2 polygons 147 us of pixel pass against 34.) Scenes without maps keep the
+// device's choice of flood or scan.
+spm::DevScene effective(const spm_scene *s) {
+    spm::DevScene d = s->ds;
+    if (d.flood_mode == 0 && d.use_flood && d.gen_maps && d.static_tile_start && spm::flood_sources_direct(d)) {
+        d.flood_mode = 3;
+        d.use_maps = 1;
+    }
+    return d;
+}
+
 spm_status upload_sources(spm_scene *s) {
     const spm::HostScene &hs = s->hs;
     spm::DevScene &ds = s->ds;
@@ -445,6 +460,7 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
                 start[vv + 1] = start[vv] + deg[vv];
             }
             const long long E_s = start[nv];
+            ds.open_scene = E_s >= 8LL * nv;
             if (E_s <= ds.edge_cap) {
                 for (int uu = 0; uu < nv; ++uu) {
                     out_init[ns + uu + 1] = out_start[uu + 1];
@@ -475,6 +491,14 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
                 ds.st_len = len;
             }
         }
+    }
+    ds.cull_items = nullptr;
+    ds.cull_count = nullptr;
+    if (ds.open_scene && ds.static_tile_start) {
+        auto tiles = [&](int t) { return (size_t)((hs.Nx + t - 1) / t) * ((hs.Ny + t - 1) / t); };
+        ds.cull_items = dalloc<int32_t>(s, std::max(tiles(spm::kTileSmall) * spm::cull_cap(spm::kTileSmall),
+                                                    tiles(spm::kTile) * spm::cull_cap(spm::kTile)));
+        ds.cull_count = dalloc<int32_t>(s, tiles(spm::kTileSmall));
     }
     if (!ok || s->alloc_failed) {
         free_all(s);
@@ -592,9 +616,10 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(cs, &cap);
     const bool timed = cap == cudaStreamCaptureStatusNone;
-    const bool side = s->ds.use_flood && s->ds.flood_mode == 3;  // geometric flood beside the vertex phase
-    s->ds.static_lists = side && s->ds.static_tile_start ? 1 : 0;  // the pixel pass reads the kept lists too
-    s->ds.src_direct = s->ds.static_lists && spm::flood_sources_direct(s->ds) ? 1 : 0;
+    spm::DevScene ds = effective(s);
+    const bool side = ds.use_flood && ds.flood_mode == 3;  // geometric flood beside the vertex phase
+    ds.static_lists = side && ds.static_tile_start ? 1 : 0;  // the pixel pass reads the kept lists too
+    ds.src_direct = ds.static_lists && spm::flood_sources_direct(s->ds) ? 1 : 0;
     NvtxRange range_all("spm_compute");
     if (timed) cudaEventRecord(s->ev[0], cs);
     // the geometric flood needs nothing from the vertex phase (costs and
@@ -603,47 +628,48 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     if (side) cudaEventRecord(s->fork, cs);
     {
         NvtxRange r("spm vertex phase");
-        spm::launch_vertex_phase(s->ds, cs, &s->vside);
+        spm::launch_vertex_phase(ds, cs, &s->vside);
     }
     if (side) {
         NvtxRange r("spm flood (side stream)");
         // the obstacle vertices' flood depends on the obstacles alone: built
         // once for this tile size and map setting, then only the sources flood
-        const bool maps = s->ds.use_maps && s->ds.gen_maps;
-        const bool reuse = s->flood_static_ok && s->flood_static_tile == s->ds.tile &&
-                           s->flood_static_maps == (int)maps && s->ds.static_tile_start;
+        const bool maps = ds.use_maps && ds.gen_maps;
+        const bool reuse = s->flood_static_ok && s->flood_static_tile == ds.tile &&
+                           s->flood_static_maps == (int)maps && ds.static_tile_start;
         cudaStreamWaitEvent(s->side, s->fork, 0);
-        spm::launch_flood(s->ds, s->side,
-                          !s->ds.static_tile_start ? spm::FloodStatic::kNone
+        spm::launch_flood(ds, s->side,
+                          !ds.static_tile_start ? spm::FloodStatic::kNone
                           : reuse                  ? spm::FloodStatic::kReuse
                                                    : spm::FloodStatic::kBuild);
         cudaEventRecord(s->join, s->side);
-        s->flood_static_ok = s->ds.static_tile_start != nullptr;
-        s->flood_static_tile = s->ds.tile;
+        // (a build recorded into a graph runs with every replay, and none has run yet)
+        s->flood_static_ok = ds.static_tile_start != nullptr && (timed || reuse);
+        s->flood_static_tile = ds.tile;
         s->flood_static_maps = (int)maps;
     }
     if (timed) cudaEventRecord(s->ev[1], cs);
     if (side) {
         cudaStreamWaitEvent(cs, s->join, 0);
-    } else if (s->ds.use_flood) {
-        spm::launch_flood(s->ds, cs);
+    } else if (ds.use_flood) {
+        spm::launch_flood(ds, cs);
         s->flood_static_ok = false;  // the lists and maps now hold this flood's
     } else {
         static const int32_t off[4] = {0, 0, 1, 0};
-        cudaMemcpyAsync(s->ds.flood_counts, off, sizeof off, cudaMemcpyHostToDevice, cs);
+        cudaMemcpyAsync(ds.flood_counts, off, sizeof off, cudaMemcpyHostToDevice, cs);
     }
     if (timed) cudaEventRecord(s->ev[3], cs);
     if (!dist_host) {
         NvtxRange r("spm pixel phase");
-        spm::launch_pixel_phase(s->ds, cs, dist, parent, tile_row0, tile_row1);
+        spm::launch_pixel_phase(ds, cs, dist, parent, tile_row0, tile_row1);
     } else {
         NvtxRange r("spm pixel phase with host copies");
         const int rows = tile_row1 - tile_row0, nslab = std::min(rows, (int)(sizeof s->slab_ev / sizeof s->slab_ev[0]));
         const size_t Nx = (size_t)s->hs.Nx, Ny = (size_t)s->hs.Ny;
         auto slab_rows = [&](int k, size_t &r0, size_t &r1) {
             const int t0 = tile_row0 + rows * k / nslab, t1 = tile_row0 + rows * (k + 1) / nslab;
-            r0 = (size_t)t0 * s->ds.tile;
-            r1 = std::min((size_t)t1 * s->ds.tile, Ny);
+            r0 = (size_t)t0 * ds.tile;
+            r1 = std::min((size_t)t1 * ds.tile, Ny);
         };
         auto drain = [&](int k) {  // host: slab k from its bounce buffer into the caller's planes
             size_t r0, r1;
@@ -655,7 +681,7 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
         };
         for (int k = 0; k < nslab; ++k) {
             const int t0 = tile_row0 + rows * k / nslab, t1 = tile_row0 + rows * (k + 1) / nslab;
-            spm::launch_pixel_phase(s->ds, cs, dist, parent, t0, t1);
+            spm::launch_pixel_phase(ds, cs, dist, parent, t0, t1);
             cudaEventRecord(s->slab_ev[k], cs);
             cudaStreamWaitEvent(s->copy, s->slab_ev[k], 0);
             size_t r0, r1;
@@ -898,7 +924,7 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     std::vector<int32_t *> pv(parent, parent + n);
     int max_gen = 0;
     for (int k = 0; k < n; ++k) {
-        descs[k] = scenes[k]->ds;
+        descs[k] = effective(scenes[k]);
         descs[k].warm = 0;  // the batched fixpoint starts every scene from its sources
         // geometric floods reuse the obstacle vertices' static lists: built
         // here if the scene has none for this tile size and map setting
@@ -914,6 +940,7 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         // reusing scenes cull their sources directly where the maps allow it
         const spm::DevScene &d = descs[k];
         descs[k].src_direct = d.flood_reuse && spm::flood_sources_direct(d) ? 1 : 0;
+        descs[k].cull_on = spm::tiles_culled(d) ? 1 : 0;
         const long long direct = descs[k].src_direct, ntl = (long long)d.tiles_x * d.tiles_y;
         src_map_off[k + 1] = src_map_off[k] + direct * d.n_src * spm::kAngBins;
         src_ins_off[k + 1] = src_ins_off[k] + direct * d.n_src * spm::src_edge_warps(d.n_edge);
@@ -957,6 +984,7 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     b->src_tiles = src_tile_off[n];
     bd.order = bupload(b, order, ok);
     bd.tile_off = bupload(b, tile_off, ok);
+    bd.total_tiles = tile_off[n];
     bd.blk_off = bupload(b, blk_off, ok);
     bd.total_blocks = blk_off[n];
     bd.tile_counter = balloc<int32_t>(b, 1);
@@ -984,6 +1012,8 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     bd.flood_smem = 0;
     bd.any_maps = 0;
     bd.any_lists = 0;
+    bd.any_cull = 0;
+    for (int k = 0; k < n; ++k) bd.any_cull |= spm::tiles_culled(descs[k]);
     for (int k = 0; k < n; ++k)
         bd.any_lists |= descs[k].use_flood && descs[k].flood_mode != 2 && !descs[k].src_direct;
     for (int k = 0; k < n; ++k) bd.any_maps |= descs[k].use_flood && descs[k].flood_mode != 2 && descs[k].use_maps;
@@ -1228,18 +1258,19 @@ spm_status spm_scene_info(spm_scene *s, int64_t *info) {
     info[7] = s->ds.tile;
     info[8] = (s->ds.use_flood && fc[2] == 0) ? 1 : 0;
     info[9] = s->ds.flood_mode;
-    const bool floods = s->ds.use_flood && s->ds.flood_mode != 2;
+    const spm::DevScene run = effective(s);
+    const bool floods = run.use_flood && run.flood_mode != 2;
     // the geometric mode over kept obstacle-vertex lists: the sources' culling
     // (list reset, the walk and the list scan and fill, or maps from every
     // polygon and the tile tests)
-    const bool reuse = floods && s->ds.flood_mode == 3 && s->ds.static_tile_start;
-    const int src_cull = !spm::flood_sources_direct(s->ds) ? 4 : s->ds.n_poly > 0 ? 3 : 2;
+    const bool reuse = floods && run.flood_mode == 3 && run.static_tile_start;
+    const int src_cull = !spm::flood_sources_direct(run) ? 4 : s->ds.n_poly > 0 ? 3 : 2;
     // vertex phase (prep, pairs, edges, the tree's kernels, fixpoint kernels,
     // and after the many-CTA one its finalisation); flood, list scan and
     // fill; pixels
     const int many_cta = s->ds.fix_launch & (spm::kFixSoloSure | spm::kFixClusterSure) ? 0 : 2;
     info[10] = 1 + (s->hs.n_vert > 0 ? 4 : 0) + (s->ds.warm && s->ds.vtab ? 4 : 0) + (s->ds.fix_launch & spm::kFixSolo ? 1 : 0) +
-               (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull : 3) : 0) + 1;
+               (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull : 3) : 0) + (spm::tiles_culled(run) ? 1 : 0) + 1;
     return SPM_OK;
 }
 

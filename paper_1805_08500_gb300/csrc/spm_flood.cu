@@ -211,6 +211,53 @@ __device__ void insert_polygon_warp(const DevScene &ds, float *depth2, float *lo
     }
 }
 
+// Edges e0 .. e0 + kSrcEdges - 1 into the map of a generator at g, one warp: a
+// lane views an edge, then the bins they span are dealt to the lanes evenly (a
+// wall next to the generator spans hundreds, a far one two or three). With up
+// to check_most bins in all, they are read before they are written (far edges
+// lower few bins; the wide ones are near and lower most).
+constexpr int kSrcEdges = 16;
+template <bool MAPS>
+__device__ __forceinline__ void insert_edges_warp(const DevScene &ds, float *up, float *low, int2 g, int e0, int stride,
+                                                  int check_most) {
+    const int lane = threadIdx.x & 31;
+    EdgeView v = {};
+    int span = 0;
+    if (lane < kSrcEdges && e0 + lane < ds.n_edge && edge_view(g, __ldg(ds.edges + e0 + lane), v))
+        span = v.k1 - v.k0 + 1;
+    int incl = span;
+#pragma unroll
+    for (int o = 1; o < kSrcEdges; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, kSrcEdges - 1);
+    for (int r0 = 0; r0 < total; r0 += 32) {
+        const int r = r0 + lane;
+        int own = 0;  // the first edge whose bins end beyond r
+#pragma unroll
+        for (int o = kSrcEdges / 2; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, incl, own + o - 1) <= r) own += o;
+        own = min(own, kSrcEdges - 1);
+        EdgeView o;
+        auto take = [&](float x) { return __shfl_sync(0xffffffffu, x, own); };
+        o.ex = __shfl_sync(0xffffffffu, v.ex, own);
+        o.ey = __shfl_sync(0xffffffffu, v.ey, own);
+        o.nx = -o.ey;
+        o.ny = o.ex;
+        o.N2 = take(v.N2);
+        o.h2 = take(v.h2);
+        o.lo = take(v.lo);
+        o.hi = take(v.hi);
+        o.c2 = take(v.c2);
+        o.a2 = take(v.a2);
+        o.sc = take(v.sc);
+        o.sa = take(v.sa);
+        const int k = r - __shfl_sync(0xffffffffu, incl - span - v.k0, own);
+        if (r < total) edge_into_bin<MAPS>(o, k, up, low, stride, total <= check_most);
+    }
+}
+
 // Floods generator g of scene ds: one CTA, a breadth-first level at a time.
 // MAPS: also keep g's depth map (with the lower-bound bins) for the pixel pass.
 template <bool MAPS>
@@ -395,6 +442,74 @@ __device__ void flood_one(const DevScene &ds, FloodSmem &sm, unsigned *fdyn, int
     SPM_TFLUSH();
 }
 
+// Geometric culling of generator g without the walk: one CTA enters every
+// polygon edge into its map and tests every tile against the complete map. In
+// an open scene a generator reaches much of the grid, and the walk's levels
+// (four barriers each, the whole grid's width deep) cost far more: first
+// compute of the 1024^2 polygons, 1188 generators, 1.2 ms of walks.
+// hit: a bit per tile. A superset of what the walk reaches.
+template <bool MAPS>
+__device__ void flood_direct(const DevScene &ds, float *up, float *low, unsigned *hit, int g) {
+    __shared__ long long wsum[32];
+    __shared__ int base;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gl8 = lane & 7;
+    const int ntiles = ds.tiles_x * ds.tiles_y, words = (ntiles + 31) / 32;
+    const int2 gl = ds.gen_lat[g];
+    __syncthreads();  // the previous generator is done with smem
+    for (int k = tid; k < kAng; k += kFloodThreads) up[k] = low[k] = INFINITY;
+    for (int w = tid; w < words; w += kFloodThreads) hit[w] = 0u;
+    __syncthreads();
+    for (int e = warp * kSrcEdges; e < ds.n_edge; e += kFloodThreads / 32 * kSrcEdges)
+        insert_edges_warp<MAPS>(ds, up, low, gl, e, 1, 1 << 30);
+    __syncthreads();
+    const unsigned gmask = 0xffu << (lane & 24);
+    for (int t0 = warp * 4; t0 < ntiles; t0 += kFloodThreads / 32 * 4) {
+        const int t = t0 + (lane >> 3);
+        if (t >= ntiles) continue;  // whole groups
+        const int4 area = tile_area(ds, t % ds.tiles_x, t / ds.tiles_x);
+        const bool inside = gl.x >= area.x && gl.x <= area.z && gl.y >= area.y && gl.y <= area.w;
+        const bool seen = inside || !box_hidden_ang<8>(up, gl, area, gl8, gmask, 1);
+        if (seen && gl8 == 0) atomicOr(&hit[t >> 5], 1u << (t & 31));
+    }
+    __syncthreads();
+    int mine = 0;
+    for (int w = tid; w < words; w += kFloodThreads) mine += __popc(hit[w]);
+    const long long before = cta_exclusive_scan(mine, wsum);
+    if (tid == kFloodThreads - 1) base = atomicAdd(&ds.flood_counts[0], (int)before + mine);
+    __syncthreads();
+    int slot = base + (int)before;
+    for (int w = tid; w < words; w += kFloodThreads)
+        for (unsigned m = hit[w]; m; m &= m - 1, ++slot) {
+            const int t = 32 * w + __ffs(m) - 1;
+            if (slot < ds.pair_cap) {
+                ds.pairs[slot] = make_int2(t, g);
+                atomicAdd(&ds.tile_count[t], 1);
+            } else {
+                atomicOr(&ds.flood_counts[2], 1);
+            }
+        }
+    if (MAPS) {
+        float2 *mp = ds.gen_maps + (size_t)g * kAng;
+        for (int k = tid; k < kAng; k += kFloodThreads) mp[k] = make_float2(up[k], low[k]);
+    }
+    if (tid == 0 && ds.gen_map_ok) ds.gen_map_ok[g] = MAPS ? 1 : 0;
+}
+
+// Resident CTAs take the obstacle vertices [g0, g1) from the work counter.
+template <bool MAPS>
+__global__ void __launch_bounds__(kFloodThreads, 6) k_flood_direct(const __grid_constant__ DevScene ds, int g0, int g1) {
+    extern __shared__ unsigned fdyn[];
+    __shared__ float up[kAng], low[kAng];
+    __shared__ int next_g;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) next_g = g0 + atomicAdd(&ds.flood_counts[3], 1);
+        __syncthreads();
+        if (next_g >= g1) break;
+        flood_direct<MAPS>(ds, up, low, fdyn, next_g);
+    }
+}
+
 // Direct culling of the sources (generators [0, n_src)) in the geometric
 // mode: few generators, each reaching much of the grid, which one CTA per
 // generator would walk a breadth-first level at a time. Instead every
@@ -422,50 +537,11 @@ __device__ __forceinline__ void src_prep(const DevScene &ds, int i0, int stride)
     if (i0 < 4) ds.flood_counts[i0] = i0 == 1 || i0 == 2 ? ds.static_counts[i0] : 0;
 }
 
-// Edges e0 .. e0 + kSrcEdges - 1 into source g's map, one warp: a lane views
-// an edge, then the bins they span are dealt to the lanes evenly (a wall next
-// to the source spans hundreds, a far one two or three).
-constexpr int kSrcEdges = 16;
 template <bool MAPS>
 __device__ __forceinline__ void src_insert(const DevScene &ds, int g, int e0) {
-    const int lane = threadIdx.x & 31;
     if (!src_on_grid(ds, g)) return;  // the same for the whole warp
     float *mp = reinterpret_cast<float *>(ds.gen_maps + (size_t)g * kAng);
-    EdgeView v = {};
-    int span = 0;
-    if (lane < kSrcEdges && e0 + lane < ds.n_edge && edge_view(ds.gen_lat[g], __ldg(ds.edges + e0 + lane), v))
-        span = v.k1 - v.k0 + 1;
-    int incl = span;
-#pragma unroll
-    for (int o = 1; o < kSrcEdges; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, kSrcEdges - 1);
-    for (int r0 = 0; r0 < total; r0 += 32) {
-        const int r = r0 + lane;
-        int own = 0;  // the first edge whose bins end beyond r
-#pragma unroll
-        for (int o = kSrcEdges / 2; o > 0; o >>= 1)
-            if (__shfl_sync(0xffffffffu, incl, own + o - 1) <= r) own += o;
-        own = min(own, kSrcEdges - 1);
-        EdgeView o;
-        auto take = [&](float x) { return __shfl_sync(0xffffffffu, x, own); };
-        o.ex = __shfl_sync(0xffffffffu, v.ex, own);
-        o.ey = __shfl_sync(0xffffffffu, v.ey, own);
-        o.nx = -o.ey;
-        o.ny = o.ex;
-        o.N2 = take(v.N2);
-        o.h2 = take(v.h2);
-        o.lo = take(v.lo);
-        o.hi = take(v.hi);
-        o.c2 = take(v.c2);
-        o.a2 = take(v.a2);
-        o.sc = take(v.sc);
-        o.sa = take(v.sa);
-        const int k = r - __shfl_sync(0xffffffffu, incl - span - v.k0, own);
-        if (r < total) edge_into_bin<MAPS>(o, k, mp, mp + 1, 2, total <= 64);  // wide ones are near and lower most bins
-    }
+    insert_edges_warp<MAPS>(ds, mp, mp + 1, ds.gen_lat[g], e0, 2, 64);
 }
 
 // Tile t's bits: a warp, its groups of kSrcGrp lanes a source each (most tiles
@@ -771,7 +847,14 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
         if (how == FloodStatic::kBuild) {  // the obstacle vertices' lists, kept for every later compute
             cudaMemsetAsync(ds.tile_count, 0, sizeof(int32_t) * ntiles, st);
             cudaMemsetAsync(ds.flood_counts, 0, sizeof(int32_t) * 4, st);
-            flood(ds.n_src, ds.n_gen);
+            if (flood_verts_direct(ds)) {
+                const size_t bits = sizeof(unsigned) * (size_t)((ntiles + 31) / 32);
+                const int blocks = std::min(max(sms, 1) * 6, ds.n_vert);
+                if (maps) k_flood_direct<true><<<blocks, kFloodThreads, bits, st>>>(ds, ds.n_src, ds.n_gen);
+                else k_flood_direct<false><<<blocks, kFloodThreads, bits, st>>>(ds, ds.n_src, ds.n_gen);
+            } else {
+                flood(ds.n_src, ds.n_gen);
+            }
             k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
             k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 1);
             k_flood_static<<<sblocks, 256, 0, st>>>(ds, 1);
@@ -796,6 +879,14 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
 bool flood_sources_direct(const DevScene &ds) {
     const long long ntiles = (long long)ds.tiles_x * ds.tiles_y;
     return ds.gen_maps && ds.n_src > 0 && (long long)ds.n_src * (ds.n_poly + ntiles) <= (1LL << 24);
+}
+
+// The obstacle vertices without the walk: in open scenes, where a vertex sees
+// many others (mazes: 3 tangent edges a vertex, polygon scenes: 8 to 45), and
+// while a generator's edges and tiles stay a few thousand.
+bool flood_verts_direct(const DevScene &ds) {
+    const long long ntiles = (long long)ds.tiles_x * ds.tiles_y;
+    return ds.n_vert > 0 && (ds.open_scene || ds.n_edge + ntiles <= 1024) && ds.n_edge + ntiles <= (1 << 16);
 }
 
 int src_edge_warps(int n_edge) { return (n_edge + kSrcEdges - 1) / kSrcEdges; }

@@ -171,6 +171,7 @@ struct DevScene {
     // tiles and their candidate lists (flood)
     int32_t tile;                      // tile side in pixels: 16 or 32
     int32_t tiles_x, tiles_y;
+    int32_t open_scene;                // an obstacle vertex has 8 tangent edges or more on average
     int32_t use_flood;                 // 0: flood impossible (too many tiles for smem)
     int32_t flood_mode;                // 0 auto (sparse visibility graph), 1 on, 2 off, 3 geometric (concurrent)
     int32_t hidden_chunk;              // first hidden-test chunk in the pixel pass
@@ -200,6 +201,10 @@ struct DevScene {
     int32_t *static_tile_items;        // pair_cap
     int32_t *static_counts;            // 4
     int32_t static_lists;              // the pixel pass reads the static lists as well (this compute)
+    // open scenes: per tile the entries of those lists that can win somewhere in
+    // it, at most cull_cap(tile) of them (cull_count -1: more, take the lists)
+    int32_t *cull_items, *cull_count;
+    int32_t cull_on;                   // this compute culls them
     int32_t flood_reuse;               // in a batch's copy: flood the sources only, over the static part
     // this compute's sources are culled directly (complete maps): instead of
     // pairs and lists, a bit per source, src_words words a tile
@@ -220,6 +225,7 @@ struct BatchDev {
     // pixel pass: scenes in processing order (costliest tiles first)
     const int32_t *order;              // n scene indices
     const int32_t *tile_off;           // n + 1 prefix of tiles in that order
+    int32_t total_tiles;
     const int32_t *blk_off;            // n + 1 prefix of 16 x 16 pixel blocks in that order
     int32_t total_blocks;
     int32_t *tile_counter;             // persistent-kernel work counter
@@ -238,6 +244,7 @@ struct BatchDev {
     const long long *src_ins_off;      // warp tasks of the map building: n_src * src_edge_warps(n_edge)
     const long long *src_tile_off;     // warp tasks of the tile tests: tiles
     int32_t walk_tasks;                // (scene, generator) walks of the batched flood
+    int32_t any_cull;                  // some scene culls its lists per tile
     int32_t any_lists;                 // some scene sorts lists per compute (its sources are not culled directly)
     // vertex fixpoint on resident clusters, one scene at a time
     const int32_t *cl_order;           // n scene indices, most generators first
@@ -256,6 +263,9 @@ struct VertexSide {
     cudaEvent_t fork, join;
 };
 void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *side = nullptr);
+// entries a tile's culled list may hold: 32 KB of them a 128 x 128 pixels
+constexpr int cull_cap(int tile) { return tile == kTile ? 512 : 128; }
+bool tiles_culled(const DevScene &ds);  // the pixel pass culls its lists per tile first
 // pixel kernel over the tiles of tile rows [tile_row0, tile_row1)
 void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int tile_row0,
                         int tile_row1);
@@ -291,6 +301,7 @@ int flood_smem_attr();
 // the geometric mode culls the sources directly (complete depth maps, every
 // tile tested at once) rather than by the per-generator walk
 bool flood_sources_direct(const DevScene &ds);
+bool flood_verts_direct(const DevScene &ds);  // the same for the obstacle vertices, once per scene
 int src_edge_warps(int n_edge);  // warps that put a scene's edges into one source's map
 int sssp_grid_blocks();  // co-resident CTAs for the cooperative fixpoint kernel
 int solo_smem_bytes();   // shared memory granted to the single-CTA fixpoint kernel (0 if refused)

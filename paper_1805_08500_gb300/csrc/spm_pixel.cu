@@ -13,11 +13,11 @@
 //     lower bound lb = cost + dist(g, block) below the block's current worst;
 //   * order: candidates in order of lb; the warp stops once every pixel's best
 //     is <= lb (no later candidate can win);
-//   * depth maps (when the flood kept them): the bins the block spans may show
-//     that it sees the candidate as a whole or not at all; otherwise a pixel
-//     nearer than the lower bound of its bin sees it, one beyond the
-//     full-blocking upper bound does not, and only the pixels in between take
-//     the exact test below;
+//   * depth maps (when the flood kept them): a pixel nearer than the lower
+//     bound of its bin sees the candidate, one beyond the full-blocking upper
+//     bound does not, and only the pixels in between take the exact test below
+//     (deciding whole blocks from the bins they span first cost as much as it
+//     saved: half of the blocks are neither);
 //   * visibility: the warp lists the polygons whose interior may meet the hull
 //     of (block, g), and every undecided pixel runs the exact integer
 //     separating-axis test against that list (none when the list is empty);
@@ -63,7 +63,8 @@ __device__ __forceinline__ float segment_lower_bound(const DevScene &ds, int s, 
 // ---------------------------------------------------------------------------
 // One warp, one block of pixels (16 x 16, smaller on small grids), no barrier.
 // ---------------------------------------------------------------------------
-constexpr int kWarpCand = 96;    // candidates a warp holds before it works them off
+constexpr int kWarpCand = 160;   // candidates a warp holds before it works them off: nearly every block's at once
+                                 // (in parts, a block's true generators may come last: 50 processed where 16 would do)
 constexpr int kWarpPoly = 64;    // blocker polygons a warp lists at a time
 constexpr int kBlocked = 1 << 15; // an undecided pixel found blocked
 
@@ -108,6 +109,57 @@ __device__ __forceinline__ float point_dist(float cf, float dx, float dy) { retu
 __device__ __forceinline__ float pixel_x(const DevScene &ds, int i) { return ((float)i + 0.5f) * ds.hx; }
 __device__ __forceinline__ float pixel_y(const DevScene &ds, int j) { return ((float)j + 0.5f) * ds.hy; }
 
+// The candidates of a tile's pixels: the list culled for the tile, or the kept
+// list of obstacle vertices, this compute's entries (a bit per source, or a
+// list) and the global list, or every generator.
+struct TileList {
+    const int32_t *a, *l, *gl;  // entries [0, na), [na, nl) and [nl, total)
+    const uint32_t *bits;       // or the middle part's bits
+    int na, nl, total;
+    bool lists;
+    __device__ __forceinline__ TileList(const DevScene &ds, int tile, bool culled) {
+        lists = ds.use_flood && ds.flood_counts[2] == 0;
+        a = l = gl = ds.glob_list;
+        bits = nullptr;
+        na = nl = 0;
+        total = ds.n_gen;
+        if (!lists) return;
+        if (culled && ds.cull_on) {
+            na = nl = total = ds.cull_count[tile];
+            a = ds.cull_items + (size_t)tile * cull_cap(ds.tile);
+            if (total >= 0) return;
+            na = 0;
+        }
+        if (ds.static_lists) {
+            const int s0 = ds.static_tile_start[tile];
+            na = ds.static_tile_start[tile + 1] - s0;
+            a = ds.static_tile_items + s0;
+        }
+        if (ds.static_lists && ds.src_direct) {
+            bits = ds.src_mask + (size_t)tile * ds.src_words;
+            nl = na + ds.n_src;
+        } else {
+            const int l0 = ds.tile_start[tile];
+            nl = na + ds.tile_start[tile + 1] - l0;
+            l = ds.tile_items + l0;
+        }
+        total = nl + ds.flood_counts[1];
+    }
+    // entry e's generator, or false when there is none
+    __device__ __forceinline__ bool entry(const DevScene &ds, int e, int &g) const {
+        if (e >= total) return false;
+        g = e;
+        if (!lists) return true;
+        const int r = e - na;
+        if (r >= 0 && e < nl && bits) {
+            g = r;
+            return __ldg(bits + (r >> 5)) >> (r & 31) & 1u;
+        }
+        g = __ldg(r < 0 ? a + e : e < nl ? l + r : gl + (e - nl));
+        return true;
+    }
+};
+
 // Generator g as a candidate of the block: its lower bound and flags; false
 // when it cannot win anywhere in the block. Most entries of a list go by their
 // cost or cone, one 16-byte load.
@@ -141,41 +193,6 @@ __device__ __forceinline__ bool block_candidate(const DevScene &ds, int g, const
     if ((lo1 | lo2) >= 0 && (q.y != q.z || q.y == 0)) cand |= kCandInCone;
     if (maps && ds.gen_map_ok[g]) cand |= kCandMap;
     return true;
-}
-
-// What the depth map says about the whole block: 0 every pixel sees the
-// generator, 1 none does, 2 neither is shown. The block's box spans less than
-// half a turn seen from a point outside it, so its corners bound its angles.
-__device__ __forceinline__ int block_class(const float2 *map, int2 gl, const int4 box) {
-    const int lane = threadIdx.x & 31;
-    if (gl.x >= box.x - 1 && gl.x <= box.z + 1 && gl.y >= box.y - 1 && gl.y <= box.w + 1) return 2;
-    const float x0 = (float)(box.x - gl.x), x1 = (float)(box.z - gl.x), y0 = (float)(box.y - gl.y),
-                y1 = (float)(box.w - gl.y);
-    const float a = pang(lane & 1 ? x1 : x0, lane & 2 ? y1 : y0);
-    const float a0 = __shfl_sync(0xffffffffu, a, 0);
-    float d = a - a0;
-    if (d > 2.f) d -= 4.f;
-    if (d < -2.f) d += 4.f;
-    const float d1 = __shfl_xor_sync(0xffffffffu, d, 1);
-    float lo = fminf(d, d1), hi = fmaxf(d, d1);
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, 2));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 2));
-    const int k0 = (int)floorf((a0 + lo - kAngEps) / kAngW), k1 = (int)floorf((a0 + hi + kAngEps) / kAngW);
-    if (k1 - k0 >= 256) return 2;  // a generator next to the block: pixel by pixel
-    float up = 0.f, low = INFINITY;
-    for (int k = k0 + lane; k <= k1; k += 32) {
-        const float2 b = __ldg(map + ((k + kAngBins) & (kAngBins - 1)));
-        up = fmaxf(up, b.x);
-        low = fminf(low, b.y);
-    }
-    // non-negative floats order as their bits
-    const float l = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(low)));
-    const float u = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(up)));
-    const float fx = fmaxf(fabsf(x0), fabsf(x1)), fy = fmaxf(fabsf(y0), fabsf(y1));
-    if (fmaf(fx, fx, fy * fy) * (1.f + 1e-5f) < l) return 0;
-    const float nx = fmaxf(fmaxf(x0, -x1), 0.f), ny = fmaxf(fmaxf(y0, -y1), 0.f);
-    if (fmaf(nx, nx, ny * ny) * (1.f - 1e-5f) >= u) return 1;
-    return 2;
 }
 
 // Depth-map bins a pixel at offset (rx, ry) != 0 may lie in.
@@ -391,9 +408,6 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX 
     const bool seg = (__float_as_int(rec.w) & 7) == kSegI;
     const int seg_id = seg ? ds.gen_aux[g] : -1;
     const float2 *map = c & kCandMap ? ds.gen_maps + (size_t)g * kAngBins : nullptr;
-    const int cls = map ? block_class(map, gl, b.box) : 2;
-    if (lane == 0) SPM_CNT(cls == 0 ? 2 : cls == 1 ? 3 : 8, 1);
-    if (cls == 1) return;
     float4 sf = make_float4(0.f, 0.f, 0.f, 0.f);
     float il = 0.f;
     if (seg) {
@@ -401,39 +415,32 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX 
         const float fux = sf.z - sf.x, fuy = sf.w - sf.y;
         il = 1.0f / sqrtf(fux * fux + fuy * fuy);
     }
-    auto dist_at = [&](int k) {
-        const float fx = pixel_x(ds, b.i + k % PX), fy = pixel_y(ds, b.j + k / PX * kStep);
-        return seg ? fabsf((sf.z - sf.x) * (fy - sf.y) - (sf.w - sf.y) * (fx - sf.x)) * il
-                   : point_dist(rec.z, fx - rec.x, fy - rec.y);
-    };
-    const bool take_all = cls == 0 && (c & kCandInCone);
     unsigned want = 0;
-    float worst = -INFINITY;
 #pragma unroll 1
     for (int h = 0; h < PY; ++h) {
-#pragma unroll
+#pragma unroll 2
         for (int k4 = 0; k4 < PX; ++k4) {
             const int k = PX * h + k4, at = k * 32 + lane;
-            const float d = dist_at(k);
-            float old = ws.bd[at];
+            const float d = point_dist(rec.z, pixel_x(ds, b.i + k4) - rec.x, pixel_y(ds, b.j + h * kStep) - rec.y);
+            const float old = ws.bd[at];
             bool better = d < old;
             if (d == old) better = g < ws.bi[at];
             if (better) want |= 1u << k;
-            if (!take_all) {
-                ws.d[at] = d;
-            } else if (better) {
-                ws.bd[at] = d;
-                ws.bi[at] = g;
-                old = d;
-            }
-            worst = fmaxf(worst, old);
+            ws.d[at] = d;
+        }
+    }
+    if (seg) {
+        want = 0;
+#pragma unroll 1
+        for (int k = 0; k < PX * PY; ++k) {
+            const float fx = pixel_x(ds, b.i + k % PX), fy = pixel_y(ds, b.j + k / PX * kStep);
+            const float d = fabsf((sf.z - sf.x) * (fy - sf.y) - (sf.w - sf.y) * (fx - sf.x)) * il, old = ws.bd[k * 32 + lane];
+            ws.d[k * 32 + lane] = d;
+            if (d < old || (d == old && g < ws.bi[k * 32 + lane])) want |= 1u << k;
         }
     }
     SPM_CNT(14, __popc(want));
-    if (take_all) {
-        b.worst = worst;
-        return;
-    }
+    if (!__any_sync(0xffffffffu, want)) return;
     unsigned vis = 0, und = 0;
     float clear = INFINITY;
     const int rx0 = ds.pitch_x * b.i + ds.pitch_x / 2 - gl.x, ry0 = ds.pitch_y * b.j + ds.pitch_y / 2 - gl.y;
@@ -459,9 +466,7 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX 
                 if (!(want & bit)) continue;
                 const int ix = rx0 + k4 * ds.pitch_x, iy = ry0 + h * kStep * ds.pitch_y;
                 if (!(c & kCandInCone) && !in_cone(ct, cone, ix, iy)) continue;
-                if (cls == 0) {
-                    vis |= bit;
-                } else if (!map) {
+                if (!map) {
                     und |= bit;
                 } else {
                     const float rx = (float)ix, ry = (float)iy, r2 = fmaf(rx, rx, ry * ry);
@@ -486,18 +491,19 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX 
         const float near = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(clear)));
         vis |= resolve_pixels<PX, PY>(ds, ws, b, gl, seg_id, map ? sqrtf(near) : 0.f, und);
     }
-    if (vis) {
-#pragma unroll 1
-        for (unsigned m = vis; m; m &= m - 1) {
-            const int k = __ffs(m) - 1;
-            ws.bd[k * 32 + lane] = ws.d[k * 32 + lane];
-            ws.bi[k * 32 + lane] = g;
-        }
-        worst = -INFINITY;
+    float worst = -INFINITY;
 #pragma unroll
-        for (int k = 0; k < PX * PY; ++k) worst = fmaxf(worst, ws.bd[k * 32 + lane]);
-        b.worst = worst;
+    for (int k = 0; k < PX * PY; ++k) {
+        const int at = k * 32 + lane;
+        float d = ws.bd[at];
+        if (vis >> k & 1u) {
+            d = ws.d[at];
+            ws.bd[at] = d;
+            ws.bi[at] = g;
+        }
+        worst = fmaxf(worst, d);
     }
+    b.worst = worst;
 }
 
 // The n candidates the warp holds, in order of their lower bounds, until none
@@ -585,34 +591,17 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
         b.j1 = min(b.j0 + S::kH, ds.Ny) - 1;
         b.box = make_int4(ds.pitch_x * b.i0 + ds.pitch_x / 2, ds.pitch_y * b.j0 + ds.pitch_y / 2,
                           ds.pitch_x * b.i1 + ds.pitch_x / 2, ds.pitch_y * b.j1 + ds.pitch_y / 2);
-        b.lists = ds.use_flood && ds.flood_counts[2] == 0;
         const int sh = ds.tile == kTile ? 5 : 4, tile = (j0 >> sh) * ds.tiles_x + (i0 >> sh);  // tiles of 32 or 16 pixels
-        const bool stat = b.lists && ds.static_lists, maps = b.lists && ds.use_maps && ds.gen_maps;
-        // the kept list of obstacle vertices, this compute's entries (a bit per
-        // source, or a list), the global list; or every generator
-        const bool bits = stat && ds.src_direct;
-        const int s0 = stat ? ds.static_tile_start[tile] : 0, ns = stat ? ds.static_tile_start[tile + 1] - s0 : 0;
-        const int l0 = b.lists && !bits ? ds.tile_start[tile] : 0;
-        const int nl = ns + (bits ? ds.n_src : b.lists ? ds.tile_start[tile + 1] - l0 : 0);
-        const int total = b.lists ? nl + ds.flood_counts[1] : ds.n_gen;
+        const TileList tl(ds, tile, true);
+        b.lists = tl.lists;
+        const bool maps = b.lists && ds.use_maps && ds.gen_maps;
         float ub = INFINITY;  // no pixel of the block can take more
         int n = 0;
-        for (int e0 = 0; e0 < total; e0 += 32) {
-            const int e = e0 + lane;
+        for (int e0 = 0; e0 < tl.total; e0 += 32) {
             bool keep = false;
             float lb = 0.f;
-            int c = 0;
-            int g = e;
-            bool in = e < total;
-            if (in && b.lists) {
-                const int r = e - ns;
-                if (r >= 0 && e < nl && bits) {
-                    g = r;
-                    in = __ldg(ds.src_mask + (size_t)tile * ds.src_words + (r >> 5)) >> (r & 31) & 1u;
-                } else {
-                    g = __ldg(r < 0 ? ds.static_tile_items + s0 + e : e < nl ? ds.tile_items + l0 + r : ds.glob_list + e - nl);
-                }
-            }
+            int c = 0, g = 0;
+            const bool in = tl.entry(ds, e0 + lane, g);
             if (in) keep = block_candidate(ds, g, b, ub, maps, lb, c);
             const unsigned bal = __ballot_sync(0xffffffffu, keep);
             if (keep) {
@@ -621,7 +610,7 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
                 ws.cand[slot] = c;
             }
             n += __popc(bal);
-            const bool last = e0 + 32 >= total;
+            const bool last = e0 + 32 >= tl.total;
             if (n > kWarpCand - 32 || (last && n > 0)) {
                 if (lane == 0) SPM_CNT(1, n);
                 apply_candidates<PX, PY, SCAN>(ds, ws, n, b);
@@ -665,6 +654,58 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
     }
 }
 
+// Open scenes: most of a tile's list (every obstacle vertex that sees some of
+// it) goes by its shadow cone, alike for the tile's blocks: one CTA culls the
+// list for the tile. (Each block culling the whole list was half of the pixel
+// pass of the differentiable scene, 900 entries a tile.)
+constexpr int kCullThreads = 128;
+__device__ __forceinline__ void cull_tile(const DevScene &ds, int tile) {
+    __shared__ int n;
+    const int lane = threadIdx.x & 31, cap = cull_cap(ds.tile);
+    if (threadIdx.x == 0) n = 0;
+    __syncthreads();
+    Block b;
+    b.i0 = tile % ds.tiles_x * ds.tile;
+    b.j0 = tile / ds.tiles_x * ds.tile;
+    b.i1 = min(b.i0 + ds.tile, ds.Nx) - 1;
+    b.j1 = min(b.j0 + ds.tile, ds.Ny) - 1;
+    b.box = make_int4(ds.pitch_x * b.i0 + ds.pitch_x / 2, ds.pitch_y * b.j0 + ds.pitch_y / 2,
+                      ds.pitch_x * b.i1 + ds.pitch_x / 2, ds.pitch_y * b.j1 + ds.pitch_y / 2);
+    const TileList tl(ds, tile, false);
+    int32_t *out = ds.cull_items + (size_t)tile * cap;
+    for (int e0 = threadIdx.x & ~31; tl.lists && e0 < tl.total; e0 += kCullThreads) {
+        int g = 0, c;
+        float lb;
+        const bool keep = tl.entry(ds, e0 + lane, g) && block_candidate(ds, g, b, INFINITY, false, lb, c);
+        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+        int at = 0;
+        if (lane == 0 && bal) at = atomicAdd(&n, __popc(bal));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (keep && at < cap) out[at] = g;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) ds.cull_count[tile] = n <= cap ? n : -1;
+}
+
+__global__ void __launch_bounds__(kCullThreads) k_tile_cull(const __grid_constant__ DevScene ds, int tile0) {
+    chain_start();
+    cull_tile(ds, tile0 + blockIdx.x);
+}
+
+__global__ void __launch_bounds__(kCullThreads) k_tile_cull_b(const __grid_constant__ BatchDev b) {
+    for (int t = blockIdx.x; t < b.total_tiles; t += gridDim.x) {
+        int lo = 0, hi = b.n;  // last order index with tile_off <= t
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (__ldg(b.tile_off + mid) <= t) lo = mid;
+            else hi = mid;
+        }
+        const DevScene &ds = b.scenes[b.order[lo]];
+        if (ds.cull_on) cull_tile(ds, t - b.tile_off[lo]);  // the same for the whole CTA
+        __syncthreads();
+    }
+}
+
 constexpr long long kTwoWaves = 2 * 152 * 28;
 #ifndef SPM_BLK_MINB
 #define SPM_BLK_MINB 28  // warps per SM the kernels are compiled for
@@ -678,6 +719,7 @@ __global__ void __launch_bounds__(32, SPM_BLK_MINB) k_pixel_blocks(const __grid_
                                                                    int32_t *__restrict__ parent, int row0) {
     __shared__ WarpSmem<PX * PY> sm;
     using S = Shape<PX, PY>;
+    chain_start();
     pixel_block<PX, PY, SCAN>(ds, blockIdx.x * S::kW, row0 + blockIdx.y * S::kH, dist, parent, sm);
 }
 
@@ -824,13 +866,21 @@ void launch_free_mask(const DevScene &ds, cudaStream_t st, uint32_t *bits) {
     k_free_mask<<<(unsigned)((words + per_block - 1) / per_block), NT, 0, st>>>(ds, bits);
 }
 
-void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int tile_row0,
+bool tiles_culled(const DevScene &ds) {
+    return ds.cull_items && ds.use_flood && ds.flood_mode == 3 && ds.static_tile_start;
+}
+
+void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int32_t *parent, int tile_row0,
                         int tile_row1) {
+    DevScene ds = scene;
     const int row0 = tile_row0 * ds.tile, rows = std::min(tile_row1 * ds.tile, ds.Ny) - row0;
     if (rows <= 0) return;
+    ds.cull_on = tiles_culled(ds) ? 1 : 0;
+    if (ds.cull_on) k_tile_cull<<<ds.tiles_x * (tile_row1 - tile_row0), kCullThreads, 0, st>>>(ds, tile_row0 * ds.tiles_x);
     auto run = [&](auto shape, auto kern) {
         const dim3 grid((ds.Nx + shape.kW - 1) / shape.kW, (rows + shape.kH - 1) / shape.kH);
-        kern<<<grid, 32, 0, st>>>(ds, dist, parent, row0);
+        if (ds.cull_on) launch_chained(kern, grid, dim3(32), 0, st, ds, dist, parent, row0);
+        else kern<<<grid, 32, 0, st>>>(ds, dist, parent, row0);
     };
     // The largest blocks that still give the GPU about two waves of warps
     // (28 an SM): large blocks cull and order their candidates for more pixels
@@ -857,6 +907,7 @@ void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pixel_blocks_b, 32 * kBatchWarps, 0);
     const int grid = max(1, min((b.total_blocks + kBatchWarps - 1) / kBatchWarps, sms * max(per_sm, 1)));
+    if (b.any_cull) k_tile_cull_b<<<std::min(b.total_tiles, sms * 16), kCullThreads, 0, st>>>(b);
     k_pixel_blocks_b<<<grid, 32 * kBatchWarps, 0, st>>>(b);
 }
 
