@@ -188,6 +188,16 @@ spm::DevScene effective(const spm_scene *s) {
         d.flood_mode = 3;
         d.use_maps = 1;
     }
+    // Where the vertices are culled without the walk and once a tile, large
+    // tiles pay (1024^2 polygons 167 us with 32 pixels, 178 with 16) until they
+    // span the obstacles' spacing and hide from nothing (batch of 64, its coarse
+    // grids on 32 pixels: 1.9 ms of pixel pass against 1.6)
+    if (d.flood_mode == 3 && d.static_tile_start && d.tile == spm::kTileSmall && d.n_poly > 0) {
+        spm::DevScene wide = d;
+        set_tile(wide, spm::kTile);
+        const double side = spm::kTile * (double)std::max(d.hx, d.hy);
+        if (spm::flood_verts_direct(wide) && side * side * d.n_poly <= 0.4 * (double)d.Wx * (double)d.Wy) return wide;
+    }
     return d;
 }
 
@@ -494,8 +504,15 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
     }
     ds.cull_items = nullptr;
     ds.cull_count = nullptr;
+    auto tiles = [&](int t) { return (size_t)((hs.Nx + t - 1) / t) * ((hs.Ny + t - 1) / t); };
+    ds.vert_mask = nullptr;
+    ds.vert_words = (hs.n_vert + 31) / 32;
+    ds.vert_bits = 0;
+    const size_t mask_words = tiles(spm::kTileSmall) * ds.vert_words;
+    if (hs.n_vert > 0 && ds.static_tile_start && mask_words <= ((size_t)64 << 20) &&
+        (ds.open_scene || ds.n_edge + tiles(spm::kTile) <= 1024))
+        ds.vert_mask = dalloc<uint32_t>(s, mask_words);
     if (ds.open_scene && ds.static_tile_start) {
-        auto tiles = [&](int t) { return (size_t)((hs.Nx + t - 1) / t) * ((hs.Ny + t - 1) / t); };
         ds.cull_items = dalloc<int32_t>(s, std::max(tiles(spm::kTileSmall) * spm::cull_cap(spm::kTileSmall),
                                                     tiles(spm::kTile) * spm::cull_cap(spm::kTile)));
         ds.cull_count = dalloc<int32_t>(s, tiles(spm::kTileSmall));
@@ -610,7 +627,7 @@ spm_status spm_scene_update_sources_device(spm_scene *s, void *stream, const flo
 // copy stream while the next slab computes, and the host moves the previous
 // slab from its bounce buffer into the caller's memory meanwhile. Returns
 // once every row is in place.
-static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t *parent, int tile_row0, int tile_row1,
+static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t *parent, int row0, int row1,
                         float *dist_host = nullptr, int32_t *parent_host = nullptr) {
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -619,7 +636,8 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     spm::DevScene ds = effective(s);
     const bool side = ds.use_flood && ds.flood_mode == 3;  // geometric flood beside the vertex phase
     ds.static_lists = side && ds.static_tile_start ? 1 : 0;  // the pixel pass reads the kept lists too
-    ds.src_direct = ds.static_lists && spm::flood_sources_direct(s->ds) ? 1 : 0;
+    ds.src_direct = ds.static_lists && spm::flood_sources_direct(ds) ? 1 : 0;
+    ds.vert_bits = ds.static_lists && spm::flood_verts_direct(ds) ? 1 : 0;
     NvtxRange range_all("spm_compute");
     if (timed) cudaEventRecord(s->ev[0], cs);
     // the geometric flood needs nothing from the vertex phase (costs and
@@ -661,15 +679,14 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     if (timed) cudaEventRecord(s->ev[3], cs);
     if (!dist_host) {
         NvtxRange r("spm pixel phase");
-        spm::launch_pixel_phase(ds, cs, dist, parent, tile_row0, tile_row1);
+        spm::launch_pixel_phase(ds, cs, dist, parent, row0, row1);
     } else {
         NvtxRange r("spm pixel phase with host copies");
-        const int rows = tile_row1 - tile_row0, nslab = std::min(rows, (int)(sizeof s->slab_ev / sizeof s->slab_ev[0]));
-        const size_t Nx = (size_t)s->hs.Nx, Ny = (size_t)s->hs.Ny;
-        auto slab_rows = [&](int k, size_t &r0, size_t &r1) {
-            const int t0 = tile_row0 + rows * k / nslab, t1 = tile_row0 + rows * (k + 1) / nslab;
-            r0 = (size_t)t0 * ds.tile;
-            r1 = std::min((size_t)t1 * ds.tile, Ny);
+        const int rows = (row1 - row0 + ds.tile - 1) / ds.tile, nslab = std::min(rows, (int)(sizeof s->slab_ev / sizeof s->slab_ev[0]));
+        const size_t Nx = (size_t)s->hs.Nx;
+        auto slab_rows = [&](int k, size_t &r0, size_t &r1) {  // whole rows of tiles
+            r0 = (size_t)row0 + (size_t)(rows * k / nslab) * ds.tile;
+            r1 = std::min((size_t)row0 + (size_t)(rows * (k + 1) / nslab) * ds.tile, (size_t)row1);
         };
         auto drain = [&](int k) {  // host: slab k from its bounce buffer into the caller's planes
             size_t r0, r1;
@@ -680,12 +697,11 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
             std::memcpy(parent_host + r0 * Nx, s->bounce[k & 1] + sizeof(float) * cnt, sizeof(int32_t) * cnt);
         };
         for (int k = 0; k < nslab; ++k) {
-            const int t0 = tile_row0 + rows * k / nslab, t1 = tile_row0 + rows * (k + 1) / nslab;
-            spm::launch_pixel_phase(ds, cs, dist, parent, t0, t1);
-            cudaEventRecord(s->slab_ev[k], cs);
-            cudaStreamWaitEvent(s->copy, s->slab_ev[k], 0);
             size_t r0, r1;
             slab_rows(k, r0, r1);
+            spm::launch_pixel_phase(ds, cs, dist, parent, (int)r0, (int)r1);
+            cudaEventRecord(s->slab_ev[k], cs);
+            cudaStreamWaitEvent(s->copy, s->slab_ev[k], 0);
             const size_t off = r0 * Nx, cnt = (r1 - r0) * Nx;
             // bounce buffer k & 1 was emptied by the host when slab k - 2 drained
             cudaMemcpyAsync(s->bounce[k & 1], dist + off, sizeof(float) * cnt, cudaMemcpyDeviceToHost, s->copy);
@@ -700,7 +716,7 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     s->ev_valid = timed;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_err(s, SPM_ERR_CUDA, cudaGetErrorString(e));
-    const bool whole = tile_row0 == 0 && tile_row1 == s->ds.tiles_y;
+    const bool whole = row0 == 0 && row1 == s->hs.Ny;
     s->last_dist = whole ? dist : nullptr;  // queries need the whole field
     s->last_parent = whole ? parent : nullptr;
     s->last_stream = cs;
@@ -711,7 +727,7 @@ spm_status spm_compute(spm_scene *s, void *stream, float *dist, int32_t *parent)
     if (!s || !dist || !parent) return set_err(s, SPM_ERR_INVALID_ARG, "null argument");
     spm_status st = check_device(s);
     if (st != SPM_OK) return st;
-    return compute_impl(s, stream, dist, parent, 0, s->ds.tiles_y);
+    return compute_impl(s, stream, dist, parent, 0, s->hs.Ny);
 }
 
 spm_status spm_compute_rows(spm_scene *s, void *stream, int32_t row0, int32_t row1, float *dist, int32_t *parent) {
@@ -721,7 +737,7 @@ spm_status spm_compute_rows(spm_scene *s, void *stream, int32_t row0, int32_t ro
         return set_err(s, SPM_ERR_INVALID_ARG, "rows must be tile-aligned within the grid");
     spm_status st = check_device(s);
     if (st != SPM_OK) return st;
-    return compute_impl(s, stream, dist, parent, row0 / T, (row1 + T - 1) / T);
+    return compute_impl(s, stream, dist, parent, row0, row1);
 }
 
 spm_status spm_scene_sync(spm_scene *s, void *stream) {
@@ -784,7 +800,7 @@ spm_status spm_compute_host(spm_scene *s, void *stream, float *dist_host, int32_
     cudaGetLastError();  // a pageable pointer is not an error here
     if (direct) {
         st = compute_impl(s, stream, static_cast<float *>(ad.devicePointer), static_cast<int32_t *>(ap.devicePointer),
-                          0, s->ds.tiles_y);
+                          0, s->hs.Ny);
         // the caller may unpin or free these buffers at any time after the
         // call: queries must not read them (they need a device compute)
         s->last_dist = nullptr;
@@ -792,7 +808,8 @@ spm_status spm_compute_host(spm_scene *s, void *stream, float *dist_host, int32_
     } else {
         st = ensure_stage(s);
         if (st != SPM_OK) return st;
-        const size_t slab_rows = (size_t)((s->ds.tiles_y + 7) / 8 + 1) * s->ds.tile;
+        const spm::DevScene run = effective(s);
+        const size_t slab_rows = (size_t)((run.tiles_y + 7) / 8 + 1) * run.tile;
         const size_t need = slab_rows * (size_t)s->hs.Nx * (sizeof(float) + sizeof(int32_t));
         if (s->bounce_bytes < need) {  // page-locked bounce buffers, on first use or growth
             for (int k = 0; k < 2; ++k)
@@ -811,7 +828,7 @@ spm_status spm_compute_host(spm_scene *s, void *stream, float *dist_host, int32_
             }
             s->bounce_bytes = need;
         }
-        st = compute_impl(s, stream, s->stage_dist, s->stage_par, 0, s->ds.tiles_y, dist_host, parent_host);
+        st = compute_impl(s, stream, s->stage_dist, s->stage_par, 0, s->hs.Ny, dist_host, parent_host);
     }
     if (st != SPM_OK) return st;
     return spm_scene_sync(s, stream);
@@ -941,6 +958,7 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         const spm::DevScene &d = descs[k];
         descs[k].src_direct = d.flood_reuse && spm::flood_sources_direct(d) ? 1 : 0;
         descs[k].cull_on = spm::tiles_culled(d) ? 1 : 0;
+        descs[k].vert_bits = d.flood_reuse && spm::flood_verts_direct(d) ? 1 : 0;
         const long long direct = descs[k].src_direct, ntl = (long long)d.tiles_x * d.tiles_y;
         src_map_off[k + 1] = src_map_off[k] + direct * d.n_src * spm::kAngBins;
         src_ins_off[k + 1] = src_ins_off[k] + direct * d.n_src * spm::src_edge_warps(d.n_edge);

@@ -447,17 +447,18 @@ __device__ void flood_one(const DevScene &ds, FloodSmem &sm, unsigned *fdyn, int
 // an open scene a generator reaches much of the grid, and the walk's levels
 // (four barriers each, the whole grid's width deep) cost far more: first
 // compute of the 1024^2 polygons, 1188 generators, 1.2 ms of walks.
-// hit: a bit per tile. A superset of what the walk reaches.
+// The result is a bit per tile and vertex (a superset of what the walk
+// reaches), turned into the kept lists where they fit: with bits alone there is
+// no capacity to outgrow (8836 tiles of the 1501^2 polygons hold 5 M pairs,
+// over the lists' 4 M: every block scanned), with lists a tile's culling skips
+// what it does not see (batch of 64: 1.6 ms of pixel pass against 1.9).
 template <bool MAPS>
-__device__ void flood_direct(const DevScene &ds, float *up, float *low, unsigned *hit, int g) {
-    __shared__ long long wsum[32];
-    __shared__ int base;
+__device__ void flood_direct(const DevScene &ds, float *up, float *low, int g) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gl8 = lane & 7;
-    const int ntiles = ds.tiles_x * ds.tiles_y, words = (ntiles + 31) / 32;
+    const int ntiles = ds.tiles_x * ds.tiles_y, v = g - ds.n_src;
     const int2 gl = ds.gen_lat[g];
     __syncthreads();  // the previous generator is done with smem
     for (int k = tid; k < kAng; k += kFloodThreads) up[k] = low[k] = INFINITY;
-    for (int w = tid; w < words; w += kFloodThreads) hit[w] = 0u;
     __syncthreads();
     for (int e = warp * kSrcEdges; e < ds.n_edge; e += kFloodThreads / 32 * kSrcEdges)
         insert_edges_warp<MAPS>(ds, up, low, gl, e, 1, 1 << 30);
@@ -469,25 +470,8 @@ __device__ void flood_direct(const DevScene &ds, float *up, float *low, unsigned
         const int4 area = tile_area(ds, t % ds.tiles_x, t / ds.tiles_x);
         const bool inside = gl.x >= area.x && gl.x <= area.z && gl.y >= area.y && gl.y <= area.w;
         const bool seen = inside || !box_hidden_ang<8>(up, gl, area, gl8, gmask, 1);
-        if (seen && gl8 == 0) atomicOr(&hit[t >> 5], 1u << (t & 31));
+        if (seen && gl8 == 0) atomicOr(&ds.vert_mask[(size_t)t * ds.vert_words + (v >> 5)], 1u << (v & 31));
     }
-    __syncthreads();
-    int mine = 0;
-    for (int w = tid; w < words; w += kFloodThreads) mine += __popc(hit[w]);
-    const long long before = cta_exclusive_scan(mine, wsum);
-    if (tid == kFloodThreads - 1) base = atomicAdd(&ds.flood_counts[0], (int)before + mine);
-    __syncthreads();
-    int slot = base + (int)before;
-    for (int w = tid; w < words; w += kFloodThreads)
-        for (unsigned m = hit[w]; m; m &= m - 1, ++slot) {
-            const int t = 32 * w + __ffs(m) - 1;
-            if (slot < ds.pair_cap) {
-                ds.pairs[slot] = make_int2(t, g);
-                atomicAdd(&ds.tile_count[t], 1);
-            } else {
-                atomicOr(&ds.flood_counts[2], 1);
-            }
-        }
     if (MAPS) {
         float2 *mp = ds.gen_maps + (size_t)g * kAng;
         for (int k = tid; k < kAng; k += kFloodThreads) mp[k] = make_float2(up[k], low[k]);
@@ -498,7 +482,6 @@ __device__ void flood_direct(const DevScene &ds, float *up, float *low, unsigned
 // Resident CTAs take the obstacle vertices [g0, g1) from the work counter.
 template <bool MAPS>
 __global__ void __launch_bounds__(kFloodThreads, 6) k_flood_direct(const __grid_constant__ DevScene ds, int g0, int g1) {
-    extern __shared__ unsigned fdyn[];
     __shared__ float up[kAng], low[kAng];
     __shared__ int next_g;
     for (;;) {
@@ -506,7 +489,42 @@ __global__ void __launch_bounds__(kFloodThreads, 6) k_flood_direct(const __grid_
         if (threadIdx.x == 0) next_g = g0 + atomicAdd(&ds.flood_counts[3], 1);
         __syncthreads();
         if (next_g >= g1) break;
-        flood_direct<MAPS>(ds, up, low, fdyn, next_g);
+        flood_direct<MAPS>(ds, up, low, next_g);
+    }
+}
+
+// The kept lists from the bits: a warp a tile counts them, and after the scan
+// (static_tile_start) writes the list, in order; static_counts[3] says whether
+// they fit.
+__global__ void k_bits_count(const __grid_constant__ DevScene ds) {
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (t >= ds.tiles_x * ds.tiles_y) return;  // whole warps
+    int n = 0;
+    for (int w = lane; w < ds.vert_words; w += 32) n += __popc(ds.vert_mask[(size_t)t * ds.vert_words + w]);
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) ds.tile_count[t] = n;
+}
+
+__global__ void k_bits_fill(const __grid_constant__ DevScene ds) {
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int ntiles = ds.tiles_x * ds.tiles_y;
+    if (t >= ntiles) return;  // whole warps
+    const bool fit = ds.static_tile_start[ntiles] <= ds.pair_cap;
+    if (t == 0 && lane == 0) ds.static_counts[3] = fit;
+    if (!fit) return;
+    int at = ds.static_tile_start[t];
+    for (int w0 = 0; w0 < ds.vert_words; w0 += 32) {
+        const int w = w0 + lane;
+        const uint32_t bits = w < ds.vert_words ? ds.vert_mask[(size_t)t * ds.vert_words + w] : 0u;
+        int incl = __popc(bits);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        int slot = at + incl - __popc(bits);
+        for (uint32_t m = bits; m; m &= m - 1) ds.static_tile_items[slot++] = ds.n_src + 32 * w + __ffs(m) - 1;
+        at += __shfl_sync(0xffffffffu, incl, 31);
     }
 }
 
@@ -848,15 +866,18 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
             cudaMemsetAsync(ds.tile_count, 0, sizeof(int32_t) * ntiles, st);
             cudaMemsetAsync(ds.flood_counts, 0, sizeof(int32_t) * 4, st);
             if (flood_verts_direct(ds)) {
-                const size_t bits = sizeof(unsigned) * (size_t)((ntiles + 31) / 32);
+                cudaMemsetAsync(ds.vert_mask, 0, sizeof(uint32_t) * (size_t)ntiles * ds.vert_words, st);
                 const int blocks = std::min(max(sms, 1) * 6, ds.n_vert);
-                if (maps) k_flood_direct<true><<<blocks, kFloodThreads, bits, st>>>(ds, ds.n_src, ds.n_gen);
-                else k_flood_direct<false><<<blocks, kFloodThreads, bits, st>>>(ds, ds.n_src, ds.n_gen);
+                if (maps) k_flood_direct<true><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen);
+                else k_flood_direct<false><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen);
+                k_bits_count<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
+                k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
+                k_bits_fill<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
             } else {
                 flood(ds.n_src, ds.n_gen);
+                k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
+                k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 1);
             }
-            k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
-            k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 1);
             k_flood_static<<<sblocks, 256, 0, st>>>(ds, 1);
         }
         if (flood_sources_direct(ds)) {  // a bit per source and tile: nothing to sort
@@ -886,7 +907,7 @@ bool flood_sources_direct(const DevScene &ds) {
 // while a generator's edges and tiles stay a few thousand.
 bool flood_verts_direct(const DevScene &ds) {
     const long long ntiles = (long long)ds.tiles_x * ds.tiles_y;
-    return ds.n_vert > 0 && (ds.open_scene || ds.n_edge + ntiles <= 1024) && ds.n_edge + ntiles <= (1 << 16);
+    return ds.vert_mask && (ds.open_scene || ds.n_edge + ntiles <= 1024) && ds.n_edge + ntiles <= (1 << 17);
 }
 
 int src_edge_warps(int n_edge) { return (n_edge + kSrcEdges - 1) / kSrcEdges; }

@@ -201,8 +201,13 @@ struct DevScene {
     int32_t *static_tile_items;        // pair_cap
     int32_t *static_counts;            // 4
     int32_t static_lists;              // the pixel pass reads the static lists as well (this compute)
+    // the same as a bit per obstacle vertex, vert_words words a tile, where the
+    // vertices are culled without the walk (vert_bits: in this compute; the
+    // lists are kept beside it when they fit, static_counts[3])
+    uint32_t *vert_mask;
+    int32_t vert_words, vert_bits;
     // open scenes: per tile the entries of those lists that can win somewhere in
-    // it, at most cull_cap(tile) of them (cull_count -1: more, take the lists)
+    // it, at most cull_cap of them (cull_count -1: more, take the lists)
     int32_t *cull_items, *cull_count;
     int32_t cull_on;                   // this compute culls them
     int32_t flood_reuse;               // in a batch's copy: flood the sources only, over the static part
@@ -263,12 +268,11 @@ struct VertexSide {
     cudaEvent_t fork, join;
 };
 void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *side = nullptr);
-// entries a tile's culled list may hold: 32 KB of them a 128 x 128 pixels
-constexpr int cull_cap(int tile) { return tile == kTile ? 512 : 128; }
+// entries a tile's culled list may hold
+constexpr int cull_cap(int tile) { return tile == kTile ? 512 : 256; }
 bool tiles_culled(const DevScene &ds);  // the pixel pass culls its lists per tile first
-// pixel kernel over the tiles of tile rows [tile_row0, tile_row1)
-void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int tile_row0,
-                        int tile_row1);
+// pixel kernel over the grid rows [row0, row1); row0 a multiple of the small tile's side
+void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int row0, int row1);
 // flood of the per-tile candidate lists. FloodStatic::kNone floods every
 // generator; kBuild (geometric mode) floods the obstacle vertices, keeps
 // their lists as the static part, then floods the sources; kReuse restores

@@ -110,17 +110,17 @@ __device__ __forceinline__ float pixel_x(const DevScene &ds, int i) { return ((f
 __device__ __forceinline__ float pixel_y(const DevScene &ds, int j) { return ((float)j + 0.5f) * ds.hy; }
 
 // The candidates of a tile's pixels: the list culled for the tile, or the kept
-// list of obstacle vertices, this compute's entries (a bit per source, or a
-// list) and the global list, or every generator.
+// list of obstacle vertices and this compute's entries (each a list, or a bit
+// per vertex or source) and the global list, or every generator.
 struct TileList {
-    const int32_t *a, *l, *gl;  // entries [0, na), [na, nl) and [nl, total)
-    const uint32_t *bits;       // or the middle part's bits
+    const int32_t *a, *l, *gl;       // entries [0, na), [na, nl) and [nl, total)
+    const uint32_t *abits, *lbits;   // or the first two parts' bits
     int na, nl, total;
     bool lists;
     __device__ __forceinline__ TileList(const DevScene &ds, int tile, bool culled) {
         lists = ds.use_flood && ds.flood_counts[2] == 0;
         a = l = gl = ds.glob_list;
-        bits = nullptr;
+        abits = lbits = nullptr;
         na = nl = 0;
         total = ds.n_gen;
         if (!lists) return;
@@ -130,13 +130,16 @@ struct TileList {
             if (total >= 0) return;
             na = 0;
         }
-        if (ds.static_lists) {
+        if (ds.static_lists && ds.vert_bits && !ds.static_counts[3]) {
+            abits = ds.vert_mask + (size_t)tile * ds.vert_words;
+            na = ds.n_vert;
+        } else if (ds.static_lists) {
             const int s0 = ds.static_tile_start[tile];
             na = ds.static_tile_start[tile + 1] - s0;
             a = ds.static_tile_items + s0;
         }
         if (ds.static_lists && ds.src_direct) {
-            bits = ds.src_mask + (size_t)tile * ds.src_words;
+            lbits = ds.src_mask + (size_t)tile * ds.src_words;
             nl = na + ds.n_src;
         } else {
             const int l0 = ds.tile_start[tile];
@@ -150,12 +153,14 @@ struct TileList {
         if (e >= total) return false;
         g = e;
         if (!lists) return true;
-        const int r = e - na;
-        if (r >= 0 && e < nl && bits) {
-            g = r;
+        const bool first = e < na, second = !first && e < nl;
+        const int r = first ? e : second ? e - na : e - nl;
+        const uint32_t *bits = first ? abits : second ? lbits : nullptr;
+        if (bits) {
+            g = first ? r + ds.n_src : r;
             return __ldg(bits + (r >> 5)) >> (r & 31) & 1u;
         }
-        g = __ldg(r < 0 ? a + e : e < nl ? l + r : gl + (e - nl));
+        g = __ldg((first ? a : second ? l : gl) + r);
         return true;
     }
 };
@@ -661,7 +666,7 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
 constexpr int kCullThreads = 128;
 __device__ __forceinline__ void cull_tile(const DevScene &ds, int tile) {
     __shared__ int n;
-    const int lane = threadIdx.x & 31, cap = cull_cap(ds.tile);
+    const int lane = threadIdx.x & 31;
     if (threadIdx.x == 0) n = 0;
     __syncthreads();
     Block b;
@@ -672,7 +677,7 @@ __device__ __forceinline__ void cull_tile(const DevScene &ds, int tile) {
     b.box = make_int4(ds.pitch_x * b.i0 + ds.pitch_x / 2, ds.pitch_y * b.j0 + ds.pitch_y / 2,
                       ds.pitch_x * b.i1 + ds.pitch_x / 2, ds.pitch_y * b.j1 + ds.pitch_y / 2);
     const TileList tl(ds, tile, false);
-    int32_t *out = ds.cull_items + (size_t)tile * cap;
+    int32_t *out = ds.cull_items + (size_t)tile * cull_cap(ds.tile);
     for (int e0 = threadIdx.x & ~31; tl.lists && e0 < tl.total; e0 += kCullThreads) {
         int g = 0, c;
         float lb;
@@ -681,10 +686,10 @@ __device__ __forceinline__ void cull_tile(const DevScene &ds, int tile) {
         int at = 0;
         if (lane == 0 && bal) at = atomicAdd(&n, __popc(bal));
         at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
-        if (keep && at < cap) out[at] = g;
+        if (keep && at < cull_cap(ds.tile)) out[at] = g;
     }
     __syncthreads();
-    if (threadIdx.x == 0) ds.cull_count[tile] = n <= cap ? n : -1;
+    if (threadIdx.x == 0) ds.cull_count[tile] = n <= cull_cap(ds.tile) ? n : -1;
 }
 
 __global__ void __launch_bounds__(kCullThreads) k_tile_cull(const __grid_constant__ DevScene ds, int tile0) {
@@ -867,16 +872,18 @@ void launch_free_mask(const DevScene &ds, cudaStream_t st, uint32_t *bits) {
 }
 
 bool tiles_culled(const DevScene &ds) {
-    return ds.cull_items && ds.use_flood && ds.flood_mode == 3 && ds.static_tile_start;
+    return ds.cull_items && ds.use_flood && ds.flood_mode == 3 && flood_verts_direct(ds);
 }
 
-void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int32_t *parent, int tile_row0,
-                        int tile_row1) {
+void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int32_t *parent, int row0, int row1) {
     DevScene ds = scene;
-    const int row0 = tile_row0 * ds.tile, rows = std::min(tile_row1 * ds.tile, ds.Ny) - row0;
+    const int rows = row1 - row0;
     if (rows <= 0) return;
     ds.cull_on = tiles_culled(ds) ? 1 : 0;
-    if (ds.cull_on) k_tile_cull<<<ds.tiles_x * (tile_row1 - tile_row0), kCullThreads, 0, st>>>(ds, tile_row0 * ds.tiles_x);
+    if (ds.cull_on) {
+        const int t0 = row0 / ds.tile, t1 = (row1 + ds.tile - 1) / ds.tile;
+        k_tile_cull<<<ds.tiles_x * (t1 - t0), kCullThreads, 0, st>>>(ds, t0 * ds.tiles_x);
+    }
     auto run = [&](auto shape, auto kern) {
         const dim3 grid((ds.Nx + shape.kW - 1) / shape.kW, (rows + shape.kH - 1) / shape.kH);
         if (ds.cull_on) launch_chained(kern, grid, dim3(32), 0, st, ds, dist, parent, row0);
