@@ -934,12 +934,13 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     b->scenes.assign(scenes, scenes + n);
     b->device = dev;
     std::vector<spm::DevScene> descs(n);
-    std::vector<long long> pair_off(n + 1, 0), src_map_off(n + 1, 0), src_ins_off(n + 1, 0),
+    std::vector<long long> src_map_off(n + 1, 0), src_ins_off(n + 1, 0),
         src_tile_off(n + 1, 0);
     std::vector<int32_t> vert_off(n + 1, 0), gen_off(n + 1, 0), order(n), tile_off(n + 1, 0), flood_off(n + 1, 0);
     std::vector<float *> dv(dist, dist + n);
     std::vector<int32_t *> pv(parent, parent + n);
     int max_gen = 0;
+    const int cluster_grid = spm::cluster_batched_grid();
     for (int k = 0; k < n; ++k) {
         descs[k] = effective(scenes[k]);
         descs[k].warm = 0;  // the batched fixpoint starts every scene from its sources
@@ -958,6 +959,8 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         const spm::DevScene &d = descs[k];
         descs[k].src_direct = d.flood_reuse && spm::flood_sources_direct(d) ? 1 : 0;
         descs[k].cull_on = spm::tiles_culled(d) ? 1 : 0;
+        descs[k].cl_lists =
+            cluster_grid > 0 && spm::cluster_lists(d, d.fix_launch, spm::kFixClusterFits | spm::kFixBatchLists) ? 1 : 0;
         descs[k].vert_bits = d.flood_reuse && spm::flood_verts_direct(d) ? 1 : 0;
         const long long direct = descs[k].src_direct, ntl = (long long)d.tiles_x * d.tiles_y;
         src_map_off[k + 1] = src_map_off[k] + direct * d.n_src * spm::kAngBins;
@@ -966,7 +969,6 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         const bool floods = d.use_flood && d.flood_mode != 2;
         flood_off[k + 1] =
             flood_off[k] + (floods && !direct ? (d.flood_reuse ? d.n_src : d.n_gen) : 0);
-        pair_off[k + 1] = pair_off[k] + (long long)descs[k].n_vert * descs[k].pair_words;
         vert_off[k + 1] = vert_off[k] + descs[k].n_vert;
         gen_off[k + 1] = gen_off[k] + descs[k].n_gen;
         max_gen = std::max(max_gen, descs[k].n_gen);
@@ -990,7 +992,6 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     spm::BatchDev &bd = b->dev;
     bd.n = n;
     bd.scenes = bupload(b, descs, ok);
-    bd.pair_off = bupload(b, pair_off, ok);
     bd.vert_off = bupload(b, vert_off, ok);
     bd.gen_off = bupload(b, gen_off, ok);
     bd.flood_off = bupload(b, flood_off, ok);
@@ -1021,7 +1022,7 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         bd.cl_order = bupload(b, cl_order, ok);
         bd.cl_done = balloc<int32_t>(b, n);
         bd.cl_counter = balloc<int32_t>(b, 1);
-        bd.cl_grid = spm::cluster_batched_grid();
+        bd.cl_grid = cluster_grid;
         bd.cl_all = bd.cl_grid > 0 ? 1 : 0;
         for (int k = 0; k < n; ++k) bd.cl_all &= (descs[k].fix_launch & spm::kFixClusterFits) ? 1 : 0;
     }
@@ -1030,6 +1031,8 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     bd.flood_smem = 0;
     bd.any_maps = 0;
     bd.any_lists = 0;
+    bd.max_src_words = 0;
+    for (int k = 0; k < n; ++k) bd.max_src_words = std::max(bd.max_src_words, (descs[k].n_src + 31) / 32);
     bd.any_cull = 0;
     for (int k = 0; k < n; ++k) bd.any_cull |= spm::tiles_culled(descs[k]);
     for (int k = 0; k < n; ++k)
@@ -1283,11 +1286,13 @@ spm_status spm_scene_info(spm_scene *s, int64_t *info) {
     // polygon and the tile tests)
     const bool reuse = floods && run.flood_mode == 3 && run.static_tile_start;
     const int src_cull = !spm::flood_sources_direct(run) ? 4 : s->ds.n_poly > 0 ? 3 : 2;
-    // vertex phase (prep, pairs, edges, the tree's kernels, fixpoint kernels,
+    // vertex phase (prep, pairs, edge lists, the tree's kernels, fixpoint kernels,
     // and after the many-CTA one its finalisation); flood, list scan and
     // fill; pixels
     const int many_cta = s->ds.fix_launch & (spm::kFixSoloSure | spm::kFixClusterSure) ? 0 : 2;
-    info[10] = 1 + (s->hs.n_vert > 0 ? 4 : 0) + (s->ds.warm && s->ds.vtab ? 4 : 0) + (s->ds.fix_launch & spm::kFixSolo ? 1 : 0) +
+    const bool own_lists = spm::cluster_lists(run, run.fix_launch, spm::kFixClusterSure | spm::kFixClusterLists) &&
+                           !(run.fix_launch & spm::kFixSolo);
+    info[10] = 1 + (s->hs.n_vert > 0 ? (own_lists ? 1 : 4) : 0) + (s->ds.warm && s->ds.vtab ? 4 : 0) + (s->ds.fix_launch & spm::kFixSolo ? 1 : 0) +
                (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull : 3) : 0) + (spm::tiles_culled(run) ? 1 : 0) + 1;
     return SPM_OK;
 }

@@ -146,48 +146,6 @@ __device__ __forceinline__ void arrival_dir(const DevScene &ds, int u, int2 vl, 
     dy = vl.y - ul.y;
 }
 
-// Conservative bin enumeration for the segment p->q thickened by r (lattice
-// units, float). Calls f(bin) for every bin the thick segment may touch, in
-// columns ordered from p toward q; stops early when f returns true.
-template <class F>
-__device__ __forceinline__ bool walk_bins(const DevScene &ds, float px, float py, float qx, float qy,
-                                          float r, F &&f) {
-    const float bs = (float)ds.bin_size, x0 = (float)ds.bin_x0, y0 = (float)ds.bin_y0;
-    const float m = r + 1.0f;
-    auto bin_of = [&](float v, float o, int n) {
-        int b = (int)floorf((v - o) / bs);
-        return b < 0 ? 0 : (b >= n ? n - 1 : b);
-    };
-    const int c0 = bin_of(fminf(px, qx) - m, x0, ds.bin_nx), c1 = bin_of(fmaxf(px, qx) + m, x0, ds.bin_nx);
-    const float dx = qx - px, dy = qy - py;
-    const int step = dx >= 0.f ? 1 : -1;
-    const int cs = step > 0 ? c0 : c1, ce = step > 0 ? c1 : c0;
-    for (int c = cs;; c += step) {
-        float ylo, yhi;
-        if (fabsf(dx) < 0.5f) {
-            ylo = fminf(py, qy);
-            yhi = fmaxf(py, qy);
-        } else {
-            float a = x0 + c * bs - m, b = x0 + (c + 1) * bs + m;
-            float t0 = (a - px) / dx, t1 = (b - px) / dx;
-            float tl = fmaxf(0.f, fminf(t0, t1)), th = fminf(1.f, fmaxf(t0, t1));
-            if (tl > th) { tl = 0.f; th = 1.f; }  // rounding guard: keep it conservative
-            float ya = py + tl * dy, yb = py + th * dy;
-            ylo = fminf(ya, yb);
-            yhi = fmaxf(ya, yb);
-        }
-        int r0 = bin_of(ylo - m, y0, ds.bin_ny), r1 = bin_of(yhi + m, y0, ds.bin_ny);
-        int rstep = dy >= 0.f ? 1 : -1;
-        int rs = rstep > 0 ? r0 : r1, re = rstep > 0 ? r1 : r0;
-        for (int rr = rs;; rr += rstep) {
-            if (f(rr * ds.bin_nx + c)) return true;
-            if (rr == re) break;
-        }
-        if (c == ce) break;
-    }
-    return false;
-}
-
 // Does the open segment p->q meet the open interior of convex CCW polygon
 // V[0..m)? Separating-axis test on the segment and the polygon (both convex):
 // they are disjoint in the interiors iff some outward edge normal of the
@@ -212,21 +170,16 @@ __device__ __forceinline__ bool segment_meets_poly(const int2 *V, int m, int px,
     return pos && neg && !apart;
 }
 
-// Calls f(V, m) for every polygon that blocks the open segment between lattice
-// points p and q (its open interior meets it) until f returns true; returns
-// whether one did. One thread: walks the bins the segment crosses, cell to
-// cell. Only the first share `part` of the segment from p is walked: 1, or
-// less when no obstacle is met beyond it (a polygon that blocks the segment
-// then meets that part, and is listed in one of its bins). The float steps are
-// off by far less than the unit the polygons' boxes are grown by when they are
-// binned. (A walk by columns with both their row ranges, grown by a margin,
-// took four divisions a column and visited more bins: vertex phase of the
-// 1024^2 polygons 0.106 -> 0.092 ms.)
+// Calls f(bin) for the bins that the segment from (x, y) by (dx, dy) (lattice
+// units) crosses, cell to cell, until f returns true; returns whether it did.
+// The float steps are off by far less than the unit the polygons' boxes are
+// grown by when they are binned. (A walk by columns with both their row
+// ranges, grown by a margin, took four divisions a column and visited more
+// bins: vertex phase of the 1024^2 polygons 0.106 -> 0.092 ms.)
 template <class F>
-__device__ __forceinline__ bool walk_blockers(const DevScene &ds, int px, int py, int qx, int qy, float part, F &&f) {
-    const float dx = (float)(qx - px), dy = (float)(qy - py);
-    const float u = (float)(px - ds.bin_x0) * ds.bin_inv, v = (float)(py - ds.bin_y0) * ds.bin_inv;
-    const float du = dx * part * ds.bin_inv, dv = dy * part * ds.bin_inv;
+__device__ __forceinline__ bool walk_cells(const DevScene &ds, float x, float y, float dx, float dy, F &&f) {
+    const float u = (x - (float)ds.bin_x0) * ds.bin_inv, v = (y - (float)ds.bin_y0) * ds.bin_inv;
+    const float du = dx * ds.bin_inv, dv = dy * ds.bin_inv;
     auto cell = [](float w, int n) { return min(max((int)floorf(w), 0), n - 1); };
     int cx = cell(u, ds.bin_nx), cy = cell(v, ds.bin_ny);
     const int ex = cell(u + du, ds.bin_nx), ey = cell(v + dv, ds.bin_ny);
@@ -235,10 +188,31 @@ __device__ __forceinline__ bool walk_blockers(const DevScene &ds, int px, int py
     const float ix = __fdividef(1.f, fabsf(du)), iy = __fdividef(1.f, fabsf(dv));
     float nx = (float)(sx > 0 ? cx + 1 : cx), ny = (float)(sy > 0 ? cy + 1 : cy);
     float tx = ex == cx ? INFINITY : fabsf(nx - u) * ix, ty = ey == cy ? INFINITY : fabsf(ny - v) * iy;
-    const int bx0 = min(px, qx), bx1 = max(px, qx), by0 = min(py, qy), by1 = max(py, qy);
     for (int left = abs(ex - cx) + abs(ey - cy);; --left) {
         SPM_CNT(24, 1);  // a bin walked
-        const int bin = cy * ds.bin_nx + cx, end = __ldg(ds.bin_start + bin + 1);
+        if (f(cy * ds.bin_nx + cx)) return true;
+        if (left <= 0) return false;
+        if (tx < ty) {
+            cx += sx;
+            nx += (float)sx;
+            tx = cx == ex ? INFINITY : fabsf(nx - u) * ix;
+        } else {
+            cy += sy;
+            ny += (float)sy;
+            ty = cy == ey ? INFINITY : fabsf(ny - v) * iy;
+        }
+    }
+}
+
+// Calls f(V, m) for every polygon that blocks the open segment between lattice
+// points p and q (its open interior meets it) until f returns true; returns
+// whether one did. One thread.
+template <class F>
+__device__ __forceinline__ bool walk_blockers(const DevScene &ds, int px, int py, int qx, int qy, F &&f) {
+    const float dx = (float)(qx - px), dy = (float)(qy - py);
+    const int bx0 = min(px, qx), bx1 = max(px, qx), by0 = min(py, qy), by1 = max(py, qy);
+    return walk_cells(ds, (float)px, (float)py, dx, dy, [&](int bin) {
+        const int end = __ldg(ds.bin_start + bin + 1);
         for (int it = __ldg(ds.bin_start + bin); it < end; ++it) {
             const int4 *rp = reinterpret_cast<const int4 *>(ds.bin_recs + it);
             const int4 bx = __ldg(rp);
@@ -253,24 +227,15 @@ __device__ __forceinline__ bool walk_blockers(const DevScene &ds, int px, int py
             SPM_CNT(25, 1);  // a polygon tested
             if (segment_meets_poly(ds.poly_v + rec.y, rec.z, px, py, qx, qy) && f(ds.poly_v + rec.y, rec.z)) return true;
         }
-        if (left <= 0) return false;
-        if (tx < ty) {
-            cx += sx;
-            nx += (float)sx;
-            tx = cx == ex ? INFINITY : fabsf(nx - u) * ix;
-        } else {
-            cy += sy;
-            ny += (float)sy;
-            ty = cy == ey ? INFINITY : fabsf(ny - v) * iy;
-        }
-    }
+        return false;
+    });
 }
 
 // Exact visibility between lattice point p and generator target q (a point),
 // one thread.
 __device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int py, int qx, int qy) {
     if (px == qx && py == qy) return true;
-    return !walk_blockers(ds, px, py, qx, qy, 1.f, [](const int2 *, int) { return true; });
+    return !walk_blockers(ds, px, py, qx, qy, [](const int2 *, int) { return true; });
 }
 
 // Does one polygon hide every point of the box from the point generator at
@@ -280,7 +245,7 @@ __device__ __forceinline__ bool visible_points(const DevScene &ds, int px, int p
 __device__ __forceinline__ bool box_hidden(const DevScene &ds, int4 box, int2 g) {
     const int cx = (box.x + box.z) >> 1, cy = (box.y + box.w) >> 1;
     if (cx == g.x && cy == g.y) return false;
-    return walk_blockers(ds, cx, cy, g.x, g.y, 1.f, [&](const int2 *V, int m) {
+    return walk_blockers(ds, cx, cy, g.x, g.y, [&](const int2 *V, int m) {
         bool all = true;
 #pragma unroll 1
         for (int k = 0; k < 4 && all; ++k)
@@ -290,31 +255,96 @@ __device__ __forceinline__ bool box_hidden(const DevScene &ds, int4 box, int2 g)
 }
 
 // Exact visibility between lattice point p and its perpendicular foot on
-// segment source s (0 < num < den), one thread. The bins are walked from p,
-// or from the foot (from_foot); the result is the same (each bin's test is
-// the whole segment's, and the walks cover every bin the segment crosses).
-__device__ __forceinline__ bool visible_foot(const DevScene &ds, int s, int px, int py, long long num,
-                                             long long den, bool from_foot = false) {
-    int4 L = ds.seg_lat[s];
-    int ux = L.z - L.x, uy = L.w - L.y;
-    int side = cross32(ux, uy, px - L.x, py - L.y);
-    if (side == 0) return true;
-    double t = (double)num / (double)den;
-    float fx = (float)(L.x + t * ux), fy = (float)(L.y + t * uy);
-    int4 sb = make_int4((int)floorf(fminf((float)px, fx)) - 1, (int)floorf(fminf((float)py, fy)) - 1,
-                        (int)ceilf(fmaxf((float)px, fx)) + 1, (int)ceilf(fmaxf((float)py, fy)) + 1);
-    const float wx0 = from_foot ? fx : (float)px, wy0 = from_foot ? fy : (float)py;
-    const float wx1 = from_foot ? (float)px : fx, wy1 = from_foot ? (float)py : fy;
-    bool blocked = walk_bins(ds, wx0, wy0, wx1, wy1, 0.f, [&](int bin) {
-        for (int it = ds.bin_start[bin]; it < ds.bin_start[bin + 1]; ++it) {
-            const BinRec rec = ds.bin_recs[it];
-            const int4 bx = rec.box;
+// segment source s (0 < num < den), one thread.
+__device__ __forceinline__ bool visible_foot(const DevScene &ds, int s, int px, int py, long long num, long long den) {
+    const int4 L = ds.seg_lat[s];
+    const int ux = L.z - L.x, uy = L.w - L.y;
+    if (cross32(ux, uy, px - L.x, py - L.y) == 0) return true;
+    // the foot, to a hundredth of a unit: it only chooses bins and boxes to test
+    const float t = __fdividef((float)num, (float)den);
+    const float fx = (float)L.x + t * (float)ux, fy = (float)L.y + t * (float)uy;
+    const int4 sb = make_int4((int)floorf(fminf((float)px, fx)) - 1, (int)floorf(fminf((float)py, fy)) - 1,
+                              (int)ceilf(fmaxf((float)px, fx)) + 1, (int)ceilf(fmaxf((float)py, fy)) + 1);
+    const float dx = (float)px - fx, dy = (float)py - fy;
+    return !walk_cells(ds, fx, fy, dx, dy, [&](int bin) {
+        const int end = __ldg(ds.bin_start + bin + 1);
+        for (int it = __ldg(ds.bin_start + bin); it < end; ++it) {
+            const int4 *rp = reinterpret_cast<const int4 *>(ds.bin_recs + it);
+            const int4 bx = __ldg(rp);
             if (bx.z < sb.x || bx.x > sb.z || bx.w < sb.y || bx.y > sb.w) continue;
-            if (foot_meets_poly(ds.poly_v + rec.voff, rec.m, L, px, py, num, den)) return true;
+            const int4 rec = __ldg(rp + 1);
+            if (foot_meets_poly(ds.poly_v + rec.y, rec.z, L, px, py, num, den)) return true;
         }
         return false;
     });
-    return !blocked;
+}
+
+// Does test(rec) hold for a polygon (its record's second half: id, first vertex,
+// vertices) whose box the segment from (x, y) by (dx, dy) comes near? One warp,
+// every lane with the same arguments: a lane takes a bin the segment crosses,
+// then the bins' records are dealt to the lanes evenly, so that a whole walk is
+// three loads deep where a lane's own would be a hundred instructions and
+// three loads a polygon.
+template <class F>
+__device__ __forceinline__ bool any_poly_near_warp(const DevScene &ds, float x, float y, float dx, float dy, F &&test) {
+    const int lane = threadIdx.x & 31;
+    constexpr float m = 1.f;  // slack of the float steps
+    const float bs = (float)ds.bin_size, ibs = ds.bin_inv;
+    auto col_of = [&](float v) { return min(max((int)floorf((v - (float)ds.bin_x0) * ibs), 0), ds.bin_nx - 1); };
+    auto row_of = [&](float v) { return min(max((int)floorf((v - (float)ds.bin_y0) * ibs), 0), ds.bin_ny - 1); };
+    const int c0 = col_of(fminf(x, x + dx) - m), c1 = col_of(fmaxf(x, x + dx) + m);
+    const bool steep = fabsf(dx) < 0.5f;
+    const float idx = steep ? 0.f : __fdividef(1.0f, dx);
+    const float span = (steep ? fabsf(dy) : fminf(fabsf(dy * idx) * (bs + 2.f * m), fabsf(dy))) + 2.f * m;
+    const int K = min((int)(span * ibs) + 3, ds.bin_ny), items = (c1 - c0 + 1) * K;  // an upper bound of a column's rows
+    for (int j0 = 0; j0 < items; j0 += 32) {
+        int first = 0, cnt = 0;
+        if (j0 + lane < items) {
+            const int c = (j0 + lane) / K, kr = j0 + lane - c * K;
+            float ylo = fminf(0.f, dy), yhi = fmaxf(0.f, dy);
+            if (!steep) {
+                const float xa = (float)(ds.bin_x0 + (c0 + c) * ds.bin_size) - x;
+                const float ta = (xa - m) * idx, tb = (xa + bs + m) * idx;
+                const float ya = __saturatef(fminf(ta, tb)) * dy, yb = __saturatef(fmaxf(ta, tb)) * dy;
+                ylo = fminf(ya, yb);
+                yhi = fmaxf(ya, yb);
+            }
+            const int row = row_of(y + ylo - m) + kr;
+            if (row <= row_of(y + yhi + m)) {
+                const int bin = row * ds.bin_nx + c0 + c;
+                first = __ldg(ds.bin_start + bin);
+                cnt = __ldg(ds.bin_start + bin + 1) - first;
+            }
+        }
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        const int recs = __shfl_sync(0xffffffffu, incl, 31);
+        for (int r0 = 0; r0 < recs; r0 += 32) {
+            const int r = r0 + lane;
+            int own = 0;  // the first lane whose records end beyond r
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, incl, (own + o - 1) & 31) <= r) own += o;
+            own &= 31;
+            const int it = r + __shfl_sync(0xffffffffu, first - incl + cnt, own);
+            bool hit = false;
+            if (r < recs) {
+                const int4 *rp = reinterpret_cast<const int4 *>(ds.bin_recs + it);
+                const int4 bx = __ldg(rp), rec = __ldg(rp + 1);
+                const float hx = 0.5f * (float)(bx.z - bx.x) + m, hy = 0.5f * (float)(bx.w - bx.y) + m;
+                const float qx = 0.5f * (float)(bx.x + bx.z) - x, qy = 0.5f * (float)(bx.y + bx.w) - y;
+                hit = fabsf(dx * qy - dy * qx) <= fabsf(dx) * hy + fabsf(dy) * hx &&
+                      fabsf(qx - 0.5f * dx) <= 0.5f * fabsf(dx) + hx && fabsf(qy - 0.5f * dy) <= 0.5f * fabsf(dy) + hy &&
+                      test(rec);
+            }
+            if (__any_sync(0xffffffffu, hit)) return true;
+        }
+    }
+    return false;
 }
 
 // Pseudo-angle of direction (x, y) != 0: monotone in the true angle, [0, 4),

@@ -152,6 +152,7 @@ struct DevScene {
     int32_t *counters;                 // [0,1] frontier sizes, [2,3] dirty-list sizes
     int32_t sssp_blocks;               // cooperative grid size (CTAs)
     int32_t solo_smem;                 // shared memory the single-CTA fixpoint may use (0: not available)
+    int32_t cl_lists;                  // this compute's cluster kernel builds its in-lists itself
     int32_t fix_launch;                // fixpoint kernels a compute launches (kFix* bits)
     // finalised generator table (read by the pixel kernel)
     float *gen_costf;                  // n_gen (inf when unreached)
@@ -223,7 +224,6 @@ struct BatchDev {
     int32_t n;                         // scenes
     const DevScene *scenes;            // n descriptors (device memory)
     // prefix offsets over scenes (n + 1 entries each)
-    const long long *pair_off;         // warp tasks of the visibility pairs: n_vert * pair_words
     const int32_t *vert_off;           // obstacle-vertex generators
     const int32_t *gen_off;            // generators
     const int32_t *flood_off;          // generators the batched flood takes per scene (sources only when reusing)
@@ -241,6 +241,7 @@ struct BatchDev {
     int2 *frontier[2];
     int32_t *counters;                 // [0,1] frontier sizes, [2,3] dirty sizes, [4] rounds
     int32_t max_rounds;
+    int32_t max_src_words;             // the most source words a scene has
     int32_t sssp_blocks;
     int32_t flood_smem;                // dynamic shared memory of the batched flood (0: no scene floods)
     int32_t any_maps;                  // some scene keeps depth maps
@@ -316,6 +317,8 @@ int cluster_ctas();      // CTAs of a single scene's cluster fixpoint (16, or 8 
 // many-CTA kernel is not launched)
 constexpr int kFixSolo = 1, kFixCluster = 2, kFixSoloSure = 4, kFixClusterSure = 8;
 constexpr int kFixClusterFits = 16;  // the cluster kernel takes every compute's graph (batched form)
+constexpr int kFixClusterLists = 64, kFixBatchLists = 128;  // in-lists with lengths fit its shared memory (16 or 8 CTAs; 8)
+bool cluster_lists(const DevScene &ds, int fix, int need);
 constexpr int kFixClusterWide = 32;  // the cluster kernel runs on 16 CTAs (else 8)
 // from the static in-degrees (scene creation)
 int fixpoint_launches(const DevScene &ds, const std::vector<int32_t> &deg);

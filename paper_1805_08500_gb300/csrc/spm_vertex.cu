@@ -164,20 +164,42 @@ __device__ __forceinline__ bool loc_hidden(const DevScene &ds, int v, int2 vl, i
                                        __ldg(map + (b1 & (kLocBins - 1))));
 }
 
-// Exact visibility of a pair that passed the filter. The predicate is
-// symmetric in the two ends; a source's pairs are walked from the source,
-// since the vertex end already passed its local depth map (what blocks such
-// a pair lies farther from the vertex, often near the source).
-__device__ bool pair_visible(const DevScene &ds, int u, int v) {
+// Exact visibility of a pair that passed the filter, one thread. The predicate
+// is symmetric in the two ends.
+__device__ __forceinline__ bool pair_visible(const DevScene &ds, int u, int v) {
     const int2 vl = ds.gen_lat[v];
     if (ds.gen_kind[u] == kSegI) {
         const int s = ds.gen_aux[u];
         const int4 L = ds.seg_lat[s];
         const long long ux = L.z - L.x, uy = L.w - L.y;
-        return visible_foot(ds, s, vl.x, vl.y, (vl.x - L.x) * ux + (vl.y - L.y) * uy, ux * ux + uy * uy, true);
+        return visible_foot(ds, s, vl.x, vl.y, (vl.x - L.x) * ux + (vl.y - L.y) * uy, ux * ux + uy * uy);
     }
     const int2 ul = ds.gen_lat[u];
-    return u < ds.n_src ? visible_points(ds, ul.x, ul.y, vl.x, vl.y) : visible_points(ds, vl.x, vl.y, ul.x, ul.y);
+    return visible_points(ds, vl.x, vl.y, ul.x, ul.y);
+}
+
+// The same by one warp.
+__device__ __forceinline__ bool pair_visible_warp(const DevScene &ds, int u, int v) {
+    const int2 vl = ds.gen_lat[v], ul = ds.gen_lat[u];
+    const bool seg = ds.gen_kind[u] == kSegI;
+    int4 L = make_int4(0, 0, 0, 0);
+    float x = (float)ul.x, y = (float)ul.y;
+    long long num = 0, den = 0;
+    if (seg) {
+        L = ds.seg_lat[ds.gen_aux[u]];
+        const int ux = L.z - L.x, uy = L.w - L.y;
+        if (cross32(ux, uy, vl.x - L.x, vl.y - L.y) == 0) return true;
+        num = (long long)(vl.x - L.x) * ux + (long long)(vl.y - L.y) * uy;
+        den = (long long)ux * ux + (long long)uy * uy;
+        const float t = __fdividef((float)num, (float)den);  // only chooses what to test
+        x = (float)L.x + t * (float)ux;
+        y = (float)L.y + t * (float)uy;
+    }
+    return !any_poly_near_warp(ds, x, y, (float)vl.x - x, (float)vl.y - y, [&](const int4 &rec) {
+        const int2 *V = ds.poly_v + rec.y;
+        return seg ? foot_meets_poly(V, rec.z, L, vl.x, vl.y, num, den)
+                   : segment_meets_poly(V, rec.z, vl.x, vl.y, ul.x, ul.y);
+    });
 }
 
 // Sets the bit of edge u -> v (row v) and, between two obstacle vertices,
@@ -276,6 +298,52 @@ __global__ void __launch_bounds__(kVisThreads) k_vis_pairs(const __grid_constant
             sc = 0;
             lt = t;
         });
+}
+
+// The source columns of kRowsCta rows, by one CTA: a warp a row picks the
+// sources whose pair passes the filter (a lane each), then the CTA's warps take
+// the pairs one by one. A compute has few such pairs (1871 on the 1024^2
+// polygons, two a row) and its vertex phase waits for the longest of them.
+constexpr int kRowsCta = 4;
+struct SrcPairs {
+    int2 e[kRowsCta * 32];  // (row, source)
+    int n;
+};
+template <class Row>
+__device__ __forceinline__ void src_pairs(SrcPairs &q, int words, Row row) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int w = 0; w < words; ++w) {
+        if (threadIdx.x == 0) q.n = 0;
+        __syncthreads();
+        int vv;
+        if (const DevScene *ds = warp < kRowsCta ? row(warp, vv) : nullptr) {
+            const int u = 32 * w + lane, v = ds->n_src + vv;
+            bool c = u < ds->n_src && pair_filter(*ds, u, v);
+            if (c && ds->vert_maps && ds->gen_kind[u] != kSegI) c = !loc_hidden(*ds, v, ds->gen_lat[v], ds->gen_lat[u]);
+            if (c) q.e[atomicAdd(&q.n, 1)] = make_int2(warp, u);
+        }
+        __syncthreads();
+        for (int i = warp; i < q.n; i += kVisThreads / 32) {
+            const int2 pr = q.e[i];
+            const DevScene *ds = row(pr.x, vv);
+            const bool vis = pair_visible_warp(*ds, pr.y, ds->n_src + vv);
+            if (lane == 0 && vis) atomicOr(&ds->vis_bits[(size_t)vv * ds->vis_words + (pr.y >> 5)], 1u << (pr.y & 31));
+            if (lane == 0) {
+                SPM_CNT(13, 1);
+                SPM_CNT(14, vis);
+            }
+        }
+        __syncthreads();  // the list is rewritten for the next word
+    }
+}
+
+__global__ void __launch_bounds__(kVisThreads) k_src_pairs(const __grid_constant__ DevScene ds) {
+    __shared__ SrcPairs q;
+    chain_start();
+    src_pairs(q, (ds.n_src + 31) / 32, [&](int r, int &vv) -> const DevScene * {
+        vv = blockIdx.x * kRowsCta + r;
+        return vv < ds.n_vert ? &ds : nullptr;
+    });
 }
 
 // In-degree per vertex row and out-degree per generator: one warp per row,
@@ -980,8 +1048,10 @@ __device__ bool cl_solve(const DevScene &ds, int max_rounds, cg::cluster_group &
         }
         return true;
     }
-    const long long E = ds.in_start[nv];
-    if (n >= 32768 || E > ds.edge_cap) return false;
+    // direct: the in-lists straight from the row's source bits and the kept
+    // obstacle-vertex lists; the host has seen that they fit, lengths and all
+    const bool direct = ds.cl_lists;
+    if (!direct && (n >= 32768 || ds.in_start[nv] > ds.edge_cap)) return false;
     static_assert(C <= kClGrp, "a changed vertex's group writes every CTA's copy");
     const int nmax = (nv + C - 1) / C;
     const int n_own = rank < nv ? (nv - rank + C - 1) / C : 0;  // vertices vv = rank + C * k
@@ -991,7 +1061,7 @@ __device__ bool cl_solve(const DevScene &ds, int max_rounds, cg::cluster_group &
     if (L0.lin_src > (size_t)kClSmem) return false;
     // every CTA's in-edge count, in each CTA (warp r sums CTA r's vertices):
     // the largest decides the layout, the same in all, with no exchange
-    if (warp < C) {
+    if (!direct && warp < C) {
         long long m = 0;
         for (int vv = warp + C * lane; vv < nv; vv += 32 * C) m += ds.in_start[vv + 1] - ds.in_start[vv];
 #pragma unroll
@@ -1005,15 +1075,28 @@ __device__ bool cl_solve(const DevScene &ds, int max_rounds, cg::cluster_group &
     long long mine = 0;
     int *lin_start = (int *)(sm_raw + L0.lin_start);
     for (int k = lo; k < hi; ++k) {
-        const int a = ds.in_start[rank + C * k], d = ds.in_start[rank + C * k + 1] - a;
+        const int vv = rank + C * k;
+        int a = 0, d = 0;
+        if (direct) {
+            d = ds.st_start[vv + 1] - ds.st_start[vv];
+            for (int w = 0; w < ds.src_words; ++w)
+                d += __popc(ds.vis_bits[(size_t)vv * ds.vis_words + w] & src_word_mask(ds, w));
+        } else {
+            a = ds.in_start[vv];
+            d = ds.in_start[vv + 1] - a;
+        }
         gstart[k] = a;
         lin_start[k] = d;  // the degree, until the offsets replace it
         mine += d;
     }
     const long long before = cta_exclusive_scan(mine, sh.wsum);  // its barriers publish own_e too
+    if (direct) {
+        if (tid == kClThreads - 1) sh.own_e[rank] = before + mine;
+        __syncthreads();
+    }
     long long mx = 0;
-    for (int r = 0; r < C; ++r) mx = max(mx, sh.own_e[r]);
-    const int fit = cl_layout(n, nv, mx, true, C).end <= (size_t)kClSmem ? 2 : cl_layout(n, nv, mx, false, C).end <= (size_t)kClSmem ? 1 : 0;
+    for (int r = 0; !direct && r < C; ++r) mx = max(mx, sh.own_e[r]);
+    const int fit = direct ? 2 : cl_layout(n, nv, mx, true, C).end <= (size_t)kClSmem ? 2 : cl_layout(n, nv, mx, false, C).end <= (size_t)kClSmem ? 1 : 0;
     if (!fit) return false;
     const bool with_len = fit == 2;
     const ClLayout L = cl_layout(n, nv, sh.own_e[rank], with_len, C);
@@ -1064,6 +1147,25 @@ __device__ bool cl_solve(const DevScene &ds, int max_rounds, cg::cluster_group &
     }
     for (int k = warp; k < n_own; k += nwarps) {  // this CTA's in-lists, a warp per vertex
         const int e0 = gstart[k], b = lin_start[k], m = lin_start[k + 1] - b;
+        if (direct) {  // in generator order: the sources' bits, then the kept list
+            const int vv = rank + C * k;
+            int at = b;
+            for (int w = 0; w < ds.src_words; ++w) {
+                const uint32_t bits = ds.vis_bits[(size_t)vv * ds.vis_words + w] & src_word_mask(ds, w);
+                if (bits >> lane & 1u) {
+                    const int i = at + __popc(bits & ((1u << lane) - 1u)), u = 32 * w + lane;
+                    lin_src[i] = (unsigned short)u;
+                    lin_len[i] = edge_len(ds, u, ns + vv);
+                }
+                at += __popc(bits);
+            }
+            const int s0 = ds.st_start[vv];
+            for (int j = lane; at + j < b + m; j += 32) {
+                lin_src[at + j] = (unsigned short)ds.st_src[s0 + j];
+                lin_len[at + j] = ds.st_len[s0 + j];
+            }
+            continue;
+        }
         for (int j = lane; j < m; j += 32) {
             lin_src[b + j] = (unsigned short)ds.in_src[e0 + j];
             if (with_len) lin_len[b + j] = ds.in_len[e0 + j];
@@ -1218,6 +1320,7 @@ __device__ bool cl_solve(const DevScene &ds, int max_rounds, cg::cluster_group &
         finalize_gen(ds, g, cost[g], pg);
     }
     if (rank == 0 && tid == 0) ds.stats[0] = round;
+    if (direct && tid == 0) atomicAdd(&ds.stats[1], (int)sh.own_e[rank]);
     cluster.sync();  // this scene's shared memory is no longer read
     return true;
 }
@@ -1230,7 +1333,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(kClThreads)
     __shared__ ClShared sh;
     cg::cluster_group cluster = cg::this_cluster();
     bool solo_len;
-    if (solo_bytes(ds, solo_len) > 0) return;  // the single-CTA kernel handles this graph (every CTA agrees)
+    if (!ds.cl_lists && solo_bytes(ds, solo_len) > 0) return;  // the single-CTA kernel handles this graph (every CTA agrees)
     const bool done = cl_solve<C>(ds, max_rounds, cluster, sh, sm_raw);
     if (cluster.block_rank() == 0 && threadIdx.x == 0) ds.counters[4] = done ? 1 : 0;  // else the many-CTA kernel
 }
@@ -1292,8 +1395,6 @@ __global__ void k_prepare_b(const __grid_constant__ BatchDev b) {
         const int nw = ds.st_start ? (ds.n_src + 31) / 32 : ds.vis_words;
         for (int w = 0; w < nw; ++w) row[w] = srow && !ds.st_start ? srow[w] : 0u;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        *reinterpret_cast<unsigned long long *>(b.counters + 6) = 0ull;  // visibility-pair work counter
     const int total = b.gen_off[b.n];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total + b.n; i += gridDim.x * blockDim.x) {
         // entries 0..total-1: one per generator; total..total+n-1: one per scene
@@ -1306,18 +1407,21 @@ __global__ void k_prepare_b(const __grid_constant__ BatchDev b) {
         } else {
             const DevScene &ds = b.scenes[i - total];
             ds.out_start[0] = 0;
+            if (ds.cl_lists) ds.stats[1] = 0;
             if (ds.n_vert == 0) ds.in_start[0] = 0;
         }
     }
 }
 
 __global__ void __launch_bounds__(kVisThreads) k_vis_pairs_b(const __grid_constant__ BatchDev b) {
-    __shared__ PairQ q;
-    vis_pairs_run(
-        q, b.pair_off[b.n], 4, reinterpret_cast<unsigned long long *>(b.counters + 6), [&](int s) { return b.scenes + s; },
-        [&](long long t, int &sc, long long &lt) {
-            sc = scene_of(b.pair_off, b.n, t);
-            lt = t - b.pair_off[sc];
+    __shared__ SrcPairs q;
+    for (int i0 = blockIdx.x * kRowsCta; i0 < b.vert_off[b.n]; i0 += gridDim.x * kRowsCta)
+        src_pairs(q, b.max_src_words, [&](int r, int &vv) -> const DevScene * {
+            const int i = i0 + r;
+            if (i >= b.vert_off[b.n]) return nullptr;
+            const int s = scene_of(b.vert_off, b.n, i);
+            vv = i - b.vert_off[s];
+            return b.scenes + s;
         });
 }
 
@@ -1325,14 +1429,14 @@ __global__ void k_edges_count_b(const __grid_constant__ BatchDev b) {
     const int lane = threadIdx.x & 31, nw = gridDim.x * (blockDim.x >> 5);
     for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < b.vert_off[b.n]; i += nw) {
         const int s = scene_of(b.vert_off, b.n, i);
-        edges_count_row(b.scenes[s], i - b.vert_off[s], lane);
+        if (!b.scenes[s].cl_lists) edges_count_row(b.scenes[s], i - b.vert_off[s], lane);
     }
 }
 
 __global__ void __launch_bounds__(1024) k_edges_scan_b(const __grid_constant__ BatchDev b) {
     __shared__ long long part[32];
     const DevScene &ds = b.scenes[blockIdx.x];
-    if (ds.n_vert > 0) edges_scan_block(ds, part);
+    if (ds.n_vert > 0 && !ds.cl_lists) edges_scan_block(ds, part);
 }
 
 __global__ void k_edges_fill_b(const __grid_constant__ BatchDev b) {
@@ -1340,7 +1444,7 @@ __global__ void k_edges_fill_b(const __grid_constant__ BatchDev b) {
     for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < b.vert_off[b.n]; i += nw) {
         const int s = scene_of(b.vert_off, b.n, i);
         const DevScene &ds = b.scenes[s];
-        if (ds.in_start[ds.n_vert] > ds.edge_cap) continue;
+        if (ds.cl_lists || ds.in_start[ds.n_vert] > ds.edge_cap) continue;
         edges_fill_row(ds, i - b.vert_off[s], lane);
         if (ds.st_start) edges_out_copy(ds, i - b.vert_off[s], lane);  // vertex i's kept out-list
     }
@@ -1515,6 +1619,7 @@ __global__ void k_vertex_prep(const __grid_constant__ DevScene ds) {
             *reinterpret_cast<unsigned long long *>(ds.stats + 2) = 0ull;  // the pair kernel's work counter
             ds.counters[4] = 0;
             ds.counters[6] = 0;
+            if (ds.cl_lists) ds.stats[1] = 0;  // the edges, summed by the cluster's CTAs
         }
     }
 }
@@ -1582,6 +1687,10 @@ int fixpoint_launches(const DevScene &ds, const std::vector<int32_t> &deg) {
     // the batched form's clusters are of the portable size
     if (cluster_ok && cl_layout(ds.n_gen, nv, own_max(kClCtas), false, kClCtas).end <= (size_t)kClSmem)
         f |= kFixClusterFits;
+    // with their lengths as well: the cluster can build its in-lists itself
+    if (cluster_sure && cl_layout(ds.n_gen, nv, own_max(C), true, C).end <= (size_t)kClSmem) f |= kFixClusterLists;
+    if ((f & kFixClusterFits) && cl_layout(ds.n_gen, nv, own_max(kClCtas), true, kClCtas).end <= (size_t)kClSmem)
+        f |= kFixBatchLists;
     if (solo_sure) f = (f & ~kFixCluster) | kFixSoloSure;
     if (cluster_sure && !solo_sure) f |= kFixClusterSure;
     return f;
@@ -1822,9 +1931,7 @@ __global__ void __launch_bounds__(256) k_warm_verify(const __grid_constant__ Dev
     const int2 vl = ds.gen_lat[v];
     long long best = 0x7ff0000000000000ll;  // +inf bits
     int bpar = -1;
-    const int e0 = act ? ds.in_start[vv] : 0, e1 = act ? ds.in_start[vv + 1] : 0;
-    for (int e = e0 + gl; e < e1; e += kWarmGrp) {  // in generator order within the lane
-        const int u = ds.in_src[e];
+    auto pull = [&](int u, double len) {
         const double cu = ds.warm_cost[u];
         const int pu = ds.warm_par[u];
         const int2 ul = ds.gen_lat[u];
@@ -1834,11 +1941,17 @@ __global__ void __launch_bounds__(256) k_warm_verify(const __grid_constant__ Dev
         const short4 w = make_short4((short)w4.x, (short)w4.y, (short)w4.z, (short)w4.w);
         const bool valid = (__double_as_longlong(cu) < 0x7ff0000000000000ll) &
                            ((u < ns) | ((pu >= 0) & in_shadow_cone(dx, dy, w, vl.x - ul.x, vl.y - ul.y)));
-        const long long cand = __double_as_longlong(__dadd_rn(cu, ds.in_len[e]));
+        const long long cand = __double_as_longlong(__dadd_rn(cu, len));
         if (valid & (cand < best)) {
             best = cand;
             bpar = u;
         }
+    };
+    if (act) {  // in generator order within the lane: the sources' bits, then the kept list
+        const uint32_t *row = ds.vis_bits + (size_t)vv * ds.vis_words;
+        for (int u = gl; u < ns; u += kWarmGrp)
+            if ((row[u >> 5] >> (u & 31)) & 1u) pull(u, edge_len(ds, u, v));
+        for (int j = ds.st_start[vv] + gl, j1 = ds.st_start[vv + 1]; j < j1; j += kWarmGrp) pull(ds.st_src[j], ds.st_len[j]);
     }
 #pragma unroll
     for (int o = kWarmGrp / 2; o > 0; o >>= 1) {  // the fixpoint's lexicographic minimum over the group
@@ -2044,17 +2157,28 @@ cudaError_t launch_vtab_build(const DevScene &ds, double *tab, int32_t *counter,
     return cudaGetLastError();
 }
 
+// The cluster kernel builds its in-lists itself, with the launch bits `need`
+// (the device's choice of flood or scan reads the edge count: it keeps them).
+bool cluster_lists(const DevScene &ds, int fix, int need) {
+    return ds.st_start && ds.vis_static && (fix & need) == need && !(ds.use_flood && ds.flood_mode == 0);
+}
+
 void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *side) {
     int f = ds.fix_launch;
     if (g_many_cta_override.load() && !(f & kFixSoloSure)) f &= ~(kFixCluster | kFixClusterSure);  // test hook
     // the warm start needs a fixpoint kernel that takes it (the many-CTA one
     // always starts from the sources)
     const bool warm = warm_start_used(ds, f);
+    // a graph that only the cluster kernel takes, in-lists and lengths in its
+    // shared memory: it builds them itself, and the edge lists (count, scan,
+    // fill: 18 us on the 1024^2 polygons) are not needed
+    const bool lists = cluster_lists(ds, f, kFixClusterSure | kFixClusterLists) && !(f & kFixSolo);
     // one kernel sets every per-compute start value (out-degrees, cursors,
     // the source columns of the bit matrix, counters, estimates)
     {
         DevScene arg = ds;
         arg.warm = warm ? 1 : 0;
+        arg.cl_lists = lists ? 1 : 0;
         const long long items = std::max<long long>(
             ds.n_gen + 1, ds.st_start ? (long long)ds.n_vert * ((ds.n_src + 31) / 32) : 0);
         k_vertex_prep<<<(int)std::max(1LL, std::min((items + 255) / 256, 152LL * 4)), 256, 0, st>>>(arg);
@@ -2068,12 +2192,14 @@ void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *
             if (ds.vis_static) cudaMemcpyAsync(ds.vis_bits, ds.vis_static, bytes, cudaMemcpyDeviceToDevice, st);
             else cudaMemsetAsync(ds.vis_bits, 0, bytes, st);
         }
-        launch_pairs(ds, st, false);
         const int eb = (ds.n_vert + 7) / 8;  // one warp per row
-        if (warm && side) {
+        if (ds.vis_static) launch_chained(k_src_pairs, dim3((ds.n_vert + kRowsCta - 1) / kRowsCta), dim3(kVisThreads), 0, st, ds);
+        else launch_pairs(ds, st, false);
+        if (lists) {
+        } else if (warm && side) {
             // the tree's estimates, parents and fold read the source columns
-            // and kept lists themselves: the edge lists, which only the
-            // verification and the fixpoint read, are built beside them
+            // and kept lists themselves, and so does the verification: the
+            // edge lists, which only the fixpoint reads, are built beside them
             cudaEventRecord(side->fork, st);
             cudaStreamWaitEvent(side->st, side->fork, 0);
             k_edges_count<<<eb, 256, 0, side->st>>>(ds);
@@ -2095,20 +2221,25 @@ void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *
     // own; the scene's bounds on the edge count skip the launches that
     // cannot apply
     arg.warm = warm ? 1 : 0;
+    arg.cl_lists = lists ? 1 : 0;
     if (arg.warm) {
         const int vb = (ds.n_vert + 255) / 256;
         launch_chained(k_warm_entry, dim3(vb, (ds.n_vert + kEntryRows - 1) / kEntryRows), dim3(256), 0, st, arg);
         const int gb = (ds.n_vert * kWarmGrp + 255) / 256;
         launch_chained(k_warm_tree, dim3(gb), dim3(256), 0, st, arg);
         launch_chained(k_warm_fold, dim3(1), dim3(kFoldThreads), fold_bytes(ds.n_gen), st, arg);
-        if (side && ds.n_vert > 0) {  // the edge lists are complete before the verification reads them
-            cudaStreamWaitEvent(st, side->join, 0);
-            k_warm_verify<<<gb, 256, 0, st>>>(arg);
-        } else {
-            launch_chained(k_warm_verify, dim3(gb), dim3(256), 0, st, arg);
-        }
+        launch_chained(k_warm_verify, dim3(gb), dim3(256), 0, st, arg);
     }
-    if (f & kFixSolo) launch_chained(k_sssp_solo, dim3(1), dim3(kSoloThreads), (size_t)ds.solo_smem, st, arg, max_rounds);
+    if (f & kFixSolo) {
+        if (arg.warm && side && ds.n_vert > 0) {  // the edge lists are complete before the fixpoint reads them
+            cudaStreamWaitEvent(st, side->join, 0);
+            k_sssp_solo<<<1, kSoloThreads, ds.solo_smem, st>>>(arg, max_rounds);
+        } else {
+            launch_chained(k_sssp_solo, dim3(1), dim3(kSoloThreads), (size_t)ds.solo_smem, st, arg, max_rounds);
+        }
+    } else if (arg.warm && side && ds.n_vert > 0 && !lists) {
+        cudaStreamWaitEvent(st, side->join, 0);
+    }
     if (f & kFixCluster) {
         if (f & kFixClusterWide)
             launch_chained(k_sssp_cluster<kClCtasWide>, dim3(kClCtasWide), dim3(kClThreads), (size_t)kClSmem, st, arg,
