@@ -13,6 +13,7 @@ points without it raises ``SpmLibraryMissing``.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 import re
 
@@ -145,7 +146,8 @@ def _stream_handle(stream):
     if stream is None:
         try:
             import torch
-            return torch.cuda.current_stream().cuda_stream
+            # the handle alone: a Stream object costs 3 us a call
+            return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
         except Exception:  # pragma: no cover - torch missing
             return None
     if isinstance(stream, int):
@@ -561,8 +563,8 @@ def _make_autograd():
             # the sources move on the device: no host round trip in the step
             pts = points.detach().to(scene.device, torch.float32).contiguous()
             sgs = segs.detach().to(scene.device, torch.float32).contiguous()
-            spm_scene_update_sources_device(scene.handle, None, pts.reshape(-1) if pts.numel() else None,
-                                            sgs.reshape(-1) if sgs.numel() else None)
+            spm_scene_update_sources_device(scene.handle, None, pts if pts.numel() else None,
+                                            sgs if sgs.numel() else None)
             dist, parent = scene.compute()
             loss = torch.empty((), dtype=torch.float32, device=scene.device)
             n = int(agents.shape[0])
@@ -577,12 +579,15 @@ def _make_autograd():
         @staticmethod
         def backward(ctx, grad_out):
             scene = ctx.scene
-            gp = torch.zeros(ctx.shapes[0], dtype=torch.float32, device=scene.device)
-            gs = torch.zeros(ctx.shapes[1], dtype=torch.float32, device=scene.device)
-            spm_agents_backward(scene.handle, None, ctx.tape, ctx.n, gp if gp.numel() else None,
-                                gs if gs.numel() else None)
-            g = grad_out.to(scene.device)
-            return (gp * g).to(ctx.devices[0]), (gs * g).to(ctx.devices[1]), None, None
+            # both gradients in one buffer, every entry of it written by the kernel:
+            # one multiplication by grad_out, none to clear
+            n_p, n_s = (math.prod(x) for x in ctx.shapes)
+            both = torch.empty(n_p + n_s, dtype=torch.float32, device=scene.device)
+            spm_agents_backward(scene.handle, None, ctx.tape, ctx.n, both[:n_p] if n_p else None,
+                                both[n_p:] if n_s else None)
+            both = both * grad_out.to(scene.device)
+            return (both[:n_p].view(ctx.shapes[0]).to(ctx.devices[0]),
+                    both[n_p:].view(ctx.shapes[1]).to(ctx.devices[1]), None, None)
 
     return AgentLoss
 
