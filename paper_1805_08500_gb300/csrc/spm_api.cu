@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -35,6 +36,9 @@ struct spm_scene {
     // phase timing events (vertex start, pixel start, end)
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     bool ev_valid = false;
+    std::mutex path_lock;
+    spm::PathOut *path_out = nullptr;  // page-locked, on first use
+    size_t path_bytes = 0;
     double *query_out = nullptr;  // exact query result: distance, then parent (device)
     // side stream of the geometric flood (flood mode 3), with fork/join events
     cudaStream_t side = nullptr;
@@ -148,6 +152,10 @@ void free_all(spm_scene *s) {
             cudaFreeHost(s->bounce[k]);
             s->bounce[k] = nullptr;
         }
+    }
+    if (s->path_out) {
+        cudaFreeHost(s->path_out);
+        s->path_out = nullptr;
     }
     if (s->copy) {
         cudaStreamDestroy(s->copy);
@@ -1157,17 +1165,24 @@ spm_status spm_compute_batched(spm_scene *const *scenes, int32_t n, void *stream
     return st;
 }
 
-spm_status spm_query_parent(spm_scene *s, float x, float y, int32_t *parent, float *dist) {
-    if (!s || !parent || !dist) return set_err(s, SPM_ERR_INVALID_ARG, "null argument");
+// The pixel of world point (x, y) in the last computed field.
+static spm_status query_pixel(spm_scene *s, float x, float y, size_t &idx) {
     if (!s->last_dist) return set_err(s, SPM_ERR_INVALID_ARG, "nothing computed yet");
     if (!(x >= 0.f && y >= 0.f && x < (float)s->hs.Wx && y < (float)s->hs.Wy))
         return set_err(s, SPM_ERR_INVALID_ARG, "query point outside the world");
     spm_status st = check_device(s);
     if (st != SPM_OK) return st;
-    int i = (int)std::floor(x / s->ds.hx), j = (int)std::floor(y / s->ds.hy);
-    i = std::min(i, s->hs.Nx - 1);
-    j = std::min(j, s->hs.Ny - 1);
-    const size_t idx = (size_t)j * s->hs.Nx + i;
+    const int i = std::min((int)std::floor(x / s->ds.hx), s->hs.Nx - 1);
+    const int j = std::min((int)std::floor(y / s->ds.hy), s->hs.Ny - 1);
+    idx = (size_t)j * s->hs.Nx + i;
+    return SPM_OK;
+}
+
+spm_status spm_query_parent(spm_scene *s, float x, float y, int32_t *parent, float *dist) {
+    if (!s || !parent || !dist) return set_err(s, SPM_ERR_INVALID_ARG, "null argument");
+    size_t idx;
+    spm_status st = query_pixel(s, x, y, idx);
+    if (st != SPM_OK) return st;
     if (cudaStreamSynchronize(s->last_stream) != cudaSuccess ||
         cudaMemcpy(parent, s->last_parent + idx, sizeof(int32_t), cudaMemcpyDefault) != cudaSuccess ||
         cudaMemcpy(dist, s->last_dist + idx, sizeof(float), cudaMemcpyDefault) != cudaSuccess)
@@ -1206,40 +1221,45 @@ spm_status spm_query_exact(spm_scene *s, float x, float y, int32_t *parent, floa
 
 spm_status spm_extract_path(spm_scene *s, float x, float y, float *out_xy, int32_t cap, int32_t *n) {
     if (!s || !out_xy || !n || cap < 1) return set_err(s, SPM_ERR_INVALID_ARG, "bad argument");
-    int32_t g;
-    float d;
-    spm_status st = spm_query_parent(s, x, y, &g, &d);
+    size_t idx;
+    spm_status st = query_pixel(s, x, y, idx);
     if (st != SPM_OK) return st;
-    st = refresh_host_sources(s);
-    if (st != SPM_OK) return st;
-    std::vector<int32_t> par(s->hs.n_gen);
-    if (cudaMemcpy(par.data(), s->ds.gen_par, sizeof(int32_t) * s->hs.n_gen, cudaMemcpyDeviceToHost) != cudaSuccess)
-        return set_err(s, SPM_ERR_CUDA, "parent table copy failed");
-    int cnt = 0;
+    cudaPointerAttributes at{};  // a field that was freed since is an error here, not a fault there
+    if (cudaPointerGetAttributes(&at, s->last_parent + idx) != cudaSuccess || at.type == cudaMemoryTypeUnregistered) {
+        cudaGetLastError();
+        return set_err(s, SPM_ERR_CUDA, "query copy failed");
+    }
+    std::lock_guard<std::mutex> hold(s->path_lock);  // one page-locked buffer a scene
+    // a chain visits no generator twice (the walk stops after n_gen + 2)
+    const int room = std::min(cap - 1, s->hs.n_gen + 2);
+    const size_t bytes = sizeof(spm::PathOut) + sizeof(float2) * (size_t)room;
+    if (s->path_bytes < bytes) {
+        if (s->path_out) cudaFreeHost(s->path_out);
+        s->path_out = nullptr;
+        s->path_bytes = 0;
+        const size_t most = std::max(bytes, (size_t)4096);
+        if (cudaHostAlloc((void **)&s->path_out, most, cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            return set_err(s, SPM_ERR_OOM, "page-locked path buffer allocation failed");
+        }
+        s->path_bytes = most;
+    }
+    spm::launch_path(s->ds, s->last_stream, s->last_parent, idx, room, s->path_out);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s->last_stream) != cudaSuccess)
+        return set_err(s, SPM_ERR_CUDA, "path query failed");
+    const spm::PathOut &o = *s->path_out;
+    if (o.more) return set_err(s, SPM_ERR_CAPACITY, "path longer than cap");
     out_xy[0] = x;
     out_xy[1] = y;
-    cnt = 1;
-    float lx = x, ly = y;
-    const spm::HostScene &hs = s->hs;
-    for (int guard = 0; g >= 0 && guard <= hs.n_gen + 1; ++guard) {
-        if (cnt >= cap) return set_err(s, SPM_ERR_CAPACITY, "path longer than cap");
-        const int kind = hs.gen_kind[g];
-        if (kind == spm::kSegI) {
-            const float *F = &hs.segs[4 * hs.gen_aux[g]];
-            const float ux = F[2] - F[0], uy = F[3] - F[1];
-            const float t = ((lx - F[0]) * ux + (ly - F[1]) * uy) / (ux * ux + uy * uy);
-            out_xy[2 * cnt] = F[0] + t * ux;
-            out_xy[2 * cnt + 1] = F[1] + t * uy;
-            ++cnt;
-            break;
-        }
-        lx = hs.gen_pos[2 * g];
-        ly = hs.gen_pos[2 * g + 1];
-        out_xy[2 * cnt] = lx;
-        out_xy[2 * cnt + 1] = ly;
+    std::memcpy(out_xy + 2, o.pt, sizeof(float2) * (size_t)o.n);
+    int cnt = 1 + o.n;
+    if (o.seg) {
+        const float *F = &o.f.x, lx = out_xy[2 * cnt - 2], ly = out_xy[2 * cnt - 1];
+        const float ux = F[2] - F[0], uy = F[3] - F[1];
+        const float t = ((lx - F[0]) * ux + (ly - F[1]) * uy) / (ux * ux + uy * uy);
+        out_xy[2 * cnt] = F[0] + t * ux;
+        out_xy[2 * cnt + 1] = F[1] + t * uy;
         ++cnt;
-        if (kind != spm::kVert) break;
-        g = par[g];
     }
     *n = cnt;
     return SPM_OK;

@@ -298,6 +298,16 @@ void launch_flood_batched(const BatchDev &b, cudaStream_t st, long long src_ins,
 // exact query at lattice point (qx, qy), world (fx, fy), pixel (i, j) of the last field
 void launch_query_exact(const DevScene &ds, cudaStream_t st, const int32_t *field_parent, int i, int j, int qx,
                         int qy, double fx, double fy, int32_t *out_par, double *out_dist);
+// the parent chain of pixel idx, into page-locked memory (n points at most)
+struct PathOut {
+    int32_t n;                         // points written (generator positions, in order)
+    int32_t seg;                       // the chain ends at a segment's interior: its foot comes after them
+    int32_t more;                      // the chain goes on (n is all the caller has room for)
+    int32_t parent;                    // the pixel's parent, -1: none
+    float4 f;                          // that segment
+    float2 pt[1];
+};
+void launch_path(const DevScene &ds, cudaStream_t st, const int32_t *field_parent, size_t idx, int room, PathOut *out);
 int sssp_batched_grid_blocks();
 int fixpoint_round_cap(int n_gen);  // rounds the vertex fixpoint may take (test hook aside: 4 n_gen + 64)
 bool flood_possible(int tiles, int polys);

@@ -711,7 +711,7 @@ __global__ void __launch_bounds__(kCullThreads) k_tile_cull_b(const __grid_const
     }
 }
 
-constexpr long long kTwoWaves = 2 * 152 * 28;
+constexpr long long kFourWaves = 4 * 152 * 28;
 #ifndef SPM_BLK_MINB
 #define SPM_BLK_MINB 28  // warps per SM the kernels are compiled for
 #endif
@@ -821,6 +821,38 @@ __global__ void k_query_exact(const __grid_constant__ DevScene ds, const int32_t
     }
 }
 
+// Parent chain of a pixel (Sec. 1), one thread: a few dependent loads, written
+// straight to the host's page-locked buffer, so that a path costs one launch
+// and one wait (three copies and a wait, one of them of the whole parent
+// table, took 33 us a path).
+__global__ void k_path(const __grid_constant__ DevScene ds, const int32_t *__restrict__ field_parent, size_t idx,
+                       int room, PathOut *out) {
+    int g = field_parent[idx], n = 0, seg = 0, more = 0;
+    out->parent = g;
+    for (int guard = 0; g >= 0 && guard <= ds.n_gen + 1; ++guard) {
+        if (n >= room) {
+            more = 1;
+            break;
+        }
+        const int kind = ds.gen_kind[g], next = ds.gen_par[g];
+        if (kind == kSegI) {
+            out->f = ds.seg_pos[ds.gen_aux[g]];
+            seg = 1;
+            break;
+        }
+        out->pt[n++] = ds.gen_pos[g];
+        if (kind != kVert) break;
+        g = next;
+    }
+    out->n = n;
+    out->seg = seg;
+    out->more = more;
+}
+
+void launch_path(const DevScene &ds, cudaStream_t st, const int32_t *field_parent, size_t idx, int room, PathOut *out) {
+    k_path<<<1, 1, 0, st>>>(ds, field_parent, idx, room, out);
+}
+
 void launch_query_exact(const DevScene &ds, cudaStream_t st, const int32_t *field_parent, int i, int j, int qx,
                         int qy, double fx, double fy, int32_t *out_par, double *out_dist) {
     k_query_exact<<<1, 32, 0, st>>>(ds, field_parent, i, j, make_int2(qx, qy), make_double2(fx, fy), out_par,
@@ -889,21 +921,22 @@ void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int
         if (ds.cull_on) launch_chained(kern, grid, dim3(32), 0, st, ds, dist, parent, row0);
         else kern<<<grid, 32, 0, st>>>(ds, dist, parent, row0);
     };
-    // The largest blocks that still give the GPU about two waves of warps
-    // (28 an SM): large blocks cull and order their candidates for more pixels
-    // at once, but a small grid of them waits for its slowest few. Pixel pass
-    // in us with 16 x 16 / 16 x 8 / 8 x 8 / 8 x 4 blocks: 256^2 rectangles 33 /
-    // 22 / 17 / 15, 512^2 polygons 73 / 47 / 34 / 41, 1024^2 polygons 92 / 81 /
-    // 90 / 118, 1501^2 156 / 161 / 210 / 421, maze 4096^2 264 / 334 / 447 / 860.
+    // The smallest blocks that make at most four waves of warps (28 an SM):
+    // large blocks cull and order their candidates for more pixels at once, but
+    // a grid of few blocks waits for its slowest. Pixel pass in us with one /
+    // two / four / eight waves for the line: squares 1000^2 109 / 84 / 72 / 70,
+    // 512^2 polygons 37 / 35 / 35 / 35, 1024^2 79 / 70 / 70 / 76, 1501^2 127 /
+    // 127 / 127 / 123, maze 2048^2 80 / 80 / 80 / 90, differentiable 112 / 112 /
+    // 113 / 124.
     const bool scan = !ds.use_flood || ds.flood_mode == 2 || ds.flood_mode == 0;  // (or may, decided on the device)
     auto pick = [&](auto shape, auto lists, auto scans) {
         if (scan) run(shape, scans);
         else run(shape, lists);
     };
     const long long blocks = (long long)((ds.Nx + 15) / 16) * ((rows + 15) / 16);
-    if (blocks * 8 <= kTwoWaves) pick(Shape<1, 1>(), k_pixel_blocks<1, 1, false>, k_pixel_blocks<1, 1, true>);
-    else if (blocks * 4 <= kTwoWaves) pick(Shape<2, 1>(), k_pixel_blocks<2, 1, false>, k_pixel_blocks<2, 1, true>);
-    else if (blocks * 2 <= kTwoWaves) pick(Shape<4, 1>(), k_pixel_blocks<4, 1, false>, k_pixel_blocks<4, 1, true>);
+    if (blocks * 8 <= kFourWaves) pick(Shape<1, 1>(), k_pixel_blocks<1, 1, false>, k_pixel_blocks<1, 1, true>);
+    else if (blocks * 4 <= kFourWaves) pick(Shape<2, 1>(), k_pixel_blocks<2, 1, false>, k_pixel_blocks<2, 1, true>);
+    else if (blocks * 2 <= kFourWaves) pick(Shape<4, 1>(), k_pixel_blocks<4, 1, false>, k_pixel_blocks<4, 1, true>);
     else pick(Shape<4, 2>(), k_pixel_blocks<4, 2, false>, k_pixel_blocks<4, 2, true>);
 }
 
