@@ -439,7 +439,9 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX 
 #pragma unroll 1
         for (int k = 0; k < PX * PY; ++k) {
             const float fx = pixel_x(ds, b.i + k % PX), fy = pixel_y(ds, b.j + k / PX * kStep);
-            const float d = fabsf((sf.z - sf.x) * (fy - sf.y) - (sf.w - sf.y) * (fx - sf.x)) * il, old = ws.bd[k * 32 + lane];
+            // the roundings named: which product is contracted is otherwise the compiler's choice
+            const float cross = fmaf(-(sf.w - sf.y), fx - sf.x, __fmul_rn(sf.z - sf.x, fy - sf.y));
+            const float d = fabsf(cross) * il, old = ws.bd[k * 32 + lane];
             ws.d[k * 32 + lane] = d;
             if (d < old || (d == old && g < ws.bi[k * 32 + lane])) want |= 1u << k;
         }
