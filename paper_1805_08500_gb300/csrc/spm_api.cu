@@ -994,7 +994,8 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     for (int k = 0; k < n; ++k) {
         const spm::DevScene &d = descs[order[k]];
         tile_off[k + 1] = tile_off[k] + d.tiles_x * d.tiles_y;
-        blk_off[k + 1] = blk_off[k] + (d.Nx + 15) / 16 * ((d.Ny + 15) / 16);
+        blk_off[k + 1] = blk_off[k] + (d.Nx + spm::kBatchBlkW - 1) / spm::kBatchBlkW *
+                                          ((d.Ny + spm::kBatchBlkH - 1) / spm::kBatchBlkH);
     }
     bool ok = true;
     spm::BatchDev &bd = b->dev;

@@ -219,6 +219,8 @@ struct DevScene {
     uint32_t *src_mask;
 };
 
+constexpr int kBatchBlkW = 16, kBatchBlkH = 8;  // pixels of a batch's blocks
+
 // A batch of scenes computed together (device-side descriptor).
 struct BatchDev {
     int32_t n;                         // scenes
@@ -231,7 +233,7 @@ struct BatchDev {
     const int32_t *order;              // n scene indices
     const int32_t *tile_off;           // n + 1 prefix of tiles in that order
     int32_t total_tiles;
-    const int32_t *blk_off;            // n + 1 prefix of 16 x 16 pixel blocks in that order
+    const int32_t *blk_off;            // n + 1 prefix of the pixel blocks in that order
     int32_t total_blocks;
     int32_t *tile_counter;             // persistent-kernel work counter
     float *const *dist;                // n output planes (device pointers)

@@ -732,12 +732,17 @@ __global__ void __launch_bounds__(32, SPM_BLK_MINB) k_pixel_blocks(const __grid_
 
 // Persistent form over a batch of scenes: each warp takes the next
 // (scene, block) from a global counter (costliest tiles first), copies that
-// scene's descriptor into shared memory and runs the same code.
-constexpr int kBatchWarps = 4;  // per CTA: neighbouring blocks share their lists and maps in L1
-__global__ void __launch_bounds__(32 * kBatchWarps, SPM_BLK_MINB / kBatchWarps) k_pixel_blocks_b(const __grid_constant__ BatchDev b) {
-    __shared__ WarpSmem<8> sm[kBatchWarps];
+// scene's descriptor into shared memory and runs the same code. Blocks of
+// 16 x 8: a batch's grids are coarse, and a larger block evaluates generators
+// for pixels they cannot win (64 polygon scenes, 22.4 Mpixel: 16 x 16 1674 us,
+// 16 x 8 1220, 8 x 8 1306). 24 warps an SM (1206 us; 28: 1220, 32: 1293, more
+// of them contend for L1), four a CTA (one to sixteen: within 2 %).
+constexpr int kBatchWarps = 4, kBatchSm = 24;
+__global__ void __launch_bounds__(32 * kBatchWarps, kBatchSm / kBatchWarps) k_pixel_blocks_b(const __grid_constant__ BatchDev b) {
+    using S = Shape<4, 1>;
+    static_assert(S::kW == kBatchBlkW && S::kH == kBatchBlkH, "the batch counts these blocks");
+    __shared__ WarpSmem<S::kPix> sm[kBatchWarps];
     __shared__ DevScene sds[kBatchWarps];
-    using S = Shape<4, 2>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     DevScene &ds = sds[warp];
     int held = -1;
@@ -761,7 +766,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, SPM_BLK_MINB / kBatchWarps) 
             held = sc;
         }
         const int across = (ds.Nx + S::kW - 1) / S::kW;
-        pixel_block<4, 2, false>(ds, blk % across * S::kW, blk / across * S::kH, b.dist[sc], b.parent[sc], sm[warp]);
+        pixel_block<4, 1, false>(ds, blk % across * S::kW, blk / across * S::kH, b.dist[sc], b.parent[sc], sm[warp]);
         __syncwarp();
     }
 }
@@ -929,7 +934,9 @@ void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int
     // two / four / eight waves for the line: squares 1000^2 109 / 84 / 72 / 70,
     // 512^2 polygons 37 / 35 / 35 / 35, 1024^2 79 / 70 / 70 / 76, 1501^2 127 /
     // 127 / 127 / 123, maze 2048^2 80 / 80 / 80 / 90, differentiable 112 / 112 /
-    // 113 / 124.
+    // 113 / 124. Halving a 16 x 16 block costs the least work, and pays up to six
+    // waves (four / six: 1560^2 polygons 120 / 113, 1700^2 150 / 138, maze 1536^2
+    // 68 / 64).
     const bool scan = !ds.use_flood || ds.flood_mode == 2 || ds.flood_mode == 0;  // (or may, decided on the device)
     auto pick = [&](auto shape, auto lists, auto scans) {
         if (scan) run(shape, scans);
@@ -938,7 +945,7 @@ void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int
     const long long blocks = (long long)((ds.Nx + 15) / 16) * ((rows + 15) / 16);
     if (blocks * 8 <= kFourWaves) pick(Shape<1, 1>(), k_pixel_blocks<1, 1, false>, k_pixel_blocks<1, 1, true>);
     else if (blocks * 4 <= kFourWaves) pick(Shape<2, 1>(), k_pixel_blocks<2, 1, false>, k_pixel_blocks<2, 1, true>);
-    else if (blocks * 2 <= kFourWaves) pick(Shape<4, 1>(), k_pixel_blocks<4, 1, false>, k_pixel_blocks<4, 1, true>);
+    else if (blocks * 2 <= kFourWaves / 2 * 3) pick(Shape<4, 1>(), k_pixel_blocks<4, 1, false>, k_pixel_blocks<4, 1, true>);
     else pick(Shape<4, 2>(), k_pixel_blocks<4, 2, false>, k_pixel_blocks<4, 2, true>);
 }
 
