@@ -22,6 +22,8 @@ struct spm_scene {
     int device = 0;
     std::string err;
     std::vector<void *> allocs;
+    unsigned char *chunk = nullptr;  // small buffers are cut from this allocation
+    size_t chunk_left = 0;
     const float *last_dist = nullptr;
     const int32_t *last_parent = nullptr;
     cudaStream_t last_stream = nullptr;
@@ -103,13 +105,29 @@ T *dalloc(spm_scene *s, size_t n) {
             }
             break;
         }
+    // A scene has about sixty buffers, most of a few KB, and an allocation
+    // takes some 10 us of host time: those of up to kSmall bytes are cut, 256
+    // bytes apart at least, from chunks that are freed with the rest.
+    constexpr size_t kSmall = (size_t)64 << 10, kChunk = (size_t)1 << 20;
+    const size_t bytes = sizeof(T) * (n ? n : 1), cut = (bytes + 255) & ~(size_t)255;
+    const bool small = bytes <= kSmall;
+    if (small && cut <= s->chunk_left) {
+        unsigned char *p = s->chunk;
+        s->chunk += cut;
+        s->chunk_left -= cut;
+        return reinterpret_cast<T *>(p);
+    }
     void *p = nullptr;
-    if (cudaMalloc(&p, sizeof(T) * (n ? n : 1)) != cudaSuccess) {
+    if (cudaMalloc(&p, small ? kChunk : bytes) != cudaSuccess) {
         cudaGetLastError();  // not sticky: clear it, the caller reports SPM_ERR_OOM
         s->alloc_failed = true;
         return nullptr;
     }
     s->allocs.push_back(p);
+    if (small) {
+        s->chunk = static_cast<unsigned char *>(p) + cut;
+        s->chunk_left = kChunk - cut;
+    }
     return static_cast<T *>(p);
 }
 
@@ -128,6 +146,8 @@ T *dupload(spm_scene *s, const std::vector<T> &v, bool &ok) {
 void free_all(spm_scene *s) {
     for (void *p : s->allocs) cudaFree(p);
     s->allocs.clear();
+    s->chunk = nullptr;
+    s->chunk_left = 0;
     for (cudaEvent_t &e : s->ev)
         if (e) {
             cudaEventDestroy(e);
@@ -1249,6 +1269,7 @@ spm_status spm_extract_path(spm_scene *s, float x, float y, float *out_xy, int32
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s->last_stream) != cudaSuccess)
         return set_err(s, SPM_ERR_CUDA, "path query failed");
     const spm::PathOut &o = *s->path_out;
+    if (o.more == 2) return set_err(s, SPM_ERR_INVALID_ARG, "the parent plane no longer holds this scene's map");
     if (o.more) return set_err(s, SPM_ERR_CAPACITY, "path longer than cap");
     out_xy[0] = x;
     out_xy[1] = y;

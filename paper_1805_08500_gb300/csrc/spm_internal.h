@@ -304,7 +304,7 @@ void launch_query_exact(const DevScene &ds, cudaStream_t st, const int32_t *fiel
 struct PathOut {
     int32_t n;                         // points written (generator positions, in order)
     int32_t seg;                       // the chain ends at a segment's interior: its foot comes after them
-    int32_t more;                      // the chain goes on (n is all the caller has room for)
+    int32_t more;                      // 1: the chain goes on (n is all the caller has room for), 2: not a generator
     int32_t parent;                    // the pixel's parent, -1: none
     float4 f;                          // that segment
     float2 pt[1];

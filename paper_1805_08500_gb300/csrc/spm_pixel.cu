@@ -837,8 +837,8 @@ __global__ void k_path(const __grid_constant__ DevScene ds, const int32_t *__res
     int g = field_parent[idx], n = 0, seg = 0, more = 0;
     out->parent = g;
     for (int guard = 0; g >= 0 && guard <= ds.n_gen + 1; ++guard) {
-        if (n >= room) {
-            more = 1;
+        if (n >= room || g >= ds.n_gen) {
+            more = g >= ds.n_gen ? 2 : 1;  // 2: the plane no longer holds this scene's map
             break;
         }
         const int kind = ds.gen_kind[g], next = ds.gen_par[g];

@@ -1069,3 +1069,105 @@ def test_pixel_blocks_at_their_edges(spm, oracle_mod, n, tile):
             s.sync()
             check_parity(scene, d.cpu().numpy().reshape(Ny, Nx), p.cpu().numpy().reshape(Ny, Nx), rd, rp, rd2,
                          f"blocks n={n} tile={tile} mode={mode} maps={maps} off={off}", rp2)
+
+
+def _route_scene(which):
+    rng = np.random.default_rng(11)
+    if which == "rects":
+        return sg.plain_rects(5, W=400, N=100, n_rects=8)
+    if which == "polys":
+        return sg.plain_polys(9, W=2000, N=250, n_polys=60, n_segs=2)
+    if which == "maze":
+        return sg.maze(4, cells=24, N=768)
+    if which == "many_sources":  # more sources than one word of their bits
+        s = sg.plain_polys(9, n_polys=80, N=256, n_segs=1)
+        pts = [(x, y) for x, y in rng.uniform(0, s.world[0], (400, 2))
+               if not any(q[:, 0].min() - 2 <= x <= q[:, 0].max() + 2 and q[:, 1].min() - 2 <= y <= q[:, 1].max() + 2
+                          for q in s.polys)]
+        return sg.Scene(s.world, s.grid, s.polys, [(float(x), float(y)) for x, y in pts[:37]], s.segs)
+
+    def triangles(side, n, step):
+        at = rng.permutation((side // step) ** 2)[:n]
+        return [np.array([(x, y), (x + step // 2, y + 1), (x + 1, y + step // 2)])
+                for x, y in ((step * int(a % (side // step)) + 8, step * int(a // (side // step)) + 8) for a in at)]
+    if which == "crowded_tile":  # hundreds of vertices that win in one tile: more than its culled list holds
+        return sg.Scene((4096, 4096), (64, 64), triangles(1024, 400, 48), [(3000.0, 2900.0)], [(2000.0, 100.0, 3900.0, 200.0)])
+    # "many_tiles": the vertices' tiles are more entries than the kept lists hold
+    return sg.Scene((4096, 4096), (2048, 2048), triangles(4096, 420, 150), [(5.0, 5.0)], [(4000.0, 5.0, 4090.0, 5.0)])
+
+
+@pytest.mark.parametrize("which", ["rects", "polys", "maze", "many_sources", "crowded_tile", "many_tiles"])
+def test_chosen_route_agrees_with_a_full_scan(spm, which):
+    """The route the library chooses by itself (culling, block and tile size,
+    kept lists or bits, sources' bits, the fixpoint's kernels), in its first
+    compute, recorded into a CUDA graph as its first compute, in a later one, by
+    row slabs and at the other tile size, against a scan of every generator by
+    every tile: the same bits."""
+    scene = _route_scene(which)
+    s = spm.Scene(scene)
+    first = s.compute()
+    s.sync()
+    again = s.compute()
+    s.sync()
+    c = spm.Scene(scene)
+    st, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    graphed = c.empty_outputs()
+    with torch.cuda.graph(g, stream=st):
+        spm.spm_compute(c.handle, st, *graphed)
+    g.replay()
+    torch.cuda.synchronize()
+    direct = c.compute()  # after a compute that was only recorded
+    c.sync()
+    g.replay()
+    torch.cuda.synchronize()
+    slabs = s.empty_outputs()
+    side = 32
+    for r in range(0, scene.grid[1], 3 * side):
+        s.compute_rows(r, min(r + 3 * side, scene.grid[1]), *slabs)
+    s.sync()
+    got = {"first": first, "again": again, "graph": graphed, "after the graph": direct, "slabs": slabs}
+    for tile in (16, 32):
+        spm.spm_scene_set_tuning(s.handle, 3, 32, tile, 1)
+        got[f"geometric, tile {tile}"] = s.compute()
+        s.sync()
+    for tile in (16, 32):
+        spm.spm_scene_set_tuning(s.handle, 2, 32, tile, 0)
+        rd, rp = s.compute()
+        s.sync()
+        for name, (d, p) in got.items():
+            assert torch.equal(p, rp), f"{which}, {name}: parents differ from the scan's (tile {tile})"
+            assert torch.equal(d.view(torch.int32), rd.view(torch.int32)), f"{which}, {name}: distances differ"
+
+
+def test_extracted_path_is_the_parent_chain(spm):
+    """A path's points are the parent chain's generators, ended by a segment's
+    foot point, at the smallest cap that holds it; one less is refused."""
+    scene = sg.plain_polys(7, n_polys=80, N=256, n_segs=2)
+    s, gd, gp = gpu_field(spm, scene)
+    kind, lat, _, par = s.generators()
+    S, h = s.info()["lattice_scale"], scene.world[0] / scene.grid[0]
+    rng = np.random.default_rng(1)
+    feet = 0
+    for j, i in rng.integers(0, 256, (150, 2)):
+        if gp[j, i] < 0:
+            continue
+        want, g = [], int(gp[j, i])
+        while True:
+            want.append(g)
+            if kind[g] != 4:
+                break
+            g = int(par[g])
+        path = s.extract_path((i + 0.5) * h, (j + 0.5) * h, cap=1 + len(want))
+        assert len(path) == 1 + len(want)
+        for k, g in enumerate(want):
+            if kind[g] == 3:  # a foot point on the segment
+                feet += 1
+                a, b = (lat[e] / S for e in (g - 2, g - 1)) if kind[g - 1] == 2 else (None, None)
+                assert a is not None
+                away = abs((b[0] - a[0]) * (path[1 + k][1] - a[1]) - (b[1] - a[1]) * (path[1 + k][0] - a[0]))
+                assert away <= 1.0 * np.hypot(*(b - a)) + 1e-3  # snapping moves an endpoint by under a unit
+            else:
+                assert np.all(np.abs(path[1 + k] - lat[g] / S) <= 1.0)
+        with pytest.raises(spm.SpmError):
+            s.extract_path((i + 0.5) * h, (j + 0.5) * h, cap=len(want))
+    assert feet > 0
