@@ -175,7 +175,7 @@ struct DevScene {
     int32_t open_scene;                // an obstacle vertex has 8 tangent edges or more on average
     int32_t use_flood;                 // 0: flood impossible (too many tiles for smem)
     int32_t flood_mode;                // 0 auto (sparse visibility graph), 1 on, 2 off, 3 geometric (concurrent)
-    int32_t hidden_chunk;              // first hidden-test chunk in the pixel pass
+    int32_t hidden_chunk;              // checked and reported, no longer read by a kernel
     int32_t use_maps;                  // keep and use the flood's depth maps (needs gen_maps)
     int32_t *tile_start;               // ntiles + 1 (CSR by tile)
     int32_t *tile_count;               // ntiles (counts, then fill cursors)

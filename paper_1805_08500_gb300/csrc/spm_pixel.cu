@@ -575,6 +575,7 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
     using S = Shape<PX, PY>;
     constexpr int kStep = 32 / S::kRow;
     const int lane = threadIdx.x & 31;
+    SPM_T0();
     Block b;
     b.i0 = i0;
     b.j0 = j0;
@@ -602,6 +603,7 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
         const TileList tl(ds, tile, true);
         b.lists = tl.lists;
         const bool maps = b.lists && ds.use_maps && ds.gen_maps;
+        SPM_LAP(0);
         float ub = INFINITY;  // no pixel of the block can take more
         int n = 0;
         for (int e0 = 0; e0 < tl.total; e0 += 32) {
@@ -620,7 +622,9 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
             const bool last = e0 + 32 >= tl.total;
             if (n > kWarpCand - 32 || (last && n > 0)) {
                 if (lane == 0) SPM_CNT(1, n);
+                SPM_LAP(1);
                 apply_candidates<PX, PY, SCAN>(ds, ws, n, b);
+                SPM_LAP(2);
                 n = 0;
                 if (!last) {
                     float w = b.worst;
@@ -659,6 +663,8 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
                 }
         }
     }
+    SPM_LAP(3);
+    SPM_TFLUSH();
 }
 
 // Open scenes: most of a tile's list (every obstacle vertex that sees some of
@@ -976,7 +982,8 @@ extern "C" int spm_debug_counters(unsigned long long *out32) {
 #endif
 
 #ifdef SPM_TIME
-// Instrumentation build only: reads and clears the pixel kernel's phase clocks.
+// Instrumentation build only: reads and clears the pixel kernel's phase clocks
+// (0 set-up, 1 candidates, 2 their pixels, 3 output; of each CTA's first warp).
 extern "C" int spm_debug_times(unsigned long long *out8) {
     cudaDeviceSynchronize();
     if (cudaMemcpyFromSymbol(out8, spm::g_time, sizeof(unsigned long long) * 8) != cudaSuccess) return 1;
