@@ -495,7 +495,10 @@ __global__ void __launch_bounds__(kFloodThreads, 6) k_flood_direct(const __grid_
 
 // The kept lists from the bits: a warp a tile counts them, and after the scan
 // (static_tile_start) writes the list, in order; static_counts[3] says whether
-// they fit.
+// they fit. Up to kBitsOnly words a tile they would save a block nothing -- it
+// takes 32 entries at a time -- and the first compute does without them (and
+// saves the counts in the sources' first kernel: rectangles 256^2 130 -> 120 us).
+constexpr int kBitsOnly = 2;
 __global__ void k_bits_count(const __grid_constant__ DevScene ds) {
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (t >= ds.tiles_x * ds.tiles_y) return;  // whole warps
@@ -545,14 +548,19 @@ __device__ __forceinline__ bool src_on_grid(const DevScene &ds, int g) {
 }
 
 // Before the sources' culling: empty maps, the global list and the overflow
-// flag as the obstacle vertices' flood left them.
-__device__ __forceinline__ void src_prep(const DevScene &ds, int i0, int stride) {
+// flag as the obstacle vertices' flood left them (keep: just now, to be saved;
+// 2: as bits alone).
+__device__ __forceinline__ void src_prep(const DevScene &ds, int i0, int stride, int keep) {
     const bool maps = ds.use_maps && ds.gen_maps;
     for (int i = i0; i < ds.n_src * kAng; i += stride) {
         ds.gen_maps[i] = make_float2(INFINITY, INFINITY);
         if (i < ds.n_src) ds.gen_map_ok[i] = maps && src_on_grid(ds, i);  // complete by the time the pixel pass reads it
     }
-    if (i0 < 4) ds.flood_counts[i0] = i0 == 1 || i0 == 2 ? ds.static_counts[i0] : 0;
+    if (i0 < 4) {
+        if (keep && i0 < 3) ds.static_counts[i0] = ds.flood_counts[i0];
+        if (keep == 2 && i0 == 3) ds.static_counts[3] = 0;
+        ds.flood_counts[i0] = i0 == 1 || i0 == 2 ? ds.static_counts[i0] : 0;
+    }
 }
 
 template <bool MAPS>
@@ -595,8 +603,8 @@ __device__ __forceinline__ void src_tile(const DevScene &ds, int t) {
     }
 }
 
-__global__ void k_src_prep(const __grid_constant__ DevScene ds) {
-    src_prep(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+__global__ void k_src_prep(const __grid_constant__ DevScene ds, int keep) {
+    src_prep(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, keep);
 }
 
 template <bool MAPS>
@@ -641,7 +649,7 @@ __global__ void __launch_bounds__(kFloodThreads, MAPS ? 6 : 8) k_flood(DevScene 
     }
 }
 
-// After the obstacle vertices' flood (keep = 1) its counts are saved; before
+// After the obstacle vertices' flood (keep = 1, 2: as bits alone) its counts are saved; before
 // the sources' flood (keep = 0) the lists start empty, the global list after
 // the vertices' entries, the overflow flag as the vertices' flood left it,
 // and the work counter from zero.
@@ -653,6 +661,7 @@ __global__ void k_flood_static(DevScene ds, int keep) {
         const int k = threadIdx.x;
         if (keep) {
             if (k < 3) ds.static_counts[k] = ds.flood_counts[k];
+            else if (keep == 2) ds.static_counts[3] = 0;
         } else {
             ds.flood_counts[k] = k == 1 || k == 2 ? ds.static_counts[k] : 0;
         }
@@ -862,26 +871,30 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
         cudaMemsetAsync(ds.flood_counts, 0, sizeof(int32_t) * 4, st);
         flood(0, ds.n_gen);
     } else {
+        int keep = 0;
         if (how == FloodStatic::kBuild) {  // the obstacle vertices' lists, kept for every later compute
-            cudaMemsetAsync(ds.tile_count, 0, sizeof(int32_t) * ntiles, st);
+            keep = 1;
             cudaMemsetAsync(ds.flood_counts, 0, sizeof(int32_t) * 4, st);
             if (flood_verts_direct(ds)) {
                 cudaMemsetAsync(ds.vert_mask, 0, sizeof(uint32_t) * (size_t)ntiles * ds.vert_words, st);
                 const int blocks = std::min(max(sms, 1) * 6, ds.n_vert);
                 if (maps) k_flood_direct<true><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen);
                 else k_flood_direct<false><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen);
-                k_bits_count<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
-                k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
-                k_bits_fill<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
+                if (ds.vert_words <= kBitsOnly) keep = 2;
+                else {
+                    k_bits_count<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
+                    k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
+                    k_bits_fill<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
+                }
             } else {
+                cudaMemsetAsync(ds.tile_count, 0, sizeof(int32_t) * ntiles, st);
                 flood(ds.n_src, ds.n_gen);
                 k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
                 k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 1);
             }
-            k_flood_static<<<sblocks, 256, 0, st>>>(ds, 1);
         }
         if (flood_sources_direct(ds)) {  // a bit per source and tile: nothing to sort
-            k_src_prep<<<std::min((ds.n_src * kAng + 255) / 256, 152 * 8), 256, 0, st>>>(ds);
+            k_src_prep<<<std::min((ds.n_src * kAng + 255) / 256, 152 * 8), 256, 0, st>>>(ds, keep);
             // ordinary launches: a dependent one would hold SMs, waiting, that
             // the vertex phase beside it needs
             const dim3 grid((ds.n_edge + 4 * kSrcEdges - 1) / (4 * kSrcEdges), std::min(ds.n_src, 65535));
@@ -890,6 +903,7 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
             k_src_tiles<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
             return;
         }
+        if (keep) k_flood_static<<<sblocks, 256, 0, st>>>(ds, keep);
         k_flood_static<<<sblocks, 256, 0, st>>>(ds, 0);
         flood(0, ds.n_src);
     }
