@@ -656,7 +656,7 @@ spm_status spm_scene_update_sources_device(spm_scene *s, void *stream, const flo
 // slab from its bounce buffer into the caller's memory meanwhile. Returns
 // once every row is in place.
 static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t *parent, int row0, int row1,
-                        float *dist_host = nullptr, int32_t *parent_host = nullptr) {
+                        float *dist_host = nullptr, int32_t *parent_host = nullptr, bool to_host = false) {
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(cs, &cap);
@@ -707,7 +707,7 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     if (timed) cudaEventRecord(s->ev[3], cs);
     if (!dist_host) {
         NvtxRange r("spm pixel phase");
-        spm::launch_pixel_phase(ds, cs, dist, parent, row0, row1);
+        spm::launch_pixel_phase(ds, cs, dist, parent, row0, row1, to_host);
     } else {
         NvtxRange r("spm pixel phase with host copies");
         const int rows = (row1 - row0 + ds.tile - 1) / ds.tile, nslab = std::min(rows, (int)(sizeof s->slab_ev / sizeof s->slab_ev[0]));
@@ -828,7 +828,7 @@ spm_status spm_compute_host(spm_scene *s, void *stream, float *dist_host, int32_
     cudaGetLastError();  // a pageable pointer is not an error here
     if (direct) {
         st = compute_impl(s, stream, static_cast<float *>(ad.devicePointer), static_cast<int32_t *>(ap.devicePointer),
-                          0, s->hs.Ny);
+                          0, s->hs.Ny, nullptr, nullptr, true);
         // the caller may unpin or free these buffers at any time after the
         // call: queries must not read them (they need a device compute)
         s->last_dist = nullptr;

@@ -274,8 +274,10 @@ void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *
 // entries a tile's culled list may hold
 constexpr int cull_cap(int tile) { return tile == kTile ? 512 : 256; }
 bool tiles_culled(const DevScene &ds);  // the pixel pass culls its lists per tile first
-// pixel kernel over the grid rows [row0, row1); row0 a multiple of the small tile's side
-void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int row0, int row1);
+// pixel kernel over the grid rows [row0, row1); row0 a multiple of the small
+// tile's side; to_host: the planes lie in page-locked host memory
+void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int row0, int row1,
+                        bool to_host = false);
 // flood of the per-tile candidate lists. FloodStatic::kNone floods every
 // generator; kBuild (geometric mode) floods the obstacle vertices, keeps
 // their lists as the static part, then floods the sources; kReuse restores

@@ -76,10 +76,10 @@ constexpr int kCandMap = 1 << 21;     // its depth map is complete
 // The pixels' state lives in shared memory (a lane's eight pixels at
 // k * 32 + lane), not in registers: the loops over them stay rolled, nothing
 // spills around the exact tests, and more warps are resident.
-template <int PX, int PY>
+template <int PX, int PY, int ROW = PX == 1 ? 8 : 4>
 struct Shape {                       // a lane's pixels: PX consecutive ones of PY rows
     static constexpr int kPix = PX * PY;
-    static constexpr int kRow = PX == 1 ? 8 : 4;                  // lanes across the block
+    static constexpr int kRow = ROW;                              // lanes across the block
     static constexpr int kW = PX * kRow, kH = PY * (32 / kRow);   // block size in pixels
 };
 
@@ -223,10 +223,10 @@ __device__ __forceinline__ int2 pixel_bins(float rx, float ry) {
 // takes a listed polygon. (Lanes walking bins of their own, record by record
 // and vertex by vertex, waited on some 80 loads in a row: 57k cycles a list on
 // the 2048^2 maze.)
-template <int PX, int PY>
+template <int PX, int PY, int ROW>
 __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem<PX * PY> &ws, const Block &b, int2 gl, int seg_id,
                                                    float clear, unsigned und) {
-    using S = Shape<PX, PY>;
+    using S = Shape<PX, PY, ROW>;
     constexpr int N = S::kPix;
     const int lane = threadIdx.x & 31;
     if (lane == 0) SPM_CNT(5, 1);
@@ -403,9 +403,9 @@ __device__ __forceinline__ unsigned resolve_pixels(const DevScene &ds, WarpSmem<
 }
 
 // Candidate c against the block's pixels.
-template <int PX, int PY>
+template <int PX, int PY, int ROW>
 __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX * PY> &ws, Block &b, int c) {
-    constexpr int kStep = 32 / Shape<PX, PY>::kRow;  // rows between a lane's pixels
+    constexpr int kStep = 32 / ROW;  // rows between a lane's pixels
     const int lane = threadIdx.x & 31, g = c & kCandId;
     const float4 rec = __ldg(ds.gen_rec + g);
     const int4 q = __ldg(ds.gen_cull + g);
@@ -496,7 +496,7 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX 
     if (__any_sync(0xffffffffu, und)) {
         // squared distances are non-negative: they order as their bits
         const float near = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(clear)));
-        vis |= resolve_pixels<PX, PY>(ds, ws, b, gl, seg_id, map ? sqrtf(near) : 0.f, und);
+        vis |= resolve_pixels<PX, PY, ROW>(ds, ws, b, gl, seg_id, map ? sqrtf(near) : 0.f, und);
     }
     float worst = -INFINITY;
 #pragma unroll
@@ -515,7 +515,7 @@ __device__ __forceinline__ void apply_candidate(const DevScene &ds, WarpSmem<PX 
 
 // The n candidates the warp holds, in order of their lower bounds, until none
 // can improve a pixel.
-template <int PX, int PY, bool SCAN>
+template <int PX, int PY, int ROW, bool SCAN>
 __device__ __forceinline__ void apply_candidates(const DevScene &ds, WarpSmem<PX * PY> &ws, int n, Block &b) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
@@ -543,7 +543,7 @@ __device__ __forceinline__ void apply_candidates(const DevScene &ds, WarpSmem<PX
         }
         c = __shfl_sync(0xffffffffu, c, from);
         if (lane == 0) SPM_CNT(4, 1);
-        apply_candidate<PX, PY>(ds, ws, b, ws.cand[32 * c + from]);
+        apply_candidate<PX, PY, ROW>(ds, ws, b, ws.cand[32 * c + from]);
         if (SCAN && !b.lists && !tested) {
             // flooded lists were tested on the tile's area; a scan's candidates
             // that one polygon hides from the block go here, a lane each,
@@ -569,10 +569,10 @@ __device__ __forceinline__ void apply_candidates(const DevScene &ds, WarpSmem<PX
     __syncwarp();
 }
 
-template <int PX, int PY, bool SCAN>
+template <int PX, int PY, int ROW, bool SCAN>
 __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, const int j0, float *__restrict__ dist,
                                             int32_t *__restrict__ parent, WarpSmem<PX * PY> &ws) {
-    using S = Shape<PX, PY>;
+    using S = Shape<PX, PY, ROW>;
     constexpr int kStep = 32 / S::kRow;
     const int lane = threadIdx.x & 31;
     SPM_T0();
@@ -623,7 +623,7 @@ __device__ __forceinline__ void pixel_block(const DevScene &ds, const int i0, co
             if (n > kWarpCand - 32 || (last && n > 0)) {
                 if (lane == 0) SPM_CNT(1, n);
                 SPM_LAP(1);
-                apply_candidates<PX, PY, SCAN>(ds, ws, n, b);
+                apply_candidates<PX, PY, ROW, SCAN>(ds, ws, n, b);
                 SPM_LAP(2);
                 n = 0;
                 if (!last) {
@@ -726,14 +726,14 @@ constexpr long long kFourWaves = 4 * 152 * 28;
 // One warp a CTA, so that a finished block's place is taken at once: with four
 // warps a CTA (sharing nothing) the early ones waited for the slowest, 15 %
 // on the 4096^2 maze.
-template <int PX, int PY, bool SCAN>
+template <int PX, int PY, int ROW, bool SCAN>
 __global__ void __launch_bounds__(32, SPM_BLK_MINB) k_pixel_blocks(const __grid_constant__ DevScene ds,
                                                                    float *__restrict__ dist,
                                                                    int32_t *__restrict__ parent, int row0) {
     __shared__ WarpSmem<PX * PY> sm;
-    using S = Shape<PX, PY>;
+    using S = Shape<PX, PY, ROW>;
     chain_start();
-    pixel_block<PX, PY, SCAN>(ds, blockIdx.x * S::kW, row0 + blockIdx.y * S::kH, dist, parent, sm);
+    pixel_block<PX, PY, ROW, SCAN>(ds, blockIdx.x * S::kW, row0 + blockIdx.y * S::kH, dist, parent, sm);
 }
 
 // Persistent form over a batch of scenes: each warp takes the next
@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, kBatchSm / kBatchWarps) k_pi
             held = sc;
         }
         const int across = (ds.Nx + S::kW - 1) / S::kW;
-        pixel_block<4, 1, false>(ds, blk % across * S::kW, blk / across * S::kH, b.dist[sc], b.parent[sc], sm[warp]);
+        pixel_block<4, 1, 4, false>(ds, blk % across * S::kW, blk / across * S::kH, b.dist[sc], b.parent[sc], sm[warp]);
         __syncwarp();
     }
 }
@@ -920,7 +920,8 @@ bool tiles_culled(const DevScene &ds) {
     return ds.cull_items && ds.use_flood && ds.flood_mode == 3 && flood_verts_direct(ds);
 }
 
-void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int32_t *parent, int row0, int row1) {
+void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int32_t *parent, int row0, int row1,
+                        bool to_host) {
     DevScene ds = scene;
     const int rows = row1 - row0;
     if (rows <= 0) return;
@@ -949,10 +950,20 @@ void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int
         else run(shape, lists);
     };
     const long long blocks = (long long)((ds.Nx + 15) / 16) * ((rows + 15) / 16);
-    if (blocks * 8 <= kFourWaves) pick(Shape<1, 1>(), k_pixel_blocks<1, 1, false>, k_pixel_blocks<1, 1, true>);
-    else if (blocks * 4 <= kFourWaves) pick(Shape<2, 1>(), k_pixel_blocks<2, 1, false>, k_pixel_blocks<2, 1, true>);
-    else if (blocks * 2 <= kFourWaves / 2 * 3) pick(Shape<4, 1>(), k_pixel_blocks<4, 1, false>, k_pixel_blocks<4, 1, true>);
-    else pick(Shape<4, 2>(), k_pixel_blocks<4, 2, false>, k_pixel_blocks<4, 2, true>);
+    // A large grid's planes in the host's memory: blocks 32 wide, within a tile,
+    // whose rows are whole 128-byte lines. The link takes 193 GB/s of those, as
+    // of copies, but 172 of a 16 x 16 block's 64-byte rows, and such a map waits
+    // for it (16 x 16 or 16 x 8 / 32 x 4, wall clock of the whole call: maze
+    // 4096^2 934 / 845 us, differentiable 2048^2 328 / 303, maze 2048^2 318 /
+    // 314). Smaller grids wait for their slowest block (1024^2 polygons 194 / 205).
+    if (to_host && !scan && ds.tile == kTile && blocks * 4 > kFourWaves) {
+        run(Shape<4, 1, 8>(), k_pixel_blocks<4, 1, 8, false>);
+        return;
+    }
+    if (blocks * 8 <= kFourWaves) pick(Shape<1, 1>(), k_pixel_blocks<1, 1, 8, false>, k_pixel_blocks<1, 1, 8, true>);
+    else if (blocks * 4 <= kFourWaves) pick(Shape<2, 1>(), k_pixel_blocks<2, 1, 4, false>, k_pixel_blocks<2, 1, 4, true>);
+    else if (blocks * 2 <= kFourWaves / 2 * 3) pick(Shape<4, 1>(), k_pixel_blocks<4, 1, 4, false>, k_pixel_blocks<4, 1, 4, true>);
+    else pick(Shape<4, 2>(), k_pixel_blocks<4, 2, 4, false>, k_pixel_blocks<4, 2, 4, true>);
 }
 
 void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st) {

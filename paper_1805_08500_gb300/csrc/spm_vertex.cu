@@ -6,7 +6,8 @@
 //     cost(v) = min over generators u that see v, with v inside u's shadow
 //               cone, of cost(u) + |u - v|
 // computed on the GPU in three steps:
-//   1. k_vis_pairs: one bit per (generator u, obstacle vertex v) pair, set when
+//   1. k_vis_pairs (the obstacle vertices' pairs, once per scene) and
+//      k_src_pairs (the sources', per compute): one bit per (generator u, obstacle vertex v) pair, set when
 //      u sees v exactly and the line uv is tangent to the obstacle wedges of u
 //      and of v (a vertex passes a path on only along a tangent: other edges
 //      never carry a shortest path to a pixel); segment interiors reach v
@@ -16,7 +17,8 @@
 //      the obstacle vertices (k_vert_maps, once per scene) reject most hidden
 //      pairs before the exact test.
 //   2. k_edges_*: the bits become CSR in-lists (by v) with FP64 edge lengths
-//      and out-lists (by u) for frontier marking.
+//      and out-lists (by u) for frontier marking; left out where the cluster
+//      kernel builds its in-lists from the bits itself.
 //   3. k_sssp_solo: for sparse graphs, one CTA with the graph in shared
 //      memory runs rounds over the vertices whose in-neighbours changed, each
 //      pulling its in-neighbours' current state; k_sssp_cluster: for denser

@@ -1171,3 +1171,16 @@ def test_extracted_path_is_the_parent_chain(spm):
         with pytest.raises(spm.SpmError):
             s.extract_path((i + 0.5) * h, (j + 0.5) * h, cap=len(want))
     assert feet > 0
+
+
+@pytest.mark.parametrize("n", [1060, 1066, 1088])
+def test_host_planes_of_a_large_grid(spm, n):
+    """Page-locked planes of a grid large enough for the wide blocks (rows that
+    are and are not whole lines or 16-byte stores): the device compute's bits."""
+    scene = sg.plain_polys(3, W=4 * n, N=n, n_polys=120, n_segs=1)
+    s, gd, gp = gpu_field(spm, scene)
+    spm.spm_scene_set_tuning(s.handle, 3, 32, 32, 1)
+    d = torch.full((n, n), -5.0).pin_memory()
+    p = torch.full((n, n), -5, dtype=torch.int32).pin_memory()
+    spm.spm_compute_host(s.handle, None, d, p)
+    assert np.array_equal(p.numpy(), gp) and np.array_equal(d.numpy().view(np.int32), gd.view(np.int32))
