@@ -41,14 +41,14 @@ FLOPS_PER_PIXEL = 7  # winning-generator distance: 2 sub, mul, fma(2), sqrt, add
 # full-size launch (dram__bytes_read.sum + dram__bytes_write.sum,
 # smsp__issue_active and the ALU / FMA pipe shares; the first timed step,
 # right after the L2 flush) and from the instrumentation build's work
-# counters (orientation tests and exact polygon tests per pixel); valid for
-# those workloads and that kernel version only (re-captured after a change).
-KPIXELS_TRAFFIC = {"maze4096": 104_169_728, "batched256": 1_310_612_480, "polys1024": 6_548_736}
-KPIXELS_UTIL = {"maze4096": {"issue_frac": 0.437, "alu_pipe_frac": 0.304, "fma_pipe_frac": 0.131,
-                             "orient_per_px": 0.254, "exact_tests_per_px": 0.0636},
-                "batched256": {"issue_frac": 0.414, "alu_pipe_frac": 0.289, "fma_pipe_frac": 0.123},
-                "polys1024": {"issue_frac": 0.452, "alu_pipe_frac": 0.296, "fma_pipe_frac": 0.117,
-                              "orient_per_px": 0.360, "exact_tests_per_px": 0.0611}}
+# counters (exact polygon tests per pixel); valid for those workloads and
+# that kernel version only (re-captured after a change).
+KPIXELS_TRAFFIC = {"maze4096": 89_678_336, "batched256": 1_065_832_704, "polys1024": 2_030_336}
+KPIXELS_UTIL = {"maze4096": {"issue_frac": 0.647, "alu_pipe_frac": 0.457, "fma_pipe_frac": 0.207,
+                             "exact_tests_per_px": 0.0200},
+                "batched256": {"issue_frac": 0.627, "alu_pipe_frac": 0.461, "fma_pipe_frac": 0.209},
+                "polys1024": {"issue_frac": 0.521, "alu_pipe_frac": 0.376, "fma_pipe_frac": 0.135,
+                              "exact_tests_per_px": 0.0512}}
 
 
 def fixpoint_start(spm, s, args, tuning):
@@ -428,7 +428,7 @@ def run_batched(args, cfg_desc, scenes):
                        "launch": "one CUDA graph per step", "tuning_by_grid_side": tunings},
             "mpixel_per_s": npx_all / (ms * 1e-3) / 1e6, "clocks": clk.summary(),
             "phases_ms": {"vertex_and_lists": vert_ms, "pixel": pix_ms},
-            "roofline": {"bound": "alu", "kernel": "k_pixels_batched", "achieved": achieved, "peak": peak_tflops,
+            "roofline": {"bound": "alu", "kernel": "k_pixel_blocks_b", "achieved": achieved, "peak": peak_tflops,
                          "unit": "TFLOP/s", "frac": achieved / peak_tflops,
                          "traffic": KPIXELS_TRAFFIC.get("batched256"), **KPIXELS_UTIL.get("batched256", {}),
                          "note": f"algorithmic = {FLOPS_PER_PIXEL} FP32 flops/pixel (winning distance) over the "
@@ -441,7 +441,7 @@ def run_batched(args, cfg_desc, scenes):
             "e2e": {"value": len(all_scenes) / e2e_s, "unit": "scenes/s",
                     "h2d_bytes_per_step": int(4 * offs[-1]), "d2h_bytes_per_step": int(8 * npx),
                     "host_buffers": "page-locked"},
-            # vertex phase (7), list reset, flood, scan, fill, the persistent pixel kernel
+            # vertex phase (7), list reset, the sources' culling (2), the tiles' culling, the persistent pixel kernel
             "gpu_launches": 12 * args.steps}
     if world > 1:
         line["config"]["parallelism"] = f"scenes sharded longest-first over {world} ranks"
@@ -635,7 +635,7 @@ def run_differentiable(args, cfg_desc, scene):
             "phases_ms": {"vertex": float(np.mean([p[0] for p in phases])),
                           "cull": float(np.mean([p[1] for p in phases])), "pixel": pix_ms},
             "fixpoint_rounds": s.info()["rounds"],
-            "roofline": {"bound": "alu", "kernel": "k_pixels", "achieved": achieved, "peak": peak_tflops,
+            "roofline": {"bound": "alu", "kernel": "k_pixel_blocks", "achieved": achieved, "peak": peak_tflops,
                          "unit": "TFLOP/s", "frac": achieved / peak_tflops, "traffic": None,
                          "note": f"the forward's map: algorithmic = {FLOPS_PER_PIXEL} FP32 flops/pixel (winning "
                                  f"distance) over the pixel pass's event-timed duration; peak = FP32 lanes x SMs "
@@ -946,7 +946,7 @@ def main():
     peaks, peak_src = load_peaks()
     vert_ms = float(np.mean([p[0] for p in phases]))
     cull_ms = float(np.mean([p[1] for p in phases]))
-    pix_ms = float(np.mean([p[2] for p in phases]))  # k_pixels, one launch per step
+    pix_ms = float(np.mean([p[2] for p in phases]))  # k_pixel_blocks, one launch per step (open scenes: and k_tile_cull)
     clock_mhz = float(peaks.get("sm_max_mhz", 2070.0))
     peak_tflops = FP32_LANES * N_SMS * 2 * clock_mhz * 1e6 / 1e12
     achieved = FLOPS_PER_PIXEL * npx / (pix_ms * 1e-3) / 1e12
@@ -970,14 +970,14 @@ def main():
                              "upload and the obstacles' static structures (free-space mask, vertex depth "
                              "maps, obstacle-vertex visibility and edges, the table of geodesic distances "
                              "between obstacle vertices; the obstacle vertices' flood at the first compute)"},
-        "roofline": {"bound": "alu", "kernel": "k_pixels", "achieved": achieved,
+        "roofline": {"bound": "alu", "kernel": "k_pixel_blocks", "achieved": achieved,
                      "peak": peak_tflops, "unit": "TFLOP/s", "frac": achieved / peak_tflops,
                      "traffic": KPIXELS_TRAFFIC.get(args.workload),
                      **KPIXELS_UTIL.get(args.workload, {}),
                      "note": f"algorithmic = {FLOPS_PER_PIXEL} FP32 flops/pixel (winning distance); "
                              f"peak = FP32 lanes x SMs x 2 x max SM clock ({peak_src}); issue_frac and the "
-                             f"pipe shares: ncu on one launch of this kernel; orient_per_px: counted "
-                             f"orientation tests of the exact visibility per pixel"},
+                             f"pipe shares: ncu on one launch of this kernel; exact_tests_per_px: "
+                             f"counted polygon tests of the exact visibility per pixel"},
         "hbm_write": {"achieved": write_gbs, "peak": hbm_peak, "unit": "GB/s",
                       "frac": write_gbs / hbm_peak, "bytes_per_pixel": 8,
                       "peak_source": peak_src},
