@@ -934,6 +934,8 @@ int flood_smem_attr() {
            cudaFuncSetAttribute(k_flood_b<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) == cudaSuccess;
 }
 
+bool flood_batched_direct(const BatchDev &b) { return b.flood_smem > 0 && b.walk_tasks <= 0 && !b.any_lists; }
+
 void launch_flood_batched(const BatchDev &b, cudaStream_t st, long long src_ins, long long src_tiles) {
     k_flood_reset_b<<<152 * 4, 256, 0, st>>>(b);
     if (b.flood_smem <= 0) return;  // every scene scans

@@ -298,6 +298,7 @@ void launch_update_sources(const DevScene &ds, cudaStream_t st, const float *pts
 void launch_vertex_phase_batched(const BatchDev &b, cudaStream_t st);
 void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st);
 // src_ins / src_tiles: the totals of b.src_ins_off / b.src_tile_off (host copies)
+bool flood_batched_direct(const BatchDev &b);  // no scene's culling walks or reads the vertex phase
 void launch_flood_batched(const BatchDev &b, cudaStream_t st, long long src_ins, long long src_tiles);
 // exact query at lattice point (qx, qy), world (fx, fy), pixel (i, j) of the last field
 void launch_query_exact(const DevScene &ds, cudaStream_t st, const int32_t *field_parent, int i, int j, int qx,

@@ -1184,3 +1184,30 @@ def test_host_planes_of_a_large_grid(spm, n):
     p = torch.full((n, n), -5, dtype=torch.int32).pin_memory()
     spm.spm_compute_host(s.handle, None, d, p)
     assert np.array_equal(p.numpy(), gp) and np.array_equal(d.numpy().view(np.int32), gd.view(np.int32))
+
+
+def test_batch_recorded_in_a_callers_graph(spm):
+    """A batch whose culling runs beside its vertex phase, recorded into the
+    caller's CUDA graph and replayed after the sources moved: the bits of the
+    scenes' own computes."""
+    scenes = [sg.plain_polys(k, n_polys=60 + 10 * k, N=128 << (k % 3), n_segs=k % 2) for k in range(6)]
+    objs = [spm.Scene(x) for x in scenes]
+    for s in objs:
+        spm.spm_scene_set_tuning(s.handle, 3, 32, 32, 1)
+    batch = spm.Batch(objs)
+    batch.compute()
+    torch.cuda.synchronize()
+    st, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        batch.compute(st)
+    for s, x in zip(objs, scenes):
+        s.update_sources(np.asarray(x.points, np.float32).reshape(-1, 2)[::-1].copy(),
+                         np.asarray(x.segs, np.float32).reshape(-1, 4))
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    out = [(d.clone(), p.clone()) for d, p in batch.outputs]
+    for s, (d, p) in zip(objs, out):
+        rd, rp = s.compute()
+        s.sync()
+        assert torch.equal(p, rp) and torch.equal(d.view(torch.int32), rd.view(torch.int32))
