@@ -359,6 +359,17 @@ __device__ __forceinline__ float pang(float x, float y) {
     return x < 0.f ? 2.f + r : 4.f - r;
 }
 
+// Counter-clockwise pseudo-angle from lo to hi, the ends of an edge seen from
+// its outer side: less than half a turn, so that a difference below -1 has
+// passed 4. One that is merely negative is rounding (an edge in line with the
+// viewer spans less than pang resolves: 1e-9 to 1e-7 where the lattice unit is
+// the world's) and the edge covers nothing. Taken for a turn, it covered the
+// whole circle at its line's distance, often below a unit, and hid everything.
+__device__ __forceinline__ float pang_span(float lo, float hi) {
+    const float d = hi - lo;
+    return d < -1.f ? d + 4.f : fmaxf(d, 0.f);
+}
+
 // Exclusive prefix sum of one value per thread over a CTA of blockDim.x
 // threads (a multiple of 32, at most 1024); every thread must call it.
 // wsum: 32 shared slots. Returns the sum of the values of lower threads.

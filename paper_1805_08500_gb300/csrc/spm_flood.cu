@@ -153,9 +153,7 @@ __device__ __forceinline__ bool edge_view(int2 g, int4 e, EdgeView &v) {
     v.N2 = (float)N * (float)N;
     v.h2 = __fdividef(v.N2, (float)v.ex * (float)v.ex + (float)v.ey * (float)v.ey) * (1.f - 1e-5f);
     v.lo = pang((float)cx, (float)cy);
-    float d = pang((float)ax, (float)ay) - v.lo;
-    if (d < 0.f) d += 4.f;
-    v.hi = v.lo + d;
+    v.hi = v.lo + pang_span(v.lo, pang((float)ax, (float)ay));
     v.c2 = (float)cx * (float)cx + (float)cy * (float)cy;
     v.a2 = (float)ax * (float)ax + (float)ay * (float)ay;
     v.sc = (float)v.ex * (float)cx + (float)v.ey * (float)cy;
@@ -173,7 +171,8 @@ __device__ __forceinline__ bool edge_view(int2 g, int4 e, EdgeView &v) {
 // as a lower bound of where a ray can first meet an obstacle: a ray enters an
 // obstacle through a front-facing edge or a vertex of one. Boundary rays are
 // exact multiples of 1/kAngQ, so their products with n are exact in integers;
-// a 1e-5 margin covers the few float roundings.
+// a 1e-5 margin covers the few float roundings of the distances, kAngEps those
+// of the range's ends (whose order pang_span keeps).
 // check: read a bin first and leave it when the edge does not lower it (saves
 // the atomic, costs the load's latency).
 template <bool MAPS>

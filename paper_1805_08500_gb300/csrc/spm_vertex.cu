@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(256) k_vert_maps(const __grid_constant__ DevSc
                     const float fN2 = (float)N * (float)N;
                     // the edge runs clockwise seen from g: counter-clockwise from c to a
                     const float lo = pang((float)(c.x - g.x), (float)(c.y - g.y));
-                    const float hi = lo + fmodf(pang((float)(a.x - g.x), (float)(a.y - g.y)) - lo + 4.f, 4.f);
+                    const float hi = lo + pang_span(lo, pang((float)(a.x - g.x), (float)(a.y - g.y)));
                     const int k0 = (int)ceilf((lo + kAngEps) / kLocW), k1 = (int)floorf((hi - kAngEps) / kLocW) - 1;
                     auto bdist2 = [&](int mb) {
                         const int2 u = loc_boundary_dir(mb);

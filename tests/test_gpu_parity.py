@@ -1211,3 +1211,116 @@ def test_batch_recorded_in_a_callers_graph(spm):
         rd, rp = s.compute()
         s.sync()
         assert torch.equal(p, rp) and torch.equal(d.view(torch.int32), rd.view(torch.int32))
+
+
+def _pseudo_angle_step(g, a, c):
+    """Float32 difference of the pseudo-angles of edge ends c and a as seen
+    from g (with correctly rounded quotients: the device's may differ by a
+    unit in the last place, so tests take many edges)."""
+    one, two, four = np.float32(1), np.float32(2), np.float32(4)
+
+    def pang(x, y):
+        x, y = np.float32(x), np.float32(y)
+        r = abs(y) * (one / (abs(x) + abs(y)))
+        if y >= 0:
+            return r if x >= 0 else two - r
+        return two + r if x < 0 else four - r
+    return pang(a[0] - g[0], a[1] - g[1]) - pang(c[0] - g[0], c[1] - g[1])
+
+
+def _near_radial_triangles(g, W, n, seed, reach, keep, below=False):
+    """n triangles apart from each other, each with a front-facing edge whose
+    line passes g within a unit: its two ends differ by less in angle, as seen
+    from g, than float32 resolves. keep(step): which rounded differences to take."""
+    rng = np.random.default_rng(seed)
+    out, boxes = [], []
+    while len(out) < n:
+        p, q = (int(v) for v in rng.integers(-24, 25, 2))
+        if math.gcd(p, q) != 1 or abs(p) + abs(q) < 8 or p == 0 or q == 0:
+            continue
+        u = pow(q % abs(p), -1, abs(p)) if abs(p) > 1 else 0  # u q - w p = 1
+        w = (u * q - 1) // p
+        k = int(rng.uniform(*reach) / math.hypot(p, q))
+        c = (g[0] + k * p + u, g[1] + k * q + w)
+        a, t = (c[0] + p, c[1] + q), (c[0] + q, c[1] - p)
+        assert (c[0] - g[0]) * (a[1] - g[1]) - (c[1] - g[1]) * (a[0] - g[0]) == 1
+        tri = np.array([a, c, t])
+        lo, hi = tri.min(0) - 2, tri.max(0) + 2
+        if lo.min() < 4 or hi.max() > W - 4 or (below and hi[1] > g[1] - 400) or not keep(_pseudo_angle_step(g, a, c)):
+            continue
+        if all((lo > b[1]).any() or (hi < b[0]).any() for b in boxes):
+            boxes.append((lo, hi))
+            out.append(tri)
+    return out
+
+
+@pytest.mark.parametrize("seed", range(4))
+@pytest.mark.parametrize("who", ["source", "vertex"])
+def test_edges_in_line_with_a_generator(spm, oracle_mod, who, seed):
+    """Edges that a source, or an obstacle vertex, sees end on: the rounded
+    range of angles of such an edge must not become the whole circle, which
+    would hide everything from that generator. Every route with depth maps
+    against a scan without them, bit for bit, and the oracle."""
+    W, g = 32000, (16000, 16000)
+    polys = _near_radial_triangles(g, W, 10, seed, (4000.0, 15000.0), lambda d: -1 < d < 0)
+    source = g
+    if who == "vertex":  # of an obstacle behind which it is the parent
+        polys.append(np.array([g, (g[0] + 700, g[1] - 900), (g[0] + 800, g[1] - 300)]))
+        source = (g[0] + 1500, g[1] - 1100)
+    scene = sg.Scene((W, W), (250, 250), polys, [tuple(float(v) for v in source)], np.zeros((0, 4)))
+    s = spm.Scene(scene)
+    assert s.info()["lattice_scale"] == 1
+    spm.spm_scene_set_tuning(s.handle, 2, 32, 32, 0)
+    rd, rp = s.compute()
+    s.sync()
+    for mode, tile, maps in ((0, 0, 0), (3, 16, 1), (3, 32, 1), (1, 16, 1), (1, 32, 1)):
+        spm.spm_scene_set_tuning(s.handle, mode, 32, tile, maps)
+        d, p = s.compute()
+        s.sync()
+        assert torch.equal(p, rp) and torch.equal(d.view(torch.int32), rd.view(torch.int32)), (mode, tile, maps)
+    od, op, od2, op2 = oracle_mod.Oracle(scene).field()
+    check_parity(scene, rd.cpu().numpy(), rp.cpu().numpy(), od, op, od2, f"in line with a {who}", op2)
+
+
+@pytest.mark.parametrize("W,n_polys,r,seed", [(32000, 600, (60.0, 500.0), 0), (32000, 600, (60.0, 500.0), 1),
+                                              (32000, 600, (60.0, 500.0), 2), (16384, 300, (60.0, 450.0), 3)])
+def test_large_polygon_worlds(spm, oracle_mod, W, n_polys, r, seed):
+    """Polygon scenes whose lattice is the world's own units, the largest
+    spans: the chosen route and the walk with depth maps against a scan without
+    them, bit for bit, and the oracle at sampled pixels."""
+    scene = sg.tiny(seed, W=W, N=W // 64, n_polys=n_polys, n_points=3, n_segs=1, r=r, k=(4, 8))
+    s = spm.Scene(scene)
+    assert s.info()["lattice_scale"] == 1
+    spm.spm_scene_set_tuning(s.handle, 2, 32, 32, 0)
+    rd, rp = s.compute()
+    s.sync()
+    for mode, tile, maps in ((0, 0, 0), (1, 16, 1), (3, 32, 1)):
+        spm.spm_scene_set_tuning(s.handle, mode, 32, tile, maps)
+        d, p = s.compute()
+        s.sync()
+        assert torch.equal(p, rp) and torch.equal(d.view(torch.int32), rd.view(torch.int32)), (mode, tile, maps)
+    ij = np.random.default_rng(seed).integers(0, W // 64, (4000, 2)).astype(np.int32)
+    od, op, od2, op2 = oracle_mod.Oracle(scene).pixels(ij)
+    gd, gp = (t.cpu().numpy()[ij[:, 1], ij[:, 0]] for t in (rd, rp))
+    check_parity(scene, gd, gp, od, op, od2, f"world {W}, seed {seed}", op2)
+
+
+def test_vertex_pairs_past_edges_in_line(spm, oracle_mod):
+    """The local depth maps that filter vertex pairs: an edge the vertex sees
+    end on must not hide every other generator from it. Vertex costs against
+    the oracle's, over scenes with few, near polygons."""
+    W, g = 32000, (16000, 20000)
+
+    def whole_circle(d):  # a range that a remainder of 4 does not bring back to nothing
+        return -1 < d < 1 and float(np.fmod(np.float32(d + np.float32(4)), np.float32(4))) > 1
+    for seed in range(24):
+        polys = _near_radial_triangles(g, W, 6, seed, (3000.0, 8500.0), whole_circle, below=True)
+        polys.append(np.array([g, (g[0] + 300, g[1] + 800), (g[0] - 300, g[1] + 800)]))
+        scene = sg.Scene((W, W), (250, 250), polys, [(float(g[0] - 6000), float(g[1] + 7))], np.zeros((0, 4)))
+        s = spm.Scene(scene)
+        s.compute()
+        s.sync()
+        _, _, cost, par = s.generators()
+        o = oracle_mod.Oracle(scene)
+        used = o.cside != oracle_mod.CONE_EMPTY
+        assert np.array_equal(cost[used], o.cost[used]) and np.array_equal(par[used], o.parent[used]), seed
