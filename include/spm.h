@@ -121,7 +121,9 @@ spm_status spm_scene_update_sources_device(spm_scene *scene, void *stream,
  * foot, Sec. 4). Asynchronous on `stream` (a cudaStream_t, NULL = legacy
  * default stream). dist_dev / parent_dev: caller-owned DEVICE buffers of
  * grid_w * grid_h elements, row-major. Allocates nothing. Device-side errors
- * surface through spm_scene_sync. */
+ * surface through spm_scene_sync. May be captured in a CUDA graph: a replay
+ * runs with the tuning of its capture and the sources of its moment, whatever
+ * tuning the scene was computed with in between. */
 spm_status spm_compute(spm_scene *scene, void *stream, float *dist_dev,
                        int32_t *parent_dev);
 

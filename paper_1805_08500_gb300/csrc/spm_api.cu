@@ -66,6 +66,9 @@ struct spm_scene {
     // device for this tile size and depth-map setting
     bool flood_static_ok = false;
     int flood_static_tile = 0, flood_static_maps = 0;
+    // a graph holds work of this scene that writes it: what the device has is
+    // not known here any more, and computes go by the device's own tag
+    bool flood_recorded = false;
     // the warm start of the fixpoint: the rounds the table build's deepest
     // root took, whether that makes the warm start the default, and the
     // caller's choice (spm_tuning.fixpoint_start)
@@ -438,7 +441,8 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
             ds.gen_map_ok = dalloc<uint8_t>(s, hs.n_gen);
             if (ds.gen_map_ok) cudaMemset(ds.gen_map_ok, 0, hs.n_gen);
         }
-        ds.flood_counts = dalloc<int32_t>(s, 4);
+        ds.flood_counts = dalloc<int32_t>(s, spm::kFloodCounts);
+        if (ds.flood_counts) cudaMemset(ds.flood_counts, 0, sizeof(int32_t) * spm::kFloodCounts);
         ds.static_tile_start = ds.use_flood ? dalloc<int32_t>(s, ntiles + 1) : nullptr;
         ds.static_tile_items = ds.use_flood ? dalloc<int32_t>(s, ds.pair_cap) : nullptr;
         ds.static_counts = ds.use_flood ? dalloc<int32_t>(s, 4) : nullptr;
@@ -683,14 +687,18 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
         const bool maps = ds.use_maps && ds.gen_maps;
         const bool reuse = s->flood_static_ok && s->flood_static_tile == ds.tile &&
                            s->flood_static_maps == (int)maps && ds.static_tile_start;
+        // recorded into a graph, now or before: the host does not know what the
+        // device holds when this runs (the checks' kernels, at most six, end at
+        // once beside the vertex phase)
+        if (!timed) s->flood_recorded = true;
         cudaStreamWaitEvent(s->side, s->fork, 0);
         spm::launch_flood(ds, s->side,
                           !ds.static_tile_start ? spm::FloodStatic::kNone
-                          : reuse                  ? spm::FloodStatic::kReuse
-                                                   : spm::FloodStatic::kBuild);
+                          : s->flood_recorded   ? spm::FloodStatic::kEnsure
+                          : reuse               ? spm::FloodStatic::kReuse
+                                                : spm::FloodStatic::kBuild);
         cudaEventRecord(s->join, s->side);
-        // (a build recorded into a graph runs with every replay, and none has run yet)
-        s->flood_static_ok = ds.static_tile_start != nullptr && (timed || reuse);
+        s->flood_static_ok = ds.static_tile_start != nullptr && !s->flood_recorded;
         s->flood_static_tile = ds.tile;
         s->flood_static_maps = (int)maps;
     }
@@ -700,6 +708,7 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
     } else if (ds.use_flood) {
         spm::launch_flood(ds, cs);
         s->flood_static_ok = false;  // the lists and maps now hold this flood's
+        if (!timed) s->flood_recorded = true;
     } else {
         static const int32_t off[4] = {0, 0, 1, 0};
         cudaMemcpyAsync(ds.flood_counts, off, sizeof off, cudaMemcpyHostToDevice, cs);
@@ -926,7 +935,7 @@ void batch_free(spm_batch *b) {
 bool build_flood_static(spm_scene *s, const spm::DevScene &d) {
     spm::launch_flood(d, nullptr, spm::FloodStatic::kBuild);
     if (cudaStreamSynchronize(nullptr) != cudaSuccess) return false;
-    s->flood_static_ok = true;
+    s->flood_static_ok = !s->flood_recorded;
     s->flood_static_tile = d.tile;
     s->flood_static_maps = d.use_maps && d.gen_maps ? 1 : 0;
     return true;
@@ -1121,18 +1130,23 @@ spm_status spm_batch_compute(spm_batch *b, void *stream) {
     if (cudaGetDevice(&dev) != cudaSuccess || dev != b->device)
         return set_err(nullptr, SPM_ERR_INVALID_ARG, "batch used on another device");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &cap);
     // a single-scene compute in another flood mode may have replaced a
     // scene's static lists since: rebuild them before the batch reads them
+    // (where a graph may have, the device checks)
     for (size_t k = 0; k < b->scenes.size(); ++k)
         if (b->descs[k].flood_reuse && !flood_static_matches(b->scenes[k], b->descs[k])) {
-            if (cudaStreamSynchronize(st) != cudaSuccess || !build_flood_static(b->scenes[k], b->descs[k]))
+            if (cap != cudaStreamCaptureStatusNone || b->scenes[k]->flood_recorded) {
+                spm::launch_flood_kept(b->descs[k], st);
+                b->scenes[k]->flood_recorded = true;
+            } else if (cudaStreamSynchronize(st) != cudaSuccess || !build_flood_static(b->scenes[k], b->descs[k])) {
                 return set_err(nullptr, SPM_ERR_CUDA, "static flood rebuild failed");
+            }
         }
     // the caller's stream may be the legacy default stream, which cannot be
     // captured: the graph is captured and replayed on the batch's own
     // stream, after the caller's prior work and before its later work
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(st, &cap);
     if (cap != cudaStreamCaptureStatusNone) {  // inside the caller's own capture: record the launches there
         batch_launch(b, st, true);
     } else {
@@ -1172,8 +1186,10 @@ spm_status spm_batch_compute(spm_batch *b, void *stream) {
         s->last_parent = nullptr;
         s->ev_valid = false;
         // the batched flood rewrote the lists of scenes that flood every generator
-        if (!b->descs[k].flood_reuse && b->descs[k].use_flood && b->descs[k].flood_mode != 2)
+        if (!b->descs[k].flood_reuse && b->descs[k].use_flood && b->descs[k].flood_mode != 2) {
             s->flood_static_ok = false;
+            if (cap != cudaStreamCaptureStatusNone) s->flood_recorded = true;
+        }
     }
     return SPM_OK;
 }
@@ -1356,7 +1372,8 @@ spm_status spm_scene_info(spm_scene *s, int64_t *info) {
     const bool own_lists = spm::cluster_lists(run, run.fix_launch, spm::kFixClusterSure | spm::kFixClusterLists) &&
                            !(run.fix_launch & spm::kFixSolo);
     info[10] = 1 + (s->hs.n_vert > 0 ? (own_lists ? 1 : 4) : 0) + (s->ds.warm && s->ds.vtab ? 4 : 0) + (s->ds.fix_launch & spm::kFixSolo ? 1 : 0) +
-               (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull : 3) : 0) + (spm::tiles_culled(run) ? 1 : 0) + 1;
+               (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull : 3) : 0) +
+               (reuse && s->flood_recorded ? spm::flood_kept_kernels(run) : 0) + (spm::tiles_culled(run) ? 1 : 0) + 1;
     return SPM_OK;
 }
 

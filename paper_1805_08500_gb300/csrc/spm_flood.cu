@@ -50,6 +50,30 @@ __device__ __forceinline__ bool cone_meets_box(int ct, int4 c, int2 v, int4 box)
     return !(out1 || out2);
 }
 
+// What the kept part of the obstacle vertices is built for. Whoever overwrites
+// it clears the tag in flood_counts; its last kernel sets it. A build whose
+// kernels get the tag as `unless` does nothing when the device has that part
+// already: recorded computes are replayed in whatever order the caller likes,
+// between computes of other tunings.
+__host__ __device__ __forceinline__ int kept_tag(const DevScene &ds) {
+    return 4 | (ds.tile == kTile ? 2 : 0) | (ds.use_maps && ds.gen_maps ? 1 : 0);
+}
+__device__ __forceinline__ bool kept_already(const DevScene &ds, int unless) {
+    return unless && ds.flood_counts[kKeptTag] == unless;
+}
+
+// Before the obstacle vertices' flood: no counts, no bits or tile counts.
+__global__ void k_kept_reset(const __grid_constant__ DevScene ds, int unless) {
+    if (kept_already(ds, unless)) return;
+    const size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    const size_t ntiles = (size_t)ds.tiles_x * ds.tiles_y;
+    if (i0 < 4) ds.flood_counts[i0] = 0;
+    if (ds.vert_bits)
+        for (size_t i = i0; i < ntiles * ds.vert_words; i += step) ds.vert_mask[i] = 0u;
+    else
+        for (size_t i = i0; i < ntiles; i += step) ds.tile_count[i] = 0;
+}
+
 __device__ __forceinline__ void push_global(const DevScene &ds, int g) {
     ds.glob_list[atomicAdd(&ds.flood_counts[1], 1)] = g;
 }
@@ -480,9 +504,11 @@ __device__ void flood_direct(const DevScene &ds, float *up, float *low, int g) {
 
 // Resident CTAs take the obstacle vertices [g0, g1) from the work counter.
 template <bool MAPS>
-__global__ void __launch_bounds__(kFloodThreads, 6) k_flood_direct(const __grid_constant__ DevScene ds, int g0, int g1) {
+__global__ void __launch_bounds__(kFloodThreads, 6) k_flood_direct(const __grid_constant__ DevScene ds, int g0, int g1,
+                                                                   int unless) {
     __shared__ float up[kAng], low[kAng];
     __shared__ int next_g;
+    if (kept_already(ds, unless)) return;
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) next_g = g0 + atomicAdd(&ds.flood_counts[3], 1);
@@ -498,19 +524,19 @@ __global__ void __launch_bounds__(kFloodThreads, 6) k_flood_direct(const __grid_
 // takes 32 entries at a time -- and the first compute does without them (and
 // saves the counts in the sources' first kernel: rectangles 256^2 130 -> 120 us).
 constexpr int kBitsOnly = 2;
-__global__ void k_bits_count(const __grid_constant__ DevScene ds) {
+__global__ void k_bits_count(const __grid_constant__ DevScene ds, int unless) {
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (t >= ds.tiles_x * ds.tiles_y) return;  // whole warps
+    if (t >= ds.tiles_x * ds.tiles_y || kept_already(ds, unless)) return;  // whole warps
     int n = 0;
     for (int w = lane; w < ds.vert_words; w += 32) n += __popc(ds.vert_mask[(size_t)t * ds.vert_words + w]);
     n = __reduce_add_sync(0xffffffffu, n);
     if (lane == 0) ds.tile_count[t] = n;
 }
 
-__global__ void k_bits_fill(const __grid_constant__ DevScene ds) {
+__global__ void k_bits_fill(const __grid_constant__ DevScene ds, int unless) {
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int ntiles = ds.tiles_x * ds.tiles_y;
-    if (t >= ntiles) return;  // whole warps
+    if (t >= ntiles || kept_already(ds, unless)) return;  // whole warps
     const bool fit = ds.static_tile_start[ntiles] <= ds.pair_cap;
     if (t == 0 && lane == 0) ds.static_counts[3] = fit;
     if (!fit) return;
@@ -546,20 +572,28 @@ __device__ __forceinline__ bool src_on_grid(const DevScene &ds, int g) {
     return ds.gen_kind[g] != kSegI && gl.x >= 0 && gl.y >= 0 && gl.x <= ds.Nx * ds.pitch_x && gl.y <= ds.Ny * ds.pitch_y;
 }
 
-// Before the sources' culling: empty maps, the global list and the overflow
-// flag as the obstacle vertices' flood left them (keep: just now, to be saved;
-// 2: as bits alone).
-__device__ __forceinline__ void src_prep(const DevScene &ds, int i0, int stride, int keep) {
+// The obstacle vertices' flood is done (keep = 1, 2: as bits alone; 0: some
+// time ago): its counts are saved and its tag is set. restore: the counts a
+// compute's sources start from, the global list and the overflow flag as that
+// flood left them. One whole warp.
+__device__ __forceinline__ void kept_counts(const DevScene &ds, int keep, int unless, bool restore) {
+    const int k = threadIdx.x & 31;
+    const bool built = keep && !kept_already(ds, unless);
+    __syncwarp();  // every lane has read the tag
+    if (k < 3 && built) ds.static_counts[k] = ds.flood_counts[k];
+    if (k == 3 && built && keep == 2) ds.static_counts[3] = 0;
+    if (k == kKeptTag && built) ds.flood_counts[k] = kept_tag(ds);
+    if (k < 4 && restore) ds.flood_counts[k] = k == 1 || k == 2 ? ds.static_counts[k] : 0;
+}
+
+// Before the sources' culling: empty maps and the counts they start from.
+__device__ __forceinline__ void src_prep(const DevScene &ds, int i0, int stride, int keep, int unless) {
     const bool maps = ds.use_maps && ds.gen_maps;
     for (int i = i0; i < ds.n_src * kAng; i += stride) {
         ds.gen_maps[i] = make_float2(INFINITY, INFINITY);
         if (i < ds.n_src) ds.gen_map_ok[i] = maps && src_on_grid(ds, i);  // complete by the time the pixel pass reads it
     }
-    if (i0 < 4) {
-        if (keep && i0 < 3) ds.static_counts[i0] = ds.flood_counts[i0];
-        if (keep == 2 && i0 == 3) ds.static_counts[3] = 0;
-        ds.flood_counts[i0] = i0 == 1 || i0 == 2 ? ds.static_counts[i0] : 0;
-    }
+    if (i0 < 32) kept_counts(ds, keep, unless, true);
 }
 
 template <bool MAPS>
@@ -602,8 +636,8 @@ __device__ __forceinline__ void src_tile(const DevScene &ds, int t) {
     }
 }
 
-__global__ void k_src_prep(const __grid_constant__ DevScene ds, int keep) {
-    src_prep(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, keep);
+__global__ void k_src_prep(const __grid_constant__ DevScene ds, int keep, int unless) {
+    src_prep(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, keep, unless);
 }
 
 template <bool MAPS>
@@ -630,10 +664,11 @@ __device__ __forceinline__ bool flood_declined(const DevScene &ds) {
 // kernel waiting for the CTAs that drew several deep generators.
 // Generators [g0, g1) are flooded.
 template <bool MAPS>
-__global__ void __launch_bounds__(kFloodThreads, MAPS ? 6 : 8) k_flood(DevScene ds, int g0, int g1) {
+__global__ void __launch_bounds__(kFloodThreads, MAPS ? 6 : 8) k_flood(DevScene ds, int g0, int g1, int unless) {
     extern __shared__ unsigned fdyn[];
     __shared__ FloodSmem sm;
     __shared__ int next_g;
+    if (kept_already(ds, unless)) return;
     if (flood_declined(ds)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) ds.flood_counts[2] = 1;
         return;
@@ -648,23 +683,15 @@ __global__ void __launch_bounds__(kFloodThreads, MAPS ? 6 : 8) k_flood(DevScene 
     }
 }
 
-// After the obstacle vertices' flood (keep = 1, 2: as bits alone) its counts are saved; before
-// the sources' flood (keep = 0) the lists start empty, the global list after
-// the vertices' entries, the overflow flag as the vertices' flood left it,
-// and the work counter from zero.
-__global__ void k_flood_static(DevScene ds, int keep) {
+// After the obstacle vertices' flood (keep) its counts are saved; before the
+// sources' flood (keep = 0) the lists start empty, the global list after the
+// vertices' entries, the overflow flag as the vertices' flood left it, and the
+// work counter from zero.
+__global__ void k_flood_static(DevScene ds, int keep, int unless) {
     const int ntiles = ds.tiles_x * ds.tiles_y;
     if (!keep)
         for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x) ds.tile_count[t] = 0;
-    if (blockIdx.x == 0 && threadIdx.x < 4) {
-        const int k = threadIdx.x;
-        if (keep) {
-            if (k < 3) ds.static_counts[k] = ds.flood_counts[k];
-            else if (keep == 2) ds.static_counts[3] = 0;
-        } else {
-            ds.flood_counts[k] = k == 1 || k == 2 ? ds.static_counts[k] : 0;
-        }
-    }
+    if (blockIdx.x == 0 && threadIdx.x < 32) kept_counts(ds, keep, unless, !keep);
 }
 
 
@@ -720,10 +747,14 @@ __global__ void k_flood_reset_b(const __grid_constant__ BatchDev b) {
         } else {  // reusing scenes: the global list after the vertices' entries
             const DevScene &ds = b.scenes[(int)(i - total)];
             const bool on = ds.use_flood && ds.flood_mode != 2;
+            // a kept part of another tuning (only a batch recorded in its
+            // caller's graph meets one): the scene scans every generator
+            const bool kept = ds.flood_reuse && ds.flood_counts[kKeptTag] == kept_tag(ds);
             ds.flood_counts[0] = 0;
-            ds.flood_counts[1] = ds.flood_reuse ? ds.static_counts[1] : 0;
-            ds.flood_counts[2] = ds.flood_reuse ? ds.static_counts[2] : (on ? 0 : 1);
+            ds.flood_counts[1] = kept ? ds.static_counts[1] : 0;
+            ds.flood_counts[2] = kept ? ds.static_counts[2] : (on && !ds.flood_reuse ? 0 : 1);
             ds.flood_counts[3] = 0;
+            if (on && !ds.flood_reuse) ds.flood_counts[kKeptTag] = 0;  // its flood overwrites the kept part
         }
     }
 }
@@ -815,9 +846,12 @@ __device__ __forceinline__ void tiles_fill(const DevScene &ds, int i0, int strid
     }
 }
 
-__global__ void __launch_bounds__(1024) k_tiles_scan(DevScene ds, int to_static) { tiles_scan_block(ds, to_static); }
+__global__ void __launch_bounds__(1024) k_tiles_scan(DevScene ds, int to_static, int unless) {
+    if (!kept_already(ds, unless)) tiles_scan_block(ds, to_static);
+}
 
-__global__ void k_tiles_fill(DevScene ds, int to_static) {
+__global__ void k_tiles_fill(DevScene ds, int to_static, int unless) {
+    if (kept_already(ds, unless)) return;
     tiles_fill(ds, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, to_static);
 }
 
@@ -845,6 +879,58 @@ bool flood_possible(int tiles, int polys) {
     return flood_smem_bytes(tiles, polys, true) + sizeof(FloodSmem) <= 200 * 1024;
 }
 
+// Generators [g0, g1) walked by resident CTAs.
+static void flood_walk(const DevScene &ds, cudaStream_t st, int g0, int g1, int unless) {
+    if (g1 <= g0) return;
+    const bool maps = ds.use_maps && ds.gen_maps;
+    const size_t smem = flood_smem_bytes(ds.tiles_x * ds.tiles_y, ds.n_poly, maps);
+    int per_sm = 0, dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, maps ? k_flood<true> : k_flood<false>, kFloodThreads, smem);
+    const int blocks = max(1, min(max(sms, 1) * max(per_sm, 1), g1 - g0));
+    if (maps) k_flood<true><<<blocks, kFloodThreads, smem, st>>>(ds, g0, g1, unless);
+    else k_flood<false><<<blocks, kFloodThreads, smem, st>>>(ds, g0, g1, unless);
+}
+
+// The obstacle vertices' lists, kept for every later compute, up to their
+// counts and tag: kept_counts(keep) is what is left to do, with what this
+// returns. unless: kept_already's.
+static int flood_kept(const DevScene &scene, cudaStream_t st, int unless) {
+    DevScene ds = scene;
+    ds.vert_bits = flood_verts_direct(ds) ? 1 : 0;
+    const int ntiles = ds.tiles_x * ds.tiles_y;
+    const size_t clear = (size_t)ntiles * (ds.vert_bits ? ds.vert_words : 1);
+    k_kept_reset<<<(int)std::max<size_t>(1, std::min<size_t>((clear + 255) / 256, 152 * 8)), 256, 0, st>>>(ds, unless);
+    if (!ds.vert_bits) {
+        flood_walk(ds, st, ds.n_src, ds.n_gen, unless);
+        k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1, unless);
+        k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 1, unless);
+        return 1;
+    }
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int blocks = std::min(max(sms, 1) * 6, ds.n_vert);
+    if (ds.use_maps && ds.gen_maps) k_flood_direct<true><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen, unless);
+    else k_flood_direct<false><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen, unless);
+    if (ds.vert_words <= kBitsOnly) return 2;
+    k_bits_count<<<(ntiles + 7) / 8, 256, 0, st>>>(ds, unless);
+    k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1, unless);
+    k_bits_fill<<<(ntiles + 7) / 8, 256, 0, st>>>(ds, unless);
+    return 1;
+}
+
+int flood_kept_kernels(const DevScene &ds) {
+    const int build = !flood_verts_direct(ds) ? 3 + (ds.n_vert > 0) : ds.vert_words <= kBitsOnly ? 2 : 5;
+    return build + (flood_sources_direct(ds) ? 0 : 1);
+}
+
+void launch_flood_kept(const DevScene &ds, cudaStream_t st) {
+    const int tag = kept_tag(ds), keep = flood_kept(ds, st, tag);
+    k_flood_static<<<1, 32, 0, st>>>(ds, keep, tag);
+}
+
 void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
     const int ntiles = ds.tiles_x * ds.tiles_y;
     if (ds.flood_mode == 2) {  // never: the pixel pass scans every generator
@@ -853,47 +939,16 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
         return;
     }
     const bool maps = ds.use_maps && ds.gen_maps;
-    const size_t smem = flood_smem_bytes(ntiles, ds.n_poly, maps);
-    int per_sm = 0, dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, maps ? k_flood<true> : k_flood<false>, kFloodThreads, smem);
-    auto flood = [&](int g0, int g1) {
-        if (g1 <= g0) return;
-        const int blocks = max(1, min(max(sms, 1) * max(per_sm, 1), g1 - g0));  // resident CTAs only
-        if (maps) k_flood<true><<<blocks, kFloodThreads, smem, st>>>(ds, g0, g1);
-        else k_flood<false><<<blocks, kFloodThreads, smem, st>>>(ds, g0, g1);
-    };
     const int sblocks = max(1, min((ntiles + 255) / 256, 152));
     if (how == FloodStatic::kNone) {
         cudaMemsetAsync(ds.tile_count, 0, sizeof(int32_t) * ntiles, st);
-        cudaMemsetAsync(ds.flood_counts, 0, sizeof(int32_t) * 4, st);
-        flood(0, ds.n_gen);
+        cudaMemsetAsync(ds.flood_counts, 0, sizeof(int32_t) * kFloodCounts, st);  // the tag too: the kept part goes
+        flood_walk(ds, st, 0, ds.n_gen, 0);
     } else {
-        int keep = 0;
-        if (how == FloodStatic::kBuild) {  // the obstacle vertices' lists, kept for every later compute
-            keep = 1;
-            cudaMemsetAsync(ds.flood_counts, 0, sizeof(int32_t) * 4, st);
-            if (flood_verts_direct(ds)) {
-                cudaMemsetAsync(ds.vert_mask, 0, sizeof(uint32_t) * (size_t)ntiles * ds.vert_words, st);
-                const int blocks = std::min(max(sms, 1) * 6, ds.n_vert);
-                if (maps) k_flood_direct<true><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen);
-                else k_flood_direct<false><<<blocks, kFloodThreads, 0, st>>>(ds, ds.n_src, ds.n_gen);
-                if (ds.vert_words <= kBitsOnly) keep = 2;
-                else {
-                    k_bits_count<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
-                    k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
-                    k_bits_fill<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
-                }
-            } else {
-                cudaMemsetAsync(ds.tile_count, 0, sizeof(int32_t) * ntiles, st);
-                flood(ds.n_src, ds.n_gen);
-                k_tiles_scan<<<1, 1024, 0, st>>>(ds, 1);
-                k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 1);
-            }
-        }
+        const int unless = how == FloodStatic::kEnsure ? kept_tag(ds) : 0;
+        const int keep = how == FloodStatic::kReuse ? 0 : flood_kept(ds, st, unless);
         if (flood_sources_direct(ds)) {  // a bit per source and tile: nothing to sort
-            k_src_prep<<<std::min((ds.n_src * kAng + 255) / 256, 152 * 8), 256, 0, st>>>(ds, keep);
+            k_src_prep<<<std::min((ds.n_src * kAng + 255) / 256, 152 * 8), 256, 0, st>>>(ds, keep, unless);
             // ordinary launches: a dependent one would hold SMs, waiting, that
             // the vertex phase beside it needs
             const dim3 grid((ds.n_edge + 4 * kSrcEdges - 1) / (4 * kSrcEdges), std::min(ds.n_src, 65535));
@@ -902,12 +957,12 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
             k_src_tiles<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
             return;
         }
-        if (keep) k_flood_static<<<sblocks, 256, 0, st>>>(ds, keep);
-        k_flood_static<<<sblocks, 256, 0, st>>>(ds, 0);
-        flood(0, ds.n_src);
+        if (keep) k_flood_static<<<1, 32, 0, st>>>(ds, keep, unless);
+        k_flood_static<<<sblocks, 256, 0, st>>>(ds, 0, 0);
+        flood_walk(ds, st, 0, ds.n_src, 0);
     }
-    k_tiles_scan<<<1, 1024, 0, st>>>(ds, 0);
-    k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 0);
+    k_tiles_scan<<<1, 1024, 0, st>>>(ds, 0, 0);
+    k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 0, 0);
 }
 
 bool flood_sources_direct(const DevScene &ds) {

@@ -191,7 +191,10 @@ struct DevScene {
     uint8_t *gen_map_ok;
     int32_t pair_cap;
     int32_t *glob_list;                // generators every tile scans
-    int32_t *flood_counts;             // [0] pairs, [1] global list size, [2] overflow, [3] work counter
+    // [0] pairs, [1] global list size, [2] overflow, [3] work counter,
+    // [kKeptTag] the tile size and map setting the kept part below was built
+    // for (0: none, or overwritten since)
+    int32_t *flood_counts;
     // the geometric flood (mode 3) of the obstacle-vertex generators depends
     // on the obstacles alone: its per-tile lists are kept here (CSR), with
     // its global entries at the front of `glob_list`, its depth maps in
@@ -281,9 +284,14 @@ void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_
 // flood of the per-tile candidate lists. FloodStatic::kNone floods every
 // generator; kBuild (geometric mode) floods the obstacle vertices, keeps
 // their lists as the static part, then floods the sources; kReuse restores
-// the static part and floods the sources only.
-enum class FloodStatic { kNone, kBuild, kReuse };
+// the static part and floods the sources only; kEnsure is one or the other, by
+// what the device holds when it runs (the host does not know when a recorded
+// compute does).
+enum class FloodStatic { kNone, kBuild, kReuse, kEnsure };
+constexpr int kKeptTag = 4, kFloodCounts = 5;
 void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how = FloodStatic::kNone);
+void launch_flood_kept(const DevScene &ds, cudaStream_t st);  // kEnsure's static part alone
+int flood_kept_kernels(const DevScene &ds);  // kernels kEnsure launches beside kReuse's
 // visibility bits of the obstacle-vertex pairs into ds.vis_static (once per scene)
 void launch_vis_static(const DevScene &ds, cudaStream_t st, uint32_t *vis_static);
 // free-space mask of the pixel centres (once per scene)

@@ -1324,3 +1324,81 @@ def test_vertex_pairs_past_edges_in_line(spm, oracle_mod):
         o = oracle_mod.Oracle(scene)
         used = o.cside != oracle_mod.CONE_EMPTY
         assert np.array_equal(cost[used], o.cost[used]) and np.array_equal(par[used], o.parent[used]), seed
+
+
+def _scan(spm, scene, points=None):
+    """(dist, parent) of a scan of every generator, by a scene of its own."""
+    s = spm.Scene(scene)
+    if points is not None:
+        s.update_sources(points, np.asarray(scene.segs, np.float32).reshape(-1, 4))
+    spm.spm_scene_set_tuning(s.handle, 2, 32, 32, 0)
+    out = s.compute()
+    s.sync()
+    return out
+
+
+def _same(got, want, what):
+    assert torch.equal(got[1], want[1]), f"{what}: parents differ"
+    assert torch.equal(got[0].view(torch.int32), want[0].view(torch.int32)), f"{what}: distances differ"
+
+
+def _bars():
+    """Bars across the world, open at alternate ends: a corridor's tiles see few of the vertices."""
+    bars = [np.array([(x, y), (x + 330, y), (x + 330, y + 6), (x, y + 6)])
+            for x, y in ((60 if k % 2 else 10, 30 * k + 20) for k in range(12))]
+    return sg.Scene((400, 400), (100, 100), bars, [(200.0, 5.0)], np.zeros((0, 4)))
+
+
+@pytest.mark.parametrize("which", ["bars", "polys", "maze"])
+@pytest.mark.parametrize("mode,maps", [(3, 1), (3, 0), (1, 1)])
+@pytest.mark.parametrize("warm", [True, False])
+def test_graphs_and_later_tuning(spm, which, mode, maps, warm):
+    """A compute recorded into a graph, before or after the scene's first
+    compute, replayed after the scene was computed with other tiles, other maps
+    or another kind of flood and its sources moved; the same for a batch
+    recorded by its caller; and computes and batches after those replays."""
+    scene = _bars() if which == "bars" else _route_scene(which)
+    s, other = spm.Scene(scene), spm.Scene(_route_scene("rects"))
+    t0 = s.tuning()
+    tile = 48 - t0["tile"]
+
+    def tune(m, t, mp):
+        spm.spm_scene_set_tuning(s.handle, m, 32, t, mp)
+    if warm:
+        s.compute()
+        s.sync()
+    st, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    graphed = s.empty_outputs()
+    with torch.cuda.graph(g, stream=st):
+        spm.spm_compute(s.handle, st, *graphed)
+    batch, gb = spm.Batch([s, other]), torch.cuda.CUDAGraph()
+    if warm:
+        batch.compute()
+        torch.cuda.synchronize()
+    with torch.cuda.graph(gb, stream=st):
+        batch.compute(st)
+    pts = np.asarray(scene.points, np.float32).reshape(-1, 2)
+    here = _scan(spm, scene)
+    moved = (pts + np.float32([1.0, -1.0])).astype(np.float32)
+    there = _scan(spm, scene, moved)
+    segs = np.asarray(scene.segs, np.float32).reshape(-1, 4)
+    for k in range(2):
+        tune(mode, tile, maps)
+        _same(s.compute(), here, "retuned")
+        s.sync()
+        s.update_sources(moved, segs)
+        gb.replay()
+        torch.cuda.synchronize()
+        _same(batch.outputs[0], there, "recorded batch")
+        g.replay()
+        torch.cuda.synchronize()
+        _same(graphed, there, "graph")
+        _same(s.compute(), there, "retuned, after the replays")
+        s.sync()
+        batch.compute()
+        torch.cuda.synchronize()
+        _same(batch.outputs[0], there, "batch")
+        tune(t0["flood_mode"], t0["tile"], t0["maps"])
+        _same(s.compute(), there, "first tuning")
+        s.sync()
+        s.update_sources(pts, segs)
