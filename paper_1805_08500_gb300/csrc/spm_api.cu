@@ -60,6 +60,9 @@ struct spm_scene {
     // the device holds sources moved by spm_scene_update_sources_device that
     // the host copy in hs has not seen yet
     bool host_src_stale = false;
+    // the stream of that update; unordered: there were several, or a graph holds it
+    cudaStream_t src_stream = nullptr;
+    bool src_unordered = false;
     bool alloc_failed = false;  // some device allocation of this scene failed
     int seq_blocks = 0;  // co-resident CTAs of the sequential kernel
     // the static part of the geometric flood (obstacle vertices) is on the
@@ -649,6 +652,11 @@ spm_status spm_scene_update_sources_device(spm_scene *s, void *stream, const flo
     if ((np > 0 && !pts_dev) || (ns > 0 && !segs_dev)) return set_err(s, SPM_ERR_INVALID_ARG, "null source array");
     spm::launch_update_sources(s->ds, static_cast<cudaStream_t>(stream), pts_dev, segs_dev);
     if (cudaPeekAtLastError() != cudaSuccess) return set_err(s, SPM_ERR_CUDA, "source update launch failed");
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap);
+    s->src_unordered = cap != cudaStreamCaptureStatusNone ||
+                       (s->host_src_stale && (s->src_unordered || s->src_stream != stream));
+    s->src_stream = static_cast<cudaStream_t>(stream);
     s->host_src_stale = true;
     return SPM_OK;
 }
@@ -1288,6 +1296,12 @@ spm_status spm_extract_path(spm_scene *s, float x, float y, float *out_xy, int32
         return set_err(s, SPM_ERR_CUDA, "query copy failed");
     }
     std::lock_guard<std::mutex> hold(s->path_lock);  // one page-locked buffer a scene
+    // the kernel below reads the sources: a move that is not in its stream is
+    // waited for (once: the host copy is then up to date)
+    if (s->host_src_stale && (s->src_unordered || s->src_stream != s->last_stream)) {
+        st = refresh_host_sources(s);
+        if (st != SPM_OK) return st;
+    }
     // a chain visits no generator twice (the walk stops after n_gen + 2)
     const int room = std::min(cap - 1, s->hs.n_gen + 2);
     const size_t bytes = sizeof(spm::PathOut) + sizeof(float2) * (size_t)room;

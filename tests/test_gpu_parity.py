@@ -1402,3 +1402,30 @@ def test_graphs_and_later_tuning(spm, which, mode, maps, warm):
         _same(s.compute(), there, "first tuning")
         s.sync()
         s.update_sources(pts, segs)
+
+
+def test_path_after_a_source_move_on_another_stream(spm):
+    """A path asked for while a device-side source move is still on its way on
+    another stream shows the moved source: it waits for the move."""
+    scene = sg.plain_polys(7, n_polys=80, N=256, n_segs=0, n_points=1)
+    s = spm.Scene(scene)
+    s.compute()
+    s.sync()
+    pts = torch.tensor(scene.points, dtype=torch.float32, device="cuda")
+    moved = pts + 2.0
+    other = torch.cuda.Stream()
+    torch.cuda._sleep(1000)
+    torch.cuda.synchronize()
+    h = scene.world[0] / scene.grid[0]
+    d, p = s.compute()
+    s.sync()
+    j, i = torch.nonzero(p >= 0)[0].tolist()
+    s.update_sources_device(pts, None)
+    s.extract_path((i + 0.5) * h, (j + 0.5) * h)  # its buffer allocated, the kernels loaded
+    torch.cuda.synchronize()
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(100_000_000)  # some 50 ms
+        s.update_sources_device(moved, None, stream=other)
+    path = s.extract_path((i + 0.5) * h, (j + 0.5) * h)
+    s.sync()
+    assert np.allclose(path[-1], moved[0].cpu().numpy()), (path[-1], moved)
