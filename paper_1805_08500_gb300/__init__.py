@@ -146,10 +146,13 @@ def _stream_handle(stream):
     if stream is None:
         try:
             import torch
-            # the handle alone: a Stream object costs 3 us a call
-            return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
-        except Exception:  # pragma: no cover - torch missing
+            device = torch.cuda.current_device()
+        except Exception:  # no torch or no device: the library call says so itself
             return None
+        # the handle alone: a Stream object costs 3 us a call; never another
+        # stream than torch's current one, where the private call is missing
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return raw(device) if raw is not None else torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -93,6 +93,21 @@ def test_null_scene_and_arguments_are_rejected(spm):
     assert lib.spm_query_exact(None, 1.0, 1.0, None, None) == spm.SPM_ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("private", [True, False])
+def test_current_stream_handle(spm, monkeypatch, private):
+    """Without a stream, torch's current one, also on a torch build whose
+    private shortcut to its handle is missing."""
+    class Current:
+        cuda_stream = 1234
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: Current)
+    if private:
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda d: 1234, raising=False)
+    else:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert spm._stream_handle(None) == 1234
+
+
 def test_device_source_update_wants_cuda_float32(spm):
     """The binding refuses host or non-float32 tensors for the device-side
     source update before calling the library."""
