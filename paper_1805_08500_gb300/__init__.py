@@ -444,6 +444,7 @@ class Scene:
         self.device = torch.device("cuda", torch.cuda.current_device())
         self.handle = spm_scene_create(scene)
         self.grid = (int(scene.grid[0]), int(scene.grid[1]))
+        self.source_numel = (int(np.size(scene.points)), int(np.size(scene.segs)))
 
     def close(self):
         if getattr(self, "handle", None):
@@ -582,10 +583,12 @@ def _make_autograd():
         @staticmethod
         def backward(ctx, grad_out):
             scene = ctx.scene
-            # both gradients in one buffer, every entry of it written by the kernel:
-            # one multiplication by grad_out, none to clear
+            # both gradients in one buffer, the scene's sources' entries written by
+            # the kernel: one multiplication by grad_out, and none to clear unless
+            # the tensors have rows beyond those sources (their gradient is zero)
             n_p, n_s = (math.prod(x) for x in ctx.shapes)
-            both = torch.empty(n_p + n_s, dtype=torch.float32, device=scene.device)
+            new = torch.empty if (n_p, n_s) == scene.source_numel else torch.zeros
+            both = new(n_p + n_s, dtype=torch.float32, device=scene.device)
             spm_agents_backward(scene.handle, None, ctx.tape, ctx.n, both[:n_p] if n_p else None,
                                 both[n_p:] if n_s else None)
             both = both * grad_out.to(scene.device)

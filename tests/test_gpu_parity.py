@@ -1429,3 +1429,23 @@ def test_path_after_a_source_move_on_another_stream(spm):
     path = s.extract_path((i + 0.5) * h, (j + 0.5) * h)
     s.sync()
     assert np.allclose(path[-1], moved[0].cpu().numpy()), (path[-1], moved)
+
+
+def test_loss_gradient_of_rows_beyond_the_sources(spm):
+    """Tensors with more rows than the scene has sources: the rows beyond them
+    take no part in the map and get no gradient."""
+    scene = sg.differentiable(5, W=1024, N=256, n_polys=15, n_agents=2000)
+    s = spm.Scene(scene)
+    agents = torch.tensor(scene.agents, device="cuda")
+
+    def grads(extra):
+        p = np.concatenate([scene.points, np.full((extra, 2), 7.0)]).astype(np.float32)
+        q = np.concatenate([scene.segs, np.full((extra, 4), 7.0)]).astype(np.float32)
+        p, q = (torch.tensor(v, device="cuda", requires_grad=True) for v in (p, q))
+        loss = spm.agent_loss(s, p, q, agents)
+        held = [torch.full((n,), float("nan"), device="cuda") for n in (16, 32, 64, 128) for _ in range(8)]
+        del held  # memory that an uncleared buffer would show
+        return torch.autograd.grad(loss, (p, q))
+    want, got = grads(0), grads(3)
+    for w, g in zip(want, got):
+        assert torch.equal(g[:len(w)], w) and (g[len(w):] == 0).all(), g
