@@ -388,7 +388,8 @@ const char *spm_last_error(const spm_scene *scene);
  * next device allocation of the library fails (n = 0: the next one), as if
  * the device were out of memory; n < 0 switches it off (the default). The
  * call that meets the failure returns SPM_ERR_OOM and frees what it had
- * allocated. Process-wide; has no effect unless called. */
+ * allocated, unless only a faster route needs that memory: the scene is then
+ * created without the route. Process-wide; has no effect unless called. */
 void spm_debug_fail_alloc_after(int32_t n);
 
 /* Test hook for the fixpoint's failure path (no counterpart in the paper):

@@ -101,12 +101,14 @@ struct NvtxRange {
     ~NvtxRange() { nvtxRangePop(); }
 };
 
+// optional: a buffer that only a faster route needs; without it the scene takes
+// another
 template <class T>
-T *dalloc(spm_scene *s, size_t n) {
+T *dalloc(spm_scene *s, size_t n, bool optional = false) {
     for (int k = g_fail_alloc_after.load(); k >= 0; k = g_fail_alloc_after.load())
         if (g_fail_alloc_after.compare_exchange_weak(k, k - 1)) {
             if (k == 0) {
-                s->alloc_failed = true;
+                s->alloc_failed |= !optional;
                 return nullptr;
             }
             break;
@@ -126,7 +128,7 @@ T *dalloc(spm_scene *s, size_t n) {
     void *p = nullptr;
     if (cudaMalloc(&p, small ? kChunk : bytes) != cudaSuccess) {
         cudaGetLastError();  // not sticky: clear it, the caller reports SPM_ERR_OOM
-        s->alloc_failed = true;
+        s->alloc_failed |= !optional;
         return nullptr;
     }
     s->allocs.push_back(p);
@@ -233,6 +235,32 @@ spm::DevScene effective(const spm_scene *s) {
         if (spm::flood_verts_direct(wide) && side * side * d.n_poly <= 0.4 * (double)d.Wx * (double)d.Wy) return wide;
     }
     return d;
+}
+
+// Buffers of the direct culling, after every other one: only where a tile size
+// is within its bounds (100000 sources on 4096^2 would take 0.8 GB of bits that
+// nothing reads), and no scene is refused for want of them.
+void alloc_direct_culling(spm_scene *s) {
+    spm::DevScene &ds = s->ds;
+    if (!ds.use_flood || !ds.static_tile_start) return;
+    spm::DevScene at[2] = {ds, ds};
+    set_tile(at[0], spm::kTileSmall);
+    set_tile(at[1], spm::kTile);
+    auto tiles = [](const spm::DevScene &d) { return (size_t)d.tiles_x * d.tiles_y; };
+    size_t src = 0, vert = 0, cull = 0;
+    for (const spm::DevScene &d : at) {
+        if (spm::flood_sources_fit(d)) src = std::max(src, tiles(d) * d.src_words);
+        if (!spm::flood_verts_fit(d)) continue;
+        vert = std::max(vert, tiles(d) * d.vert_words);
+        cull = std::max(cull, tiles(d) * spm::cull_cap(d.tile));
+    }
+    if (src) ds.src_mask = dalloc<uint32_t>(s, src, true);
+    if (vert && tiles(at[0]) * ds.vert_words <= ((size_t)64 << 20)) ds.vert_mask = dalloc<uint32_t>(s, vert, true);
+    if (ds.vert_mask && ds.open_scene) {
+        ds.cull_items = dalloc<int32_t>(s, cull, true);
+        ds.cull_count = dalloc<int32_t>(s, tiles(at[0]), true);
+        if (!ds.cull_count) ds.cull_items = nullptr;
+    }
 }
 
 spm_status upload_sources(spm_scene *s) {
@@ -452,7 +480,7 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
         ds.static_lists = 0;
         ds.src_direct = 0;
         ds.src_words = (hs.n_src + 31) / 32;
-        ds.src_mask = ds.use_flood ? dalloc<uint32_t>(s, (size_t)ntiles * ds.src_words) : nullptr;
+        ds.src_mask = nullptr;
     }
     ds.free_words = (hs.Nx + 31) / 32;
     uint32_t *free_bits = dalloc<uint32_t>(s, (size_t)hs.Ny * ds.free_words);
@@ -539,19 +567,9 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
     }
     ds.cull_items = nullptr;
     ds.cull_count = nullptr;
-    auto tiles = [&](int t) { return (size_t)((hs.Nx + t - 1) / t) * ((hs.Ny + t - 1) / t); };
     ds.vert_mask = nullptr;
     ds.vert_words = (hs.n_vert + 31) / 32;
     ds.vert_bits = 0;
-    const size_t mask_words = tiles(spm::kTileSmall) * ds.vert_words;
-    if (hs.n_vert > 0 && ds.static_tile_start && mask_words <= ((size_t)64 << 20) &&
-        (ds.open_scene || ds.n_edge + tiles(spm::kTile) <= 1024))
-        ds.vert_mask = dalloc<uint32_t>(s, mask_words);
-    if (ds.open_scene && ds.static_tile_start) {
-        ds.cull_items = dalloc<int32_t>(s, std::max(tiles(spm::kTileSmall) * spm::cull_cap(spm::kTileSmall),
-                                                    tiles(spm::kTile) * spm::cull_cap(spm::kTile)));
-        ds.cull_count = dalloc<int32_t>(s, tiles(spm::kTileSmall));
-    }
     if (!ok || s->alloc_failed) {
         free_all(s);
         delete s;
@@ -593,6 +611,7 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
         delete s;
         return set_err(nullptr, SPM_ERR_CUDA, "scene preparation kernels failed to launch");
     }
+    alloc_direct_culling(s);
     for (cudaEvent_t &e : s->ev)
         if (cudaEventCreate(&e) != cudaSuccess) ok = false;
     if (cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) != cudaSuccess ||

@@ -965,18 +965,20 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
     k_tiles_fill<<<152 * 4, 256, 0, st>>>(ds, 0, 0);
 }
 
-bool flood_sources_direct(const DevScene &ds) {
+bool flood_sources_fit(const DevScene &ds) {
     const long long ntiles = (long long)ds.tiles_x * ds.tiles_y;
     return ds.gen_maps && ds.n_src > 0 && (long long)ds.n_src * (ds.n_poly + ntiles) <= (1LL << 24);
 }
+bool flood_sources_direct(const DevScene &ds) { return ds.src_mask && flood_sources_fit(ds); }
 
 // The obstacle vertices without the walk: in open scenes, where a vertex sees
 // many others (mazes: 3 tangent edges a vertex, polygon scenes: 8 to 45), and
 // while a generator's edges and tiles stay a few thousand.
-bool flood_verts_direct(const DevScene &ds) {
+bool flood_verts_fit(const DevScene &ds) {
     const long long ntiles = (long long)ds.tiles_x * ds.tiles_y;
-    return ds.vert_mask && (ds.open_scene || ds.n_edge + ntiles <= 1024) && ds.n_edge + ntiles <= (1 << 17);
+    return ds.n_vert > 0 && (ds.open_scene || ds.n_edge + ntiles <= 1024) && ds.n_edge + ntiles <= (1 << 17);
 }
+bool flood_verts_direct(const DevScene &ds) { return ds.vert_mask && flood_verts_fit(ds); }
 
 int src_edge_warps(int n_edge) { return (n_edge + kSrcEdges - 1) / kSrcEdges; }
 

@@ -330,6 +330,9 @@ int flood_smem_attr();
 // tile tested at once) rather than by the per-generator walk
 bool flood_sources_direct(const DevScene &ds);
 bool flood_verts_direct(const DevScene &ds);  // the same for the obstacle vertices, once per scene
+// their bounds alone, at the descriptor's tile size (the buffers are allocated where these hold)
+bool flood_sources_fit(const DevScene &ds);
+bool flood_verts_fit(const DevScene &ds);
 int src_edge_warps(int n_edge);  // warps that put a scene's edges into one source's map
 int sssp_grid_blocks();  // co-resident CTAs for the cooperative fixpoint kernel
 int solo_smem_bytes();   // shared memory granted to the single-CTA fixpoint kernel (0 if refused)

@@ -1449,3 +1449,57 @@ def test_loss_gradient_of_rows_beyond_the_sources(spm):
     want, got = grads(0), grads(3)
     for w, g in zip(want, got):
         assert torch.equal(g[:len(w)], w) and (g[len(w):] == 0).all(), g
+
+
+@pytest.mark.parametrize("which,limit", [("many_sources", 200), ("large_grid", 350)])
+def test_scene_takes_no_memory_for_routes_it_cannot_take(spm, which, limit):
+    """Scenes past the bounds of the direct culling (so many sources, or so
+    many tiles) allocate nothing for it (MB in all)."""
+    square = [np.array([(40, 40), (60, 40), (60, 60), (40, 60)])]
+    if which == "many_sources":
+        x, y = np.meshgrid(np.arange(200), np.arange(200))
+        pts = np.stack([100 + 70 * x, 100 + 70 * y], -1).reshape(-1, 2).astype(np.float64)
+        scene = sg.Scene((16384, 16384), (4096, 4096), square, pts, np.zeros((0, 4)))
+    else:
+        scene = sg.Scene((32764, 32764), (16382, 16382), sg.tiny(1, W=32764, N=16382, n_polys=60, r=(60.0, 400.0), k=(4, 8)).polys,
+                         [(5.0, 5.0)], np.zeros((0, 4)))
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    s = spm.Scene(scene)
+    took = (before - torch.cuda.mem_get_info()[0]) / 2**20
+    s.close()
+    assert took <= limit, took
+
+
+def test_scene_without_the_memory_of_its_faster_routes(spm):
+    """An allocation that fails at creation is SPM_ERR_OOM, unless only a
+    faster route needs it: the scene then does without, with the same map."""
+    scene = sg.plain_polys(6, W=2048, N=256, n_polys=30, n_segs=1)
+    lib = spm.load_library()
+    ref = spm.Scene(scene)
+    want, kernels = ref.compute(), ref.info()["kernels_per_compute"]
+    ref.sync()
+    without = 0
+    try:
+        for k in range(100):
+            lib.spm_debug_fail_alloc_after(k)
+            try:
+                s = spm.Scene(scene)
+            except spm.SpmError as e:
+                assert e.status == spm.SPM_ERR_OOM, (k, str(e))
+                continue
+            finally:
+                lib.spm_debug_fail_alloc_after(-1)
+            without += s.info()["kernels_per_compute"] != kernels
+            for mode in (0, 3, 1):
+                spm.spm_scene_set_tuning(s.handle, mode, 32, 16, 1)
+                d, p = s.compute()
+                s.sync()
+                assert torch.equal(p, want[1]) and torch.equal(d.view(torch.int32), want[0].view(torch.int32)), (k, mode)
+            b = spm.Batch([s, ref])
+            b.compute()
+            torch.cuda.synchronize()
+            assert torch.equal(b.outputs[0][1], want[1]), k
+    finally:
+        lib.spm_debug_fail_alloc_after(-1)
+    assert without == 4, without  # the sources' bits, the vertices' bits, the tiles' culled lists and their counts
