@@ -131,8 +131,8 @@ spm_status spm_compute(spm_scene *scene, void *stream, float *dist_dev,
  * counterpart in the paper; each GPU computes its own slab, and no data is
  * exchanged). Runs the whole vertex phase and culling, then the pixel pass
  * for grid rows [row0, row1) only: row0 and row1 must be multiples of the
- * scene's tile size (spm_scene_info()[7]) or row1 == grid_h, else
- * SPM_ERR_INVALID_ARG. dist_dev / parent_dev are the full-grid buffers of
+ * scene's tile size (spm_scene_info()[7], or the smaller one that was set) or
+ * row1 == grid_h, else SPM_ERR_INVALID_ARG. dist_dev / parent_dev are the full-grid buffers of
  * spm_compute; only the slab's rows are written, with the values
  * spm_compute writes there. Queries (spm_query_parent, spm_extract_path)
  * need a whole-grid spm_compute. Asynchronous; allocates nothing. */
@@ -252,9 +252,9 @@ spm_status spm_scene_generators(spm_scene *scene, int32_t *kind, int32_t *lattic
  * segment), [2] obstacle-vertex generators, [3] lattice scale S, [4]
  * polygons, [5] vertex-phase rounds of the last compute (after sync), [6]
  * visibility-graph edges of the last compute (after sync), [7] tile size in
- * pixels, [8] 1 if the last compute used flooded per-tile candidate lists
- * (after sync), [9] flood_mode, [10] kernels one spm_compute launches with
- * the current settings. */
+ * pixels that a compute runs with (see spm_tuning), [8] 1 if the last compute
+ * used flooded per-tile candidate lists (after sync), [9] flood_mode as set,
+ * [10] kernels one spm_compute launches with the current settings. */
 spm_status spm_scene_info(spm_scene *scene, int64_t *info);
 
 /* Differentiable form. Forward: loss = mean over n agents (pixel indices,
@@ -338,7 +338,11 @@ spm_status spm_scene_phase_ms(spm_scene *scene, float *vertex_ms, float *cull_ms
  * hidden_chunk: 32..256, checked and reported; the pixel pass takes its
  *   candidates one by one in order of their lower bounds, so it has no effect.
  * tile: side of the tiles that carry the candidate lists, 16 or 32 pixels
- *   (default 16 when a pixel spans 8 world units or more, else 32).
+ *   (default 16 when a pixel spans 8 world units or more, else 32). Mode 3
+ *   (and 0 where it takes mode 3) runs 16 as 32 in open scenes, where an
+ *   obstacle vertex sees eight others or more on average, unless tiles of 32
+ *   pixels span the obstacles' spacing; spm_scene_info reports what runs, and
+ *   spm_compute_rows goes by the size that was set.
  * maps: 1 = the flood keeps each point generator's angular depth map and the
  *   pixel pass decides most pixels' visibility from it (exact bounds; only
  *   the undecided pixels take the exact polygon test), 0 = every pixel takes
@@ -371,7 +375,8 @@ spm_status spm_scene_set_tuning(spm_scene *scene, const spm_tuning *tuning);
 
 /* Autotuner: times spm_compute on this scene (device events on `stream`,
  * warm-up then the median of 3 runs) for every flood_mode x tile x maps
- * combination in {1, 2, 3} x {16, 32} x {0, 1} (maps only with a flood), keeps
+ * combination in {1, 2, 3} x {16, 32} x {0, 1} (maps only with a flood; no
+ * tile that would run as the other one), keeps
  * the fastest and writes it to *chosen (may be NULL). Synchronous. Allocates the scene's
  * output staging planes on first use; call it at set-up, not inside a
  * captured stream. */

@@ -1388,10 +1388,10 @@ spm_status spm_scene_info(spm_scene *s, int64_t *info) {
     info[4] = (int64_t)s->hs.poly_off.size() - 1;
     info[5] = stats[0];
     info[6] = stats[1];
-    info[7] = s->ds.tile;
     info[8] = (s->ds.use_flood && fc[2] == 0) ? 1 : 0;
     info[9] = s->ds.flood_mode;
     const spm::DevScene run = effective(s);
+    info[7] = run.tile;
     const bool floods = run.use_flood && run.flood_mode != 2;
     // the geometric mode over kept obstacle-vertex lists: the sources' culling
     // (list reset, the walk and the list scan and fill, or maps from every
@@ -1462,6 +1462,7 @@ spm_status spm_scene_autotune(spm_scene *s, void *stream, spm_tuning *chosen) {
         s->ds.flood_mode = modes[mi];
         s->ds.use_maps = ui;
         set_tile(s->ds, tiles[ti]);
+        if (effective(s).tile != tiles[ti]) continue;  // the other size would run
         float t[3];
         st = spm_compute(s, stream, s->stage_dist, s->stage_par);  // warm-up
         for (int k = 0; k < 3 && st == SPM_OK; ++k) {

@@ -1503,3 +1503,25 @@ def test_scene_without_the_memory_of_its_faster_routes(spm):
     finally:
         lib.spm_debug_fail_alloc_after(-1)
     assert without == 4, without  # the sources' bits, the vertices' bits, the tiles' culled lists and their counts
+
+
+def test_reported_tile_is_the_one_that_runs(spm):
+    """An open scene runs its geometric flood on 32-pixel tiles where 16 was
+    set: info reports what runs, row slabs go by either, and the autotuner does
+    not choose a size that would not run."""
+    scene = sg.plain_polys(4, n_polys=60, N=512)
+    s = spm.Scene(scene)
+    spm.spm_scene_set_tuning(s.handle, 3, 32, 16, 1)
+    assert s.info()["tile"] == 32 and s.tuning()["tile"] == 16
+    full = s.compute()
+    s.sync()
+    for side in (16, 32):
+        d, p = torch.full_like(full[0], float("nan")), torch.full_like(full[1], -7)
+        for r in range(0, 512, 3 * side):
+            s.compute_rows(r, min(r + 3 * side, 512), d, p)
+        s.sync()
+        assert torch.equal(p, full[1]) and torch.equal(d.view(torch.int32), full[0].view(torch.int32))
+    spm.spm_scene_set_tuning(s.handle, 1, 32, 16, 1)
+    assert s.info()["tile"] == 16  # the walk keeps the size that was set
+    t = s.autotune()
+    assert s.info()["tile"] == t["tile"] == s.tuning()["tile"]
