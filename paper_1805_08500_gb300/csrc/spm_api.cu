@@ -418,9 +418,6 @@ spm_status spm_scene_create(const spm_scene_desc *desc, spm_scene **out) {
     // source columns only
     uint32_t *vis_static = dalloc<uint32_t>(s, (size_t)hs.n_vert * ds.vis_words);
     ds.vis_static = vis_static;
-    ds.pair_words = (hs.n_src + 31) / 32;
-    ds.pair_u0 = 0;
-    ds.pair_u1 = hs.n_src;
     ds.in_start = dalloc<int32_t>(s, hs.n_vert + 1);
     ds.out_start = dalloc<int32_t>(s, hs.n_gen + 1);
     ds.out_fill = dalloc<int32_t>(s, hs.n_gen);

@@ -110,11 +110,8 @@ struct DevScene {
     uint32_t *vis_bits;                // n_vert rows x vis_words
     int32_t vis_words;
     // bits of the obstacle-vertex pairs alone, same layout (built once per
-    // scene: obstacles never move; null when every compute tests every pair)
+    // scene: obstacles never move; a compute tests the source columns only)
     const uint32_t *vis_static;
-    // the pair kernel's range: words 0..pair_words-1 of every row, generators
-    // u in [pair_u0, pair_u1) (with vis_static: the source columns only)
-    int32_t pair_words, pair_u0, pair_u1;
     int32_t *in_start;                 // n_vert + 1 (by target vertex)
     int32_t *in_src;                   // E
     double *in_len;                    // E

@@ -166,21 +166,7 @@ __device__ __forceinline__ bool loc_hidden(const DevScene &ds, int v, int2 vl, i
                                        __ldg(map + (b1 & (kLocBins - 1))));
 }
 
-// Exact visibility of a pair that passed the filter, one thread. The predicate
-// is symmetric in the two ends.
-__device__ __forceinline__ bool pair_visible(const DevScene &ds, int u, int v) {
-    const int2 vl = ds.gen_lat[v];
-    if (ds.gen_kind[u] == kSegI) {
-        const int s = ds.gen_aux[u];
-        const int4 L = ds.seg_lat[s];
-        const long long ux = L.z - L.x, uy = L.w - L.y;
-        return visible_foot(ds, s, vl.x, vl.y, (vl.x - L.x) * ux + (vl.y - L.y) * uy, ux * ux + uy * uy);
-    }
-    const int2 ul = ds.gen_lat[u];
-    return visible_points(ds, vl.x, vl.y, ul.x, ul.y);
-}
-
-// The same by one warp.
+// Exact visibility of a pair that passed the filter, by one warp.
 __device__ __forceinline__ bool pair_visible_warp(const DevScene &ds, int u, int v) {
     const int2 vl = ds.gen_lat[v], ul = ds.gen_lat[u];
     const bool seg = ds.gen_kind[u] == kSegI;
@@ -204,24 +190,24 @@ __device__ __forceinline__ bool pair_visible_warp(const DevScene &ds, int u, int
     });
 }
 
-// Sets the bit of edge u -> v (row v) and, between two obstacle vertices,
-// its mirror v -> u (row u). The matrix starts zeroed.
+// Sets the bit of edge u -> v (row v) between two obstacle vertices and its
+// mirror v -> u (row u). The matrix starts zeroed.
 __device__ __forceinline__ void set_edge_bits(const DevScene &ds, int u, int v) {
     atomicOr(&ds.vis_bits[(size_t)(v - ds.n_src) * ds.vis_words + (u >> 5)], 1u << (u & 31));
-    if (u >= ds.n_src) atomicOr(&ds.vis_bits[(size_t)(u - ds.n_src) * ds.vis_words + (v >> 5)], 1u << (v & 31));
+    atomicOr(&ds.vis_bits[(size_t)(u - ds.n_src) * ds.vis_words + (v >> 5)], 1u << (v & 31));
 }
 
-// Visibility pairs of one or many scenes. A warp task is row vv (vertex
-// index) of a scene's bit matrix and word w covering generators
+// Visibility pairs of a scene's obstacle vertices (once per scene). A warp task
+// is row vv (vertex index) of the bit matrix and word w covering generators
 // 32w..32w+31. A pair of obstacle vertices passes the filter and sees each
 // other symmetrically (both tangency tests and the blocking predicate are
 // symmetric in the two points), so only generators u < v are tested and an
-// edge between two vertices also sets its mirror bit. Pairs that pass the
+// edge also sets its mirror bit. Pairs that pass the
 // filter queue up per warp in shared memory and are walked 32 at a time, so
 // every lane walks (the filter passes a few lanes of each word).
 constexpr int kPairQ = 64;
 struct PairQ {
-    int3 e[kVisThreads / 32][kPairQ];  // (scene, u, v)
+    int2 e[kVisThreads / 32][kPairQ];  // (u, v)
 };
 
 // Warps take tasks `chunk` at a time, the first by their index, the rest
@@ -230,17 +216,17 @@ struct PairQ {
 // is a run of consecutive words of one row, so the row vertex's data and
 // local map stay in L1; the host sizes it so that every resident warp takes
 // about two chunks.
-template <class Scene, class Task>
-__device__ __forceinline__ void vis_pairs_run(PairQ &q, long long tasks, int chunk, unsigned long long *work,
-                                              Scene scene_of_task, Task task_of) {
+__global__ void __launch_bounds__(kVisThreads) k_vis_pairs(const __grid_constant__ DevScene ds, int chunk) {
+    __shared__ PairQ q;
+    const long long tasks = (long long)ds.n_vert * ds.vis_words;
+    unsigned long long *work = reinterpret_cast<unsigned long long *>(ds.stats + 2);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int qn = 0;  // warp-uniform queue length
     auto walk = [&](int n) {  // lanes < n walk the last n queued pairs
         if (lane < n) {
-            const int3 pr = q.e[warp][qn - n + lane];
-            const DevScene &ds = *scene_of_task(pr.x);
-            const bool vis = pair_visible(ds, pr.y, pr.z);
-            if (vis) set_edge_bits(ds, pr.y, pr.z);
+            const int2 pr = q.e[warp][qn - n + lane], ul = ds.gen_lat[pr.x], vl = ds.gen_lat[pr.y];
+            const bool vis = visible_points(ds, vl.x, vl.y, ul.x, ul.y);
+            if (vis) set_edge_bits(ds, pr.x, pr.y);
             SPM_CNT(13, 1);
             SPM_CNT(14, vis ? 1 : 0);
         }
@@ -268,38 +254,22 @@ __device__ __forceinline__ void vis_pairs_run(PairQ &q, long long tasks, int chu
             if (t >= tasks) break;
             t_end = min(t + chunk, tasks);
         }
-        const long long tt = t++;
-        int sc;
-        long long lt;
-        task_of(tt, sc, lt);
-        const DevScene &ds = *scene_of_task(sc);
-        const int vv = (int)(lt / ds.pair_words), w = (int)(lt % ds.pair_words);
+        const long long lt = t++;
+        const int vv = (int)(lt / ds.vis_words), w = (int)(lt % ds.vis_words);
         const int u = w * 32 + lane, v = ds.n_src + vv;
         if (w * 32 >= v) continue;  // the whole word lies at or above the diagonal (warp-uniform)
-        bool c = u < v && u >= ds.pair_u0 && u < ds.pair_u1 && pair_filter(ds, u, v);
-        if (c && ds.vert_maps && ds.gen_kind[u] != kSegI) {  // hidden by an obstacle near either end
+        bool c = u < v && u >= ds.n_src && pair_filter(ds, u, v);
+        if (c && ds.vert_maps) {  // hidden by an obstacle near either end
             const int2 ul = ds.gen_lat[u], vl = ds.gen_lat[v];
-            c = !loc_hidden(ds, v, vl, ul) && !(u >= ds.n_src && loc_hidden(ds, u, ul, vl));
+            c = !loc_hidden(ds, v, vl, ul) && !loc_hidden(ds, u, ul, vl);
         }
         const unsigned bal = __ballot_sync(0xffffffffu, c);
-        if (c) q.e[warp][qn + __popc(bal & ((1u << lane) - 1u))] = make_int3(sc, u, v);
+        if (c) q.e[warp][qn + __popc(bal & ((1u << lane) - 1u))] = make_int2(u, v);
         qn += __popc(bal);
         __syncwarp();
         if (qn >= 32) walk(32);
     }
     if (qn > 0) walk(qn);
-}
-
-__global__ void __launch_bounds__(kVisThreads) k_vis_pairs(const __grid_constant__ DevScene ds, int chunk) {
-    __shared__ PairQ q;
-    chain_start();
-    vis_pairs_run(
-        q, (long long)ds.n_vert * ds.pair_words, chunk, reinterpret_cast<unsigned long long *>(ds.stats + 2),
-        [&](int) { return &ds; },
-        [&](long long t, int &sc, long long &lt) {
-            sc = 0;
-            lt = t;
-        });
 }
 
 // The source columns of kRowsCta rows, by one CTA: a warp a row picks the
@@ -1393,9 +1363,9 @@ __global__ void k_prepare_b(const __grid_constant__ BatchDev b) {
         const int s = scene_of(b.vert_off, b.n, i);
         const DevScene &ds = b.scenes[s];
         uint32_t *row = ds.vis_bits + (size_t)(i - b.vert_off[s]) * ds.vis_words;
-        const uint32_t *srow = ds.vis_static ? ds.vis_static + (size_t)(i - b.vert_off[s]) * ds.vis_words : nullptr;
+        const uint32_t *srow = ds.vis_static + (size_t)(i - b.vert_off[s]) * ds.vis_words;
         const int nw = ds.st_start ? (ds.n_src + 31) / 32 : ds.vis_words;
-        for (int w = 0; w < nw; ++w) row[w] = srow && !ds.st_start ? srow[w] : 0u;
+        for (int w = 0; w < nw; ++w) row[w] = ds.st_start ? 0u : srow[w];
     }
     const int total = b.gen_off[b.n];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total + b.n; i += gridDim.x * blockDim.x) {
@@ -1600,12 +1570,9 @@ int fixpoint_round_cap(int n_gen) {
     return o > 0 ? o : 4 * n_gen + 64;
 }
 
-// Visibility-pair kernel over ds's pair range (resident CTAs, runs sized so
-// that every resident warp takes about two).
 // The start values of a compute's vertex phase, in one launch: out-degrees
 // (the kept obstacle vertices', or zero), fill cursors, the source columns of
-// the bit matrix (with kept edge lists), the pair kernel's work counter, the
-// cluster kernel's done flag and, for a warm start, the estimates (a huge
+// the bit matrix (with kept edge lists), the cluster kernel's done flag and, for a warm start, the estimates (a huge
 // value: none yet) and the count of unsatisfied vertices.
 __global__ void k_vertex_prep(const __grid_constant__ DevScene ds) {
     chain_start();
@@ -1618,7 +1585,6 @@ __global__ void k_vertex_prep(const __grid_constant__ DevScene ds) {
         if (i < n_bits) ds.vis_bits[(i / sw) * ds.vis_words + i % sw] = 0u;
         if (ds.warm && i < ds.n_vert) ds.warm_est[i] = __longlong_as_double(0x7f7f7f7f7f7f7f7fll);  // 1.4e306
         if (i == 0) {
-            *reinterpret_cast<unsigned long long *>(ds.stats + 2) = 0ull;  // the pair kernel's work counter
             ds.counters[4] = 0;
             ds.counters[6] = 0;
             if (ds.cl_lists) ds.stats[1] = 0;  // the edges, summed by the cluster's CTAs
@@ -1626,28 +1592,20 @@ __global__ void k_vertex_prep(const __grid_constant__ DevScene ds) {
     }
 }
 
-void launch_pairs(const DevScene &ds, cudaStream_t st, bool reset_counter = true) {
-    const long long tasks = (long long)ds.n_vert * ds.pair_words;
-    if (reset_counter) cudaMemsetAsync(ds.stats + 2, 0, sizeof(unsigned long long), st);  // the pair kernel's work counter
-    if (tasks == 0) return;
+// Resident CTAs, runs sized so that every resident warp takes about two.
+void launch_vis_static(const DevScene &ds, cudaStream_t st, uint32_t *vis_static) {
+    if (ds.n_vert == 0) return;
+    cudaMemsetAsync(vis_static, 0, sizeof(uint32_t) * (size_t)ds.n_vert * ds.vis_words, st);
+    cudaMemsetAsync(ds.stats + 2, 0, sizeof(unsigned long long), st);  // the pair kernel's work counter
+    DevScene d = ds;
+    d.vis_bits = vis_static;
+    const long long tasks = (long long)ds.n_vert * ds.vis_words;
     const int resident = vis_resident_blocks();
     long long blocks = (tasks + (kVisThreads / 32) - 1) / (kVisThreads / 32);  // a task per warp at least
     blocks = blocks > resident ? resident : blocks;
     const long long per_chunk = tasks / (blocks * (kVisThreads / 32) * 2);
     const int chunk = (int)(per_chunk < 1 ? 1 : (per_chunk > 32 ? 32 : per_chunk));
-    launch_chained(k_vis_pairs, dim3((int)blocks), dim3(kVisThreads), 0, st, ds, chunk);
-}
-
-void launch_vis_static(const DevScene &ds, cudaStream_t st, uint32_t *vis_static) {
-    if (ds.n_vert == 0) return;
-    cudaMemsetAsync(vis_static, 0, sizeof(uint32_t) * (size_t)ds.n_vert * ds.vis_words, st);
-    DevScene d = ds;  // every word of every row, obstacle-vertex columns only
-    d.vis_bits = vis_static;
-    d.vis_static = nullptr;
-    d.pair_words = ds.vis_words;
-    d.pair_u0 = ds.n_src;
-    d.pair_u1 = ds.n_gen;
-    launch_pairs(d, st);
+    k_vis_pairs<<<(int)blocks, kVisThreads, 0, st>>>(d, chunk);
 }
 
 
@@ -2162,7 +2120,7 @@ cudaError_t launch_vtab_build(const DevScene &ds, double *tab, int32_t *counter,
 // The cluster kernel builds its in-lists itself, with the launch bits `need`
 // (the device's choice of flood or scan reads the edge count: it keeps them).
 bool cluster_lists(const DevScene &ds, int fix, int need) {
-    return ds.st_start && ds.vis_static && (fix & need) == need && !(ds.use_flood && ds.flood_mode == 0);
+    return ds.st_start && (fix & need) == need && !(ds.use_flood && ds.flood_mode == 0);
 }
 
 void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *side) {
@@ -2186,17 +2144,14 @@ void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *
         k_vertex_prep<<<(int)std::max(1LL, std::min((items + 255) / 256, 152LL * 4)), 256, 0, st>>>(arg);
     }
     if (ds.n_vert > 0) {
-        const size_t bytes = sizeof(uint32_t) * (size_t)ds.n_vert * ds.vis_words;
         // the obstacle-vertex pairs come from the scene's static bits; the
         // pair kernel then tests the source columns only (with kept edge
         // lists only they are read: the prep kernel cleared them)
-        if (!ds.st_start) {
-            if (ds.vis_static) cudaMemcpyAsync(ds.vis_bits, ds.vis_static, bytes, cudaMemcpyDeviceToDevice, st);
-            else cudaMemsetAsync(ds.vis_bits, 0, bytes, st);
-        }
+        if (!ds.st_start)
+            cudaMemcpyAsync(ds.vis_bits, ds.vis_static, sizeof(uint32_t) * (size_t)ds.n_vert * ds.vis_words,
+                            cudaMemcpyDeviceToDevice, st);
         const int eb = (ds.n_vert + 7) / 8;  // one warp per row
-        if (ds.vis_static) launch_chained(k_src_pairs, dim3((ds.n_vert + kRowsCta - 1) / kRowsCta), dim3(kVisThreads), 0, st, ds);
-        else launch_pairs(ds, st, false);
+        launch_chained(k_src_pairs, dim3((ds.n_vert + kRowsCta - 1) / kRowsCta), dim3(kVisThreads), 0, st, ds);
         if (lists) {
         } else if (warm && side) {
             // the tree's estimates, parents and fold read the source columns
