@@ -65,13 +65,12 @@ struct spm_scene {
     bool src_unordered = false;
     bool alloc_failed = false;  // some device allocation of this scene failed
     int seq_blocks = 0;  // co-resident CTAs of the sequential kernel
-    // the static part of the geometric flood (obstacle vertices) is on the
-    // device for this tile size and depth-map setting
-    bool flood_static_ok = false;
-    int flood_static_tile = 0, flood_static_maps = 0;
-    // a graph holds work of this scene that writes it: what the device has is
-    // not known here any more, and computes go by the device's own tag
-    bool flood_recorded = false;
+    // the static part of the geometric flood (obstacle vertices) that the last
+    // work launched here left on the device (its tag, 0: none), and what graphs
+    // that hold work of this scene leave there when they are replayed (a bit a
+    // tag; bit 0: it is overwritten)
+    int flood_kept = 0;
+    unsigned flood_recorded = 0;
     // the warm start of the fixpoint: the rounds the table build's deepest
     // root took, whether that makes the warm start the default, and the
     // caller's choice (spm_tuning.fixpoint_start)
@@ -261,6 +260,12 @@ void alloc_direct_culling(spm_scene *s) {
         ds.cull_count = dalloc<int32_t>(s, tiles(at[0]), true);
         if (!ds.cull_count) ds.cull_items = nullptr;
     }
+}
+
+// The device holds descriptor d's static part, whatever was replayed since.
+// Where it is not sure, work of scenes in graphs checks on the device.
+bool flood_kept_sure(const spm_scene *s, const spm::DevScene &d) {
+    return s->flood_kept == spm::flood_kept_tag(d) && !(s->flood_recorded & ~(1u << s->flood_kept));
 }
 
 spm_status upload_sources(spm_scene *s) {
@@ -708,31 +713,30 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
         NvtxRange r("spm flood (side stream)");
         // the obstacle vertices' flood depends on the obstacles alone: built
         // once for this tile size and map setting, then only the sources flood
-        const bool maps = ds.use_maps && ds.gen_maps;
-        const bool reuse = s->flood_static_ok && s->flood_static_tile == ds.tile &&
-                           s->flood_static_maps == (int)maps && ds.static_tile_start;
-        // recorded into a graph, now or before: the host does not know what the
-        // device holds when this runs (the checks' kernels, at most six, end at
-        // once beside the vertex phase)
-        if (!timed) s->flood_recorded = true;
+        const int tag = spm::flood_kept_tag(ds);
+        if (!timed) s->flood_recorded |= 1u << tag;
         cudaStreamWaitEvent(s->side, s->fork, 0);
+        // recorded, the host does not know what the device holds when this runs;
+        // the kernels that check and need not build (at most six) end at once,
+        // beside the vertex phase (a graph of the 256^2 rectangles 36.9 -> 38.6
+        // us, of the 4096^2 maze 321 -> 324, of the polygons unchanged)
         spm::launch_flood(ds, s->side,
-                          !ds.static_tile_start ? spm::FloodStatic::kNone
-                          : s->flood_recorded   ? spm::FloodStatic::kEnsure
-                          : reuse               ? spm::FloodStatic::kReuse
-                                                : spm::FloodStatic::kBuild);
+                          !ds.static_tile_start             ? spm::FloodStatic::kNone
+                          : timed && flood_kept_sure(s, ds) ? spm::FloodStatic::kReuse
+                          : timed && !s->flood_recorded     ? spm::FloodStatic::kBuild
+                                                            : spm::FloodStatic::kEnsure);
         cudaEventRecord(s->join, s->side);
-        s->flood_static_ok = ds.static_tile_start != nullptr && !s->flood_recorded;
-        s->flood_static_tile = ds.tile;
-        s->flood_static_maps = (int)maps;
+        if (timed) s->flood_kept = ds.static_tile_start ? tag : 0;
     }
     if (timed) cudaEventRecord(s->ev[1], cs);
     if (side) {
         cudaStreamWaitEvent(cs, s->join, 0);
     } else if (ds.use_flood) {
         spm::launch_flood(ds, cs);
-        s->flood_static_ok = false;  // the lists and maps now hold this flood's
-        if (!timed) s->flood_recorded = true;
+        if (ds.flood_mode != 2) {  // the lists and maps hold this flood's when it has run
+            if (timed) s->flood_kept = 0;
+            else s->flood_recorded |= 1u;
+        }
     } else {
         static const int32_t off[4] = {0, 0, 1, 0};
         cudaMemcpyAsync(ds.flood_counts, off, sizeof off, cudaMemcpyHostToDevice, cs);
@@ -959,15 +963,8 @@ void batch_free(spm_batch *b) {
 bool build_flood_static(spm_scene *s, const spm::DevScene &d) {
     spm::launch_flood(d, nullptr, spm::FloodStatic::kBuild);
     if (cudaStreamSynchronize(nullptr) != cudaSuccess) return false;
-    s->flood_static_ok = !s->flood_recorded;
-    s->flood_static_tile = d.tile;
-    s->flood_static_maps = d.use_maps && d.gen_maps ? 1 : 0;
+    s->flood_kept = spm::flood_kept_tag(d);
     return true;
-}
-
-bool flood_static_matches(const spm_scene *s, const spm::DevScene &d) {
-    return s->flood_static_ok && s->flood_static_tile == d.tile &&
-           s->flood_static_maps == (d.use_maps && d.gen_maps ? 1 : 0);
 }
 
 void batch_launch(spm_batch *b, cudaStream_t st, bool capturing) {
@@ -1027,7 +1024,7 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         // here if the scene has none for this tile size and map setting
         descs[k].flood_reuse = 0;
         if (descs[k].use_flood && descs[k].flood_mode == 3 && descs[k].static_tile_start) {
-            if (!flood_static_matches(scenes[k], descs[k]) && !build_flood_static(scenes[k], descs[k])) {
+            if (!flood_kept_sure(scenes[k], descs[k]) && !build_flood_static(scenes[k], descs[k])) {
                 delete b;
                 return set_err(nullptr, SPM_ERR_CUDA, "static flood build failed");
             }
@@ -1160,10 +1157,14 @@ spm_status spm_batch_compute(spm_batch *b, void *stream) {
     // scene's static lists since: rebuild them before the batch reads them
     // (where a graph may have, the device checks)
     for (size_t k = 0; k < b->scenes.size(); ++k)
-        if (b->descs[k].flood_reuse && !flood_static_matches(b->scenes[k], b->descs[k])) {
-            if (cap != cudaStreamCaptureStatusNone || b->scenes[k]->flood_recorded) {
+        if (b->descs[k].flood_reuse && !flood_kept_sure(b->scenes[k], b->descs[k])) {
+            const int tag = spm::flood_kept_tag(b->descs[k]);
+            if (cap != cudaStreamCaptureStatusNone) {
                 spm::launch_flood_kept(b->descs[k], st);
-                b->scenes[k]->flood_recorded = true;
+                b->scenes[k]->flood_recorded |= 1u << tag;
+            } else if (b->scenes[k]->flood_recorded) {
+                spm::launch_flood_kept(b->descs[k], st);
+                b->scenes[k]->flood_kept = tag;
             } else if (cudaStreamSynchronize(st) != cudaSuccess || !build_flood_static(b->scenes[k], b->descs[k])) {
                 return set_err(nullptr, SPM_ERR_CUDA, "static flood rebuild failed");
             }
@@ -1211,8 +1212,8 @@ spm_status spm_batch_compute(spm_batch *b, void *stream) {
         s->ev_valid = false;
         // the batched flood rewrote the lists of scenes that flood every generator
         if (!b->descs[k].flood_reuse && b->descs[k].use_flood && b->descs[k].flood_mode != 2) {
-            s->flood_static_ok = false;
-            if (cap != cudaStreamCaptureStatusNone) s->flood_recorded = true;
+            if (cap != cudaStreamCaptureStatusNone) s->flood_recorded |= 1u;
+            else s->flood_kept = 0;
         }
     }
     return SPM_OK;
@@ -1403,7 +1404,7 @@ spm_status spm_scene_info(spm_scene *s, int64_t *info) {
                            !(run.fix_launch & spm::kFixSolo);
     info[10] = 1 + (s->hs.n_vert > 0 ? (own_lists ? 1 : 4) : 0) + (s->ds.warm && s->ds.vtab ? 4 : 0) + (s->ds.fix_launch & spm::kFixSolo ? 1 : 0) +
                (s->ds.fix_launch & spm::kFixCluster ? 1 : 0) + many_cta + (floods ? (reuse ? src_cull : 3) : 0) +
-               (reuse && s->flood_recorded ? spm::flood_kept_kernels(run) : 0) + (spm::tiles_culled(run) ? 1 : 0) + 1;
+               (reuse && s->flood_recorded && !flood_kept_sure(s, run) ? spm::flood_kept_kernels(run) : 0) + (spm::tiles_culled(run) ? 1 : 0) + 1;
     return SPM_OK;
 }
 

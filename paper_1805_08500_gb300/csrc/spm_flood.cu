@@ -921,6 +921,8 @@ static int flood_kept(const DevScene &scene, cudaStream_t st, int unless) {
     return 1;
 }
 
+int flood_kept_tag(const DevScene &ds) { return kept_tag(ds); }
+
 int flood_kept_kernels(const DevScene &ds) {
     const int build = !flood_verts_direct(ds) ? 3 + (ds.n_vert > 0) : ds.vert_words <= kBitsOnly ? 2 : 5;
     return build + (flood_sources_direct(ds) ? 0 : 1);

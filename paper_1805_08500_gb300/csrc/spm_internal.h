@@ -286,6 +286,7 @@ void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_
 // compute does).
 enum class FloodStatic { kNone, kBuild, kReuse, kEnsure };
 constexpr int kKeptTag = 4, kFloodCounts = 5;
+int flood_kept_tag(const DevScene &ds);  // the tag of this descriptor's kept part: 4 to 7
 void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how = FloodStatic::kNone);
 void launch_flood_kept(const DevScene &ds, cudaStream_t st);  // kEnsure's static part alone
 int flood_kept_kernels(const DevScene &ds);  // kernels kEnsure launches beside kReuse's
