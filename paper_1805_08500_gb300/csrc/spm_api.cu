@@ -718,8 +718,8 @@ static spm_status compute_impl(spm_scene *s, void *stream, float *dist, int32_t 
         cudaStreamWaitEvent(s->side, s->fork, 0);
         // recorded, the host does not know what the device holds when this runs;
         // the kernels that check and need not build (at most six) end at once,
-        // beside the vertex phase (a graph of the 256^2 rectangles 36.9 -> 38.6
-        // us, of the 4096^2 maze 321 -> 324, of the polygons unchanged)
+        // beside the vertex phase (a graph of the 256^2 rectangles 36.9 -> 37.6
+        // us, of the 4096^2 maze 320 -> 323, of the 1024^2 polygons unchanged)
         spm::launch_flood(ds, s->side,
                           !ds.static_tile_start             ? spm::FloodStatic::kNone
                           : timed && flood_kept_sure(s, ds) ? spm::FloodStatic::kReuse

@@ -749,10 +749,13 @@ __global__ void k_flood_reset_b(const __grid_constant__ BatchDev b) {
             const bool on = ds.use_flood && ds.flood_mode != 2;
             // a kept part of another tuning (only a batch recorded in its
             // caller's graph meets one): the scene scans every generator
-            const bool kept = ds.flood_reuse && ds.flood_counts[kKeptTag] == kept_tag(ds);
+            // (all three loads at once)
+            const int tag = ds.flood_reuse ? ds.flood_counts[kKeptTag] : 0;
+            const int globals = ds.flood_reuse ? ds.static_counts[1] : 0, over = ds.flood_reuse ? ds.static_counts[2] : 0;
+            const bool kept = tag == kept_tag(ds);
             ds.flood_counts[0] = 0;
-            ds.flood_counts[1] = kept ? ds.static_counts[1] : 0;
-            ds.flood_counts[2] = kept ? ds.static_counts[2] : (on && !ds.flood_reuse ? 0 : 1);
+            ds.flood_counts[1] = kept ? globals : 0;
+            ds.flood_counts[2] = kept ? over : (on && !ds.flood_reuse ? 0 : 1);
             ds.flood_counts[3] = 0;
             if (on && !ds.flood_reuse) ds.flood_counts[kKeptTag] = 0;  // its flood overwrites the kept part
         }
