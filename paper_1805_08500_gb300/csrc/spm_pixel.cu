@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(kCullThreads) k_tile_cull_b(const __grid_const
     }
 }
 
-constexpr long long kFourWaves = 4 * 152 * 28;
+constexpr long long kFourWaves = 4 * 152 * 28;  // GB300: 152 SMs
 #ifndef SPM_BLK_MINB
 #define SPM_BLK_MINB 28  // warps per SM the kernels are compiled for
 #endif
@@ -953,9 +953,10 @@ void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int
     // A large grid's planes in the host's memory: blocks 32 wide, within a tile,
     // whose rows are whole 128-byte lines. The link takes 193 GB/s of those, as
     // of copies, but 172 of a 16 x 16 block's 64-byte rows, and such a map waits
-    // for it (16 x 16 or 16 x 8 / 32 x 4, wall clock of the whole call: maze
-    // 4096^2 934 / 845 us, differentiable 2048^2 328 / 303, maze 2048^2 318 /
-    // 314). Smaller grids wait for their slowest block (1024^2 polygons 194 / 205).
+    // for it (16 x 16 or 16 x 8 / 32 x 4, wall clock of spm_compute_host alone:
+    // maze 4096^2 934 / 845 us, differentiable 2048^2 328 / 303, maze 2048^2 318
+    // / 314; a host move of the sources before it is another 70 to 90). Smaller
+    // grids wait for their slowest block (1024^2 polygons 194 / 205).
     if (to_host && !scan && ds.tile == kTile && blocks * 4 > kFourWaves) {
         run(Shape<4, 1, 8>(), k_pixel_blocks<4, 1, 8, false>);
         return;
