@@ -1041,7 +1041,7 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
         const long long direct = descs[k].src_direct, ntl = (long long)d.tiles_x * d.tiles_y;
         src_map_off[k + 1] = src_map_off[k] + direct * d.n_src * spm::kAngBins;
         src_ins_off[k + 1] = src_ins_off[k] + direct * d.n_src * spm::src_edge_warps(d.n_edge);
-        src_tile_off[k + 1] = src_tile_off[k] + direct * ntl;
+        src_tile_off[k + 1] = src_tile_off[k] + direct * ntl * d.src_words;
         const bool floods = d.use_flood && d.flood_mode != 2;
         flood_off[k + 1] =
             flood_off[k] + (floods && !direct ? (d.flood_reuse ? d.n_src : d.n_gen) : 0);

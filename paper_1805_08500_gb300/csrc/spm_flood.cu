@@ -603,37 +603,36 @@ __device__ __forceinline__ void src_insert(const DevScene &ds, int g, int e0) {
     insert_edges_warp<MAPS>(ds, mp, mp + 1, ds.gen_lat[g], e0, 2, 64);
 }
 
-// Tile t's bits: a warp, its groups of kSrcGrp lanes a source each (most tiles
-// span few bins). Segment interiors and sources off the grid are candidates
-// of every tile.
+// Word w of tile t's bits: a warp, its groups of kSrcGrp lanes a source each
+// (most tiles span few bins). Segment interiors and sources off the grid are
+// candidates of every tile. (A warp that went through all of a tile's words took
+// 2.9 ms for 4000 sources on the 64 tiles of 256^2 rectangles.)
 constexpr int kSrcGrp = 8;
-__device__ __forceinline__ void src_tile(const DevScene &ds, int t) {
+__device__ __forceinline__ void src_tile(const DevScene &ds, int t, int w) {
     const int lane = threadIdx.x & 31, gl8 = lane % kSrcGrp, grp = lane / kSrcGrp;
     const unsigned gmask = ((1u << kSrcGrp) - 1u) << (grp * kSrcGrp);
     const int4 area = tile_area(ds, t % ds.tiles_x, t / ds.tiles_x);
-    for (int w = 0; w < ds.src_words; ++w) {
-        const int mine = 32 * w + lane;  // one load for the word's sources
-        const int2 lat = mine < ds.n_src ? ds.gen_lat[mine] : make_int2(0, 0);
-        const bool on = mine < ds.n_src && src_on_grid(ds, mine);
-        const bool inside = lat.x >= area.x && lat.x <= area.z && lat.y >= area.y && lat.y <= area.w;
-        const unsigned every = __ballot_sync(0xffffffffu, mine < ds.n_src && (inside || !on));
-        uint32_t bits = every;
-        const int n = min(32, ds.n_src - 32 * w);
+    const int mine = 32 * w + lane;  // one load for the word's sources
+    const int2 lat = mine < ds.n_src ? ds.gen_lat[mine] : make_int2(0, 0);
+    const bool on = mine < ds.n_src && src_on_grid(ds, mine);
+    const bool inside = lat.x >= area.x && lat.x <= area.z && lat.y >= area.y && lat.y <= area.w;
+    const unsigned every = __ballot_sync(0xffffffffu, mine < ds.n_src && (inside || !on));
+    uint32_t bits = every;
+    const int n = min(32, ds.n_src - 32 * w);
 #pragma unroll 2
-        for (int j0 = 0; j0 < n; j0 += 32 / kSrcGrp) {
-            const int j = j0 + grp;
-            const int2 gl = make_int2(__shfl_sync(0xffffffffu, lat.x, j & 31), __shfl_sync(0xffffffffu, lat.y, j & 31));
-            bool seen = false;
-            if (j < n && !(every >> j & 1u))
-                seen = !box_hidden_ang<kSrcGrp>(reinterpret_cast<const float *>(ds.gen_maps + (size_t)(32 * w + j) * kAng),
-                                                gl, area, gl8, gmask, 2);
-            const unsigned bal = __ballot_sync(0xffffffffu, seen && gl8 == 0);
+    for (int j0 = 0; j0 < n; j0 += 32 / kSrcGrp) {
+        const int j = j0 + grp;
+        const int2 gl = make_int2(__shfl_sync(0xffffffffu, lat.x, j & 31), __shfl_sync(0xffffffffu, lat.y, j & 31));
+        bool seen = false;
+        if (j < n && !(every >> j & 1u))
+            seen = !box_hidden_ang<kSrcGrp>(reinterpret_cast<const float *>(ds.gen_maps + (size_t)(32 * w + j) * kAng),
+                                            gl, area, gl8, gmask, 2);
+        const unsigned bal = __ballot_sync(0xffffffffu, seen && gl8 == 0);
 #pragma unroll
-            for (int q = 0; q < 32 / kSrcGrp; ++q)
-                if (bal >> (q * kSrcGrp) & 1u) bits |= 1u << (j0 + q);
-        }
-        if (lane == 0) ds.src_mask[(size_t)t * ds.src_words + w] = bits;
+        for (int q = 0; q < 32 / kSrcGrp; ++q)
+            if (bal >> (q * kSrcGrp) & 1u) bits |= 1u << (j0 + q);
     }
+    if (lane == 0) ds.src_mask[(size_t)t * ds.src_words + w] = bits;
 }
 
 __global__ void k_src_prep(const __grid_constant__ DevScene ds, int keep, int unless) {
@@ -648,7 +647,7 @@ __global__ void k_src_insert(const __grid_constant__ DevScene ds) {  // grid: (e
 
 __global__ void k_src_tiles(const __grid_constant__ DevScene ds) {
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (t < ds.tiles_x * ds.tiles_y) src_tile(ds, t);  // whole warps
+    if (t < ds.tiles_x * ds.tiles_y) src_tile(ds, t, blockIdx.y);  // whole warps
 }
 
 // Automatic mode: flood only sparse visibility graphs (mazes); a dense one
@@ -782,7 +781,9 @@ __global__ void k_src_tiles_b(const __grid_constant__ BatchDev b) {
     for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; w < n;
          w += (gridDim.x * (long long)blockDim.x) >> 5) {
         const int sc = scene_of_b(b.src_tile_off, b.n, w);
-        src_tile(b.scenes[sc], (int)(w - b.src_tile_off[sc]));
+        const DevScene &ds = b.scenes[sc];
+        const long long i = w - b.src_tile_off[sc];
+        src_tile(ds, (int)(i / ds.src_words), (int)(i % ds.src_words));
     }
 }
 
@@ -959,7 +960,7 @@ void launch_flood(const DevScene &ds, cudaStream_t st, FloodStatic how) {
             const dim3 grid((ds.n_edge + 4 * kSrcEdges - 1) / (4 * kSrcEdges), std::min(ds.n_src, 65535));
             if (ds.n_edge > 0 && maps) k_src_insert<true><<<grid, 128, 0, st>>>(ds);
             else if (ds.n_edge > 0) k_src_insert<false><<<grid, 128, 0, st>>>(ds);
-            k_src_tiles<<<(ntiles + 7) / 8, 256, 0, st>>>(ds);
+            k_src_tiles<<<dim3((ntiles + 7) / 8, ds.src_words), 256, 0, st>>>(ds);
             return;
         }
         if (keep) k_flood_static<<<1, 32, 0, st>>>(ds, keep, unless);

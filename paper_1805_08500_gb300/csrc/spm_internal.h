@@ -250,7 +250,7 @@ struct BatchDev {
     // direct culling of the sources of scenes with src_direct (n + 1 prefixes):
     const long long *src_map_off;      // map entries: n_src * kAngBins
     const long long *src_ins_off;      // warp tasks of the map building: n_src * src_edge_warps(n_edge)
-    const long long *src_tile_off;     // warp tasks of the tile tests: tiles
+    const long long *src_tile_off;     // warp tasks of the tile tests: tiles * src_words
     int32_t walk_tasks;                // (scene, generator) walks of the batched flood
     int32_t any_cull;                  // some scene culls its lists per tile
     int32_t any_lists;                 // some scene sorts lists per compute (its sources are not culled directly)

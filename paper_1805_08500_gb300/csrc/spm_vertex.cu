@@ -272,47 +272,46 @@ __global__ void __launch_bounds__(kVisThreads) k_vis_pairs(const __grid_constant
     if (qn > 0) walk(qn);
 }
 
-// The source columns of kRowsCta rows, by one CTA: a warp a row picks the
-// sources whose pair passes the filter (a lane each), then the CTA's warps take
-// the pairs one by one. A compute has few such pairs (1871 on the 1024^2
-// polygons, two a row) and its vertex phase waits for the longest of them.
+// One word of the source columns (32 sources) of kRowsCta rows, by one CTA: a
+// warp a row picks the sources whose pair passes the filter (a lane each), then
+// the CTA's warps take the pairs one by one. A compute has few such pairs (1871
+// on the 1024^2 polygons, two a row) and its vertex phase waits for the longest
+// of them. (A CTA that went through its rows' words one after another took
+// 1.6 ms for 4000 sources around eight rectangles, whose 32 rows are 8 CTAs.)
 constexpr int kRowsCta = 4;
 struct SrcPairs {
     int2 e[kRowsCta * 32];  // (row, source)
     int n;
 };
 template <class Row>
-__device__ __forceinline__ void src_pairs(SrcPairs &q, int words, Row row) {
+__device__ __forceinline__ void src_pairs(SrcPairs &q, int w, Row row) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int w = 0; w < words; ++w) {
-        if (threadIdx.x == 0) q.n = 0;
-        __syncthreads();
-        int vv;
-        if (const DevScene *ds = warp < kRowsCta ? row(warp, vv) : nullptr) {
-            const int u = 32 * w + lane, v = ds->n_src + vv;
-            bool c = u < ds->n_src && pair_filter(*ds, u, v);
-            if (c && ds->vert_maps && ds->gen_kind[u] != kSegI) c = !loc_hidden(*ds, v, ds->gen_lat[v], ds->gen_lat[u]);
-            if (c) q.e[atomicAdd(&q.n, 1)] = make_int2(warp, u);
+    if (threadIdx.x == 0) q.n = 0;
+    __syncthreads();
+    int vv;
+    if (const DevScene *ds = warp < kRowsCta ? row(warp, vv) : nullptr) {
+        const int u = 32 * w + lane, v = ds->n_src + vv;
+        bool c = u < ds->n_src && pair_filter(*ds, u, v);
+        if (c && ds->vert_maps && ds->gen_kind[u] != kSegI) c = !loc_hidden(*ds, v, ds->gen_lat[v], ds->gen_lat[u]);
+        if (c) q.e[atomicAdd(&q.n, 1)] = make_int2(warp, u);
+    }
+    __syncthreads();
+    for (int i = warp; i < q.n; i += kVisThreads / 32) {
+        const int2 pr = q.e[i];
+        const DevScene *ds = row(pr.x, vv);
+        const bool vis = pair_visible_warp(*ds, pr.y, ds->n_src + vv);
+        if (lane == 0 && vis) atomicOr(&ds->vis_bits[(size_t)vv * ds->vis_words + (pr.y >> 5)], 1u << (pr.y & 31));
+        if (lane == 0) {
+            SPM_CNT(13, 1);
+            SPM_CNT(14, vis);
         }
-        __syncthreads();
-        for (int i = warp; i < q.n; i += kVisThreads / 32) {
-            const int2 pr = q.e[i];
-            const DevScene *ds = row(pr.x, vv);
-            const bool vis = pair_visible_warp(*ds, pr.y, ds->n_src + vv);
-            if (lane == 0 && vis) atomicOr(&ds->vis_bits[(size_t)vv * ds->vis_words + (pr.y >> 5)], 1u << (pr.y & 31));
-            if (lane == 0) {
-                SPM_CNT(13, 1);
-                SPM_CNT(14, vis);
-            }
-        }
-        __syncthreads();  // the list is rewritten for the next word
     }
 }
 
-__global__ void __launch_bounds__(kVisThreads) k_src_pairs(const __grid_constant__ DevScene ds) {
+__global__ void __launch_bounds__(kVisThreads) k_src_pairs(const __grid_constant__ DevScene ds) {  // grid: (rows, words)
     __shared__ SrcPairs q;
     chain_start();
-    src_pairs(q, (ds.n_src + 31) / 32, [&](int r, int &vv) -> const DevScene * {
+    src_pairs(q, blockIdx.y, [&](int r, int &vv) -> const DevScene * {
         vv = blockIdx.x * kRowsCta + r;
         return vv < ds.n_vert ? &ds : nullptr;
     });
@@ -1387,14 +1386,18 @@ __global__ void k_prepare_b(const __grid_constant__ BatchDev b) {
 
 __global__ void __launch_bounds__(kVisThreads) k_vis_pairs_b(const __grid_constant__ BatchDev b) {
     __shared__ SrcPairs q;
-    for (int i0 = blockIdx.x * kRowsCta; i0 < b.vert_off[b.n]; i0 += gridDim.x * kRowsCta)
-        src_pairs(q, b.max_src_words, [&](int r, int &vv) -> const DevScene * {
+    const int rows = b.vert_off[b.n], groups = (rows + kRowsCta - 1) / kRowsCta;
+    for (long long t = blockIdx.x; t < (long long)groups * b.max_src_words; t += gridDim.x) {
+        const int i0 = (int)(t % groups) * kRowsCta;
+        src_pairs(q, (int)(t / groups), [&](int r, int &vv) -> const DevScene * {
             const int i = i0 + r;
-            if (i >= b.vert_off[b.n]) return nullptr;
+            if (i >= rows) return nullptr;
             const int s = scene_of(b.vert_off, b.n, i);
             vv = i - b.vert_off[s];
             return b.scenes + s;
         });
+        __syncthreads();  // the list is rewritten for the next task
+    }
 }
 
 __global__ void k_edges_count_b(const __grid_constant__ BatchDev b) {
@@ -2151,7 +2154,8 @@ void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *
             cudaMemcpyAsync(ds.vis_bits, ds.vis_static, sizeof(uint32_t) * (size_t)ds.n_vert * ds.vis_words,
                             cudaMemcpyDeviceToDevice, st);
         const int eb = (ds.n_vert + 7) / 8;  // one warp per row
-        launch_chained(k_src_pairs, dim3((ds.n_vert + kRowsCta - 1) / kRowsCta), dim3(kVisThreads), 0, st, ds);
+        launch_chained(k_src_pairs, dim3((ds.n_vert + kRowsCta - 1) / kRowsCta, (ds.n_src + 31) / 32),
+                       dim3(kVisThreads), 0, st, ds);
         if (lists) {
         } else if (warm && side) {
             // the tree's estimates, parents and fold read the source columns
