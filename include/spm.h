@@ -327,7 +327,8 @@ spm_status spm_scene_phase_ms(spm_scene *scene, float *vertex_ms, float *cull_ms
 
 /* Tuning of the pixel pass's culling, per scene.
  * flood_mode: 0 = automatic: mode 3 with depth maps (below) where the scene
- *   has room for the maps; otherwise the per-tile candidate lists are flooded
+ *   has room for the maps (and, in mazes, at most two (source, obstacle edge)
+ *   pairs a pixel); otherwise the per-tile candidate lists are flooded
  *   when the visibility graph among generators is sparse (below 1% of all
  *   pairs, as in mazes) and every tile scans every generator when it is not,
  *   decided on the device each compute. 1 = always flood, 2 = never flood,

@@ -216,10 +216,15 @@ void set_tile(spm::DevScene &ds, int tile) {
 // obstacle vertices are kept, and a compute culls its sources beside the vertex
 // phase. (Scanning every generator, what it took on dense scenes before:
 // 512^2 polygons 147 us of pixel pass against 34.) Scenes without maps keep the
-// device's choice of flood or scan.
+// device's choice of flood or scan, and so do mazes of so many sources that
+// entering every edge into their maps outweighs what the pixels save, two
+// (source, edge) pairs a pixel (maze 1024^2, 273 walls, maps / device's choice:
+// 1000 sources 353 / 464 us, 2000 620 / 480, 6000 1646 / 883); in open scenes the
+// vertex phase hides it (1024^2 polygons 1000 436 / 627, 6000 2488 / 5087).
 spm::DevScene effective(const spm_scene *s) {
     spm::DevScene d = s->ds;
-    if (d.flood_mode == 0 && d.use_flood && d.gen_maps && d.static_tile_start && spm::flood_sources_direct(d)) {
+    const bool few = d.open_scene || (double)d.n_src * d.n_edge <= 2.0 * d.Nx * d.Ny;
+    if (d.flood_mode == 0 && d.use_flood && d.gen_maps && d.static_tile_start && few && spm::flood_sources_direct(d)) {
         d.flood_mode = 3;
         d.use_maps = 1;
     }

@@ -1610,3 +1610,23 @@ def test_scan_of_many_sources(spm, oracle_mod):
         gd, gp = (v.cpu().numpy()[ij[:, 1], ij[:, 0]] for v in (d, p))
         check_parity(scene, gd, gp, od, op, od2, f"scan, {n} sources", op2)
     assert max(pixel_ms[1:]) <= 1.1 * pixel_ms[0], pixel_ms
+
+
+def test_automatic_culling_of_many_sources_in_a_maze(spm):
+    """The automatic choice in a maze, with few sources (maps) and many (the
+    device's choice), costs no more than the better of maps and scan by a margin,
+    and gives the scan's map."""
+    base = sg.maze(0, cells=16, N=1024)
+    base = sg.Scene(base.world, base.grid, base.polys, base.points, np.zeros((0, 4)))
+    for n in (300, 6000):
+        s = spm.Scene(_with_sources(base, n))
+        us, out = {}, {}
+        for mode, maps in ((0, 0), (3, 1), (2, 0)):
+            spm.spm_scene_set_tuning(s.handle, mode, 32, 32, maps)
+            out[mode] = s.empty_outputs()
+            us[mode] = _median_us(lambda: s.compute(*out[mode]))
+            s.sync()
+        assert us[0] <= 1.3 * min(us[3], us[2]), (n, us)
+        for mode in (0, 3):
+            assert torch.equal(out[mode][1], out[2][1]), (n, mode)
+            assert torch.equal(out[mode][0].view(torch.int32), out[2][0].view(torch.int32)), (n, mode)
