@@ -1005,7 +1005,14 @@ void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int
     // 113 / 124. Halving a 16 x 16 block costs the least work, and pays up to six
     // waves (four / six: 1560^2 polygons 120 / 113, 1700^2 150 / 138, maze 1536^2
     // 68 / 64).
-    const bool scan = !ds.use_flood || ds.flood_mode == 2 || ds.flood_mode == 0;  // (or may, decided on the device)
+    // Every generator may be scanned: no flood, or the device decides, or lists
+    // that may outgrow their buffer, as an open scene's do (200 polygons, 2000
+    // sources, 4096^2, mode 1: 8.4 ms in the kernel for lists alone, 1.6 in the
+    // other, which takes 0 to 5 % longer where there are lists).
+    const long long pairs = (long long)(ds.flood_mode == 3 && ds.static_lists
+                                            ? std::max(ds.vert_bits ? 0 : ds.n_vert, ds.src_direct ? 0 : ds.n_src)
+                                            : ds.n_gen) * ds.tiles_x * ds.tiles_y;
+    const bool scan = !ds.use_flood || ds.flood_mode == 2 || ds.flood_mode == 0 || (ds.open_scene && pairs > ds.pair_cap);
     auto pick = [&](auto shape, auto lists, auto scans) {
         if (scan) run(shape, scans);
         else run(shape, lists);
