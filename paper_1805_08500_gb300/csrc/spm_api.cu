@@ -1117,6 +1117,11 @@ spm_status spm_batch_create(spm_scene *const *scenes, int32_t n, float *const *d
     for (int k = 0; k < n; ++k) bd.max_src_words = std::max(bd.max_src_words, (descs[k].n_src + 31) / 32);
     bd.any_cull = 0;
     for (int k = 0; k < n; ++k) bd.any_cull |= spm::tiles_culled(descs[k]);
+    // The scan's own tests pay in a batch where a scene has many sources (scans
+    // of eight 512^2 scenes with 100 sources 707 -> 289 us of pixel pass; with a
+    // few, sixteen such scenes 352 -> 788)
+    bd.any_scan = 0;
+    for (int k = 0; k < n; ++k) bd.any_scan |= descs[k].n_src > 32 && spm::pixels_may_scan(descs[k]);
     for (int k = 0; k < n; ++k)
         bd.any_lists |= descs[k].use_flood && descs[k].flood_mode != 2 && !descs[k].src_direct;
     for (int k = 0; k < n; ++k) bd.any_maps |= descs[k].use_flood && descs[k].flood_mode != 2 && descs[k].use_maps;

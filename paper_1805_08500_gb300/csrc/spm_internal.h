@@ -253,6 +253,7 @@ struct BatchDev {
     const long long *src_tile_off;     // warp tasks of the tile tests: tiles * src_words
     int32_t walk_tasks;                // (scene, generator) walks of the batched flood
     int32_t any_cull;                  // some scene culls its lists per tile
+    int32_t any_scan;                  // some scene of many sources may scan every generator
     int32_t any_lists;                 // some scene sorts lists per compute (its sources are not culled directly)
     // vertex fixpoint on resident clusters, one scene at a time
     const int32_t *cl_order;           // n scene indices, most generators first
@@ -274,6 +275,7 @@ void launch_vertex_phase(const DevScene &ds, cudaStream_t st, const VertexSide *
 // entries a tile's culled list may hold
 constexpr int cull_cap(int tile) { return tile == kTile ? 512 : 256; }
 bool tiles_culled(const DevScene &ds);  // the pixel pass culls its lists per tile first
+bool pixels_may_scan(const DevScene &ds);  // its blocks may take every generator
 // pixel kernel over the grid rows [row0, row1); row0 a multiple of the small
 // tile's side; to_host: the planes lie in page-locked host memory
 void launch_pixel_phase(const DevScene &ds, cudaStream_t st, float *dist, int32_t *parent, int row0, int row1,

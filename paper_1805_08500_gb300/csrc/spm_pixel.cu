@@ -805,6 +805,7 @@ __global__ void __launch_bounds__(32, SPM_BLK_MINB) k_pixel_blocks(const __grid_
 // 16 x 8 1220, 8 x 8 1306). 24 warps an SM (1206 us; 28: 1220, 32: 1293, more
 // of them contend for L1), four a CTA (one to sixteen: within 2 %).
 constexpr int kBatchWarps = 4, kBatchSm = 24;
+template <bool SCAN>  // some scene of many sources may scan
 __global__ void __launch_bounds__(32 * kBatchWarps, kBatchSm / kBatchWarps) k_pixel_blocks_b(const __grid_constant__ BatchDev b) {
     using S = Shape<4, 1>;
     static_assert(S::kW == kBatchBlkW && S::kH == kBatchBlkH, "the batch counts these blocks");
@@ -833,7 +834,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, kBatchSm / kBatchWarps) k_pi
             held = sc;
         }
         const int across = (ds.Nx + S::kW - 1) / S::kW;
-        pixel_block<4, 1, 4, false>(ds, blk % across * S::kW, blk / across * S::kH, b.dist[sc], b.parent[sc], sm[warp]);
+        pixel_block<4, 1, 4, SCAN>(ds, blk % across * S::kW, blk / across * S::kH, b.dist[sc], b.parent[sc], sm[warp]);
         __syncwarp();
     }
 }
@@ -977,6 +978,17 @@ void launch_free_mask(const DevScene &ds, cudaStream_t st, uint32_t *bits) {
     k_free_mask<<<(unsigned)((words + per_block - 1) / per_block), NT, 0, st>>>(ds, bits);
 }
 
+// Every generator may be scanned: no flood, or the device decides, or lists
+// that may outgrow their buffer, as an open scene's do (200 polygons, 2000
+// sources, 4096^2, mode 1: 8.4 ms in the kernel for lists alone, 1.6 in the
+// other, which takes 0 to 5 % longer where there are lists).
+bool pixels_may_scan(const DevScene &ds) {
+    const long long pairs = (long long)(ds.flood_mode == 3 && ds.static_lists
+                                            ? std::max(ds.vert_bits ? 0 : ds.n_vert, ds.src_direct ? 0 : ds.n_src)
+                                            : ds.n_gen) * ds.tiles_x * ds.tiles_y;
+    return !ds.use_flood || ds.flood_mode == 2 || ds.flood_mode == 0 || (ds.open_scene && pairs > ds.pair_cap);
+}
+
 bool tiles_culled(const DevScene &ds) {
     return ds.cull_items && ds.use_flood && ds.flood_mode == 3 && flood_verts_direct(ds);
 }
@@ -1005,14 +1017,7 @@ void launch_pixel_phase(const DevScene &scene, cudaStream_t st, float *dist, int
     // 113 / 124. Halving a 16 x 16 block costs the least work, and pays up to six
     // waves (four / six: 1560^2 polygons 120 / 113, 1700^2 150 / 138, maze 1536^2
     // 68 / 64).
-    // Every generator may be scanned: no flood, or the device decides, or lists
-    // that may outgrow their buffer, as an open scene's do (200 polygons, 2000
-    // sources, 4096^2, mode 1: 8.4 ms in the kernel for lists alone, 1.6 in the
-    // other, which takes 0 to 5 % longer where there are lists).
-    const long long pairs = (long long)(ds.flood_mode == 3 && ds.static_lists
-                                            ? std::max(ds.vert_bits ? 0 : ds.n_vert, ds.src_direct ? 0 : ds.n_src)
-                                            : ds.n_gen) * ds.tiles_x * ds.tiles_y;
-    const bool scan = !ds.use_flood || ds.flood_mode == 2 || ds.flood_mode == 0 || (ds.open_scene && pairs > ds.pair_cap);
+    const bool scan = pixels_may_scan(ds);
     auto pick = [&](auto shape, auto lists, auto scans) {
         if (scan) run(shape, scans);
         else run(shape, lists);
@@ -1040,10 +1045,11 @@ void launch_pixel_phase_batched(const BatchDev &b, cudaStream_t st) {
     int per_sm = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pixel_blocks_b, 32 * kBatchWarps, 0);
+    const auto kern = b.any_scan ? k_pixel_blocks_b<true> : k_pixel_blocks_b<false>;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kBatchWarps, 0);
     const int grid = max(1, min((b.total_blocks + kBatchWarps - 1) / kBatchWarps, sms * max(per_sm, 1)));
     if (b.any_cull) k_tile_cull_b<<<std::min(b.total_tiles, sms * 16), kCullThreads, 0, st>>>(b);
-    k_pixel_blocks_b<<<grid, 32 * kBatchWarps, 0, st>>>(b);
+    kern<<<grid, 32 * kBatchWarps, 0, st>>>(b);
 }
 
 int count_kernel_launches_pixel() { return 1; }
