@@ -1673,3 +1673,25 @@ def test_batch_of_scans(spm, scans):
     for (d, p), (rd, rp) in zip(batch.outputs, want):
         assert torch.equal(p, rp) and torch.equal(d.view(torch.int32), rd.view(torch.int32))
     assert batch.phase_ms()[1] <= 5.5 * maps_ms
+
+
+@pytest.mark.parametrize("N", [1024, 2048])
+def test_blocks_of_crowded_scenes_without_maps(spm, oracle_mod, N):
+    """Obstacles 20 and 40 pixels apart, whose blocks without depth maps are
+    smaller than the grid alone would have them: flooded lists and a scan against
+    the lists with maps, bit for bit, and the oracle."""
+    scene = sg.tiny(0, W=16384, N=N, n_polys=2650, n_points=3, n_segs=1, r=(20.0, 70.0), k=(4, 8))
+    s = spm.Scene(scene)
+    spm.spm_scene_set_tuning(s.handle, 3, 32, 32, 1)
+    assert s.tuning()["maps"] == 1
+    rd, rp = s.compute()
+    s.sync()
+    for mode in (1, 2):
+        spm.spm_scene_set_tuning(s.handle, mode, 32, 32, 0)
+        d, p = s.compute()
+        s.sync()
+        assert torch.equal(p, rp) and torch.equal(d.view(torch.int32), rd.view(torch.int32)), mode
+    ij = np.random.default_rng(N).integers(0, N, (3000, 2)).astype(np.int32)
+    od, op, od2, op2 = oracle_mod.Oracle(scene).pixels(ij)
+    gd, gp = (v.cpu().numpy()[ij[:, 1], ij[:, 0]] for v in (rd, rp))
+    check_parity(scene, gd, gp, od, op, od2, f"crowded {N}", op2)
