@@ -222,31 +222,19 @@ __device__ __forceinline__ void edge_into_bin(const EdgeView &v, int k, float *u
     }
 }
 
-// One warp inserts polygon q's front-facing edges into the depth map, the
-// lanes spread over each edge's bins.
-template <bool MAPS>
-__device__ void insert_polygon_warp(const DevScene &ds, float *depth2, float *lo2, int2 g, int q, int lane) {
-    const int e0 = ds.poly_off[q], e1 = ds.poly_off[q + 1];
-    for (int e = e0; e < e1; ++e) {
-        EdgeView v;
-        if (!edge_view(g, __ldg(ds.edges + e), v)) continue;
-        for (int k = v.k0 + lane; k <= v.k1; k += 32) edge_into_bin<MAPS>(v, k, depth2, lo2, 1, true);
-    }
-}
-
-// Edges e0 .. e0 + kSrcEdges - 1 into the map of a generator at g, one warp: a
+// Edges e0 .. min(e0 + kSrcEdges, end) - 1 into the map of a generator at g, one warp: a
 // lane views an edge, then the bins they span are dealt to the lanes evenly (a
 // wall next to the generator spans hundreds, a far one two or three). With up
 // to check_most bins in all, they are read before they are written (far edges
 // lower few bins; the wide ones are near and lower most).
 constexpr int kSrcEdges = 16;
 template <bool MAPS>
-__device__ __forceinline__ void insert_edges_warp(const DevScene &ds, float *up, float *low, int2 g, int e0, int stride,
-                                                  int check_most) {
+__device__ __forceinline__ void insert_edges_warp(const DevScene &ds, float *up, float *low, int2 g, int e0, int end,
+                                                  int stride, int check_most) {
     const int lane = threadIdx.x & 31;
     EdgeView v = {};
     int span = 0;
-    if (lane < kSrcEdges && e0 + lane < ds.n_edge && edge_view(g, __ldg(ds.edges + e0 + lane), v))
+    if (lane < kSrcEdges && e0 + lane < end && edge_view(g, __ldg(ds.edges + e0 + lane), v))
         span = v.k1 - v.k0 + 1;
     int incl = span;
 #pragma unroll
@@ -278,6 +266,25 @@ __device__ __forceinline__ void insert_edges_warp(const DevScene &ds, float *up,
         o.sa = take(v.sa);
         const int k = r - __shfl_sync(0xffffffffu, incl - span - v.k0, own);
         if (r < total) edge_into_bin<MAPS>(o, k, up, low, stride, total <= check_most);
+    }
+}
+
+// One warp inserts polygon q's front-facing edges into the depth map: up to four
+// edges one after another, every lane with all of them, the bins spread over the
+// lanes; more are dealt (flood of the 3400 polygons, five edges each on average,
+// 3150 us one after another, 2420 dealt; of the 160 x 160 maze 756 and 815).
+template <bool MAPS>
+__device__ void insert_polygon_warp(const DevScene &ds, float *depth2, float *lo2, int2 g, int q, int lane) {
+    const int e0 = ds.poly_off[q], e1 = ds.poly_off[q + 1];
+    static_assert(kMaxPolyVerts <= kSrcEdges, "a warp takes a polygon's edges at once");
+    if (e1 - e0 > 4) {
+        insert_edges_warp<MAPS>(ds, depth2, lo2, g, e0, e1, 1, 1 << 30);
+        return;
+    }
+    for (int e = e0; e < e1; ++e) {
+        EdgeView v;
+        if (!edge_view(g, __ldg(ds.edges + e), v)) continue;
+        for (int k = v.k0 + lane; k <= v.k1; k += 32) edge_into_bin<MAPS>(v, k, depth2, lo2, 1, true);
     }
 }
 
@@ -484,7 +491,7 @@ __device__ void flood_direct(const DevScene &ds, float *up, float *low, int g) {
     for (int k = tid; k < kAng; k += kFloodThreads) up[k] = low[k] = INFINITY;
     __syncthreads();
     for (int e = warp * kSrcEdges; e < ds.n_edge; e += kFloodThreads / 32 * kSrcEdges)
-        insert_edges_warp<MAPS>(ds, up, low, gl, e, 1, 1 << 30);
+        insert_edges_warp<MAPS>(ds, up, low, gl, e, ds.n_edge, 1, 1 << 30);
     __syncthreads();
     const unsigned gmask = 0xffu << (lane & 24);
     for (int t0 = warp * 4; t0 < ntiles; t0 += kFloodThreads / 32 * 4) {
@@ -600,7 +607,7 @@ template <bool MAPS>
 __device__ __forceinline__ void src_insert(const DevScene &ds, int g, int e0) {
     if (!src_on_grid(ds, g)) return;  // the same for the whole warp
     float *mp = reinterpret_cast<float *>(ds.gen_maps + (size_t)g * kAng);
-    insert_edges_warp<MAPS>(ds, mp, mp + 1, ds.gen_lat[g], e0, 2, 64);
+    insert_edges_warp<MAPS>(ds, mp, mp + 1, ds.gen_lat[g], e0, ds.n_edge, 2, 64);
 }
 
 // Word w of tile t's bits: a warp, its groups of kSrcGrp lanes a source each
